@@ -810,13 +810,13 @@ static sph_status create_impl(sph_handle* h, const sph_domain* dom, const sph_fi
   h->cells_cap = S.total_cells;
   SPH_TRY(grab(h, S.cstart, (size_t)S.total_cells + 1));
   SPH_TRY(grab(h, S.scan_part, (size_t)S.total_cells / 4096 + 2));
-  SPH_TRY(grab(h, S.partials, N / 128 + 2));
+  SPH_TRY(grab(h, S.partials, partial_slots(N, 128)));
   SPH_TRY(grab(h, S.scal, 2));
   SPH_TRY(grab(h, S.ctl, 1));
-  SPH_TRY(grab(h, S.tickets, 4));
+  SPH_TRY(grab(h, S.tickets, ticket_slots(N, 128)));
   SPH_TRY(grab(h, S.err, 1));
   SPH_CUDA(h, cudaMemsetAsync(S.cnt, 0, sizeof(uint32_t) * S.total_cells, h->stream));
-  SPH_CUDA(h, cudaMemsetAsync(S.tickets, 0, sizeof(unsigned) * 4, h->stream));
+  SPH_CUDA(h, cudaMemsetAsync(S.tickets, 0, sizeof(unsigned) * ticket_slots(N, 128), h->stream));
   SPH_CUDA(h, cudaMemsetAsync(S.err, 0, sizeof(int), h->stream));
   SPH_CUDA(h, cudaMemsetAsync(S.scal, 0, sizeof(Scalars) * 2, h->stream));
   SPH_CUDA(h, cudaMemsetAsync(S.lcount, 0, sizeof(uint32_t) * N, h->stream));

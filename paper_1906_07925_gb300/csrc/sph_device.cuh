@@ -100,13 +100,26 @@ struct Phys {
   T alpha;  // dimensionless Wendland constant: 7/pi (2D), 21/(2 pi) (3D)
 };
 
-// Per-block partials of the pass-A reductions (FP64), reduced in fixed order.
+// Per-block partials of the pass-A reductions, merged in fixed order, first
+// over groups of kPartialGroup consecutive blocks, then over the groups. The
+// FP64 path fills min_rc_a and err_max with values; the FP32 path names the
+// particles they belong to (r_c and |a|, rho and rho_t: exact FP32 values) and
+// divides once, at the end.
+constexpr int kPartialGroup = 128;
 struct Partial {
   double min_rc_a, max_a, sum_rho, err_l2, err_max;
   long long ipairs, fpairs;
   long long lentries;  // neighbour-list entries scanned
   long long amin;      // index (current order) of min_rc_a; -1: none
+  float rc, an;        // FP32 path: r_c and |a| of particle amin
+  float er, et;        // FP32 path: rho and rho_t where |rho / rho_t - 1| is largest (et = 0: none)
 };
+// partials of the blocks and of their groups for n particles at >= `threads` per block
+constexpr size_t partial_slots(size_t n, int threads) {
+  const size_t nb = n / threads + 2;
+  return nb + nb / kPartialGroup + 2;
+}
+constexpr size_t ticket_slots(size_t n, int threads) { return 4 + (n / threads + 2) / kPartialGroup + 2; }
 
 // Step scalars written by the last block of pass A, read by pass B.
 struct Scalars {

@@ -21,6 +21,8 @@ constexpr size_t kCap = 96;  // list entries per particle (exact neighbour sets,
 
 constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
+constexpr size_t kPartialSlots = partial_slots(kN, 128), kTicketSlots = ticket_slots(kN, 128);
+
 // segment offsets (bytes) inside the scratch array
 constexpr size_t kX0 = 0;
 constexpr size_t kX1 = kX0 + al(32 * kN);
@@ -44,10 +46,10 @@ constexpr size_t kCnt = kPc + al(4 * kN);
 constexpr size_t kCstart = kCnt + al(4 * kC);
 constexpr size_t kScanPart = kCstart + al(4 * (kC + 1));
 constexpr size_t kPartials = kScanPart + al(4 * (kC / 4096 + 2));
-constexpr size_t kScal = kPartials + al(sizeof(Partial) * (kN / 128 + 2));
+constexpr size_t kScal = kPartials + al(sizeof(Partial) * kPartialSlots);
 constexpr size_t kCtl = kScal + al(2 * sizeof(Scalars));
 constexpr size_t kTickets = kCtl + al(sizeof(StepCtl));
-constexpr size_t kErr = kTickets + al(16);
+constexpr size_t kErr = kTickets + al(4 * kTicketSlots);
 constexpr size_t kBytes = kErr + al(16);
 
 // The scratch array. Host code must not use its name as an address: the
@@ -206,7 +208,7 @@ extern "C" sph_status sph_eval_forces_noalloc(const sph_domain* dom, const sph_f
     }                                                                                      \
   } while (0)
   NA_CUDA(cudaMemsetAsync(Sd.cnt, 0, sizeof(uint32_t) * cells, st));
-  NA_CUDA(cudaMemsetAsync(Sd.tickets, 0, 16, st));
+  NA_CUDA(cudaMemsetAsync(Sd.tickets, 0, 4 * kTicketSlots, st));
   NA_CUDA(cudaMemsetAsync(Sd.err, 0, sizeof(int), st));
   NA_CUDA(cudaMemsetAsync(Sd.scal, 0, sizeof(Scalars), st));
   NA_CUDA(cudaMemcpyAsync(Sd.ctl, &ctl, sizeof ctl, cudaMemcpyHostToDevice, st));
