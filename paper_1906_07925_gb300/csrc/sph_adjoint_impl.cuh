@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n,
                                                   const typename ViewOf<T>::type* __restrict__ v0,
                                                   const typename ViewOf<T>::type* __restrict__ v1,
                                                   const uint32_t* __restrict__ plist,
-                                                  const uint32_t* __restrict__ pcount,
+                                                  const uint32_t* __restrict__ pcount, int cap,
                                                   const V4<T>* __restrict__ acc, const Scalars* __restrict__ scal,
                                                   Frame<T> F, Phys<T> P, int recomputed_dt, AdjBufs<T> B) {
   using VT = typename ViewOf<T>::type;
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n,
   if (i < n) {
     const VT* __restrict__ view = ctl->vp ? v1 : v0;
     const VT vi = view[i];
-    const T qv = F.qv, hv = view_h(vi), hi = hv * qv;
+    const T qv = F.qv, hv = view_h(F, vi), hi = hv * qv;
     const T half_kappa = T(0.5) * P.kappa;
     const T dt1 = (T)scal->dt1, dt2 = (T)scal->dt2;
     const V4<T> ai = acc[i];
@@ -283,13 +283,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n,
     struct Rec {
       V4<T> a, atb;
     };
-    for_list_x(plist, view, n, i, cnt, [&](int j) { return Rec{acc[j], B.atb[j]}; },
+    for_pairs_x(plist, view, i, cnt, cap, [&](int j) { return Rec{acc[j], B.atb[j]}; },
                [&](uint32_t e, const VT& vj, const Rec& rj) {
       const int j = (int)(e >> 8);
-      const T dx = vd<false>(F, vi.x, vj.x), dy = vd<false>(F, vi.y, vj.y);
-      const T dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
+      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
       const T r2 = dx * dx + dy * dy + dz * dz;
-      const T hvj = view_h(vj);
+      const T hvj = view_h(F, vj);
       const T Hv = half_kappa * (hv + hvj);
       if (!(r2 < Hv * Hv) || j == i) return;
       const T irv = drsqrt<T>(r2);  // 1/r, view units
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n,
     const long long k = scal->argmin;
     if (k >= 0 && mb != 0.0) {
       const VT* __restrict__ view = ctl->vp ? v1 : v0;
-      const double h = (double)view_h(view[k]) * (double)F.qv;
+      const double h = (double)view_h(F, view[k]) * (double)F.qv;
       const V4<T> a = acc[k];
       const double ax = a.x, ay = a.y, az = a.z;
       const double an = sqrt(ax * ax + ay * ay + az * az);
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? SPH_BWD_FORCE_MIN_BLOCKS
                                                    const typename ViewOf<T>::type* __restrict__ v1,
                                                    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1,
                                                    const uint32_t* __restrict__ plist,
-                                                   const uint32_t* __restrict__ pcount,
+                                                   const uint32_t* __restrict__ pcount, int cap,
                                                    const T* __restrict__ rho, const T* __restrict__ pc,
                                                    const Scalars* __restrict__ scal, Frame<T> F, Phys<T> P,
                                                    const LL4* __restrict__ X0, const LL4* __restrict__ X1,
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? SPH_BWD_FORCE_MIN_BLOCKS
     const VT* __restrict__ view = ctl->vp ? v1 : v0;
     const VT vi = view[i];
     const uint32_t ci = (ctl->buf ? m1 : m0)[i] & 0xFFu;
-    const T qv = F.qv, hv = view_h(vi), hi = hv * qv;
+    const T qv = F.qv, hv = view_h(F, vi), hi = hv * qv;
     const T half_kappa = T(0.5) * P.kappa;
     const T sigma = (T)scal->sigma, P0 = P.P0;
     const T rti = rho_t_of_h<D, T>(hi, P.inv_tau), Ti = inv_rho_t2<D, T>(hi, P.inv_tau);
@@ -515,12 +515,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? SPH_BWD_FORCE_MIN_BLOCKS
     T xx = 0, xy = 0, xz = 0, hbar = 0, Tbar = 0, Qbar = 0;
     T sb = 0, pb = 0;
     const int cnt = (int)pcount[i];
-    for_list_x(plist, view, n, i, cnt, [&](int j) { return B.ab[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& abj) {
+    for_pairs_x(plist, view, i, cnt, cap, [&](int j) { return B.ab[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& abj) {
       const int j = (int)(e >> 8);
-      const T dx = vd<false>(F, vi.x, vj.x), dy = vd<false>(F, vi.y, vj.y);
-      const T dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
+      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
       const T r2 = dx * dx + dy * dy + dz * dz;
-      const T hvj = view_h(vj);
+      const T hvj = view_h(F, vj);
       const T Hv = half_kappa * (hv + hvj);
       if (!(r2 < Hv * Hv) || j == i) return;
       const T irv = drsqrt<T>(r2);  // 1/r, view units
@@ -624,21 +624,21 @@ __global__ void __launch_bounds__(256) k_bwd_local(int n, const StepCtl* __restr
     const VT* __restrict__ view = ctl->vp ? v1 : v0;
     const int buf = ctl->buf;
     const VT vi = view[i];
-    const T qv = F.qv, hv = view_h(vi), hi = hv * qv;
+    const T qv = F.qv, hv = view_h(F, vi), hi = hv * qv;
     T hbar = B.hb[i];
     T xx = 0, xy = 0, xz = 0;
     if (DENS) {
       const T rbi = B.rhob[i];
       const T Hi = P.kappa * hi;
-      for_skin_list(list, view, n, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
+      for_skin_list(list, view, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
         const int j = (int)(e >> 8);
-        const T dx = vd<false>(F, vi.x, vj.x), dy = vd<false>(F, vi.y, vj.y);
-        const T dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
+        const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+        const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
         const T r = dsqrt(dx * dx + dy * dy + dz * dz) * qv;
         const KernelD<D, T> ki = wendland<D, T>(r, Hi, P.alpha);
         hbar += rbi * ki.WH * P.kappa;
         if (j == i || !(r > T(0))) return;
-        const T Hj = P.kappa * view_h(vj) * qv;
+        const T Hj = P.kappa * view_h(F, vj) * qv;
         const KernelD<D, T> kj = wendland<D, T>(r, Hj, P.alpha);
         const T c = (rbi * ki.Wr + B.rhob[j] * kj.Wr) / r;
         xx += c * dx * qv;
@@ -683,17 +683,17 @@ __global__ void __launch_bounds__(256) k_obj(int n, const StepCtl* __restrict__ 
     const int buf = ctl->buf;
     const VT vi = view[i];
     const uint32_t ci = (buf ? m1 : m0)[i] & 0xFFu;
-    const T qv = F.qv, hv = view_h(vi), hi = hv * qv;
+    const T qv = F.qv, hv = view_h(F, vi), hi = hv * qv;
     const T Hi = P.kappa * hi, half_kappa = T(0.5) * P.kappa;
     T rho = 0, xx = 0, xy = 0, xz = 0, hbar = 0, wi = 0;
-    for_skin_list(list, view, n, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
+    for_skin_list(list, view, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
       const int j = (int)(e >> 8);
-      const T dx = vd<false>(F, vi.x, vj.x), dy = vd<false>(F, vi.y, vj.y);
-      const T dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
+      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
       const T r2 = dx * dx + dy * dy + dz * dz;
       const T r = dsqrt(r2) * qv;
       rho += wendland<D, T>(r, Hi, P.alpha).W;
-      const T hvj = view_h(vj);
+      const T hvj = view_h(F, vj);
       const T Hv = half_kappa * (hv + hvj);
       if (j == i || (e & 0xFFu) == ci || !(r2 < Hv * Hv)) return;
       const KernelD<D, T> k = wendland<D, T>(r, Hv * qv, P.alpha);
@@ -764,13 +764,13 @@ cudaError_t launch_bwd_step(const DevState& S, const Frame<T>& F, const Phys<T>&
   const V4<T>* acc = (const V4<T>*)S.acc4;
   k_bwd_out<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, (const LL4*)S.X[0], (const LL4*)S.X[1], S.pid[0], S.pid[1], acc,
                                      (const V4<T>*)S.visc, S.scal, F, geo, B);
-  k_bwd_visc<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.plist, S.pcount, acc, S.scal, F, P, recomputed_dt, B);
+  k_bwd_visc<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.plist, S.pcount, S.cap, acc, S.scal, F, P, recomputed_dt, B);
   if (general_eos)
-    k_bwd_force<D, T, true><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], S.plist, S.pcount,
+    k_bwd_force<D, T, true><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], S.plist, S.pcount, S.cap,
                                                (const T*)S.rho, (const T*)S.pc, S.scal, F, P, (const LL4*)S.X[0],
                                                (const LL4*)S.X[1], S.pid[0], S.pid[1], geo, B);
   else  // the gamma = 2 form has no density adjoint: the target-field step is fused in
-    k_bwd_force<D, T, false><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], S.plist, S.pcount,
+    k_bwd_force<D, T, false><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], S.plist, S.pcount, S.cap,
                                                 (const T*)S.rho, (const T*)S.pc, S.scal, F, P, (const LL4*)S.X[0],
                                                 (const LL4*)S.X[1], S.pid[0], S.pid[1], geo, B);
   if (general_eos)

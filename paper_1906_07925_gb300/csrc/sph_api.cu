@@ -181,7 +181,7 @@ sph_status ensure_stage(sph_handle* h) {
   DevState& S = h->S;
   if (S.llist) return SPH_OK;
   const size_t N = (size_t)std::max<int64_t>(h->n, 1), nb = (N + kStageBlock - 1) / kStageBlock;
-  SPH_TRY(grab(h, S.llist, N * (size_t)S.cap));
+  SPH_TRY(grab(h, S.llist, list_words(N, S.cap)));
   SPH_TRY(grab(h, S.scount, nb));
   SPH_TRY(grab(h, S.sj, nb * (size_t)kStageCap));
   SPH_CUDA(h, cudaMemsetAsync(S.scount, 0xFF, sizeof(int) * nb, h->stream));
@@ -572,7 +572,7 @@ sph_status run_bwd_step(sph_handle* h, const DevState& S, const double* gin, dou
 // its control block and scalars, and with a general EOS its neighbour list.
 // Slots are allocated once (through the handle's allocator) and reused.
 sph_status ensure_tape(sph_handle* h, int slots) {
-  const size_t N = (size_t)h->n, cap = (size_t)h->S.cap;
+  const size_t N = (size_t)h->n;
   const size_t t1 = h->prec == SPH_PREC_FP64 ? 8 : 4, v4 = 4 * t1;
   const bool gen = h->par.gamma != 2.0;
   auto& tape = h->adj.tape;
@@ -583,7 +583,7 @@ sph_status ensure_tape(sph_handle* h, int slots) {
     SPH_TRY(grab(h, T.meta[0], N)); T.meta[1] = T.meta[0];
     SPH_TRY(grab(h, T.pid[0], N)); T.pid[1] = T.pid[0];
     SPH_TRY(grab(h, p, N * v4)); T.view[0] = T.view[1] = p;
-    SPH_TRY(grab(h, T.plist, N * cap));
+    SPH_TRY(grab(h, T.plist, pair_words(N, h->S.cap)));
     SPH_TRY(grab(h, T.pcount, N));
     SPH_TRY(grab(h, p, N * v4)); T.acc4 = p;
     SPH_TRY(grab(h, p, N * v4)); T.visc = p;
@@ -592,7 +592,7 @@ sph_status ensure_tape(sph_handle* h, int slots) {
     SPH_TRY(grab(h, T.ctl, 1));
     SPH_TRY(grab(h, T.scal, 1));
     if (gen) {
-      SPH_TRY(grab(h, T.list, N * cap));
+      SPH_TRY(grab(h, T.list, list_words(N, h->S.cap)));
       SPH_TRY(grab(h, T.lcount, N));
     }
     tape.push_back(T);
@@ -632,7 +632,7 @@ sph_status taped_step(sph_handle* h, const DevState& T, const double* dt_fix, do
   S2.pc = T.pc;
   SPH_TRY(launch_step(h, 1, 0, nullptr, dt_fix, dt_rec, &S2, &T));
   if (T.list != h->S.list) {
-    SPH_CUDA(h, cudaMemcpyAsync(T.list, h->S.list, (size_t)h->n * (size_t)h->S.cap * 4, cudaMemcpyDeviceToDevice,
+    SPH_CUDA(h, cudaMemcpyAsync(T.list, h->S.list, list_words((size_t)h->n, h->S.cap) * 4, cudaMemcpyDeviceToDevice,
                                 h->stream));
     SPH_CUDA(h, cudaMemcpyAsync(T.lcount, h->S.lcount, (size_t)h->n * 4, cudaMemcpyDeviceToDevice, h->stream));
   }
@@ -802,9 +802,9 @@ static sph_status create_impl(sph_handle* h, const sph_domain* dom, const sph_fi
   SPH_TRY(grab(h, tmpb, N * t1)); S.pc = tmpb;
   SPH_TRY(grab(h, S.key, N));
   SPH_TRY(grab(h, S.tmp, N));
-  SPH_TRY(grab(h, S.list, N * (size_t)S.cap));
+  SPH_TRY(grab(h, S.list, list_words(N, S.cap)));
   SPH_TRY(grab(h, S.lcount, N));
-  SPH_TRY(grab(h, S.plist, N * (size_t)S.cap));
+  SPH_TRY(grab(h, S.plist, pair_words(N, S.cap)));
   SPH_TRY(grab(h, S.pcount, N));
   SPH_TRY(grab(h, S.cnt, (size_t)S.total_cells));
   h->cells_cap = S.total_cells;

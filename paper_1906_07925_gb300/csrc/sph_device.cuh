@@ -79,6 +79,7 @@ struct Frame {
   int mbits;             // FP32: bits of 1.5 * 2^(23 - kCoarseBits); adding d encodes d 2^-kCoarseBits
   float mbias;           // FP32: 1.5 * 2^(23 - kCoarseBits)
   float vscale;          // FP32: 2^-kViewBits, one view integer in view units
+  float c2w, h2w, w2c;   // FP32: w = kappa h / 2 in view integers: from h in view units, from h, and back to view units
   T qv, inv_qv;          // physical length of one view unit (the finest cell edge c0)
   T q64t, inv_q64t;
   T lo[3];

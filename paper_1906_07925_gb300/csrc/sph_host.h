@@ -201,6 +201,10 @@ inline void make_frames(const sph_domain& dom, double kappa, double skin, const 
   out.f.mbits = bits;
   out.f.mbias = bias;
   out.f.vscale = (float)std::ldexp(1.0, -kViewBits);
+  const double c2w = 0.5 * kappa * std::ldexp(1.0, kViewBits);
+  out.f.c2w = (float)c2w;
+  out.f.h2w = (float)(c2w / c0);
+  out.f.w2c = (float)(1.0 / c2w);
   convert_grid<float>(hg, c0, out.gf);
   convert_grid<double>(hg, c0, out.gd);
 }

@@ -29,12 +29,12 @@ struct DevState {
   uint32_t* cstart = nullptr;            // exclusive prefix of cell counts, total+1 entries
   uint32_t* scan_part = nullptr;
   uint32_t total_cells = 0;
-  uint32_t* list = nullptr;              // cap x n entries (j << 8 | colour_j), column per particle
+  uint32_t* list = nullptr;              // skin lists, entries (j << 8 | colour_j), see list_at
   uint32_t* lcount = nullptr;            // entries per particle; bit 31: FP32 coarse test exact
-  uint32_t* plist = nullptr;             // cap x n: the force pairs of the current step (pass A -> B)
+  uint32_t* plist = nullptr;             // the force pairs of the current step (pass A -> B), see pair_at
   // staged pass A (FP32, 256-thread pair passes): per 256-target block its
   // distinct neighbours sj (kStageCap per block), their count scount (-1: not
-  // staged) and the list again with ranks in that set (llist, cap x n)
+  // staged) and the list again with ranks in that set (llist, as list)
   int stage = 0;
   uint32_t* llist = nullptr;
   int* scount = nullptr;
@@ -52,6 +52,24 @@ struct DevState {
   int* dbg_count = nullptr;        // 2n: density / force set sizes by particle id
   long long* dbg_sum = nullptr;    // 2n: sums of member ids
 };
+
+// Lists in tiles of one warp's 32 particles, so that everything a warp walks
+// lies together and consecutive steps are constant offsets (rows across all
+// particles put a warp's list words 4 n bytes apart, a page each).
+// The skin list: four consecutive entries of a particle side by side, the 32
+// particles' quads after one another: one 16-byte load per lane and quad, 512
+// contiguous bytes per warp.
+__host__ __device__ inline int list_rows(int cap) { return (cap + 3) & ~3; }
+__host__ __device__ inline size_t list_at(int i, int row, int cap) {
+  return ((size_t)(i >> 5) * (list_rows(cap) >> 2) + (row >> 2)) * 128 + (i & 31) * 4 + (row & 3);
+}
+inline size_t list_words(size_t n, int cap) { return (n + 31) / 32 * 32 * (size_t)list_rows(cap); }
+// The force pairs: row k holds the k-th pair of the 32 particles (the warp
+// writes them together, one pair of each lane at a time).
+__host__ __device__ inline size_t pair_at(int i, int k, int cap) {
+  return ((size_t)(i >> 5) * cap + k) * 32 + (i & 31);
+}
+inline size_t pair_words(size_t n, int cap) { return (n + 31) / 32 * 32 * (size_t)cap; }
 
 // per-step gate: flip the view buffer; start a list rebuild (flip the state
 // buffer) when pass B asked for one or `force` is set

@@ -15,9 +15,11 @@ using namespace sph;
 
 namespace {
 
-constexpr size_t kN = SPH_NOALLOC_MAX_PARTICLES;
+constexpr size_t kN = SPH_NOALLOC_MAX_PARTICLES;  // a multiple of 32, as kCap of 4: whole list tiles
 constexpr size_t kC = SPH_NOALLOC_MAX_CELLS;
 constexpr size_t kCap = 96;  // list entries per particle (exact neighbour sets, no skin)
+
+static_assert(kN % 32 == 0 && kCap % 4 == 0, "list tiles");
 
 constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 

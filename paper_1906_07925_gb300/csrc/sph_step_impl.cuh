@@ -27,7 +27,7 @@
 // resident 256-thread blocks per SM asked of the pair passes and of the list
 // build (caps registers)
 #ifndef SPH_PASS_MIN_BLOCKS
-#define SPH_PASS_MIN_BLOCKS 5
+#define SPH_PASS_MIN_BLOCKS 4
 #endif
 // store of a force-pair list word (streaming: read once, by pass B)
 #ifndef SPH_PLIST_STREAM
@@ -42,7 +42,7 @@
 // (DevState::pass_threads picks one at launch); resident blocks per SM asked
 // of them scale so that the register budget per thread is the same
 #ifndef SPH_PASSB_MIN_BLOCKS
-#define SPH_PASSB_MIN_BLOCKS SPH_PASS_MIN_BLOCKS
+#define SPH_PASSB_MIN_BLOCKS 5
 #endif
 #ifndef SPH_LIST_MIN_BLOCKS
 #define SPH_LIST_MIN_BLOCKS 4
@@ -65,25 +65,18 @@ template <> struct ViewOf<float> { using type = int4; };
 template <> struct ViewOf<double> { using type = V4<double>; };
 
 // Difference of two view coordinates, in view units (finest cell edges).
-// Precise (FAST = false): the exact integer difference, rounded once to float.
-// Coarse (FAST = true, the inside/outside test of a listed pair): the view
-// integers are dropped to 2^-kCoarseBits c0 and their difference d (|d| < 2^22,
+// vd: the exact integer difference, rounded once to float.
+// vd_coarse (the FP64 path's screen of a listed pair): the view integers are dropped to 2^-kCoarseBits c0 and their difference d (|d| < 2^22,
 // certified per particle by the list build) is added to the bits of
 // 1.5 * 2^(23 - kCoarseBits), whose low mantissa bit weighs 2^-kCoarseBits: the
 // float is then bias + d 2^-kCoarseBits exactly, converted by one integer add
 // and one float subtract instead of the conversion unit.
-template <bool FAST>
-__device__ __forceinline__ float vd(const Frame<float>& F, int a, int b) {
-  if (FAST) {
-    // the modular difference is exact; shift it, not the (wrapped) operands
-    constexpr int s = kViewBits - kCoarseBits;
-    return __int_as_float(F.mbits + ((a - b) >> s)) - F.mbias;
-  }
-  return (float)(a - b) * F.vscale;
-}
-template <bool FAST>
-__device__ __forceinline__ double vd(const Frame<double>&, double a, double b) {
-  return a - b;
+__device__ __forceinline__ float vd(const Frame<float>& F, int a, int b) { return (float)(a - b) * F.vscale; }
+__device__ __forceinline__ double vd(const Frame<double>&, double a, double b) { return a - b; }
+__device__ __forceinline__ float vd_coarse(const Frame<float>& F, int a, int b) {
+  // the modular difference is exact; shift it, not the (wrapped) operands
+  constexpr int s = kViewBits - kCoarseBits;
+  return __int_as_float(F.mbits + ((a - b) >> s)) - F.mbias;
 }
 // radius H widened for a screening test on coarse vectors: each coarse component
 // is the exact one floored to 2^-kCoarseBits c0, so |r_coarse - r| < sqrt(3) 2^-kCoarseBits;
@@ -93,13 +86,17 @@ template <class T>
 __device__ __forceinline__ T screen_radius(T H) {
   return H * T(1.0 + 1.0 / (1 << 20)) + T(1.0 / (1 << (kCoarseBits - 2)));
 }
-__device__ __forceinline__ float view_h(const int4& v) { return __int_as_float(v.w); }
-__device__ __forceinline__ double view_h(const V4<double>& v) { return v.w; }
+// w of a view: FP32 kappa h / 2 in view integers (the support of a pair is the
+// sum of the two w), FP64 h in view units; view_h: h in view units
+__device__ __forceinline__ float view_w(const int4& v) { return __int_as_float(v.w); }
+__device__ __forceinline__ double view_w(const V4<double>& v) { return v.w; }
+__device__ __forceinline__ float view_h(const Frame<float>& F, const int4& v) { return __int_as_float(v.w) * F.w2c; }
+__device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>& v) { return v.w; }
 
-// The neighbour list of particle i is column i of a cap x n array, split at
+// The neighbour list of particle i has list_rows(cap) rows (list_at), split at
 // its build: the entries then inside their support (r < max(kappa h_i,
-// kappa h_ij)) fill rows 0, 1, ... in candidate order, the others rows cap-1,
-// cap-2, ... in candidate order. A pass walks the inside part first, so the
+// kappa h_ij)) fill rows 0, 1, ... in candidate order, the others the last row,
+// the one before, ... in candidate order. A pass walks the inside part first, so the
 // entries that pass its exact tests cluster at the start of every list and a
 // warp skips the pair body on the later rows, where no lane's entry passes.
 // lcount packs both counts (bits 0-14 and 15-29); bit 31 certifies that
@@ -125,12 +122,12 @@ __device__ __forceinline__ T coord_phys(const Frame<T>& F, long long X) {
 
 // view of a particle at integer position X with smoothing length h (physical):
 // FP32 integers of 2^-kViewBits c0 (rounded; the low 32 bits suffice because
-// only differences of nearby particles are used), FP64 c0 units; w = h / c0
+// only differences of nearby particles are used), FP64 c0 units; w: view_w
 template <int D>
 __device__ __forceinline__ int4 make_view(const Frame<float>& F, const LL4& X, float h) {
   const long long half = 1LL << (F.sv - 1);
   return make_int4((int)((X.x + half) >> F.sv), (int)((X.y + half) >> F.sv), D == 3 ? (int)((X.z + half) >> F.sv) : 0,
-                   __float_as_int(h * F.inv_qv));
+                   __float_as_int(h * F.h2w));
 }
 template <int D>
 __device__ __forceinline__ V4<double> make_view(const Frame<double>& F, const LL4& X, double h) {
@@ -139,64 +136,27 @@ __device__ __forceinline__ V4<double> make_view(const Frame<double>& F, const LL
 __device__ __forceinline__ int4 with_w(int4 v, float w) { return make_int4(v.x, v.y, v.z, __float_as_int(w)); }
 __device__ __forceinline__ V4<double> with_w(V4<double> v, double w) { return V4<double>{v.x, v.y, v.z, w}; }
 
-// Visit the cnt listed entries of particle i (column i of the list) in
-// batches of SPH_LIST_BATCH: the list words, then the neighbour views, are
-// loaded before any is used, so each warp keeps several independent gathers in
-// flight. List words are streamed (read once per pass).
-#ifndef SPH_LIST_BATCH
-#define SPH_LIST_BATCH 4
-#endif
-// Entry k of a list whose first n_in entries sit in rows 0.. and the rest in
-// rows cap-1, cap-2, ... (a compact list: n_in = cnt).
-__device__ __forceinline__ size_t list_row(int k, int n_in, int cap) {
-  return (size_t)(k < n_in ? k : cap - 1 - (k - n_in));
-}
-template <class VT, class Fn>
-__device__ __forceinline__ void for_list(const uint32_t* __restrict__ list, const VT* __restrict__ view, int n, int i,
-                                         int cnt, int n_in, int cap, Fn&& pair) {
-  constexpr int B = SPH_LIST_BATCH;
-  int k = 0;
-  for (; k + B <= cnt; k += B) {
-    uint32_t e[B];
-    VT v[B];
-#pragma unroll
-    for (int q = 0; q < B; ++q) e[q] = __ldcs(list + list_row(k + q, n_in, cap) * n + i);
-#pragma unroll
-    for (int q = 0; q < B; ++q) v[q] = view[e[q] >> 8];
-#pragma unroll
-    for (int q = 0; q < B; ++q) pair(e[q], v[q]);
-  }
-  for (; k < cnt; ++k) {
-    const uint32_t e = __ldcs(list + list_row(k, n_in, cap) * n + i);
-    pair(e, view[e >> 8]);
-  }
-}
-// a compact list (rows 0 .. cnt-1)
-template <class VT, class Fn>
-__device__ __forceinline__ void for_list(const uint32_t* __restrict__ list, const VT* __restrict__ view, int n, int i,
-                                         int cnt, Fn&& pair) {
-  for_list(list, view, n, i, cnt, cnt, 0, pair);
-}
-// A compact list (rows 0 .. cnt-1) whose pair body also needs a record of
-// the neighbour (its acceleration, an adjoint): that record, fetch(j), is
-// loaded for the whole batch together with the views, so each thread keeps
-// 2 x SPH_LIST_BATCH_X independent gathers in flight instead of meeting the
-// record's latency inside every pair body.
 #ifndef SPH_LIST_BATCH_X
 #define SPH_LIST_BATCH_X 2  // 4 spilled at the 48 / 64-register budgets of the passes using it
 #endif
+// The force pairs of particle i, whose pair body also needs a record of
+// the neighbour (its acceleration, an adjoint): that record, fetch(j), is
+// loaded for the whole batch together with the views, so each thread keeps
+// 2 x SPH_LIST_BATCH_X independent gathers in flight instead of meeting the
+// record's latency inside every pair body. Words are streamed (read once).
 template <class VT, class Fetch, class Fn>
-__device__ __forceinline__ void for_list_x(const uint32_t* __restrict__ list, const VT* __restrict__ view, int n,
-                                           int i, int cnt, Fetch&& fetch, Fn&& pair) {
+__device__ __forceinline__ void for_pairs_x(const uint32_t* __restrict__ plist, const VT* __restrict__ view, int i,
+                                            int cnt, int cap, Fetch&& fetch, Fn&& pair) {
   using XT = decltype(fetch(0));
   constexpr int B = SPH_LIST_BATCH_X;
+  const uint32_t* __restrict__ p = plist + pair_at(i, 0, cap);
   int k = 0;
-  for (; k + B <= cnt; k += B) {
+  for (; k + B <= cnt; k += B, p += 32 * B) {
     uint32_t e[B];
     VT v[B];
     XT x[B];
 #pragma unroll
-    for (int q = 0; q < B; ++q) e[q] = __ldcs(list + (size_t)(k + q) * n + i);
+    for (int q = 0; q < B; ++q) e[q] = __ldcs(p + 32 * q);
 #pragma unroll
     for (int q = 0; q < B; ++q) {
       v[q] = view[e[q] >> 8];
@@ -205,16 +165,65 @@ __device__ __forceinline__ void for_list_x(const uint32_t* __restrict__ list, co
 #pragma unroll
     for (int q = 0; q < B; ++q) pair(e[q], v[q], x[q]);
   }
-  for (; k < cnt; ++k) {
-    const uint32_t e = __ldcs(list + (size_t)k * n + i);
+  for (; k < cnt; ++k, p += 32) {
+    const uint32_t e = __ldcs(p);
     pair(e, view[e >> 8], fetch((int)(e >> 8)));
   }
 }
-// the skin list of particle i (split at its build, see kFastBit)
+// The skin list of particle i as quads of entries (split at its build, see
+// kFastBit), in the order: full quads of the inside part, full quads of the
+// outside part, what is left of each. quad(e, valid): four list words, and
+// which of them are entries (bit q; std::true_type: all). The next full quad
+// is loaded before the current one is used: its words come from DRAM, the
+// neighbours' views mostly from the caches.
+template <class Quad>
+__device__ __forceinline__ void for_quads(const uint32_t* __restrict__ list, int i, uint32_t lc, int cap, Quad&& quad) {
+  const int n_in = list_in(lc), n_out = list_cnt(lc) - n_in, rows = list_rows(cap) >> 2;
+  const uint4* __restrict__ in = (const uint4*)(list + list_at(i, 0, cap));
+  const int qi = n_in >> 2, nq = qi + (n_out >> 2);
+  const auto at = [&](int q) { return in + (size_t)(q < qi ? q : rows - 1 - (q - qi)) * 32; };
+  uint4 ahead = make_uint4(0, 0, 0, 0);
+  if (nq > 0) ahead = __ldcs(at(0));
+  for (int q = 0; q < nq;) {
+    const uint4 w = ahead;
+    ++q;
+    if (q < nq) ahead = __ldcs(at(q));
+    quad(w, std::true_type{});
+  }
+#pragma unroll 1
+  for (int part = 0; part < 2; ++part) {
+    const int left = (part ? n_out : n_in) & 3;
+    if (left) quad(__ldcs(part ? at(nq) : in + (size_t)qi * 32), part ? (0xF0u >> left) & 0xFu : (1u << left) - 1u);
+  }
+}
+// row of entry k of a list whose first n_in entries sit in rows 0.. and the
+// rest in the last row, the one before, ...
+__device__ __forceinline__ int list_row(int k, int n_in, int cap) {
+  return k < n_in ? k : list_rows(cap) - 1 - (k - n_in);
+}
+// pair(e, view of e) for every entry of the skin list of particle i, what is
+// left of the inside part before the outside part. A body of FP64 arithmetic
+// costs as much for one lane as for 32, so the lanes' inside entries have to
+// stay in step (quads with their remainders last: 3 % slower).
 template <class VT, class Fn>
-__device__ __forceinline__ void for_skin_list(const uint32_t* __restrict__ list, const VT* __restrict__ view, int n,
-                                              int i, uint32_t lc, int cap, Fn&& pair) {
-  for_list(list, view, n, i, list_cnt(lc), list_in(lc), cap, pair);
+__device__ __forceinline__ void for_skin_list(const uint32_t* __restrict__ list, const VT* __restrict__ view, int i,
+                                              uint32_t lc, int cap, Fn&& pair) {
+  const int cnt = list_cnt(lc), n_in = list_in(lc);
+  int k = 0;
+  for (; k + 4 <= cnt; k += 4) {
+    uint32_t e[4];
+    VT v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) e[q] = list[list_at(i, list_row(k + q, n_in, cap), cap)];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = view[e[q] >> 8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) pair(e[q], v[q]);
+  }
+  for (; k < cnt; ++k) {
+    const uint32_t e = list[list_at(i, list_row(k, n_in, cap), cap)];
+    pair(e, view[e >> 8]);
+  }
 }
 
 // The FP64 path's skin list screened on its FP32 views (v32, kept current
@@ -225,31 +234,30 @@ __device__ __forceinline__ void for_skin_list(const uint32_t* __restrict__ list,
 // rejects cost no FP64 arithmetic (the FP64 pipe bounds that pass).
 template <class VT, class Screen, class Fn>
 __device__ __forceinline__ void for_skin_list_s32(const uint32_t* __restrict__ list, const int4* __restrict__ v32,
-                                                  const VT* __restrict__ view, int n, int i, uint32_t lc, int cap,
+                                                  const VT* __restrict__ view, int i, uint32_t lc, int cap,
                                                   Screen&& screen, Fn&& pair) {
-  constexpr int B = SPH_LIST_BATCH;
   const int cnt = list_cnt(lc), n_in = list_in(lc);
   int k = 0;
-  for (; k + B <= cnt; k += B) {
-    uint32_t e[B];
-    int4 w[B];
-    bool ok[B];
-    VT v[B];
+  for (; k + 4 <= cnt; k += 4) {
+    uint32_t e[4];
+    int4 w[4];
+    bool ok[4];
+    VT v[4];
 #pragma unroll
-    for (int q = 0; q < B; ++q) e[q] = __ldcs(list + list_row(k + q, n_in, cap) * n + i);
+    for (int q = 0; q < 4; ++q) e[q] = list[list_at(i, list_row(k + q, n_in, cap), cap)];
 #pragma unroll
-    for (int q = 0; q < B; ++q) w[q] = v32[e[q] >> 8];
+    for (int q = 0; q < 4; ++q) w[q] = v32[e[q] >> 8];
 #pragma unroll
-    for (int q = 0; q < B; ++q) {
+    for (int q = 0; q < 4; ++q) {
       ok[q] = screen(w[q]);
       if (ok[q]) v[q] = view[e[q] >> 8];
     }
 #pragma unroll
-    for (int q = 0; q < B; ++q)
+    for (int q = 0; q < 4; ++q)
       if (ok[q]) pair(e[q], v[q]);
   }
   for (; k < cnt; ++k) {
-    const uint32_t e = __ldcs(list + list_row(k, n_in, cap) * n + i);
+    const uint32_t e = list[list_at(i, list_row(k, n_in, cap), cap)];
     if (screen(v32[e >> 8])) pair(e, view[e >> 8]);
   }
 }
@@ -264,27 +272,6 @@ constexpr uint32_t kStageSelf = 1u << 20;
 __device__ __forceinline__ int stage_rank(uint32_t e) {
   const int r = (int)((e >> 8) & 0xFFFu);
   return r < kStageCap ? r : kStageCap - 1;  // in range by construction; the clamp keeps any stale word in bounds
-}
-template <class VT, class Fn>
-__device__ __forceinline__ void for_staged_list(const uint32_t* __restrict__ llist, const VT* sview, int n, int i,
-                                                uint32_t lc, int cap, Fn&& pair) {
-  constexpr int B = SPH_LIST_BATCH;
-  const int cnt = list_cnt(lc), n_in = list_in(lc);
-  int k = 0;
-  for (; k + B <= cnt; k += B) {
-    uint32_t e[B];
-    VT v[B];
-#pragma unroll
-    for (int q = 0; q < B; ++q) e[q] = __ldcs(llist + list_row(k + q, n_in, cap) * n + i);
-#pragma unroll
-    for (int q = 0; q < B; ++q) v[q] = sview[stage_rank(e[q])];
-#pragma unroll
-    for (int q = 0; q < B; ++q) pair(e[q], v[q]);
-  }
-  for (; k < cnt; ++k) {
-    const uint32_t e = __ldcs(llist + list_row(k, n_in, cap) * n + i);
-    pair(e, sview[stage_rank(e)]);
-  }
 }
 // 16-byte asynchronous copy global -> shared (cp.async, L2 only), and the wait
 // for every copy this thread issued
@@ -305,6 +292,47 @@ __device__ __forceinline__ long long state_units(double x) { return llrint(x); }
 template <class T> __device__ __forceinline__ T pair_r(T r2);
 template <> __device__ __forceinline__ float pair_r<float>(float r2) { return r2 * rsqrtf(r2); }
 template <> __device__ __forceinline__ double pair_r<double>(double r2) { return sqrt(r2); }
+
+// ---- two FP32 pairs per instruction -----------------------------------------
+// add / mul / fma on two floats at once (one issue slot for both, each rounded
+// as its scalar form)
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 max2(float2 a, float b) { return make_float2(fmaxf(a.x, b), fmaxf(a.y, b)); }
+// hardware reciprocal (1 ulp) and reciprocal square root of normal numbers
+__device__ __forceinline__ float fast_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float fast_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(fast_rcp(a.x), fast_rcp(a.y)); }
+__device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(fast_rsqrt(a.x), fast_rsqrt(a.y)); }
+// the skin list of particle i two entries at a time: two(e0, r0, e1, r1, on0,
+// on1) with r = load(e); a place without an entry (on = false) comes with e = own
+template <class Load, class Two>
+__device__ __forceinline__ void for_twos(const uint32_t* __restrict__ list, int i, uint32_t lc, int cap, uint32_t own,
+                                         Load&& load, Two&& two) {
+  for_quads(list, i, lc, cap, [&](uint4 w, auto valid) {
+    if constexpr (std::is_same<decltype(valid), std::true_type>::value) {
+      const auto r0 = load(w.x), r1 = load(w.y), r2 = load(w.z), r3 = load(w.w);
+      two(w.x, r0, w.y, r1, valid, valid);
+      two(w.z, r2, w.w, r3, valid, valid);
+    } else {
+      const bool o0 = valid & 1u, o1 = valid & 2u, o2 = valid & 4u, o3 = valid & 8u;
+      w = make_uint4(o0 ? w.x : own, o1 ? w.y : own, o2 ? w.z : own, o3 ? w.w : own);
+      const auto r0 = load(w.x), r1 = load(w.y), r2 = load(w.z), r3 = load(w.w);
+      two(w.x, r0, w.y, r1, o0, o1);
+      two(w.z, r2, w.w, r3, o2, o3);
+    }
+  });
+}
 
 template <int D, class T>
 __device__ __forceinline__ void abs_pos(const Frame<T>& F, const LL4& X, T* x) {
@@ -649,7 +677,7 @@ __global__ void __launch_bounds__(256) k_make_view(int n, const StepCtl* __restr
     const T h = h_of<D, T>(geo, x);
     const auto v = make_view<D>(F, X, h);
     (ctl->vp ? v1 : v0)[i] = v;
-    vbuild[i] = with_w(v, T(0.5) * F.skin * view_h(v));  // half the skin, view units (kappa folded in by the host)
+    vbuild[i] = with_w(v, T(0.5) * F.skin * view_h(F, v));  // half the skin, view units (kappa folded in by the host)
   }
 }
 
@@ -670,7 +698,7 @@ __global__ void __launch_bounds__(256) k_view32(int n, const StepCtl* __restrict
     const LL4 X = (ctl->buf ? X1 : X0)[i];
     const double hv = (ctl->vp ? vd1 : vd0)[i].w;  // h in view units (c0, both precisions)
     out[i] = make_int4((int)((X.x + half) >> F.sv), (int)((X.y + half) >> F.sv),
-                       D == 3 ? (int)((X.z + half) >> F.sv) : 0, __float_as_int((float)hv));
+                       D == 3 ? (int)((X.z + half) >> F.sv) : 0, __float_as_int((float)hv * F.c2w));
   }
 }
 
@@ -700,7 +728,7 @@ __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(int n, 
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
   const LL4 X = (buf ? X1 : X0)[i];
   const VT vi = view[i];
-  const T hv = view_h(vi);                 // view units
+  const T hv = view_h(F, vi);                 // view units
   const T sk = F.skin * hv;                // skin of i, view units (kappa folded in by the host)
   const T sk_hv = F.skin;                  // skin per unit h
   const T lip = G.lip_h;
@@ -717,6 +745,8 @@ __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(int n, 
   const int l0 = level_of_h(G, hlo * qv), l1 = level_of_h(G, hhi * qv);
   const T R2 = Rs * Rs;
   int cnt = 0, n_in = 0, n_out = 0;  // accepted; written inside / outside entries
+  const int rows = list_rows(cap);
+  uint32_t* __restrict__ own = list + list_at(i, 0, cap);
   bool over = false;
   T reach = 0;
   const T Hd = kappa * hv;
@@ -726,10 +756,10 @@ __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(int n, 
   // warp in nearly every iteration); only the list store is conditional
   const T cl = T(1) + T(0.5) * kappa * lip;
   auto cand = [&](int jc, const VT& vj) {
-    const T dx = vd<false>(F, vi.x, vj.x), dy2 = vd<false>(F, vi.y, vj.y);
-    const T dz2 = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
+    const T dx = vd(F, vi.x, vj.x), dy2 = vd(F, vi.y, vj.y);
+    const T dz2 = D == 3 ? vd(F, vi.z, vj.z) : T(0);
     const T r2 = dx * dx + dy2 * dy2 + dz2 * dz2;
-    const T hj = view_h(vj);
+    const T hj = view_h(F, vj);
     const T skj = sk_hv * hj;
     const T smax = sk > skj ? sk : skj;
     const T hm = hv > hj ? hv : hj;  // symmetric: j lists i whenever i lists j
@@ -746,8 +776,8 @@ __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(int n, 
     reach = acc && am > reach ? am : reach;
     if (acc) {
       if (cnt < cap) {
-        const int row = inside ? n_in++ : cap - 1 - n_out++;
-        list[(size_t)row * n + i] = ((uint32_t)jc << 8) | (meta[jc] & 0xFFu);
+        const int row = inside ? n_in++ : rows - 1 - n_out++;
+        own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)jc << 8) | (meta[jc] & 0xFFu);
       } else {
         over = true;
       }
@@ -854,7 +884,7 @@ __global__ void __launch_bounds__(kStageBlock) k_stage(int n, const StepCtl* __r
   const uint32_t lc = i < n ? lcount[i] : 0u;
   const int cnt = list_cnt(lc), n_in = list_in(lc);
   for (int k = 0; k < cnt; ++k) {
-    const int j = (int)(list[list_row(k, n_in, cap) * n + i] >> 8);
+    const int j = (int)(list[list_at(i, list_row(k, n_in, cap), cap)] >> 8);
     uint32_t q = stage_hash(j);
     int p = 0;
     for (; p < kStageProbe; ++p) {
@@ -898,7 +928,7 @@ __global__ void __launch_bounds__(kStageBlock) k_stage(int n, const StepCtl* __r
   }
   __syncthreads();
   for (int k = 0; k < cnt; ++k) {
-    const size_t pos = list_row(k, n_in, cap) * n + i;
+    const size_t pos = list_at(i, list_row(k, n_in, cap), cap);
     const uint32_t e = list[pos];
     const int j = (int)(e >> 8);
     uint32_t q = stage_hash(j);
@@ -924,36 +954,42 @@ __global__ void __launch_bounds__(256) k_density(int n, const StepCtl* __restric
   if (i >= n) return;
   const VT* __restrict__ view = ctl->vp ? v1 : v0;
   const VT vi = view[i];
-  const T hv = view_h(vi);
+  const T hv = view_h(F, vi);
   const T Hd = P.kappa * hv, Hd2 = Hd * Hd, invHd = T(1) / Hd;
   const uint32_t lc = lcount[i];
-  const int cnt = list_cnt(lc), n_in = list_in(lc);
-  const T Hs = (lc & kFastBit) ? screen_radius<T>(Hd) : Hd, Hs2 = Hs * Hs;
   T acc = 0;
-  auto loop = [&](auto fastc) {
-    constexpr bool FAST = decltype(fastc)::value;
-    for (int k = 0; k < cnt; ++k) {
-      const uint32_t e = list[list_row(k, n_in, cap) * n + i];
-      const VT vj = view[e >> 8];
-      T dx = vd<FAST>(F, vi.x, vj.x), dy = vd<FAST>(F, vi.y, vj.y);
-      T dz = D == 3 ? vd<FAST>(F, vi.z, vj.z) : T(0);
-      T r2 = dx * dx + dy * dy + dz * dz;
-      if (r2 < Hs2) {
-        if (FAST) {
-          dx = vd<false>(F, vi.x, vj.x);
-          dy = vd<false>(F, vi.y, vj.y);
-          dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
-          r2 = dx * dx + dy * dy + dz * dz;
-          if (!(r2 < Hd2)) continue;
-        }
-        const T q = r2 > T(0) ? pair_r<T>(r2) * invHd : T(0);
-        const T u = T(1) - q, u2 = u * u;
-        acc += u2 * u2 * (T(1) + T(4) * q);
+  if constexpr (std::is_same<T, float>::value) {  // two entries at a time, as pass A
+    const float2 id2 = both(-0.5f / view_w(vi)), one2 = both(1.0f);
+    float2 ds2 = both(0.0f), dq2 = both(0.0f);
+    auto two = [&](uint32_t, const VT& a, uint32_t, const VT& b, auto on0, auto on1) {
+      const float2 dx = make_float2((float)(vi.x - a.x), (float)(vi.x - b.x));
+      const float2 dy = make_float2((float)(vi.y - a.y), (float)(vi.y - b.y));
+      float2 r2 = fma2(dy, dy, mul2(dx, dx));
+      if (D == 3) {
+        const float2 dz = make_float2((float)(vi.z - a.z), (float)(vi.z - b.z));
+        r2 = fma2(dz, dz, r2);
       }
-    }
-  };
-  if (lc & kFastBit) loop(std::true_type{});
-  else loop(std::false_type{});
+      r2 = make_float2(fmaxf(r2.x, 1.0f), fmaxf(r2.y, 1.0f));
+      if (!on0) r2.x = 1e30f;
+      if (!on1) r2.y = 1e30f;
+      const float2 r = mul2(r2, rsqrt2(r2)), q = mul2(r, id2), u = max2(add2(q, one2), 0.0f), u2 = mul2(u, u), u4 = mul2(u2, u2);
+      ds2 = add2(ds2, u4);
+      dq2 = fma2(u4, q, dq2);
+    };
+    auto load = [&](uint32_t e) -> VT { return view[e >> 8]; };
+    for_twos(list, i, lc, cap, (uint32_t)i << 8, load, two);
+    acc = (ds2.x + ds2.y) - 4.0f * (dq2.x + dq2.y);
+  } else {
+    for_skin_list(list, view, i, lc, cap, [&](uint32_t, const VT& vj) {
+      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
+      const T r2 = dx * dx + dy * dy + dz * dz;
+      if (!(r2 < Hd2)) return;
+      const T q = r2 > T(0) ? pair_r<T>(r2) * invHd : T(0);
+      const T u = T(1) - q, u2 = u * u;
+      acc += u2 * u2 * (T(1) + T(4) * q);
+    });
+  }
   const T Hphys = Hd * F.qv;
   const T rho = acc * P.alpha / (D == 2 ? Hphys * Hphys : Hphys * Hphys * Hphys);
   const T irt2 = inv_rho_t2<D, T>(hv * F.qv, P.inv_tau);
@@ -1000,6 +1036,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
   using VT = typename ViewOf<T>::type;
   static_assert(!STG || (std::is_same<T, float>::value && !GENERAL && !DBG && !SURF && NT == kStageBlock),
                 "staged pass A: FP32, gamma = 2, 256-target blocks");
+  constexpr bool PACKED = std::is_same<T, float>::value && !DBG && !SURF;
   extern __shared__ __align__(16) unsigned char stage_smem[];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const StepCtl cc = *ctl;
@@ -1033,7 +1070,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // a feature-surface particle (Sec. 3.5) takes forces from surface particles
     // only (SURF: the variant launched when the handle has any)
     const bool surf = SURF && (mi & kSurfaceBit) != 0;
-    const T hv = view_h(vi);
+    const T hv = view_h(F, vi);
     const T qv = F.qv;
     const T Hd = P.kappa * hv, Hd2 = Hd * Hd, invHd = T(1) / Hd;
     const T inv_tau_v = P.inv_tau * qv;           // h in view units -> (h/tau)
@@ -1046,91 +1083,149 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     long long sd = 0, sf = 0;
     const uint32_t lc = lcount[i];
     const int cnt = list_cnt(lc);
-    // Every skin-list entry: a screening test on the coarse vectors (when the
-    // list build certified them), then the exact vectors and criteria for the
-    // pairs that pass. This step's force pairs go to column i of plist.
-    // FP64 path with current FP32 views: the screen in FP32 (for_skin_list_s32)
-    constexpr bool S32_OK = std::is_same<T, double>::value && !GENERAL && !DBG && !SURF;
-    auto loop = [&](auto fastc, auto stagedc, auto s32c) {
-      constexpr bool FAST = decltype(fastc)::value;
-      constexpr bool ST = decltype(stagedc)::value;  // e = (rank << 8 | colour), view from shared memory
-      constexpr bool S32 = decltype(s32c)::value;    // entries arrive screened on the FP32 views
-      auto pair = [&](uint32_t e, const VT& vj) {
-        const int j = ST ? -1 : (int)(e >> 8);  // global index (unstaged entries)
-        const bool self = ST ? (e & kStageSelf) != 0 : j == i;
-        T dx = vd<FAST>(F, vi.x, vj.x), dy = vd<FAST>(F, vi.y, vj.y);
-        T dz = D == 3 ? vd<FAST>(F, vi.z, vj.z) : T(0);
-        T r2 = dx * dx + dy * dy + dz * dz;
-        const T hj = view_h(vj);
-        const T Hf = half_kappa * (hv + hj);
-        if (FAST) {
-          const T Hm = screen_radius<T>(GENERAL || Hf > Hd ? Hf : Hd);
-          if (!(r2 < Hm * Hm)) return;
-          dx = vd<false>(F, vi.x, vj.x);
-          dy = vd<false>(F, vi.y, vj.y);
-          dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
-          r2 = dx * dx + dy * dy + dz * dz;
-        }
-        const bool inD = !GENERAL && r2 < Hd2;
-        const bool inF = r2 < Hf * Hf && !self && (!surf || (meta[j] & kSurfaceBit));
-        if (!(inD || inF)) return;
-        const T r = r2 > T(0) ? pair_r<T>(r2) : T(0);
-        if (inD) {
-          const T q = r * invHd;
-          const T u = T(1) - q, u2 = u * u;
-          dsum += u2 * u2 * (T(1) + T(4) * q);
-          if (DBG) {
-            ++nd;
-            sd += pid[j];
+    uint32_t* __restrict__ pw = plist + pair_at(i, 0, cap);  // this step's force pairs, for pass B
+    // FP32: the listed entries two at a time, every FP32 operation on both at
+    // once, on exact differences throughout (a coarse screen first saved the
+    // conversions but evaluated the passing two thirds twice). The kernel's
+    // factors 1 - r/H are clamped at zero, so a pair outside a support adds
+    // nothing and needs no test; only an iteration in which neither entry is
+    // inside is skipped. What bounds it: the latency of the view gathers (issue
+    // slots 51 % busy, L1 data pipe 56 %). With the reductions above, at
+    // 1,048,576 particles: 304 -> 227 us in 3D (249 -> 144 million warp
+    // instructions), 216 -> 126 us in 2D. 64 registers (four 256-thread blocks
+    // per SM): at 48 it spills (8,388,608 in 3D: 2.30 ms against 1.59), at 80
+    // too few warps hide the gathers (1.84 ms).
+    if constexpr (PACKED) {
+      // lengths in view integers, the pair's support H = w_i + w_j; powers of h_j
+      // and H relative to w_i, whose own powers come in once, after the sum
+      const float wi = view_w(vi);
+      const float2 w2 = both(wi), id2 = both(-0.5f / wi), iw2 = both(1.0f / wi), one2 = both(1.0f);
+      const float hd2 = 4.0f * wi * wi;  // (kappa h_i)^2
+      const float sq = GENERAL ? sP0 * qi : 1.0f + sigma;
+      const uint32_t own = ((uint32_t)i << 8) | ci;
+      float2 ds2 = both(0.0f), dq2 = both(0.0f), ax2 = both(0.0f), ay2 = both(0.0f), az2 = both(0.0f);
+      auto sums = [&](auto stagedc) {
+        constexpr bool ST = decltype(stagedc)::value;  // e = (rank << 8 | colour), view from shared memory
+        auto load = [&](uint32_t e) -> VT { return ST ? sview[stage_rank(e)] : view[e >> 8]; };
+        auto two = [&](uint32_t e0, const VT& v0, uint32_t e1, const VT& v1, auto on0, auto on1) {
+          const float2 dx = make_float2((float)(vi.x - v0.x), (float)(vi.x - v1.x));
+          const float2 dy = make_float2((float)(vi.y - v0.y), (float)(vi.y - v1.y));
+          float2 r2 = fma2(dy, dy, mul2(dx, dx)), dz = both(0.0f);
+          if (D == 3) {
+            dz = make_float2((float)(vi.z - v0.z), (float)(vi.z - v1.z));
+            r2 = fma2(dz, dz, r2);
           }
-        }
-        if (inF) {
-          const T invH = drcp<T>(Hf);
-          const T q = r * invH;
-          const T u = T(1) - q;
-          const T invH2 = invH * invH;
-          const T w = u * u * u * (D == 2 ? invH2 * invH2 : invH2 * invH2 * invH);
-          const T qj = inv_rho_t2<D, T>(hj, inv_tau_v);
-          const T Pj = GENERAL ? pc[j] : P.P0 * qj;
-          const bool other = (e & 0xFFu) != ci;
-          const T coef = (Pi + Pj) + (other ? sP0 * (qi + qj) : T(0));
-          const T s = coef * w;
-          ax += s * dx;
-          ay += s * dy;
-          az += s * dz;
-          // this step's force pairs (global index | colour), for pass B
-          const uint32_t eg = ST ? ((uint32_t)__ldg(sjb + stage_rank(e)) << 8) | (e & 0xFFu) : e;
-          SPH_PLIST_STORE(plist + (size_t)nf * n + i, eg);
-          ++nf;
-          ni += other;
-          if (DBG) sf += pid[j];
-        }
-      };
-      if constexpr (ST) {
-        for_staged_list(llist, (const VT*)sview, n, i, lc, cap, pair);
-      } else if constexpr (S32) {
-        const int4 wi = v32[i];
-        const float hv32 = __int_as_float(wi.w), hk32 = 0.5f * (float)P.kappa, Hd32 = (float)P.kappa * hv32;
-        auto screen = [&](const int4& w) {
-          const float cx = vd<true>(F32, wi.x, w.x), cy = vd<true>(F32, wi.y, w.y);
-          const float cz = D == 3 ? vd<true>(F32, wi.z, w.z) : 0.0f;
-          const float Hf32 = hk32 * (hv32 + __int_as_float(w.w));
-          const float Hm = screen_radius<float>(Hf32 > Hd32 ? Hf32 : Hd32);
-          return cx * cx + cy * cy + cz * cz < Hm * Hm;
+          r2 = make_float2(fmaxf(r2.x, 1.0f), fmaxf(r2.y, 1.0f));  // 1 for the particle itself: r = 2^-24 c0, dx = 0
+          if (!on0) r2.x = 1e30f;
+          if (!on1) r2.y = 1e30f;
+          const float2 wj = make_float2(view_w(v0), view_w(v1));
+          const float2 H = add2(w2, wj), H2 = mul2(H, H);
+          const bool f0 = r2.x < H2.x, f1 = r2.y < H2.y;
+          if (!(f0 || f1 || (!GENERAL && (r2.x < hd2 || r2.y < hd2)))) return;
+          const float2 r = mul2(r2, rsqrt2(r2));
+          if (!GENERAL) {  // W ~ (1 - q)^4 (1 + 4 q); q = 1 - u where u > 0
+            const float2 u = max2(fma2(r, id2, one2), 0.0f), u2 = mul2(u, u), u4 = mul2(u2, u2);
+            ds2 = add2(ds2, u4);
+            dq2 = fma2(u4, mul2(r, id2), dq2);
+          }
+          const float2 nH = rcp2(make_float2(-H.x, -H.y));
+          const float2 u = max2(fma2(r, nH, one2), 0.0f), g = mul2(nH, w2), g2 = mul2(g, g), g4 = mul2(g2, g2);
+          const float2 w = mul2(mul2(mul2(u, u), u), D == 2 ? g4 : mul2(g4, g));  // 3D: negative (g < 0)
+          const float2 t = mul2(wj, iw2), t2 = mul2(t, t);
+          const float2 ts = D == 2 ? fma2(t2, t2, one2) : fma2(mul2(t2, t2), t2, one2);  // 1 + rho_t,i^2 / rho_t,j^2
+          const bool o0 = ((e0 ^ own) & 0xFFu) != 0, o1 = ((e1 ^ own) & 0xFFu) != 0;
+          float2 s = mul2(ts, w);
+          if (GENERAL) {
+            const float2 pp = make_float2(pc[e0 >> 8], pc[e1 >> 8]);
+            s = mul2(fma2(make_float2(o0 ? sq : 0.0f, o1 ? sq : 0.0f), ts, add2(both(Pi), pp)), w);
+          } else {
+            s = mul2(s, make_float2(o0 ? sq : 1.0f, o1 ? sq : 1.0f));
+          }
+          ax2 = fma2(s, dx, ax2);
+          ay2 = fma2(s, dy, ay2);
+          if (D == 3) az2 = fma2(s, dz, az2);
+          auto push = [&](uint32_t e, bool inside, bool other) {
+            if (inside && !(ST ? (e & kStageSelf) != 0 : e == own)) {
+              SPH_PLIST_STORE(pw, ST ? ((uint32_t)__ldg(sjb + stage_rank(e)) << 8) | (e & 0xFFu) : e);
+              pw += 32;
+              ++nf;
+              ni += other;
+            }
+          };
+          push(e0, f0, o0);
+          push(e1, f1, o1);
         };
-        for_skin_list_s32(list, v32, view, n, i, lc, cap, screen, pair);
-      } else {
-        for_skin_list(list, view, n, i, lc, cap, pair);
+        for_twos(ST ? llist : list, i, lc, cap, ST ? ci | kStageSelf : own, load, two);
+      };
+      if (STG && staged) sums(std::integral_constant<bool, STG>{});
+      else sums(std::false_type{});
+      dsum = (ds2.x + ds2.y) - 4.0f * (dq2.x + dq2.y);  // dq2 holds the terms in -q
+      // back to view units: w_i^-(D+2), and P0/rho_t,i^2 (or the pressures themselves)
+      const float iw = 2.0f * invHd, iw4 = iw * iw * iw * iw;
+      const float back = F.vscale * (GENERAL ? 1.0f : P.P0 * qi) * (D == 2 ? iw4 : -iw4 * iw);
+      ax = (ax2.x + ax2.y) * back;
+      ay = (ay2.x + ay2.y) * back;
+      az = (az2.x + az2.y) * back;
+    } else {
+    // FP64, feature surfaces, diagnostics: one entry at a time, the exact
+    // criteria on every entry (FP64 path with current FP32 views: on those that
+    // pass a screen in FP32, for_skin_list_s32)
+    constexpr bool S32_OK = std::is_same<T, double>::value && !GENERAL && !DBG && !SURF;
+    auto pair = [&](uint32_t e, const VT& vj) {
+      const int j = (int)(e >> 8);
+      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
+      const T r2 = dx * dx + dy * dy + dz * dz;
+      const T hj = view_h(F, vj);
+      const T Hf = half_kappa * (hv + hj);
+      const bool inD = !GENERAL && r2 < Hd2;
+      const bool inF = r2 < Hf * Hf && j != i && (!surf || (meta[j] & kSurfaceBit));
+      if (!(inD || inF)) return;
+      const T r = r2 > T(0) ? pair_r<T>(r2) : T(0);
+      if (inD) {
+        const T q = r * invHd;
+        const T u = T(1) - q, u2 = u * u;
+        dsum += u2 * u2 * (T(1) + T(4) * q);
+        if (DBG) {
+          ++nd;
+          sd += pid[j];
+        }
+      }
+      if (inF) {
+        const T invH = drcp<T>(Hf);
+        const T q = r * invH;
+        const T u = T(1) - q;
+        const T invH2 = invH * invH;
+        const T w = u * u * u * (D == 2 ? invH2 * invH2 : invH2 * invH2 * invH);
+        const T qj = inv_rho_t2<D, T>(hj, inv_tau_v);
+        const T Pj = GENERAL ? pc[j] : P.P0 * qj;
+        const bool other = (e & 0xFFu) != ci;
+        const T coef = (Pi + Pj) + (other ? sP0 * (qi + qj) : T(0));
+        const T s = coef * w;
+        ax += s * dx;
+        ay += s * dy;
+        az += s * dz;
+        SPH_PLIST_STORE(pw, e);
+        pw += 32;
+        ++nf;
+        ni += other;
+        if (DBG) sf += pid[j];
       }
     };
-    if (STG && staged) {
-      if (lc & kFastBit) loop(std::true_type{}, std::integral_constant<bool, STG>{}, std::false_type{});
-      else loop(std::false_type{}, std::integral_constant<bool, STG>{}, std::false_type{});
-    } else if (S32_OK && v32 && (lc & kFastBit)) {
-      loop(std::false_type{}, std::false_type{}, std::integral_constant<bool, S32_OK>{});
+    if (S32_OK && v32 && (lc & kFastBit)) {
+      const int4 wi = v32[i];
+      const float ws = 2.0f / (float)(1 << kViewBits), wi32 = 0.5f * ws * view_w(wi), Hd32 = ws * view_w(wi);  // view units
+      auto screen = [&](const int4& w) {
+        const float cx = vd_coarse(F32, wi.x, w.x), cy = vd_coarse(F32, wi.y, w.y);
+        const float cz = D == 3 ? vd_coarse(F32, wi.z, w.z) : 0.0f;
+        const float Hf32 = wi32 + 0.5f * ws * view_w(w);
+        const float Hm = screen_radius<float>(Hf32 > Hd32 ? Hf32 : Hd32);
+        return cx * cx + cy * cy + cz * cz < Hm * Hm;
+      };
+      for_skin_list_s32(list, v32, view, i, lc, cap, screen, pair);
     } else {
-      if (lc & kFastBit) loop(std::true_type{}, std::false_type{}, std::false_type{});
-      else loop(std::false_type{}, std::false_type{}, std::false_type{});
+      for_skin_list(list, view, i, lc, cap, pair);
+    }
     }
     pcount[i] = (uint32_t)nf;
     // back to physical units: rho ~ 1/H^D, a ~ (view length)^-(D+1)
@@ -1297,13 +1392,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
                                                 const typename ViewOf<T>::type* __restrict__ vbuild,
                                                 LL4* __restrict__ X0, LL4* __restrict__ X1,
                                                 const uint32_t* __restrict__ plist,
-                                                const uint32_t* __restrict__ pcount,
+                                                const uint32_t* __restrict__ pcount, int cap,
                                                 const V4<T>* __restrict__ acc, Frame<T> F, Phys<T> P, Geom<T> geo,
                                                 const Scalars* __restrict__ scal, V4<T>* __restrict__ visc_out,
                                                 int* __restrict__ err, unsigned long long* __restrict__ wall_moved,
                                                 int move, const uint32_t* __restrict__ m0,
                                                 const uint32_t* __restrict__ m1, int4* __restrict__ v32out,
-                                                int sv32) {
+                                                int sv32, float c2w32) {
   using VT = typename ViewOf<T>::type;
   __shared__ int moved_sm[8];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1312,7 +1407,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
   if (i < n) {
     const VT* __restrict__ view = vp ? v1 : v0;
     const VT vi = view[i];
-    const T hv = view_h(vi);
+    const T hv = view_h(F, vi);
     const T qv = F.qv;
     const T inv_tau_v = P.inv_tau * qv;
     const T qi = inv_rho_t2<D, T>(hv, inv_tau_v);
@@ -1322,12 +1417,12 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
     // this step's pairs as pass A compacted them (same positions); the force
     // support is tested again on the exact vectors
     const int cnt = (int)pcount[i];
-    for_list_x(plist, view, n, i, cnt, [&](int j) { return acc[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& aj) {
+    for_pairs_x(plist, view, i, cnt, cap, [&](int j) { return acc[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& aj) {
       const int j = (int)(e >> 8);
-      const T dx = vd<false>(F, vi.x, vj.x), dy = vd<false>(F, vi.y, vj.y);
-      const T dz = D == 3 ? vd<false>(F, vi.z, vj.z) : T(0);
+      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
+      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
       const T r2 = dx * dx + dy * dy + dz * dz;
-      const T hj = view_h(vj);
+      const T hj = view_h(F, vj);
       const T Hf = half_kappa * (hv + hj);
       if (!(r2 < Hf * Hf) || j == i) return;
       const T gs = ai.w + aj.w;
@@ -1409,13 +1504,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       if (v32out) {  // FP64 path: its FP32 view of the next step (as k_view32 makes it)
         const long long half = 1LL << (sv32 - 1);
         v32out[i] = make_int4((int)((X.x + half) >> sv32), (int)((X.y + half) >> sv32),
-                              D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_h(vn)));
+                              D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_w(vn) * c2w32));
       }
       // skin test against the view at list build
       const VT vb = vbuild[i];
-      const T ex = vd<false>(F, vn.x, vb.x), ey = vd<false>(F, vn.y, vb.y);
-      const T ez = D == 3 ? vd<false>(F, vn.z, vb.z) : T(0);
-      const T lim = view_h(vb);
+      const T ex = vd(F, vn.x, vb.x), ey = vd(F, vn.y, vb.y);
+      const T ez = D == 3 ? vd(F, vn.z, vb.z) : T(0);
+      const T lim = view_w(vb);
       far = (ex * ex + ey * ey + ez * ez) >= lim * lim;
     } else {
       (vp ? w0 : w1)[i] = vi;
@@ -1610,9 +1705,9 @@ cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P
   unsigned long long* wm = (unsigned long long*)&S.scal->wall_moved;
   (tb == 128 ? k_pass_b<D, T, 128> : k_pass_b<D, T, 256>)<<<gb, tb, 0, st>>>(
       S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], (VT*)S.view[0], (VT*)S.view[1], (const VT*)S.vbuild,
-      (LL4*)S.X[0], (LL4*)S.X[1], S.plist, S.pcount, (const V4<T>*)S.acc4, F, P, g, S.scal,
+      (LL4*)S.X[0], (LL4*)S.X[1], S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
       f.record ? (V4<T>*)S.visc : nullptr, S.err, wm, f.move, S.meta[0], S.meta[1],
-      (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0);
+      (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0, f.f32 ? f.f32->c2w : 0.0f);
   return cudaGetLastError();
 }
 
