@@ -583,7 +583,7 @@ sph_status ensure_tape(sph_handle* h, int slots) {
     SPH_TRY(grab(h, T.meta[0], N)); T.meta[1] = T.meta[0];
     SPH_TRY(grab(h, T.pid[0], N)); T.pid[1] = T.pid[0];
     SPH_TRY(grab(h, p, N * v4)); T.view[0] = T.view[1] = p;
-    SPH_TRY(grab(h, T.plist, pair_words(N, h->S.cap)));
+    SPH_TRY(grab(h, p, pair_bytes(N, h->S.cap, h->S.fp64))); T.plist = p;
     SPH_TRY(grab(h, T.pcount, N));
     SPH_TRY(grab(h, p, N * v4)); T.acc4 = p;
     SPH_TRY(grab(h, p, N * v4)); T.visc = p;
@@ -804,7 +804,7 @@ static sph_status create_impl(sph_handle* h, const sph_domain* dom, const sph_fi
   SPH_TRY(grab(h, S.tmp, N));
   SPH_TRY(grab(h, S.list, list_words(N, S.cap)));
   SPH_TRY(grab(h, S.lcount, N));
-  SPH_TRY(grab(h, S.plist, pair_words(N, S.cap)));
+  SPH_TRY(grab(h, tmpb, pair_bytes(N, S.cap, S.fp64))); S.plist = tmpb;
   SPH_TRY(grab(h, S.pcount, N));
   SPH_TRY(grab(h, S.cnt, (size_t)S.total_cells));
   h->cells_cap = S.total_cells;

@@ -31,7 +31,7 @@ struct DevState {
   uint32_t total_cells = 0;
   uint32_t* list = nullptr;              // skin lists, entries (j << 8 | colour_j), see list_at
   uint32_t* lcount = nullptr;            // entries per particle; bit 31: FP32 coarse test exact
-  uint32_t* plist = nullptr;             // the force pairs of the current step (pass A -> B), see pair_at
+  void* plist = nullptr;                 // the force pairs of the current step (PairRec, pass A -> B), see pair_at
   // staged pass A (FP32, 256-thread pair passes): per 256-target block its
   // distinct neighbours sj (kStageCap per block), their count scount (-1: not
   // staged) and the list again with ranks in that set (llist, as list)
@@ -69,7 +69,15 @@ inline size_t list_words(size_t n, int cap) { return (n + 31) / 32 * 32 * (size_
 __host__ __device__ inline size_t pair_at(int i, int k, int cap) {
   return ((size_t)(i >> 5) * cap + k) * 32 + (i & 31);
 }
-inline size_t pair_words(size_t n, int cap) { return (n + 31) / 32 * 32 * (size_t)cap; }
+// A force pair as pass A leaves it to pass B: the list word and what the viscous
+// force needs of the pair's geometry, f = (1/rho_t,i^2 + 1/rho_t,j^2) (1 - q)^3
+// / H^(D+2) (FP32: over a factor of the target alone, pair_scale).
+template <class T> struct PairRec;
+template <> struct alignas(8) PairRec<float> { uint32_t e; float f; };
+template <> struct alignas(16) PairRec<double> { double f; uint32_t e, pad; };
+inline size_t pair_bytes(size_t n, int cap, bool fp64) {
+  return (n + 31) / 32 * 32 * (size_t)cap * (fp64 ? sizeof(PairRec<double>) : sizeof(PairRec<float>));
+}
 
 // per-step gate: flip the view buffer; start a list rebuild (flip the state
 // buffer) when pass B asked for one or `force` is set

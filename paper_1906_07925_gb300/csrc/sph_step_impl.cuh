@@ -29,20 +29,16 @@
 #ifndef SPH_PASS_MIN_BLOCKS
 #define SPH_PASS_MIN_BLOCKS 4
 #endif
-// store of a force-pair list word (streaming: read once, by pass B)
-#ifndef SPH_PLIST_STREAM
-#define SPH_PLIST_STREAM 1
-#endif
-#if SPH_PLIST_STREAM
-#define SPH_PLIST_STORE(p, v) __stcs((p), (v))
-#else
-#define SPH_PLIST_STORE(p, v) (*(p) = (v))
-#endif
 // the pair passes are compiled for 128 and 256 threads per block
 // (DevState::pass_threads picks one at launch); resident blocks per SM asked
 // of them scale so that the register budget per thread is the same
+// (pass B, FP32: 2D 73 against 77 us at 1,048,576 particles with 5 and 4 blocks,
+// 3D 1.04 against 0.85 ms at 8,388,608: it spills at 48 registers there)
 #ifndef SPH_PASSB_MIN_BLOCKS
-#define SPH_PASSB_MIN_BLOCKS 5
+#define SPH_PASSB_MIN_BLOCKS (D == 2 ? 5 : 4)
+#endif
+#ifndef SPH_PASSB_BATCH
+#define SPH_PASSB_BATCH 4
 #endif
 #ifndef SPH_LIST_MIN_BLOCKS
 #define SPH_LIST_MIN_BLOCKS 4
@@ -144,19 +140,19 @@ __device__ __forceinline__ V4<double> with_w(V4<double> v, double w) { return V4
 // loaded for the whole batch together with the views, so each thread keeps
 // 2 x SPH_LIST_BATCH_X independent gathers in flight instead of meeting the
 // record's latency inside every pair body. Words are streamed (read once).
-template <class VT, class Fetch, class Fn>
-__device__ __forceinline__ void for_pairs_x(const uint32_t* __restrict__ plist, const VT* __restrict__ view, int i,
+template <class T, class VT, class Fetch, class Fn>
+__device__ __forceinline__ void for_pairs_x(const PairRec<T>* __restrict__ plist, const VT* __restrict__ view, int i,
                                             int cnt, int cap, Fetch&& fetch, Fn&& pair) {
   using XT = decltype(fetch(0));
   constexpr int B = SPH_LIST_BATCH_X;
-  const uint32_t* __restrict__ p = plist + pair_at(i, 0, cap);
+  const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
   int k = 0;
   for (; k + B <= cnt; k += B, p += 32 * B) {
     uint32_t e[B];
     VT v[B];
     XT x[B];
 #pragma unroll
-    for (int q = 0; q < B; ++q) e[q] = __ldcs(p + 32 * q);
+    for (int q = 0; q < B; ++q) e[q] = __ldcs(&p[32 * q].e);
 #pragma unroll
     for (int q = 0; q < B; ++q) {
       v[q] = view[e[q] >> 8];
@@ -166,36 +162,67 @@ __device__ __forceinline__ void for_pairs_x(const uint32_t* __restrict__ plist, 
     for (int q = 0; q < B; ++q) pair(e[q], v[q], x[q]);
   }
   for (; k < cnt; ++k, p += 32) {
-    const uint32_t e = __ldcs(p);
+    const uint32_t e = __ldcs(&p->e);
     pair(e, view[e >> 8], fetch((int)(e >> 8)));
   }
 }
+// one 8- or 16-byte access, streamed: written once by pass A, read once by pass B
+__device__ __forceinline__ void store_pair(PairRec<float>* p, uint32_t e, float f) {
+  __stcs((uint2*)p, make_uint2(e, __float_as_uint(f)));
+}
+__device__ __forceinline__ void store_pair(PairRec<double>* p, uint32_t e, double f) {
+  const long long b = __double_as_longlong(f);
+  __stcs((uint4*)p, make_uint4((uint32_t)b, (uint32_t)(b >> 32), e, 0u));
+}
+__device__ __forceinline__ PairRec<float> load_pair(const PairRec<float>* p) {
+  const uint2 v = __ldcs((const uint2*)p);
+  return PairRec<float>{v.x, __uint_as_float(v.y)};
+}
+__device__ __forceinline__ PairRec<double> load_pair(const PairRec<double>* p) {
+  const uint4 v = __ldcs((const uint4*)p);
+  return PairRec<double>{__longlong_as_double((long long)v.x | (long long)v.y << 32), v.z, 0u};
+}
+// the target's factor of its pair records: FP32 records hold powers of h_j and
+// of the support relative to w_i = kappa h_i / 2, and 1 + rho_t,i^2/rho_t,j^2
+template <int D>
+__device__ __forceinline__ float pair_scale(float qi, float invHd) {
+  const float iw = 2.0f * invHd, iw4 = iw * iw * iw * iw;
+  return qi * (D == 2 ? iw4 : -iw4 * iw);
+}
+template <int D>
+__device__ __forceinline__ double pair_scale(double, double) { return 1.0; }
+
 // The skin list of particle i as quads of entries (split at its build, see
 // kFastBit), in the order: full quads of the inside part, full quads of the
 // outside part, what is left of each. quad(e, valid): four list words, and
 // which of them are entries (bit q; std::true_type: all). The next full quad
-// is loaded before the current one is used: its words come from DRAM, the
-// neighbours' views mostly from the caches.
+// is fetched into L2 while the current one is used: its words come from DRAM,
+// the neighbours' views mostly from the caches (holding the next quad in
+// registers instead spilled: pass A of 8,388,608 particles 1.82 ms against 1.67).
 template <class Quad>
 __device__ __forceinline__ void for_quads(const uint32_t* __restrict__ list, int i, uint32_t lc, int cap, Quad&& quad) {
-  const int n_in = list_in(lc), n_out = list_cnt(lc) - n_in, rows = list_rows(cap) >> 2;
-  const uint4* __restrict__ in = (const uint4*)(list + list_at(i, 0, cap));
-  const int qi = n_in >> 2, nq = qi + (n_out >> 2);
-  const auto at = [&](int q) { return in + (size_t)(q < qi ? q : rows - 1 - (q - qi)) * 32; };
-  uint4 ahead = make_uint4(0, 0, 0, 0);
-  if (nq > 0) ahead = __ldcs(at(0));
-  for (int q = 0; q < nq;) {
-    const uint4 w = ahead;
-    ++q;
-    if (q < nq) ahead = __ldcs(at(q));
+  const int n_in = list_in(lc), n_out = list_cnt(lc) - n_in;
+  int qi = n_in >> 2, left = qi + (n_out >> 2);
+  const uint4* __restrict__ at = (const uint4*)(list + list_at(i, 0, cap));
+  const auto last = [&] { return (const uint4*)(list + list_at(i, list_rows(cap) - 4, cap)); };
+  if (qi == 0) at = last();
+  while (left > 0) {
+    const uint4 w = __ldcs(at);
+    at += qi > 0 ? 32 : -32;
+    if (--qi == 0) at = last();
+    --left;
+    if (left > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(at));
     quad(w, std::true_type{});
   }
 #pragma unroll 1
   for (int part = 0; part < 2; ++part) {
-    const int left = (part ? n_out : n_in) & 3;
-    if (left) quad(__ldcs(part ? at(nq) : in + (size_t)qi * 32), part ? (0xF0u >> left) & 0xFu : (1u << left) - 1u);
+    const int m = (part ? n_out : n_in) & 3;
+    if (m)
+      quad(__ldcs((const uint4*)(list + list_at(i, part ? list_rows(cap) - 4 - (n_out & ~3) : n_in & ~3, cap))),
+           part ? (0xF0u >> m) & 0xFu : (1u << m) - 1u);
   }
 }
+
 // row of entry k of a list whose first n_in entries sit in rows 0.. and the
 // rest in the last row, the one before, ...
 __device__ __forceinline__ int list_row(int k, int n_in, int cap) {
@@ -1026,7 +1053,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
                                                 T* __restrict__ rho_out, Partial* __restrict__ partials,
                                                 Scalars* __restrict__ scal, unsigned* __restrict__ ticket,
                                                 int* __restrict__ err, int advance, int* __restrict__ dbg_count,
-                                                long long* __restrict__ dbg_sum, uint32_t* __restrict__ plist,
+                                                long long* __restrict__ dbg_sum, PairRec<T>* __restrict__ plist,
                                                 uint32_t* __restrict__ pcount, const double* __restrict__ dt_fix,
                                                 double* __restrict__ dt_rec, const LL4* __restrict__ X0,
                                                 const LL4* __restrict__ X1, Geom<T> geo,
@@ -1083,7 +1110,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     long long sd = 0, sf = 0;
     const uint32_t lc = lcount[i];
     const int cnt = list_cnt(lc);
-    uint32_t* __restrict__ pw = plist + pair_at(i, 0, cap);  // this step's force pairs, for pass B
+    PairRec<T>* __restrict__ pw = plist + pair_at(i, 0, cap);  // this step's force pairs, for pass B
     // FP32: the listed entries two at a time, every FP32 operation on both at
     // once, on exact differences throughout (a coarse screen first saved the
     // conversions but evaluated the passing two thirds twice). The kernel's
@@ -1103,7 +1130,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       const float hd2 = 4.0f * wi * wi;  // (kappa h_i)^2
       const float sq = GENERAL ? sP0 * qi : 1.0f + sigma;
       const uint32_t own = ((uint32_t)i << 8) | ci;
-      float2 ds2 = both(0.0f), dq2 = both(0.0f), ax2 = both(0.0f), ay2 = both(0.0f), az2 = both(0.0f);
+      uint32_t counts = 0;  // force pairs, of them other colours << 16
+      float dq = 0.0f;
+      float2 ax2 = both(0.0f), ay2 = both(0.0f), az2 = both(0.0f);
       auto sums = [&](auto stagedc) {
         constexpr bool ST = decltype(stagedc)::value;  // e = (rank << 8 | colour), view from shared memory
         auto load = [&](uint32_t e) -> VT { return ST ? sview[stage_rank(e)] : view[e >> 8]; };
@@ -1125,8 +1154,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
           const float2 r = mul2(r2, rsqrt2(r2));
           if (!GENERAL) {  // W ~ (1 - q)^4 (1 + 4 q); q = 1 - u where u > 0
             const float2 u = max2(fma2(r, id2, one2), 0.0f), u2 = mul2(u, u), u4 = mul2(u2, u2);
-            ds2 = add2(ds2, u4);
-            dq2 = fma2(u4, mul2(r, id2), dq2);
+            const float2 m = mul2(u4, mul2(r, id2));
+            dsum += u4.x + u4.y;
+            dq += m.x + m.y;
           }
           const float2 nH = rcp2(make_float2(-H.x, -H.y));
           const float2 u = max2(fma2(r, nH, one2), 0.0f), g = mul2(nH, w2), g2 = mul2(g, g), g4 = mul2(g2, g2);
@@ -1134,35 +1164,36 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
           const float2 t = mul2(wj, iw2), t2 = mul2(t, t);
           const float2 ts = D == 2 ? fma2(t2, t2, one2) : fma2(mul2(t2, t2), t2, one2);  // 1 + rho_t,i^2 / rho_t,j^2
           const bool o0 = ((e0 ^ own) & 0xFFu) != 0, o1 = ((e1 ^ own) & 0xFFu) != 0;
-          float2 s = mul2(ts, w);
+          const float2 tw = mul2(ts, w);
+          float2 s;
           if (GENERAL) {
             const float2 pp = make_float2(pc[e0 >> 8], pc[e1 >> 8]);
             s = mul2(fma2(make_float2(o0 ? sq : 0.0f, o1 ? sq : 0.0f), ts, add2(both(Pi), pp)), w);
           } else {
-            s = mul2(s, make_float2(o0 ? sq : 1.0f, o1 ? sq : 1.0f));
+            s = mul2(tw, make_float2(o0 ? sq : 1.0f, o1 ? sq : 1.0f));
           }
           ax2 = fma2(s, dx, ax2);
           ay2 = fma2(s, dy, ay2);
           if (D == 3) az2 = fma2(s, dz, az2);
-          auto push = [&](uint32_t e, bool inside, bool other) {
+          auto push = [&](uint32_t e, bool inside, bool other, float f) {
             if (inside && !(ST ? (e & kStageSelf) != 0 : e == own)) {
-              SPH_PLIST_STORE(pw, ST ? ((uint32_t)__ldg(sjb + stage_rank(e)) << 8) | (e & 0xFFu) : e);
+              store_pair(pw, ST ? ((uint32_t)__ldg(sjb + stage_rank(e)) << 8) | (e & 0xFFu) : e, f);
               pw += 32;
-              ++nf;
-              ni += other;
+              counts += other ? 0x10001u : 1u;  // at most 2^15 - 1 pairs
             }
           };
-          push(e0, f0, o0);
-          push(e1, f1, o1);
+          push(e0, f0, o0, tw.x);
+          push(e1, f1, o1, tw.y);
         };
         for_twos(ST ? llist : list, i, lc, cap, ST ? ci | kStageSelf : own, load, two);
       };
       if (STG && staged) sums(std::integral_constant<bool, STG>{});
       else sums(std::false_type{});
-      dsum = (ds2.x + ds2.y) - 4.0f * (dq2.x + dq2.y);  // dq2 holds the terms in -q
+      dsum -= 4.0f * dq;  // dq holds the terms in -q
+      nf = counts & 0xFFFFu;
+      ni = counts >> 16;
       // back to view units: w_i^-(D+2), and P0/rho_t,i^2 (or the pressures themselves)
-      const float iw = 2.0f * invHd, iw4 = iw * iw * iw * iw;
-      const float back = F.vscale * (GENERAL ? 1.0f : P.P0 * qi) * (D == 2 ? iw4 : -iw4 * iw);
+      const float back = F.vscale * pair_scale<D>(GENERAL ? 1.0f : P.P0 * qi, invHd);
       ax = (ax2.x + ax2.y) * back;
       ay = (ay2.x + ay2.y) * back;
       az = (az2.x + az2.y) * back;
@@ -1171,6 +1202,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // criteria on every entry (FP64 path with current FP32 views: on those that
     // pass a screen in FP32, for_skin_list_s32)
     constexpr bool S32_OK = std::is_same<T, double>::value && !GENERAL && !DBG && !SURF;
+    const T iscale = T(1) / pair_scale<D>(qi, invHd);
     auto pair = [&](uint32_t e, const VT& vj) {
       const int j = (int)(e >> 8);
       const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
@@ -1205,7 +1237,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
         ax += s * dx;
         ay += s * dy;
         az += s * dz;
-        SPH_PLIST_STORE(pw, e);
+        store_pair(pw, e, (qi + qj) * w * iscale);
         pw += 32;
         ++nf;
         ni += other;
@@ -1391,7 +1423,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
                                                 typename ViewOf<T>::type* __restrict__ w1,
                                                 const typename ViewOf<T>::type* __restrict__ vbuild,
                                                 LL4* __restrict__ X0, LL4* __restrict__ X1,
-                                                const uint32_t* __restrict__ plist,
+                                                const PairRec<T>* __restrict__ plist,
                                                 const uint32_t* __restrict__ pcount, int cap,
                                                 const V4<T>* __restrict__ acc, Frame<T> F, Phys<T> P, Geom<T> geo,
                                                 const Scalars* __restrict__ scal, V4<T>* __restrict__ visc_out,
@@ -1408,38 +1440,84 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
     const VT* __restrict__ view = vp ? v1 : v0;
     const VT vi = view[i];
     const T hv = view_h(F, vi);
-    const T qv = F.qv;
-    const T inv_tau_v = P.inv_tau * qv;
-    const T qi = inv_rho_t2<D, T>(hv, inv_tau_v);
+    const T qi = inv_rho_t2<D, T>(hv, P.inv_tau * F.qv);
     const V4<T> ai = acc[i];
-    const T half_kappa = T(0.5) * P.kappa;
     T bx = 0, by = 0, bz = 0;
-    // this step's pairs as pass A compacted them (same positions); the force
-    // support is tested again on the exact vectors
+    // this step's pairs as pass A left them: the geometry in a factor per pair,
+    // so only the neighbour's acceleration is gathered and no distance, root or
+    // kernel value is computed again. FP32, 8,388,608 particles in 3D: 1.40 ->
+    // 0.86 ms, and pass A, which writes the factor, 1.59 -> 1.65; FP64, where the
+    // FP64 pipe bounds both passes, 300,007 in 3D: 1.40 -> 0.43 ms.
     const int cnt = (int)pcount[i];
-    for_pairs_x(plist, view, i, cnt, cap, [&](int j) { return acc[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& aj) {
-      const int j = (int)(e >> 8);
-      const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
-      const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
-      const T r2 = dx * dx + dy * dy + dz * dz;
-      const T hj = view_h(F, vj);
-      const T Hf = half_kappa * (hv + hj);
-      if (!(r2 < Hf * Hf) || j == i) return;
-      const T gs = ai.w + aj.w;
-      const T hm = gs > T(0) ? T(2) * ai.w * aj.w * drcp<T>(gs) : T(0);
-      const T invH = drcp<T>(Hf);
-      const T q = r2 > T(0) ? pair_r<T>(r2) * invH : T(0);
-      const T u = T(1) - q;
-      const T invH2 = invH * invH;
-      const T w = u * u * u * (D == 2 ? invH2 * invH2 : invH2 * invH2 * invH);
-      const T s = hm * (qi + inv_rho_t2<D, T>(hj, inv_tau_v)) * w;
-      bx += s * (ai.x - aj.x);
-      by += s * (ai.y - aj.y);
-      bz += s * (ai.z - aj.z);
-    });
+    const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
+    if constexpr (std::is_same<T, float>::value) {
+      // two pairs per instruction; sums of (a_j - a_i), factor gi gj / (gi + gj)
+      const float2 g2 = both(ai.w), nx2 = both(-ai.x), ny2 = both(-ai.y), nz2 = both(-ai.z);
+      float2 bx2 = both(0.0f), by2 = both(0.0f), bz2 = both(0.0f);
+      auto two = [&](const PairRec<T>& r0, const V4<T>& a0, const PairRec<T>& r1, const V4<T>& a1) {
+        const float2 gj = make_float2(a0.w, a1.w);
+        float2 gs = add2(g2, gj);
+        gs = make_float2(fmaxf(gs.x, 1e-37f), fmaxf(gs.y, 1e-37f));  // both zero: 0 / 1e-37
+        const float2 s = mul2(mul2(mul2(g2, rcp2(gs)), gj), make_float2(r0.f, r1.f));
+        bx2 = fma2(s, add2(make_float2(a0.x, a1.x), nx2), bx2);
+        by2 = fma2(s, add2(make_float2(a0.y, a1.y), ny2), by2);
+        if (D == 3) bz2 = fma2(s, add2(make_float2(a0.z, a1.z), nz2), bz2);
+      };
+      constexpr int B = SPH_PASSB_BATCH;
+      int k = 0;
+      PairRec<T> ahead[B];
+      if (cnt >= B)
+#pragma unroll
+        for (int q = 0; q < B; ++q) ahead[q] = load_pair(p + 32 * q);
+      for (; k + B <= cnt; k += B) {
+        PairRec<T> r[B];
+        V4<T> a[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q) r[q] = ahead[q];
+#pragma unroll
+        for (int q = 0; q < B; ++q) a[q] = acc[r[q].e >> 8];
+        p += 32 * B;
+        if (k + 2 * B <= cnt)
+#pragma unroll
+          for (int q = 0; q < B; ++q) ahead[q] = load_pair(p + 32 * q);
+#pragma unroll
+        for (int q = 0; q < B; q += 2) two(r[q], a[q], r[q + 1], a[q + 1]);
+      }
+#pragma unroll 1
+      for (; k < cnt; k += 2, p += 64) {
+        const PairRec<T> r0 = load_pair(p);
+        PairRec<T> r1{r0.e, 0.0f};  // no second pair: a zero factor
+        if (k + 1 < cnt) r1 = load_pair(p + 32);
+        const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
+        two(r0, a0, r1, a1);
+      }
+      bx = -2.0f * (bx2.x + bx2.y);
+      by = -2.0f * (by2.x + by2.y);
+      bz = -2.0f * (bz2.x + bz2.y);
+    } else {
+      auto pair = [&](const PairRec<T>& r, const V4<T>& aj) {
+        const T gs = ai.w + aj.w;
+        const T s = gs > T(0) ? T(2) * ai.w * aj.w * drcp<T>(gs) * r.f : T(0);
+        bx += s * (ai.x - aj.x);
+        by += s * (ai.y - aj.y);
+        bz += s * (ai.z - aj.z);
+      };
+      int k = 0;
+      for (; k + 2 <= cnt; k += 2, p += 64) {
+        const PairRec<T> r0 = load_pair(p), r1 = load_pair(p + 32);
+        const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
+        pair(r0, a0);
+        pair(r1, a1);
+      }
+      if (k < cnt) {
+        const PairRec<T> r0 = load_pair(p);
+        pair(r0, acc[r0.e >> 8]);
+      }
+    }
     // dW/dr / r = -20 alpha (1-q)^3 / H^(D+2); view lengths -> physical
     const T iq = F.inv_qv;
-    const T km = T(-20) * P.alpha * (D == 2 ? iq * iq * iq * iq : iq * iq * iq * iq * iq);
+    const T km = T(-20) * P.alpha * (D == 2 ? iq * iq * iq * iq : iq * iq * iq * iq * iq) *
+                 pair_scale<D>(qi, T(1) / (P.kappa * hv));
     bx *= km;
     by *= km;
     bz *= km;
@@ -1656,7 +1734,7 @@ cudaError_t launch_pass_a(const DevState& S, const Frame<T>& F, const Phys<T>& P
                                               S.meta[0], S.meta[1], S.pid[0], S.pid[1], S.list, S.lcount, S.cap, \
                                               F, P,                                                             \
                                               pc, (V4<T>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err,   \
-                                              f.advance, S.dbg_count, S.dbg_sum, S.plist, S.pcount, f.dt_fix,     \
+                                              f.advance, S.dbg_count, S.dbg_sum, (PairRec<T>*)S.plist, S.pcount, f.dt_fix,     \
                                               f.dt_rec, (const LL4*)S.X[0], (const LL4*)S.X[1], geo, S.llist,     \
                                               S.scount, S.sj, v32, f32)
 #define SPH_PASS_A(GEN, DBG)           \
@@ -1672,7 +1750,7 @@ cudaError_t launch_pass_a(const DevState& S, const Frame<T>& F, const Phys<T>& P
           <<<grid_for(S.n, kStageBlock), kStageBlock, kStageCap * sizeof(int4), st>>>(
               S.n, S.ctl, (const int4*)S.view[0], (const int4*)S.view[1], S.meta[0], S.meta[1], S.pid[0], S.pid[1],
               S.list, S.lcount, S.cap, F, P, pc, (V4<float>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err,
-              f.advance, S.dbg_count, S.dbg_sum, S.plist, S.pcount, f.dt_fix, f.dt_rec, (const LL4*)S.X[0],
+              f.advance, S.dbg_count, S.dbg_sum, (PairRec<T>*)S.plist, S.pcount, f.dt_fix, f.dt_rec, (const LL4*)S.X[0],
               (const LL4*)S.X[1], geo, S.llist, S.scount, S.sj, nullptr, Frame<float>{});
       return cudaGetLastError();
     }
@@ -1705,7 +1783,7 @@ cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P
   unsigned long long* wm = (unsigned long long*)&S.scal->wall_moved;
   (tb == 128 ? k_pass_b<D, T, 128> : k_pass_b<D, T, 256>)<<<gb, tb, 0, st>>>(
       S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], (VT*)S.view[0], (VT*)S.view[1], (const VT*)S.vbuild,
-      (LL4*)S.X[0], (LL4*)S.X[1], S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
+      (LL4*)S.X[0], (LL4*)S.X[1], (const PairRec<T>*)S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
       f.record ? (V4<T>*)S.visc : nullptr, S.err, wm, f.move, S.meta[0], S.meta[1],
       (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0, f.f32 ? f.f32->c2w : 0.0f);
   return cudaGetLastError();
