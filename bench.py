@@ -67,7 +67,7 @@ ALG_BYTES_FP64 = {"cells": 92, "pass_a": 56, "pass_b": 83}
 # make_view, list_build (predicated: they exit at once unless the list is
 # rebuilt); pass A; pass B; with the staged pass A one more predicated
 # rebuild kernel (the blocks' neighbour sets)
-KERNELS_PER_STEP = 12
+KERNELS_PER_STEP = 7
 # pair arithmetic (FP32 flop, counted from the equations as the kernels evaluate
 # them): distance of a pair 10 (differences, squared norm, root), density term 8
 # (Eq. density_sum), pressure + surface-tension term 30 (Eqs.

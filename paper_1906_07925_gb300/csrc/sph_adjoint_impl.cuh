@@ -757,7 +757,7 @@ template <int D, class T>
 cudaError_t launch_bwd_step(const DevState& S, const Frame<T>& F, const Phys<T>& P, const Geom<T>& geo,
                             const AdjBufs<T>& B, int recomputed_dt, int general_eos, cudaStream_t st) {
   using VT = typename ViewOf<T>::type;
-  const int tb = 256, gb = grid_for(S.n, tb);
+  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 256, gb = grid_for(S.n, tb);
   if (S.n <= 0) return cudaSuccess;
   const VT* w0 = (const VT*)S.view[0];
   const VT* w1 = (const VT*)S.view[1];
@@ -783,7 +783,7 @@ template <int D, class T>
 cudaError_t launch_objective(const DevState& S, const Frame<T>& F, const Phys<T>& P, const Geom<T>& geo,
                              const AdjBufs<T>& B, double wd, double lambda, cudaStream_t st) {
   using VT = typename ViewOf<T>::type;
-  const int tb = 256, gb = grid_for(S.n, tb);
+  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 256, gb = grid_for(S.n, tb);
   if (S.n <= 0) return cudaSuccess;
   const VT* w0 = (const VT*)S.view[0];
   const VT* w1 = (const VT*)S.view[1];

@@ -208,14 +208,13 @@ sph_status launch_step(sph_handle* h, int record, int force_rebuild = 0, cudaEve
   f.surface = h->has_surface ? 1 : 0;
   cudaError_t e = cudaSuccess;
   if (ev) e = cudaEventRecord(ev[0], h->stream);
-  if (e == cudaSuccess) e = launch_gate(S, force_rebuild, h->stream);
   if (e == cudaSuccess) {
     if (h->dim == 2)
-      e = f64 ? launch_rebuild<2, double>(S, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
-              : launch_rebuild<2, float>(S, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
+      e = f64 ? launch_rebuild<2, double>(S, force_rebuild, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
+              : launch_rebuild<2, float>(S, force_rebuild, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
     else
-      e = f64 ? launch_rebuild<3, double>(S, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
-              : launch_rebuild<3, float>(S, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
+      e = f64 ? launch_rebuild<3, double>(S, force_rebuild, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
+              : launch_rebuild<3, float>(S, force_rebuild, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
   }
   if (ev && e == cudaSuccess) e = cudaEventRecord(ev[1], h->stream);
   if (e == cudaSuccess) {
@@ -259,14 +258,14 @@ sph_status launch_evaluate(sph_handle* h, int nbr_debug) {
   const bool f64 = h->prec == SPH_PREC_FP64;
   f.geo = f64 ? (const void*)&h->geod : (const void*)&h->geof;
   f.surface = h->has_surface ? 1 : 0;
-  cudaError_t e = launch_gate(S, 1, h->stream);
-  if (e == cudaSuccess) {
+  cudaError_t e = cudaSuccess;
+  {
     if (h->dim == 2)
-      e = f64 ? launch_rebuild<2, double>(S, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
-              : launch_rebuild<2, float>(S, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
+      e = f64 ? launch_rebuild<2, double>(S, 1, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
+              : launch_rebuild<2, float>(S, 1, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
     else
-      e = f64 ? launch_rebuild<3, double>(S, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
-              : launch_rebuild<3, float>(S, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
+      e = f64 ? launch_rebuild<3, double>(S, 1, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
+              : launch_rebuild<3, float>(S, 1, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
   }
   if (e == cudaSuccess) {
     if (h->dim == 2)
@@ -459,14 +458,14 @@ sph_status reverse_setup(sph_handle* h, bool forward, const double* dt_fix) {
   const bool f64 = h->prec == SPH_PREC_FP64;
   // without `forward` (the objective at x_K) the list is rebuilt only if the
   // last step asked for it: otherwise it still holds every pair of x_K
-  cudaError_t e = launch_gate(S, forward ? 1 : 0, h->stream);
-  if (e == cudaSuccess) {
+  cudaError_t e = cudaSuccess;
+  {
     if (h->dim == 2)
-      e = f64 ? launch_rebuild<2, double>(S, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
-              : launch_rebuild<2, float>(S, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
+      e = f64 ? launch_rebuild<2, double>(S, forward ? 1 : 0, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
+              : launch_rebuild<2, float>(S, forward ? 1 : 0, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
     else
-      e = f64 ? launch_rebuild<3, double>(S, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
-              : launch_rebuild<3, float>(S, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
+      e = f64 ? launch_rebuild<3, double>(S, forward ? 1 : 0, h->Gdw, h->Fd, h->geod, h->par.kappa, h->stream, &h->Gf, &h->Ff)
+              : launch_rebuild<3, float>(S, forward ? 1 : 0, h->Gf, h->Ff, h->geof, (float)h->par.kappa, h->stream);
   }
   if (forward && e == cudaSuccess) {
     if (h->dim == 2)
@@ -492,7 +491,7 @@ sph_status ensure_adj(sph_handle* h) {
   if (h->adj.ready) return SPH_OK;
   const size_t N = (size_t)h->n, d = (size_t)h->dim;
   const size_t t1 = h->prec == SPH_PREC_FP64 ? 8 : 4, v4 = 4 * t1;
-  const size_t nb = N / 256 + 2;
+  const size_t nb = N / 32 + 2;  // blocks of at least 32 particles
   auto& a = h->adj;
   uint8_t* p = nullptr;
   SPH_TRY(grab(h, p, N * 32)); a.xb = p;
@@ -809,14 +808,15 @@ static sph_status create_impl(sph_handle* h, const sph_domain* dom, const sph_fi
   SPH_TRY(grab(h, S.cnt, (size_t)S.total_cells));
   h->cells_cap = S.total_cells;
   SPH_TRY(grab(h, S.cstart, (size_t)S.total_cells + 1));
-  SPH_TRY(grab(h, S.scan_part, (size_t)S.total_cells / 4096 + 2));
-  SPH_TRY(grab(h, S.partials, partial_slots(N, 128)));
+  SPH_TRY(grab(h, S.scan_part, scan_tiles(S.total_cells) + 1));
+  SPH_TRY(grab(h, S.partials, partial_slots(N, 32)));
   SPH_TRY(grab(h, S.scal, 2));
   SPH_TRY(grab(h, S.ctl, 1));
-  SPH_TRY(grab(h, S.tickets, ticket_slots(N, 128)));
+  SPH_TRY(grab(h, S.tickets, ticket_slots(N, 32)));
   SPH_TRY(grab(h, S.err, 1));
   SPH_CUDA(h, cudaMemsetAsync(S.cnt, 0, sizeof(uint32_t) * S.total_cells, h->stream));
-  SPH_CUDA(h, cudaMemsetAsync(S.tickets, 0, sizeof(unsigned) * ticket_slots(N, 128), h->stream));
+  SPH_CUDA(h, cudaMemsetAsync(S.scan_part, 0, sizeof(uint32_t) * scan_tiles(S.total_cells), h->stream));
+  SPH_CUDA(h, cudaMemsetAsync(S.tickets, 0, sizeof(unsigned) * ticket_slots(N, 32), h->stream));
   SPH_CUDA(h, cudaMemsetAsync(S.err, 0, sizeof(int), h->stream));
   SPH_CUDA(h, cudaMemsetAsync(S.scal, 0, sizeof(Scalars) * 2, h->stream));
   SPH_CUDA(h, cudaMemsetAsync(S.lcount, 0, sizeof(uint32_t) * N, h->stream));
@@ -949,13 +949,14 @@ sph_status sph_set_tuning(sph_handle* h, int32_t pass_threads, double cell_facto
       uint32_t *cnt, *cstart, *part;
       SPH_TRY(grab(h, cnt, (size_t)cells));
       SPH_TRY(grab(h, cstart, (size_t)cells + 1));
-      SPH_TRY(grab(h, part, (size_t)cells / 4096 + 2));
+      SPH_TRY(grab(h, part, scan_tiles(cells) + 1));
       h->S.cnt = cnt;
       h->S.cstart = cstart;
       h->S.scan_part = part;
       h->cells_cap = cells;
     }
     SPH_CUDA(h, cudaMemsetAsync(h->S.cnt, 0, sizeof(uint32_t) * cells, h->stream));
+    SPH_CUDA(h, cudaMemsetAsync(h->S.scan_part, 0, sizeof(uint32_t) * scan_tiles(cells), h->stream));
     h->hg = hg;
     h->S.total_cells = cells;
     h->par.cell_factor = cell_factor;

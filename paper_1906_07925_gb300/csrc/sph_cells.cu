@@ -2,13 +2,15 @@
 //
 // At a neighbour-list rebuild, particles are ordered by cell key with a
 // counting sort over the dense key range: warp-aggregated atomic counts per
-// cell, an exclusive scan of the counts (which is also the cell-start table the
-// list build reads), an atomic scatter that counts each cell back down to zero,
-// and a gather that orders each cell by particle id (so the order is a function
-// of the keys alone: by key, then id) while it moves the particle state into
-// the other buffer. Every
-// kernel here returns at once on steps without a rebuild (ctl->rebuild == 0),
-// so one captured graph serves every step.
+// cell and per tile of cells (k_rekey, sph_step_impl.cuh), an exclusive scan of
+// the counts (which is also the cell-start table the list build reads), an
+// atomic scatter that counts each cell back down to zero, and a gather that
+// orders each cell by particle id (so the order is a function of the keys
+// alone: by key, then id) while it moves the particle state into the other
+// buffer and makes the views (k_gather_view, sph_step_impl.cuh). Every kernel
+// here returns at once on steps without a rebuild (ctl->rebuild == 0), so one
+// captured graph serves every step; an idle kernel of a graph still takes
+// 1.1 us, so there are as few of them as grid-wide dependencies allow.
 #include "sph_internal.h"
 
 namespace sph {
@@ -16,48 +18,22 @@ namespace sph {
 namespace {
 
 constexpr int kScanThreads = 256;
-constexpr int kScanItems = 16;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-__global__ void k_gate(StepCtl* __restrict__ ctl, int force) {
-  StepCtl c = *ctl;
-  c.vp ^= 1;
-  if (c.need_rebuild || force) {
-    c.rebuild = 1;
-    c.buf ^= 1;
-    c.need_rebuild = 0;
-    c.rebuilds += 1;
-    c.lmax = 0;
-  } else {
-    c.rebuild = 0;
-  }
-  *ctl = c;
-}
+constexpr int kScanItems = kScanTile / kScanThreads;
+// up to this many tiles every block of k_scan_down adds up the tiles before its
+// own (8 sums per thread at most); beyond, one block scans them first
+constexpr int kScanOwn = 2048;
 
 __global__ void k_request_rebuild(StepCtl* __restrict__ ctl) { ctl->need_rebuild = 1; }
 __global__ void k_write_ctl(StepCtl* __restrict__ ctl, StepCtl v) { *ctl = v; }
-
-__global__ void __launch_bounds__(256) k_count(int n, const StepCtl* __restrict__ ctl, const uint32_t* __restrict__ key,
-                                               uint32_t* __restrict__ cnt) {
-  if (!ctl->rebuild) return;
-  for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
-    const int i = b0 + threadIdx.x;
-    const bool active = i < n;
-    const unsigned mask = __ballot_sync(0xffffffffu, active);
-    if (!active) continue;
-    const uint32_t k = key[i];
-    const unsigned peers = __match_any_sync(mask, k);
-    const int leader = __ffs(peers) - 1;
-    if ((int)(threadIdx.x & 31) == leader) atomicAdd(&cnt[k], (uint32_t)__popc(peers));
-  }
-}
 
 __global__ void __launch_bounds__(256) k_scatter(int n, const StepCtl* __restrict__ ctl,
                                                  const uint32_t* __restrict__ key,
                                                  const uint32_t* __restrict__ cstart,
                                                  uint32_t* __restrict__ cnt,
-                                                 uint32_t* __restrict__ slots) {
+                                                 uint32_t* __restrict__ slots, uint32_t* __restrict__ part, int nb) {
   if (!ctl->rebuild) return;
+  // the tile counts are used up: zero for the next rebuild
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) part[b] = 0u;
   for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
     const int i = b0 + threadIdx.x;
     const bool active = i < n;
@@ -75,30 +51,7 @@ __global__ void __launch_bounds__(256) k_scatter(int n, const StepCtl* __restric
   }
 }
 
-// per block: sum of a tile of kScanTile counts
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const StepCtl* __restrict__ ctl,
-                                                              const uint32_t* __restrict__ in,
-                                                              uint32_t n, uint32_t* __restrict__ part) {
-  if (!ctl->rebuild) return;
-  __shared__ uint32_t red[kScanThreads / 32];
-  size_t base = (size_t)blockIdx.x * kScanTile;
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < kScanItems; ++k) {
-    size_t idx = base + (size_t)k * kScanThreads + threadIdx.x;
-    if (idx < n) s += in[idx];
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < kScanThreads / 32 ? red[threadIdx.x] : 0;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
-  }
-}
-
-// exclusive scan of the block sums, in place (one block of 1024 threads)
+// exclusive scan of the tile counts, in place (one block of 1024 threads)
 __global__ void __launch_bounds__(1024) k_scan_top(const StepCtl* __restrict__ ctl, uint32_t* __restrict__ part,
                                                    int nb) {
   if (!ctl->rebuild) return;
@@ -138,11 +91,18 @@ __global__ void __launch_bounds__(1024) k_scan_top(const StepCtl* __restrict__ c
 // exclusive scan of each tile plus its block offset; out has n + 1 entries
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const StepCtl* __restrict__ ctl,
                                                             const uint32_t* __restrict__ in, uint32_t n,
-                                                            const uint32_t* __restrict__ part,
+                                                            const uint32_t* __restrict__ part, int scanned,
                                                             uint32_t* __restrict__ out) {
   if (!ctl->rebuild) return;
-  __shared__ uint32_t wtot[kScanThreads / 32];
+  __shared__ uint32_t wtot[kScanThreads / 32], wpre[kScanThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // the counts before this tile: scanned already, or added up here
+  uint32_t pre = 0;
+  if (!scanned) {
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) pre += part[b];
+    pre = __reduce_add_sync(0xffffffffu, pre);
+    if (lane == 0) wpre[w] = pre;
+  }
   // each warp owns kScanItems * 32 consecutive entries of the tile
   size_t wbase = (size_t)blockIdx.x * kScanTile + (size_t)w * kScanItems * 32;
   uint32_t v[kScanItems];
@@ -161,7 +121,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const StepCtl* __res
   }
   if (lane == 0) wtot[w] = run;
   __syncthreads();
-  uint32_t off = part[blockIdx.x];
+  uint32_t start = 0;
+  if (scanned) start = part[blockIdx.x];
+  else
+    for (int q = 0; q < kScanThreads / 32; ++q) start += wpre[q];
+  uint32_t off = start;
   for (int q = 0; q < w; ++q) off += wtot[q];
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) {
@@ -169,37 +133,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const StepCtl* __res
     if (idx < n) out[idx] = off + v[k];
   }
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) {
-    uint32_t tot = part[blockIdx.x];
+    uint32_t tot = start;
     for (int q = 0; q < kScanThreads / 32; ++q) tot += wtot[q];
     out[n] = tot;
-  }
-}
-
-struct alignas(32) State64 {
-  long long x, y, z, w;
-};
-
-// slot s of the scatter holds old index i; its rank among the cell's members by
-// particle id gives its destination (cells ordered by key, each cell by
-// particle id), where the state is copied
-__global__ void __launch_bounds__(256) k_stable_gather(
-    int n, const StepCtl* __restrict__ ctl, const uint32_t* __restrict__ slots, const uint32_t* __restrict__ key,
-    const uint32_t* __restrict__ cstart, State64* __restrict__ X0, State64* __restrict__ X1,
-    uint32_t* __restrict__ m0, uint32_t* __restrict__ m1, uint32_t* __restrict__ p0, uint32_t* __restrict__ p1) {
-  if (!ctl->rebuild) return;
-  const int nb = ctl->buf;  // new buffer; the old order lives in the other one
-  const uint32_t* __restrict__ pold = nb ? p0 : p1;
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    const uint32_t i = slots[s];
-    const uint32_t k = key[i];
-    const uint32_t id = pold[i];
-    const uint32_t b = cstart[k], e = cstart[k + 1];
-    uint32_t rank = 0;
-    for (uint32_t t = b; t < e; ++t) rank += pold[slots[t]] < id;
-    const uint32_t d = b + rank;
-    (nb ? X1 : X0)[d] = (nb ? X0 : X1)[i];
-    (nb ? m1 : m0)[d] = (nb ? m0 : m1)[i];
-    (nb ? p1 : p0)[d] = (nb ? p0 : p1)[i];
   }
 }
 
@@ -228,11 +164,6 @@ __global__ void __launch_bounds__(256) k_get_colors(int n, const StepCtl* __rest
 
 }  // namespace
 
-cudaError_t launch_gate(const DevState& S, int force, cudaStream_t st) {
-  k_gate<<<1, 1, 0, st>>>(S.ctl, force);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_write_ctl(const DevState& S, const StepCtl& v, cudaStream_t st) {
   k_write_ctl<<<1, 1, 0, st>>>(S.ctl, v);
   return cudaGetLastError();
@@ -260,15 +191,11 @@ cudaError_t build_cells(const DevState& S, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int tb = 256;
   const int gb = rebuild_grid(n, tb, 8);
-  k_count<<<gb, tb, 0, st>>>(n, S.ctl, S.key, S.cnt);
   const uint32_t m = S.total_cells;
-  const int nb = (int)((m + kScanTile - 1) / kScanTile);
-  k_scan_reduce<<<nb, kScanThreads, 0, st>>>(S.ctl, S.cnt, m, S.scan_part);
-  k_scan_top<<<1, 1024, 0, st>>>(S.ctl, S.scan_part, nb);
-  k_scan_down<<<nb, kScanThreads, 0, st>>>(S.ctl, S.cnt, m, S.scan_part, S.cstart);
-  k_scatter<<<gb, tb, 0, st>>>(n, S.ctl, S.key, S.cstart, S.cnt, S.tmp);
-  k_stable_gather<<<gb, tb, 0, st>>>(n, S.ctl, S.tmp, S.key, S.cstart, (State64*)S.X[0], (State64*)S.X[1],
-                                     S.meta[0], S.meta[1], S.pid[0], S.pid[1]);
+  const int nb = (int)scan_tiles(m), scanned = nb > kScanOwn;
+  if (scanned) k_scan_top<<<1, 1024, 0, st>>>(S.ctl, S.scan_part, nb);
+  k_scan_down<<<nb, kScanThreads, 0, st>>>(S.ctl, S.cnt, m, S.scan_part, scanned, S.cstart);
+  k_scatter<<<gb, tb, 0, st>>>(n, S.ctl, S.key, S.cstart, S.cnt, S.tmp, S.scan_part, nb);
   return cudaGetLastError();
 }
 

@@ -106,7 +106,7 @@ struct Phys {
 // FP64 path fills min_rc_a and err_max with values; the FP32 path names the
 // particles they belong to (r_c and |a|, rho and rho_t: exact FP32 values) and
 // divides once, at the end.
-constexpr int kPartialGroup = 128;
+constexpr int kPartialGroup = 512;
 struct Partial {
   double min_rc_a, max_a, sum_rho, err_l2, err_max;
   long long ipairs, fpairs;
@@ -114,6 +114,7 @@ struct Partial {
   long long amin;      // index (current order) of min_rc_a; -1: none
   float rc, an;        // FP32 path: r_c and |a| of particle amin
   float er, et;        // FP32 path: rho and rho_t where |rho / rho_t - 1| is largest (et = 0: none)
+  float ma, pad_;      // FP32 path: the largest |a|
 };
 // partials of the blocks and of their groups for n particles at >= `threads` per block
 constexpr size_t partial_slots(size_t n, int threads) {

@@ -27,7 +27,7 @@ struct DevState {
   uint32_t* tmp = nullptr;               // scatter slots
   uint32_t* cnt = nullptr;               // per-cell counters (all zero between rebuilds)
   uint32_t* cstart = nullptr;            // exclusive prefix of cell counts, total+1 entries
-  uint32_t* scan_part = nullptr;
+  uint32_t* scan_part = nullptr;         // per-tile counters (all zero between rebuilds)
   uint32_t total_cells = 0;
   uint32_t* list = nullptr;              // skin lists, entries (j << 8 | colour_j), see list_at
   uint32_t* lcount = nullptr;            // entries per particle; bit 31: FP32 coarse test exact
@@ -79,14 +79,15 @@ inline size_t pair_bytes(size_t n, int cap, bool fp64) {
   return (n + 31) / 32 * 32 * (size_t)cap * (fp64 ? sizeof(PairRec<double>) : sizeof(PairRec<float>));
 }
 
-// per-step gate: flip the view buffer; start a list rebuild (flip the state
-// buffer) when pass B asked for one or `force` is set
-cudaError_t launch_gate(const DevState& S, int force, cudaStream_t st);
+// cells per tile of the counting sort's scan, and the tiles of a grid
+constexpr int kScanTile = 4096;
+constexpr size_t scan_tiles(size_t cells) { return (cells + kScanTile - 1) / kScanTile; }
+
 // the next step rebuilds the list (after set-up or a diagnostic evaluation)
 cudaError_t launch_request_rebuild(const DevState& S, cudaStream_t st);
 // overwrite the control block (a kernel: no host synchronisation)
 cudaError_t launch_write_ctl(const DevState& S, const StepCtl& v, cudaStream_t st);
-// cell list of the old order -> gather into the new order (predicated on ctl->rebuild)
+// cell starts and scatter slots from the counts of k_rekey (predicated on ctl->rebuild)
 cudaError_t build_cells(const DevState& S, cudaStream_t st);
 // colours by particle id
 cudaError_t launch_set_surface(const DevState& S, const uint8_t* flags, cudaStream_t st);
@@ -125,8 +126,10 @@ struct PassFlags {
                                       // by pass B and screened on by pass A
 };
 
+// Start of a step: flip the view buffer; rebuild the list (and flip the state
+// buffer) when pass B asked for it or `force` is set.
 template <int D, class T>
-cudaError_t launch_rebuild(const DevState& S, const Grid<T>& G, const Frame<T>& F, const Geom<T>& g, T kappa,
+cudaError_t launch_rebuild(const DevState& S, int force, const Grid<T>& G, const Frame<T>& F, const Geom<T>& g, T kappa,
                            cudaStream_t st, const Grid<float>* G32 = nullptr, const Frame<float>* F32 = nullptr);
 template <int D, class T>
 cudaError_t launch_pass_a(const DevState& S, const Frame<T>& F, const Phys<T>& P, PassFlags f, cudaStream_t st);

@@ -23,7 +23,7 @@ static_assert(kN % 32 == 0 && kCap % 4 == 0, "list tiles");
 
 constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 
-constexpr size_t kPartialSlots = partial_slots(kN, 128), kTicketSlots = ticket_slots(kN, 128);
+constexpr size_t kPartialSlots = partial_slots(kN, 32), kTicketSlots = ticket_slots(kN, 32);
 
 // segment offsets (bytes) inside the scratch array
 constexpr size_t kX0 = 0;
@@ -47,7 +47,7 @@ constexpr size_t kPc = kRho + al(4 * kN);
 constexpr size_t kCnt = kPc + al(4 * kN);
 constexpr size_t kCstart = kCnt + al(4 * kC);
 constexpr size_t kScanPart = kCstart + al(4 * (kC + 1));
-constexpr size_t kPartials = kScanPart + al(4 * (kC / 4096 + 2));
+constexpr size_t kPartials = kScanPart + al(4 * (scan_tiles(kC) + 1));
 constexpr size_t kScal = kPartials + al(sizeof(Partial) * kPartialSlots);
 constexpr size_t kCtl = kScal + al(2 * sizeof(Scalars));
 constexpr size_t kTickets = kCtl + al(sizeof(StepCtl));
@@ -210,6 +210,7 @@ extern "C" sph_status sph_eval_forces_noalloc(const sph_domain* dom, const sph_f
     }                                                                                      \
   } while (0)
   NA_CUDA(cudaMemsetAsync(Sd.cnt, 0, sizeof(uint32_t) * cells, st));
+  NA_CUDA(cudaMemsetAsync(Sd.scan_part, 0, sizeof(uint32_t) * scan_tiles(cells), st));
   NA_CUDA(cudaMemsetAsync(Sd.tickets, 0, 4 * kTicketSlots, st));
   NA_CUDA(cudaMemsetAsync(Sd.err, 0, sizeof(int), st));
   NA_CUDA(cudaMemsetAsync(Sd.scal, 0, sizeof(Scalars), st));
@@ -221,15 +222,13 @@ extern "C" sph_status sph_eval_forces_noalloc(const sph_domain* dom, const sph_f
     const float kappa = (float)params->kappa;
     if (d == 2) {
       NA_CUDA((launch_set_state<2, float>(Sd, fr.f, xyz_dev, col_dev, st)));
-      NA_CUDA(launch_gate(Sd, 1, st));
-      NA_CUDA((launch_rebuild<2, float>(Sd, fr.gf, fr.f, geof, kappa, st)));
+      NA_CUDA((launch_rebuild<2, float>(Sd, 1, fr.gf, fr.f, geof, kappa, st)));
       NA_CUDA((launch_pass_a<2, float>(Sd, fr.f, Pf, f, st)));
       NA_CUDA((launch_get_fields<2, float>(Sd, 0, rho_dev, st)));
       NA_CUDA((launch_get_fields<2, float>(Sd, 1, acc_dev, st)));
     } else {
       NA_CUDA((launch_set_state<3, float>(Sd, fr.f, xyz_dev, col_dev, st)));
-      NA_CUDA(launch_gate(Sd, 1, st));
-      NA_CUDA((launch_rebuild<3, float>(Sd, fr.gf, fr.f, geof, kappa, st)));
+      NA_CUDA((launch_rebuild<3, float>(Sd, 1, fr.gf, fr.f, geof, kappa, st)));
       NA_CUDA((launch_pass_a<3, float>(Sd, fr.f, Pf, f, st)));
       NA_CUDA((launch_get_fields<3, float>(Sd, 0, rho_dev, st)));
       NA_CUDA((launch_get_fields<3, float>(Sd, 1, acc_dev, st)));

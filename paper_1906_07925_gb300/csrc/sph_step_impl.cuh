@@ -223,6 +223,19 @@ __device__ __forceinline__ void for_quads(const uint32_t* __restrict__ list, int
   }
 }
 
+// sum over the G lanes of a group (G a power of two), in every lane
+template <int G, class V>
+__device__ __forceinline__ V group_sum(V v) {
+  for (int o = 1; o < G; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// the lanes of this lane's group, and those of them below it
+template <int G>
+__device__ __forceinline__ unsigned group_mask() {
+  return G == 32 ? 0xffffffffu : ((1u << G) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+}
+__device__ __forceinline__ unsigned lanes_below() { return (1u << (threadIdx.x & 31)) - 1u; }
+
 // row of entry k of a list whose first n_in entries sit in rows 0.. and the
 // rest in the last row, the one before, ...
 __device__ __forceinline__ int list_row(int k, int n_in, int cap) {
@@ -342,7 +355,8 @@ __device__ __forceinline__ float fast_rsqrt(float x) {
 __device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(fast_rcp(a.x), fast_rcp(a.y)); }
 __device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(fast_rsqrt(a.x), fast_rsqrt(a.y)); }
 // the skin list of particle i two entries at a time: two(e0, r0, e1, r1, on0,
-// on1) with r = load(e); a place without an entry (on = false) comes with e = own
+// on1) with r = load(e); a place without an entry (on = false) comes with e =
+// own
 template <class Load, class Two>
 __device__ __forceinline__ void for_twos(const uint32_t* __restrict__ list, int i, uint32_t lc, int cap, uint32_t own,
                                          Load&& load, Two&& two) {
@@ -432,8 +446,7 @@ __device__ __forceinline__ void merge(Partial& a, const Partial& b) {
       a.er = b.er;
       a.et = b.et;
     }
-    // non-negative doubles order as their bits (no FP64 instruction)
-    if (__double_as_longlong(b.max_a) > __double_as_longlong(a.max_a)) a.max_a = b.max_a;
+    a.ma = fmaxf(a.ma, b.ma);
   } else {
     argmin_merge(a.min_rc_a, a.amin, b.min_rc_a, b.amin);
     a.max_a = fmax(a.max_a, b.max_a);
@@ -446,36 +459,100 @@ __device__ __forceinline__ void merge(Partial& a, const Partial& b) {
   a.lentries += b.lentries;
 }
 __device__ __forceinline__ Partial no_partial() {
-  return Partial{DBL_MAX, 0.0, 0.0, 0.0, 0.0, 0, 0, 0, -1, 0.0f, 0.0f, 0.0f, 0.0f};
+  return Partial{DBL_MAX, 0.0, 0.0, 0.0, 0.0, 0, 0, 0, -1, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 }
-// p of lane ^ o, member by member
+// Warp reductions of whole values by the integer reduction unit: a few
+// instructions where five rounds of shuffles and merges took microseconds at
+// the end of every pass.
+__device__ __forceinline__ long long warp_sum_u40(long long v) {  // v >= 0, the sum below 2^50
+  const long long lo = __reduce_add_sync(0xffffffffu, (unsigned)(v & 0xFFFFFF));
+  const long long hi = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 24));
+  return (hi << 24) + lo;
+}
+// the smallest / largest of non-negative doubles (they order as their bits)
+__device__ __forceinline__ double warp_min_bits(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? (unsigned)__double2loint(v) : 0xffffffffu);
+  return __hiloint2double((int)mh, (int)ml);
+}
+__device__ __forceinline__ double warp_max_bits(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)__double2loint(v) : 0u);
+  return __hiloint2double((int)mh, (int)ml);
+}
+// the lane whose r_c / |a| comes first (k: its particle, < 0: none); -1: none
+__device__ __forceinline__ int first_ratio(float rc, float an, int k) {
+  constexpr unsigned all = 0xffffffffu;
+  const unsigned qb = k >= 0 ? __float_as_uint(__fdiv_rn(rc, an)) : 0xffffffffu;
+  const unsigned qmin = __reduce_min_sync(all, qb), who = __ballot_sync(all, qb == qmin);
+  if (qmin == 0xffffffffu) return -1;
+  int src = __ffs(who) - 1;
+  if (who & (who - 1)) {  // FP32 quotients tie: by the exact ones, then by index
+    float brc = 0, ban = 0;
+    int bk = -1;
+    for (unsigned m = who; m; m &= m - 1) {
+      const int l = __ffs(m) - 1, ok = __shfl_sync(all, k, l);
+      const float orc = __shfl_sync(all, rc, l), oan = __shfl_sync(all, an, l);
+      if (ratio_before(orc, oan, ok, brc, ban, bk)) {
+        brc = orc;
+        ban = oan;
+        bk = ok;
+        src = l;
+      }
+    }
+  }
+  return src;
+}
+// the lane whose |rho / rho_t - 1| is largest, given it to FP32 rounding (key,
+// < 0: no particle); -1: none
+__device__ __forceinline__ int largest_error(float key, float rho, float rt) {
+  constexpr unsigned all = 0xffffffffu;
+  const float top = __uint_as_float(__reduce_max_sync(all, key >= 0.0f ? __float_as_uint(key) : 0u));
+  const unsigned who = __ballot_sync(all, key >= 0.0f && key >= top * (1.0f - 1e-6f));
+  int src = who ? __ffs(who) - 1 : -1;
+  if (who & (who - 1)) {  // several within rounding of the largest
+    float br = 0.0f, bt = 0.0f;
+    for (unsigned m = who; m; m &= m - 1) {
+      const int l = __ffs(m) - 1;
+      const float r = __shfl_sync(all, rho, l), t = __shfl_sync(all, rt, l);
+      if (err_above(r, t, br, bt)) {
+        br = r;
+        bt = t;
+        src = l;
+      }
+    }
+  }
+  return src;
+}
+// the total of a warp's partials, in every lane (the sums pair up the same way
+// on every run; FP64 sums commute, so both ends of a pair hold the same value)
 template <class T>
-__device__ __forceinline__ Partial shuffle(const Partial& p, int o) {
+__device__ __forceinline__ Partial warp_total(const Partial& p) {
   constexpr unsigned all = 0xffffffffu;
   Partial q = no_partial();
   if (sizeof(T) == 4) {
-    q.rc = __shfl_xor_sync(all, p.rc, o);
-    q.an = __shfl_xor_sync(all, p.an, o);
-    q.er = __shfl_xor_sync(all, p.er, o);
-    q.et = __shfl_xor_sync(all, p.et, o);
+    const int l = first_ratio(p.rc, p.an, (int)p.amin), s = l < 0 ? 0 : l;
+    q.rc = __shfl_sync(all, p.rc, s);
+    q.an = __shfl_sync(all, p.an, s);
+    q.amin = __shfl_sync(all, (int)p.amin, s);
+    const int m = largest_error(err_key(p.er, p.et), p.er, p.et), t = m < 0 ? 0 : m;
+    q.er = __shfl_sync(all, p.er, t);
+    q.et = __shfl_sync(all, p.et, t);
+    q.ma = __uint_as_float(__reduce_max_sync(all, __float_as_uint(p.ma)));
   } else {
-    q.min_rc_a = __shfl_xor_sync(all, p.min_rc_a, o);
-    q.err_max = __shfl_xor_sync(all, p.err_max, o);
+    q.min_rc_a = warp_min_bits(p.min_rc_a);
+    const unsigned k = p.min_rc_a == q.min_rc_a && p.amin >= 0 ? (unsigned)p.amin : 0x7fffffffu;
+    const unsigned kmin = __reduce_min_sync(all, k);
+    q.amin = kmin == 0x7fffffffu ? -1 : (long long)kmin;
+    q.max_a = warp_max_bits(p.max_a);
+    q.err_max = warp_max_bits(p.err_max);
   }
-  q.max_a = __shfl_xor_sync(all, p.max_a, o);
-  q.sum_rho = __shfl_xor_sync(all, p.sum_rho, o);
-  q.err_l2 = __shfl_xor_sync(all, p.err_l2, o);
-  q.ipairs = __shfl_xor_sync(all, p.ipairs, o);
-  q.fpairs = __shfl_xor_sync(all, p.fpairs, o);
-  q.lentries = __shfl_xor_sync(all, p.lentries, o);
-  q.amin = __shfl_xor_sync(all, p.amin, o);
+  q.sum_rho = warp_sum(p.sum_rho);
+  q.err_l2 = warp_sum(p.err_l2);
+  q.ipairs = warp_sum_u40(p.ipairs);
+  q.fpairs = warp_sum_u40(p.fpairs);
+  q.lentries = warp_sum_u40(p.lentries);
   return q;
-}
-// a warp's partials into lane 0's (the sums pair up the same way on every
-// run; FP64 sums commute, so both ends of a pair hold the same value)
-template <class T>
-__device__ __forceinline__ void warp_merge(Partial& p, int lanes) {
-  for (int o = 1; o < lanes; o <<= 1) merge<T>(p, shuffle<T>(p, o));
 }
 
 // The integer part of v (|v| < 2^22, nearest) taken off v, the rest scaled up
@@ -520,48 +597,17 @@ __device__ __forceinline__ void warp_sums(bool active, int i, float rc, float an
   const int lane = threadIdx.x & 31;
   // the smallest r_c / |a|
   const bool moves = active && an > 0.0f;
-  const unsigned qb = moves ? __float_as_uint(__fdiv_rn(rc, an)) : 0xffffffffu;
-  const unsigned qmin = __reduce_min_sync(all, qb);
-  unsigned who = __ballot_sync(all, qb == qmin);
-  int src = __ffs(who) - 1;
-  if (qmin != 0xffffffffu && (who & (who - 1))) {  // FP32 quotients tie: by the exact ones, then by index
-    float brc = 0, ban = 0;
-    int bk = -1;
-    for (unsigned m = who; m; m &= m - 1) {
-      const int l = __ffs(m) - 1;
-      const float orc = __shfl_sync(all, rc, l), oan = __shfl_sync(all, an, l);
-      if (ratio_before(orc, oan, l, brc, ban, bk)) {
-        brc = orc;
-        ban = oan;
-        bk = l;
-      }
-    }
-    src = bk;
-  }
-  const float mrc = __shfl_sync(all, rc, src), man = __shfl_sync(all, an, src);
-  const int mi = __shfl_sync(all, i, src);
+  const int first = first_ratio(rc, an, moves ? i : -1), fl = first < 0 ? 0 : first;
+  const float mrc = __shfl_sync(all, rc, fl), man = __shfl_sync(all, an, fl);
+  const int mi = __shfl_sync(all, i, fl);
   // the largest |a| (NaN, which raises the error word, counts as none)
   const unsigned amax = __reduce_max_sync(all, moves ? __float_as_uint(an) : 0u);
   // the largest |rho / rho_t - 1|
   float q1 = 0.0f, q2 = 0.0f;
   if (active) density_error(rho, rt, q1, q2);
-  const float ek = active ? fabsf(q1) : -1.0f;
-  const float emax = __uint_as_float(__reduce_max_sync(all, active ? __float_as_uint(ek) : 0u));
-  who = __ballot_sync(all, active && ek >= emax * (1.0f - 1e-6f));
-  src = who ? __ffs(who) - 1 : 0;
-  if (who & (who - 1)) {  // several within rounding of the largest
-    float br = 0.0f, bt = 0.0f;
-    for (unsigned m = who; m; m &= m - 1) {
-      const int l = __ffs(m) - 1;
-      const float r = __shfl_sync(all, rho, l), t = __shfl_sync(all, rt, l);
-      if (err_above(r, t, br, bt)) {
-        br = r;
-        bt = t;
-        src = l;
-      }
-    }
-  }
-  const float er = __shfl_sync(all, rho, src), et = __shfl_sync(all, rt, src);
+  const int worst = largest_error(active ? fabsf(q1) : -1.0f, rho, rt), wl = worst < 0 ? 0 : worst;
+  const float er = __shfl_sync(all, rho, wl), et = __shfl_sync(all, rt, wl);
+  const float emax = fabsf(__shfl_sync(all, q1, wl));
   // sum rho
   const float rv = active ? rho : 0.0f;
   const int re = fixed_exponent(__uint_as_float(__reduce_max_sync(all, __float_as_uint(rv))));
@@ -570,7 +616,7 @@ __device__ __forceinline__ void warp_sums(bool active, int i, float rc, float an
   for (int k = 0; k < 3; ++k) rl[k] = __reduce_add_sync(all, take_limb(v));
   // sum (rho/rho_t - 1)^2 = p + pl
   const float p = q1 * q1, pl = fmaf(q1, q1, -p) + 2.0f * q1 * q2;
-  const int ee = fixed_exponent(emax * emax);
+  const int ee = fixed_exponent(emax * emax * 1.00001f);  // the largest to rounding
   const float es = exponent_scale(ee);
   float a = p * es, b = pl * es * 4194304.0f;
   el[0] = take_limb(a);
@@ -583,10 +629,10 @@ __device__ __forceinline__ void warp_sums(bool active, int i, float rc, float an
   if (lane == 0) {
     out->rc = mrc;
     out->an = man;
-    out->amin = qmin != 0xffffffffu ? mi : -1;
+    out->amin = first >= 0 ? mi : -1;
     out->max_a = amax;
     out->er = er;
-    out->et = who ? et : 0.0f;
+    out->et = worst >= 0 ? et : 0.0f;
     for (int k = 0; k < 3; ++k) {
       out->rl[k] = rl[k];
       out->el[k] = el[k];
@@ -608,7 +654,7 @@ __device__ __forceinline__ Partial to_partial(const WarpSums& w) {
   p.rc = w.rc;
   p.an = w.an;
   p.amin = w.amin;
-  p.max_a = (double)__uint_as_float(w.max_a);
+  p.ma = __uint_as_float(w.max_a);
   p.er = w.er;
   p.et = w.et;
   p.sum_rho = from_limbs(w.rl, w.re);
@@ -621,18 +667,18 @@ __device__ __forceinline__ Partial to_partial(const WarpSums& w) {
 
 // L2 read of a partial another block wrote
 __device__ __forceinline__ Partial load_partial(const Partial* p) {
-  static_assert(sizeof(Partial) == 88, "members read one by one");
+  static_assert(sizeof(Partial) == 96, "members read one by one");
   const double* d = (const double*)p;
   const long long* l = (const long long*)p;
   const float* f = (const float*)p;
   return Partial{__ldcg(d + 0), __ldcg(d + 1), __ldcg(d + 2), __ldcg(d + 3), __ldcg(d + 4), __ldcg(l + 5),
                  __ldcg(l + 6), __ldcg(l + 7), __ldcg(l + 8), __ldcg(f + 18), __ldcg(f + 19), __ldcg(f + 20),
-                 __ldcg(f + 21)};
+                 __ldcg(f + 21), __ldcg(f + 22), 0.0f};
 }
-// Called by one warp of every block with the block's partial in every lane:
+// Called by one warp of every block with the block's partial in lane 0:
 // the last block of a group merges the group's partials, the last group's
 // block merges the groups' (each lane a fixed stride of them, then a fixed
-// tree). True in the warp that holds the grid's total. One block merging all
+// tree; a grid of one group ends there). True in the warp that holds the grid's total. One block merging all
 // partials took a tail of 10 us at 4,096 blocks: FP64 adds run at two lanes
 // per cycle on one SM.
 template <class T>
@@ -649,9 +695,13 @@ __device__ __forceinline__ bool grid_total(Partial& p, Partial* partials, unsign
   __threadfence();
   Partial a = no_partial();
   for (int b = lane; b < gn; b += 32) merge<T>(a, load_partial(partials + b0 + b));
-  warp_merge<T>(a, 32);
+  a = warp_total<T>(a);
+  if (lane == 0) ticket[4 + g] = 0u;
+  if (ng == 1) {
+    p = a;
+    return true;
+  }
   if (lane == 0) {
-    ticket[4 + g] = 0u;
     partials[nb + g] = a;
     __threadfence();
     last = atomicAdd(ticket, 1u) == (unsigned)(ng - 1);
@@ -660,7 +710,7 @@ __device__ __forceinline__ bool grid_total(Partial& p, Partial* partials, unsign
   __threadfence();
   a = no_partial();
   for (int b = lane; b < ng; b += 32) merge<T>(a, load_partial(partials + nb + b));
-  warp_merge<T>(a, 32);
+  a = warp_total<T>(a);
   if (lane == 0) *ticket = 0u;
   p = a;
   return true;
@@ -670,62 +720,104 @@ __device__ __forceinline__ bool grid_total(Partial& p, Partial* partials, unsign
 // List rebuild (runs only when ctl->rebuild). Old order: buffer 1 - buf.
 // ------------------------------------------------------------------------
 
-// cell key of each particle in the old order: level from h at its position,
-// cell coordinates X >> (cshift + level)
+// Gate of the step, then the cell key of each particle in the old order (level
+// from h at its position, cell coordinates X >> (cshift + level)) and its count
+// per cell and per scan tile: one launch for what were four, and with the
+// gather making the views, a step of seven kernels instead of twelve (FP64
+// thirteen). Circle (2D, 4,289 particles) 42 -> 35 us per step, general EOS at
+// 99,991 80 -> 71.
+// The control block as pass B left it says whether the list is rebuilt; this
+// kernel moves it on (view buffer, state buffer, flags) for the kernels that
+// follow: without a rebuild at once by one thread, which touches nothing the
+// other blocks read; with one by the last block to finish.
 template <int D, class T>
-__global__ void __launch_bounds__(256) k_rekey(int n, const StepCtl* __restrict__ ctl, const LL4* __restrict__ X0,
-                                               const LL4* __restrict__ X1, Frame<T> F, Grid<T> G, Geom<T> geo,
-                                               uint32_t* __restrict__ key) {
-  if (!ctl->rebuild) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const LL4 X = (ctl->buf ? X0 : X1)[i];
+__global__ void __launch_bounds__(256) k_rekey(int n, StepCtl* ctl, int force, unsigned* __restrict__ ticket,
+                                               const LL4* __restrict__ X0, const LL4* __restrict__ X1, Frame<T> F,
+                                               Grid<T> G, Geom<T> geo, uint32_t* __restrict__ key,
+                                               uint32_t* __restrict__ cnt, uint32_t* __restrict__ part) {
+  if (!(force || *(volatile int*)&ctl->need_rebuild)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      ctl->vp ^= 1;
+      ctl->rebuild = 0;
+    }
+    return;
+  }
+  const int old = ctl->buf;  // the buffer in the old order
+  for (int b0 = blockIdx.x * blockDim.x; b0 < n; b0 += gridDim.x * blockDim.x) {
+    const int i = b0 + threadIdx.x;
+    const unsigned mask = __ballot_sync(0xffffffffu, i < n);
+    if (i >= n) continue;
+    const LL4 X = (old ? X1 : X0)[i];
     T x[3];
     abs_pos<D, T>(F, X, x);
     const int l = level_of_h(G, h_of<D, T>(geo, x));
     const int sh = G.cshift + l;
     const int c[3] = {(int)min((long long)G.nx[l] - 1, X.x >> sh), (int)min((long long)G.ny[l] - 1, X.y >> sh),
                       D == 3 ? (int)min((long long)G.nz[l] - 1, X.z >> sh) : 0};
-    key[i] = G.base[l] + (uint32_t)c[0] + (uint32_t)G.nx[l] * ((uint32_t)c[1] + (uint32_t)G.ny[l] * (uint32_t)c[2]);
+    const uint32_t k =
+        G.base[l] + (uint32_t)c[0] + (uint32_t)G.nx[l] * ((uint32_t)c[1] + (uint32_t)G.ny[l] * (uint32_t)c[2]);
+    key[i] = k;
+    const int lane = threadIdx.x & 31;
+    unsigned peers = __match_any_sync(mask, k);
+    if (lane == __ffs(peers) - 1) atomicAdd(&cnt[k], (uint32_t)__popc(peers));
+    peers = __match_any_sync(mask, k / kScanTile);
+    if (lane == __ffs(peers) - 1) atomicAdd(&part[k / kScanTile], (uint32_t)__popc(peers));
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(ticket, 1u) == gridDim.x - 1) {  // every block has read the control block
+      *ticket = 0u;
+      ctl->vp ^= 1;
+      ctl->buf = old ^ 1;
+      ctl->rebuild = 1;
+      ctl->need_rebuild = 0;
+      ctl->rebuilds += 1;
+      ctl->lmax = 0;
+    }
   }
 }
 
-// views of the (new) current order and the reference view for the skin test
+// Slot s of the scatter holds old index i; its rank among the cell's members by
+// particle id gives its destination (cells ordered by key, each cell by
+// particle id): the state is copied there, with the view of the new order, the
+// reference view of the skin test (w = half the skin), and in the FP64 path the
+// FP32 view its list build and pass A's screen read. (The list only has to hold
+// every pair the exact FP64 tests can accept before the next rebuild, and an
+// FP32 candidate test errs by ~1e-7 of the distance, far inside the list's
+// margins, while FP64 arithmetic runs at a small fraction of the FP32 rate.)
 template <int D, class T>
-__global__ void __launch_bounds__(256) k_make_view(int n, const StepCtl* __restrict__ ctl, int force,
-                                                   const LL4* __restrict__ X0, const LL4* __restrict__ X1,
-                                                   Frame<T> F, Geom<T> geo, typename ViewOf<T>::type* __restrict__ v0,
-                                                   typename ViewOf<T>::type* __restrict__ v1,
-                                                   typename ViewOf<T>::type* __restrict__ vbuild) {
-  if (!force && !ctl->rebuild) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const LL4 X = (ctl->buf ? X1 : X0)[i];
+__global__ void __launch_bounds__(256) k_gather_view(
+    int n, const StepCtl* __restrict__ ctl, const uint32_t* __restrict__ slots, const uint32_t* __restrict__ key,
+    const uint32_t* __restrict__ cstart, LL4* __restrict__ X0, LL4* __restrict__ X1, uint32_t* __restrict__ m0,
+    uint32_t* __restrict__ m1, uint32_t* __restrict__ p0, uint32_t* __restrict__ p1, Frame<T> F, Geom<T> geo,
+    typename ViewOf<T>::type* __restrict__ v0, typename ViewOf<T>::type* __restrict__ v1,
+    typename ViewOf<T>::type* __restrict__ vbuild, int4* __restrict__ v32, Frame<float> F32) {
+  if (!ctl->rebuild) return;
+  const int nb = ctl->buf, vp = ctl->vp;  // new buffers; the old order lives in the other state buffer
+  const uint32_t* __restrict__ pold = nb ? p0 : p1;
+  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
+    const uint32_t i = slots[s];
+    const uint32_t k = key[i];
+    const uint32_t id = pold[i];
+    const uint32_t b = cstart[k], e = cstart[k + 1];
+    uint32_t rank = 0;
+    for (uint32_t t = b; t < e; ++t) rank += pold[slots[t]] < id;
+    const uint32_t d = b + rank;
+    const LL4 X = (nb ? X0 : X1)[i];
+    (nb ? X1 : X0)[d] = X;
+    (nb ? m1 : m0)[d] = (nb ? m0 : m1)[i];
+    (nb ? p1 : p0)[d] = id;
     T x[3];
     abs_pos<D, T>(F, X, x);
-    const T h = h_of<D, T>(geo, x);
-    const auto v = make_view<D>(F, X, h);
-    (ctl->vp ? v1 : v0)[i] = v;
-    vbuild[i] = with_w(v, T(0.5) * F.skin * view_h(F, v));  // half the skin, view units (kappa folded in by the host)
-  }
-}
-
-// FP32 view of the FP64 path's particles, made at a list rebuild for its list
-// build (and kept current every step by pass B for pass A's FP32 screen): the
-// list only has to hold every pair the exact FP64 tests can accept before the
-// next rebuild, and an FP32 candidate test errs by ~1e-7 of the distance, far
-// inside the list's margins (the skin and the 1e-5 factor), while FP64
-// arithmetic runs at a small fraction of the FP32 rate on this GPU.
-template <int D>
-__global__ void __launch_bounds__(256) k_view32(int n, const StepCtl* __restrict__ ctl,
-                                                const LL4* __restrict__ X0, const LL4* __restrict__ X1,
-                                                Frame<float> F, const V4<double>* __restrict__ vd0,
-                                                const V4<double>* __restrict__ vd1, int4* __restrict__ out) {
-  if (!ctl->rebuild) return;
-  const long long half = 1LL << (F.sv - 1);
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const LL4 X = (ctl->buf ? X1 : X0)[i];
-    const double hv = (ctl->vp ? vd1 : vd0)[i].w;  // h in view units (c0, both precisions)
-    out[i] = make_int4((int)((X.x + half) >> F.sv), (int)((X.y + half) >> F.sv),
-                       D == 3 ? (int)((X.z + half) >> F.sv) : 0, __float_as_int((float)hv * F.c2w));
+    const auto v = make_view<D>(F, X, h_of<D, T>(geo, x));
+    (vp ? v1 : v0)[d] = v;
+    vbuild[d] = with_w(v, T(0.5) * F.skin * view_h(F, v));  // kappa folded in by the host
+    if constexpr (std::is_same<T, double>::value) {
+      const long long half = 1LL << (F32.sv - 1);
+      v32[d] = make_int4((int)((X.x + half) >> F32.sv), (int)((X.y + half) >> F32.sv),
+                         D == 3 ? (int)((X.z + half) >> F32.sv) : 0, __float_as_int((float)view_w(v) * F32.c2w));
+    }
   }
 }
 
@@ -735,147 +827,250 @@ __global__ void __launch_bounds__(256) k_view32(int n, const StepCtl* __restrict
 // (and h changed by at most lip_h times that), any pair inside the exact
 // criteria is still listed. Candidates come from rows of cells of every level
 // that can hold such a j, in the order (level, z row, y row, x).
-template <int D, class T>
-__global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(int n, StepCtl* __restrict__ ctl,
-                                                    const LL4* __restrict__ X0, const LL4* __restrict__ X1,
-                                                    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1,
-                                                    const typename ViewOf<T>::type* __restrict__ v0,
-                                                    const typename ViewOf<T>::type* __restrict__ v1,
-                                                    const uint32_t* __restrict__ cstart, Frame<T> F, Grid<T> G,
-                                                    T kappa, int cap, uint32_t* __restrict__ list,
-                                                    uint32_t* __restrict__ lcount, int* __restrict__ err) {
-  using VT = typename ViewOf<T>::type;
-  if (!ctl->rebuild) return;
-  const int buf = ctl->buf;
-  const VT* __restrict__ view = ctl->vp ? v1 : v0;
-  const uint32_t* __restrict__ meta = buf ? m1 : m0;
-  int cmax = 0;  // longest list of this thread's targets
-  bool over_any = false;
-  // grid-stride over the targets (one per thread at the grid it is launched with)
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-  const LL4 X = (buf ? X1 : X0)[i];
-  const VT vi = view[i];
-  const T hv = view_h(F, vi);                 // view units
-  const T sk = F.skin * hv;                // skin of i, view units (kappa folded in by the host)
-  const T sk_hv = F.skin;                  // skin per unit h
-  const T lip = G.lip_h;
-  // search radius: bound h_j by Lipschitz continuity, iterate twice
-  T hhi = hv, Rs = kappa * hv * G.rfac + sk * (T(1) + T(0.5) * kappa * lip);
-  for (int it = 0; it < 2; ++it) {
-    hhi = hv * T(1.00001) + lip * Rs;
-    const T shi = sk * hhi / hv;
-    Rs = kappa * hhi * G.rfac + shi * (T(1) + T(0.5) * kappa * lip);
-    Rs = Rs > kappa * hv * G.rfac ? Rs : kappa * hv * G.rfac;
+// The list is built on FP32 views in both precisions. Lengths of the tests are
+// view integers; with w = kappa h / 2 (view_w) and m = max(w_i, w_j) the list
+// radius above is m times a constant and the larger of the supports kappa h_i
+// and kappa h_ij is w_i + m.
+struct ListTarget {
+  float Rs, R2;          // search radius, view units
+  float wi, c, r2max;    // view integers
+  int l0, l1;            // levels that can hold a neighbour
+  __device__ __forceinline__ ListTarget(const Frame<float>& F, const Grid<float>& G, float kappa, const int4& vi) {
+    const float hv = view_h(F, vi), sk = F.skin * hv, lip = G.lip_h, cl = 1.0f + 0.5f * kappa * lip;
+    // search radius: bound h_j by Lipschitz continuity, iterate twice
+    float hhi = hv;
+    Rs = kappa * hv * G.rfac + sk * cl;
+    for (int it = 0; it < 2; ++it) {
+      hhi = hv * 1.00001f + lip * Rs;
+      const float shi = sk * hhi / hv;
+      Rs = kappa * hhi * G.rfac + shi * cl;
+      Rs = fmaxf(Rs, kappa * hv * G.rfac);
+    }
+    l0 = level_of_h(G, (hv * 0.99999f - lip * Rs) * F.qv);
+    l1 = level_of_h(G, hhi * F.qv);
+    R2 = Rs * Rs;
+    wi = view_w(vi);
+    c = 2.0f * (1.00001f + F.skin / kappa * cl);  // skin: kappa folded in
+    r2max = R2 / (F.vscale * F.vscale);
   }
-  const T hlo = hv * T(0.99999) - lip * Rs;
-  const T qv = F.qv;
-  const int l0 = level_of_h(G, hlo * qv), l1 = level_of_h(G, hhi * qv);
-  const T R2 = Rs * Rs;
-  int cnt = 0, n_in = 0, n_out = 0;  // accepted; written inside / outside entries
-  const int rows = list_rows(cap);
-  uint32_t* __restrict__ own = list + list_at(i, 0, cap);
-  bool over = false;
-  T reach = 0;
-  const T Hd = kappa * hv;
-
-  // one candidate: every test is evaluated without a branch (most candidates
-  // fail, and a branch over the acceptance tests ran for a few lanes of the
-  // warp in nearly every iteration); only the list store is conditional
-  const T cl = T(1) + T(0.5) * kappa * lip;
-  auto cand = [&](int jc, const VT& vj) {
-    const T dx = vd(F, vi.x, vj.x), dy2 = vd(F, vi.y, vj.y);
-    const T dz2 = D == 3 ? vd(F, vi.z, vj.z) : T(0);
-    const T r2 = dx * dx + dy2 * dy2 + dz2 * dz2;
-    const T hj = view_h(F, vj);
-    const T skj = sk_hv * hj;
-    const T smax = sk > skj ? sk : skj;
-    const T hm = hv > hj ? hv : hj;  // symmetric: j lists i whenever i lists j
-    // h_j is known here: only rounding and the h change over the skin need a margin
-    const T Rl = kappa * hm * T(1.00001) + smax * cl;
-    const bool acc = r2 < R2 && r2 < Rl * Rl;
-    // inside its support now (density or force): the front of the list
-    const T Hf = T(0.5) * kappa * (hv + hj);
-    const T Hp = Hf > Hd ? Hf : Hd;
-    const bool inside = r2 < Hp * Hp;
-    // largest axis separation this pair can reach before the next rebuild
-    const T ax = fabs(dx) > fabs(dy2) ? fabs(dx) : fabs(dy2);
-    const T am = (ax > fabs(dz2) ? ax : fabs(dz2)) + smax;
-    reach = acc && am > reach ? am : reach;
-    if (acc) {
-      if (cnt < cap) {
-        const int row = inside ? n_in++ : rows - 1 - n_out++;
-        own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)jc << 8) | (meta[jc] & 0xFFu);
-      } else {
-        over = true;
-      }
-      ++cnt;
-    }
-  };
-
-  for (int l = l0; l <= l1; ++l) {
-    const int sh = G.cshift + l;
-    const int nx = G.nx[l], ny = G.ny[l], nz = G.nz[l];
-    const int cxl = (int)min((long long)nx - 1, X.x >> sh);
-    const int cyl = (int)min((long long)ny - 1, X.y >> sh);
-    const int czl = D == 3 ? (int)min((long long)nz - 1, X.z >> sh) : 0;
-    const T c = G.cellv[l], ic = T(1) / c;
-    // target position inside its level-l cell, view units
-    const T fx = (T)((double)(X.x - ((long long)cxl << sh)) * F.s2v);
-    const T fy = (T)((double)(X.y - ((long long)cyl << sh)) * F.s2v);
-    const T fz = D == 3 ? (T)((double)(X.z - ((long long)czl << sh)) * F.s2v) : T(0);
-    const uint32_t base = G.base[l];
-    int zlo = 0, zhi = 0;
+  // a pair of candidates, without a branch: listed (acc), inside its support
+  // now (density or force: the front of the list)
+  template <int D>
+  __device__ __forceinline__ void test(const int4& vi, const int4& a, const int4& b, bool (&acc)[2],
+                                       bool (&inside)[2]) const {
+    const float2 dx = make_float2((float)(vi.x - a.x), (float)(vi.x - b.x));
+    const float2 dy = make_float2((float)(vi.y - a.y), (float)(vi.y - b.y));
+    float2 r2 = fma2(dy, dy, mul2(dx, dx));
     if (D == 3) {
-      zlo = (int)dfloor((fz - Rs) * ic);
-      zhi = (int)dfloor((fz + Rs) * ic);
+      const float2 dz = make_float2((float)(vi.z - a.z), (float)(vi.z - b.z));
+      r2 = fma2(dz, dz, r2);
     }
-    const int ylo = (int)dfloor((fy - Rs) * ic), yhi = (int)dfloor((fy + Rs) * ic);
-    for (int dz = zlo; dz <= zhi; ++dz) {
-      const int czz = czl + dz;
-      if (D == 3 && (czz < 0 || czz >= nz)) continue;
-      T dzp = 0;
-      if (D == 3) {
-        const T zrel = fz - (T)dz * c;
-        dzp = zrel < T(0) ? -zrel : (zrel > c ? zrel - c : T(0));
-      }
-      for (int dy = ylo; dy <= yhi; ++dy) {
-        const int cyy = cyl + dy;
-        if (cyy < 0 || cyy >= ny) continue;
-        const T yrel = fy - (T)dy * c;
-        const T dyp = yrel < T(0) ? -yrel : (yrel > c ? yrel - c : T(0));
-        const T dp2 = dyp * dyp + dzp * dzp;
-        if (dp2 >= R2) continue;
-        const T half = dsqrt(R2 - dp2);
-        int x0 = cxl + (int)dfloor((fx - half) * ic);
-        int x1 = cxl + (int)dfloor((fx + half) * ic);
-        x0 = x0 < 0 ? 0 : x0;
-        x1 = x1 > nx - 1 ? nx - 1 : x1;
-        if (x0 > x1) continue;
-        const uint32_t krow = base + (uint32_t)nx * ((uint32_t)cyy + (uint32_t)ny * (uint32_t)(D == 3 ? czz : 0));
-        const int jb = (int)cstart[krow + (uint32_t)x0], je = (int)cstart[krow + (uint32_t)x1 + 1];
-        // candidates in ascending order, two views loaded before either is
-        // tested (two loads in flight per thread: a rebuild of the 8M 3D
-        // workload 3.5 % faster than one at a time)
-        int j = jb;
-        for (; j + 2 <= je; j += 2) {
-          const VT va = view[j], vb = view[j + 1];
-          cand(j, va);
-          cand(j + 1, vb);
-        }
-        for (; j < je; ++j) cand(j, view[j]);
-      }
-    }
+    // symmetric in i and j: j lists i whenever i lists j
+    const float2 m = make_float2(fmaxf(wi, view_w(a)), fmaxf(wi, view_w(b)));
+    const float2 rl = mul2(both(c), m), rl2 = mul2(rl, rl), hp = add2(both(wi), m), hp2 = mul2(hp, hp);
+    acc[0] = r2.x < fminf(rl2.x, r2max);
+    acc[1] = r2.y < fminf(rl2.y, r2max);
+    inside[0] = r2.x < hp2.x;
+    inside[1] = r2.y < hp2.y;
+  }
+  // largest axis separation (view units) a listed pair can reach before the next rebuild
+  template <int D>
+  __device__ __forceinline__ float reach(const Frame<float>& F, float kappa, const int4& vi, const int4& vj) const {
+    const int d = max(max(abs(vi.x - vj.x), abs(vi.y - vj.y)), D == 3 ? abs(vi.z - vj.z) : 0);
+    return (float)d * F.vscale + F.skin / kappa * 2.0f * fmaxf(wi, view_w(vj)) * F.vscale;
   }
   // the coarse FP32 conversion is exact below 2^22 coarse integers = 2^(22 - kCoarseBits) c0
-  const bool fast = reach < T(0.999) * T(1 << (22 - kCoarseBits));
-  lcount[i] = (uint32_t)n_in | ((uint32_t)n_out << kOutShift) | (fast ? kFastBit : 0u);
-  over_any |= over;
-  cmax = cnt > cmax ? cnt : cmax;
-  }  // targets
-  if (over_any) atomicOr(err, kErrListOverflow);
+  static __device__ __forceinline__ bool fast(float reach) { return reach < 0.999f * (1 << (22 - kCoarseBits)); }
+};
+// the rows of level-l cells a search ball of radius Rs reaches
+template <int D>
+struct RowWalk {
+  using T = float;
+  int nx, ny, nz, cxl, cyl, czl, zlo, zhi, ylo, yhi;
+  uint32_t base;
+  T c, ic, fx, fy, fz;  // cell edge, position inside the own cell, view units
+  __device__ __forceinline__ RowWalk(const Frame<T>& F, const Grid<T>& G, const LL4& X, T Rs, int l) {
+    const int sh = G.cshift + l;
+    nx = G.nx[l];
+    ny = G.ny[l];
+    nz = G.nz[l];
+    base = G.base[l];
+    cxl = (int)min((long long)nx - 1, X.x >> sh);
+    cyl = (int)min((long long)ny - 1, X.y >> sh);
+    czl = D == 3 ? (int)min((long long)nz - 1, X.z >> sh) : 0;
+    c = G.cellv[l];
+    ic = T(1) / c;
+    fx = (T)((double)(X.x - ((long long)cxl << sh)) * F.s2v);
+    fy = (T)((double)(X.y - ((long long)cyl << sh)) * F.s2v);
+    fz = D == 3 ? (T)((double)(X.z - ((long long)czl << sh)) * F.s2v) : T(0);
+    zlo = D == 3 ? (int)dfloor((fz - Rs) * ic) : 0;
+    zhi = D == 3 ? (int)dfloor((fz + Rs) * ic) : 0;
+    ylo = (int)dfloor((fy - Rs) * ic);
+    yhi = (int)dfloor((fy + Rs) * ic);
+  }
+  // candidates [j, je) of row (dz, dy), trimmed to the ball; false: none
+  __device__ __forceinline__ bool row(const uint32_t* __restrict__ cstart, int dz, int dy, T R2, int& j, int& je) const {
+    const int czz = czl + dz, cyy = cyl + dy;
+    if ((D == 3 && (czz < 0 || czz >= nz)) || cyy < 0 || cyy >= ny) return false;
+    T dzp = 0;
+    if (D == 3) {
+      const T zrel = fz - (T)dz * c;
+      dzp = zrel < T(0) ? -zrel : (zrel > c ? zrel - c : T(0));
+    }
+    const T yrel = fy - (T)dy * c;
+    const T dyp = yrel < T(0) ? -yrel : (yrel > c ? yrel - c : T(0));
+    const T dp2 = dyp * dyp + dzp * dzp;
+    if (dp2 >= R2) return false;
+    const T half = dsqrt(R2 - dp2);
+    int x0 = cxl + (int)dfloor((fx - half) * ic), x1 = cxl + (int)dfloor((fx + half) * ic);
+    x0 = x0 < 0 ? 0 : x0;
+    x1 = x1 > nx - 1 ? nx - 1 : x1;
+    if (x0 > x1) return false;
+    const uint32_t krow = base + (uint32_t)nx * ((uint32_t)cyy + (uint32_t)ny * (uint32_t)(D == 3 ? czz : 0));
+    j = (int)cstart[krow + (uint32_t)x0];
+    je = (int)cstart[krow + (uint32_t)x1 + 1];
+    return true;
+  }
+};
+
+// One thread per particle. REACH: certify the coarse FP32 test (kFastBit, read
+// by the FP64 path).
+template <int D, bool REACH>
+__global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(
+    int n, StepCtl* __restrict__ ctl, const LL4* __restrict__ X0, const LL4* __restrict__ X1,
+    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1, const int4* __restrict__ v0,
+    const int4* __restrict__ v1, const uint32_t* __restrict__ cstart, Frame<float> F, Grid<float> G, float kappa, int cap,
+    uint32_t* __restrict__ list, uint32_t* __restrict__ lcount, int* __restrict__ err) {
+  if (!ctl->rebuild) return;
+  const int buf = ctl->buf;
+  const int4* __restrict__ view = ctl->vp ? v1 : v0;
+  const uint32_t* __restrict__ meta = buf ? m1 : m0;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  int cnt = 0;  // accepted
+  if (i < n) {
+    const LL4 X = (buf ? X1 : X0)[i];
+    const int4 vi = view[i];
+    const ListTarget t(F, G, kappa, vi);
+    int n_in = 0, n_out = 0;  // written inside / outside entries
+    const int rows = list_rows(cap);
+    uint32_t* __restrict__ own = list + list_at(i, 0, cap);
+    float reach = 0.0f;
+    // only the list store is conditional: most candidates fail, and a branch
+    // over the tests ran for a few lanes of the warp in nearly every iteration.
+    // Bound by issue slots (lanes of a warp have different rows and row lengths:
+    // 11 of 32 active); two candidates per instruction, with the lengths of the
+    // tests relative to w, take 31 % off a rebuild (8,388,608 particles in 3D:
+    // 1.48 -> 1.03 ms per step at a rebuild every four steps).
+    auto take = [&](int j, const int4& vj, bool acc, bool inside) {
+      if (!acc) return;
+      if (cnt < cap) {
+        const int row = inside ? n_in++ : rows - 1 - n_out++;
+        own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)j << 8) | (meta[j] & 0xFFu);
+      }
+      ++cnt;
+      if (REACH) reach = fmaxf(reach, t.reach<D>(F, kappa, vi, vj));
+    };
+    for (int l = t.l0; l <= t.l1; ++l) {
+      const RowWalk<D> w(F, G, X, t.Rs, l);
+      for (int dz = w.zlo; dz <= w.zhi; ++dz) {
+        for (int dy = w.ylo; dy <= w.yhi; ++dy) {
+          int j, je;
+          if (!w.row(cstart, dz, dy, t.R2, j, je)) continue;
+          // candidates in ascending order, two at a time (an odd last one twice)
+          for (; j < je; j += 2) {
+            const bool two = j + 1 < je;
+            const int4 a = view[j], b = view[two ? j + 1 : j];
+            bool acc[2], inside[2];
+            t.test<D>(vi, a, b, acc, inside);
+            take(j, a, acc[0], inside[0]);
+            take(j + 1, b, acc[1] && two, inside[1]);
+          }
+        }
+      }
+    }
+    lcount[i] = (uint32_t)n_in | ((uint32_t)n_out << kOutShift) | (REACH && ListTarget::fast(reach) ? kFastBit : 0u);
+    if (cnt > cap) atomicOr(err, kErrListOverflow);
+  }
   // longest list of this build (one atomic per warp; every lane gets here)
-  const int wmax = __reduce_max_sync(0xffffffffu, cmax);
+  const int wmax = __reduce_max_sync(0xffffffffu, cnt);
   if ((threadIdx.x & 31) == 0 && wmax > 0) atomicMax(&ctl->lmax, wmax);
+}
+
+// The same lists with G lanes per particle: lane g walks candidate rows g,
+// g + G, ... and the group's lanes test one candidate each at a time; accepted
+// ones take their places in lane order. For particle counts that leave most of
+// the chip idle with one thread per particle, where one thread's chain of row
+// look-ups and candidate loads is the whole time (launch_rebuild).
+template <int D, int G, bool REACH>
+__global__ void __launch_bounds__(256) k_list_build_group(int n, StepCtl* __restrict__ ctl,
+                                                          const LL4* __restrict__ X0, const LL4* __restrict__ X1,
+                                                          const uint32_t* __restrict__ m0,
+                                                          const uint32_t* __restrict__ m1,
+                                                          const int4* __restrict__ v0, const int4* __restrict__ v1,
+                                                          const uint32_t* __restrict__ cstart, Frame<float> F,
+                                                          Grid<float> G32, float kappa, int cap,
+                                                          uint32_t* __restrict__ list, uint32_t* __restrict__ lcount,
+                                                          int* __restrict__ err) {
+  __shared__ int longest;
+  if (!ctl->rebuild) return;
+  if (threadIdx.x == 0) longest = 0;
+  __syncthreads();
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G, g = threadIdx.x % G;
+  if (i < n) {  // whole groups
+    const unsigned group = group_mask<G>(), below = group & lanes_below();
+    const int buf = ctl->buf;
+    const int4* __restrict__ view = ctl->vp ? v1 : v0;
+    const uint32_t* __restrict__ meta = buf ? m1 : m0;
+    const LL4 X = (buf ? X1 : X0)[i];
+    const int4 vi = view[i];
+    const ListTarget t(F, G32, kappa, vi);
+    const int rows = list_rows(cap);
+    uint32_t* __restrict__ own = list + list_at(i, 0, cap);
+    int n_in = 0, n_out = 0, cnt = 0;  // written inside / outside entries, accepted: uniform over the group
+    float reach = 0.0f;
+    for (int l = t.l0; l <= t.l1; ++l) {
+      const RowWalk<D> w(F, G32, X, t.Rs, l);
+      const int ny = w.yhi - w.ylo + 1, nr = ny * (w.zhi - w.zlo + 1);
+      for (int r = g; __any_sync(group, r < nr); r += G) {
+        int j = 0, je = 0;
+        if (r < nr) w.row(cstart, w.zlo + r / ny, w.ylo + r % ny, t.R2, j, je);
+        for (; __any_sync(group, j < je); j += 2) {
+          bool acc[2] = {false, false}, inside[2] = {false, false};
+          if (j < je) {
+            const bool two = j + 1 < je;
+            const int4 a = view[j], b = view[two ? j + 1 : j];
+            t.test<D>(vi, a, b, acc, inside);
+            acc[1] = acc[1] && two;
+            if (REACH && acc[0]) reach = fmaxf(reach, t.reach<D>(F, kappa, vi, a));
+            if (REACH && acc[1]) reach = fmaxf(reach, t.reach<D>(F, kappa, vi, b));
+          }
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            unsigned all = __ballot_sync(group, acc[q]), in = __ballot_sync(group, acc[q] && inside[q]);
+            cnt += __popc(all);
+            if (cnt > cap) {  // a full list keeps the first of them
+              for (int room = cap - n_in - n_out; __popc(all) > room;) all &= ~(1u << (31 - __clz(all)));
+              in &= all;
+            }
+            if (all >> (threadIdx.x & 31) & 1u) {
+              const int row = inside[q] ? n_in + __popc(in & below) : rows - 1 - (n_out + __popc(all & ~in & below));
+              own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)(j + q) << 8) | (meta[j + q] & 0xFFu);
+            }
+            n_in += __popc(in);
+            n_out += __popc(all & ~in);
+          }
+        }
+      }
+    }
+    for (int o = 1; o < G; o <<= 1) reach = fmaxf(reach, __shfl_xor_sync(group, reach, o));
+    if (g == 0) {
+      lcount[i] = (uint32_t)n_in | ((uint32_t)n_out << kOutShift) | (REACH && ListTarget::fast(reach) ? kFastBit : 0u);
+      if (cnt > cap) atomicOr(err, kErrListOverflow);
+      atomicMax(&longest, cnt);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && longest > 0) atomicMax(&ctl->lmax, longest);
 }
 
 // Staged pass A, set up at a list rebuild: one block per kStageBlock targets
@@ -1025,6 +1220,89 @@ __global__ void __launch_bounds__(256) k_density(int n, const StepCtl* __restric
   pc_out[i] = P.P0 * (T)pow((double)(rho / rt), (double)P.gamma) / (rho * rho);
 }
 
+// The end of pass A, called by warp 0 of every block with the block's partial in
+// lane 0: the grid's total, the step sizes, the statistics, the schedule. A
+// function of its own: inlined, its registers spilled into the pair loop.
+template <class T>
+__device__ __noinline__ void finish_step(Partial part, Partial* partials, unsigned* ticket, StepCtl* ctl,
+                                         Scalars* scal, int advance, const double* __restrict__ dt_fix,
+                                         double* __restrict__ dt_rec) {
+  if (!grid_total<T>(part, partials, ticket)) return;
+  if ((threadIdx.x & 31) == 0) {
+    const Partial& acc = part;
+    const StepCtl cc = *ctl;  
+    const long long step = cc.step;
+    // Eq. time_step_size with v_n = 0 (the velocity reset of Algorithm 1): the
+    // first time step keeps only the body-force term, dt1 = min_i 0.25
+    // sqrt(r_c,i/|a_i|). With v~_i = a_i dt1/2 and nu_i = 0.1 r_c,i |v~_i|, the
+    // second time step's terms are
+    // r_c/(40|v~|) = m/(20 dt1) and 0.125 r_c^2/nu = 2.5 m/dt1, m = min r_c/|a|
+    // (all three are monotone in r_c,i/|a_i|, so their minima share the argmin).
+    constexpr bool f32 = std::is_same<T, float>::value;
+    const double m = !f32 ? acc.min_rc_a : acc.amin >= 0 ? (double)acc.rc / (double)acc.an : DBL_MAX;
+    double dt1 = 0.0, dt2 = 0.0;
+    if (m < DBL_MAX) {
+      dt1 = 0.25 * sqrt(m);
+      dt2 = fmin(dt1, fmin(m / (20.0 * dt1), 2.5 * m / dt1));
+    }
+    if (dt_fix) {  // prescribed step sizes
+      dt1 = dt_fix[0];
+      dt2 = dt_fix[1];
+    }
+    if (dt_rec) {
+      dt_rec[0] = dt1;
+      dt_rec[1] = dt2;
+    }
+    // the step-size history of a reverse-pass run: replay or record
+    const long long hk = step - cc.dt_base;
+    if (cc.dt_mode && cc.dt_hist && hk >= 0 && hk < cc.dt_len) {
+      if (cc.dt_mode == 2) {
+        dt1 = cc.dt_hist[2 * hk];
+        dt2 = cc.dt_hist[2 * hk + 1];
+      } else {
+        cc.dt_hist[2 * hk] = dt1;
+        cc.dt_hist[2 * hk + 1] = dt2;
+      }
+    }
+    scal->dt1 = dt1;
+    scal->dt2 = dt2;
+    scal->min_rc_a = m;
+    scal->argmin = acc.amin;
+    scal->max_a = f32 ? (double)acc.ma : acc.max_a;
+    scal->sum_rho = acc.sum_rho;
+    scal->err_l2 = acc.err_l2;
+    scal->err_max = f32 ? fmax(err_exact(acc.er, acc.et), 0.0) : acc.err_max;
+    scal->sigma = (double)(T)sigma_of(cc, step);
+    scal->ipairs = acc.ipairs / 2;
+    scal->fpairs = acc.fpairs / 2;
+    scal->lentries = acc.lentries;
+    scal->wall_moved = 0;
+    scal->step_of_stats = step;
+    if (advance && cc.auto_on && !cc.auto_done) {
+      // convergence of the partition (Sec. 3.3): the interface-pair count stays
+      // within auto_tol of the count that opened the run for auto_window steps;
+      // then the ramp of Eq. sph_st_sigma starts: t0 = this step, t1 = (1 + theta) t0
+      const long long ip = acc.ipairs / 2;
+      long long ref = cc.auto_ref;
+      int stable = cc.auto_stable;
+      if (ref >= 0 && fabs((double)(ip - ref)) <= cc.auto_tol * (double)ref) {
+        ++stable;
+      } else {
+        ref = ip;
+        stable = 0;
+      }
+      ctl->auto_ref = ref;
+      ctl->auto_stable = stable;
+      if (stable >= cc.auto_window) {
+        ctl->t0 = (double)step;
+        ctl->t1 = (1.0 + cc.auto_theta) * (double)step;
+        ctl->auto_done = 1;
+      }
+    }
+    if (advance) ctl->step = step + 1;
+  }
+}
+
 // --------------------------------------------------------------------------
 // Pass A (Algorithm 1: velocity reset, forces, first time step): per target i,
 // over its listed j
@@ -1041,7 +1319,7 @@ __global__ void __launch_bounds__(256) k_density(int n, const StepCtl* __restric
 // pair counts; the last block reduces them in fixed order and sets dt1, dt2
 // (Eq. time_step_size, see below).
 // --------------------------------------------------------------------------
-template <int D, class T, bool GENERAL, bool DBG, bool SURF, int NT, bool STG = false>
+template <int D, class T, bool GENERAL, bool DBG, bool SURF, int NT, bool STG = false, int G = 1>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64 : SPH_PASS_MIN_BLOCKS) * 256 / NT) k_pass_a(int n, StepCtl* ctl,
                                                 const typename ViewOf<T>::type* __restrict__ v0,
                                                 const typename ViewOf<T>::type* __restrict__ v1,
@@ -1064,13 +1342,18 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
   static_assert(!STG || (std::is_same<T, float>::value && !GENERAL && !DBG && !SURF && NT == kStageBlock),
                 "staged pass A: FP32, gamma = 2, 256-target blocks");
   constexpr bool PACKED = std::is_same<T, float>::value && !DBG && !SURF;
+  static_assert(G == 1 || (sizeof(T) == 8 && !DBG && !SURF && NT == 32 * G),
+                "several lanes per particle: FP64, 32 particles per block");
   extern __shared__ __align__(16) unsigned char stage_smem[];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const StepCtl cc = *ctl;
-  const long long step = cc.step;
-  const int buf = cc.buf;
-  const VT* __restrict__ view = cc.vp ? v1 : v0;
-  const T sigma = (T)sigma_of(cc, step);
+  // G lanes per particle (fp64_lanes): all of a warp's lanes stay together in
+  // the loop, those past the end with an empty list; warp 0 holds the block's 32
+  // particles afterwards
+  const int slot = (blockIdx.x * NT + threadIdx.x) / G;
+  int i = G == 1 ? slot : min(slot, n - 1);
+  bool lead = slot < n;
+  const int buf = ctl->buf;
+  const VT* __restrict__ view = ctl->vp ? v1 : v0;
+  const T sigma = (T)sigma_of(*ctl, ctl->step);
   Partial part = no_partial();
   float own_rc = 0, own_an = 0, own_rho = 0, own_rt = 0;  // FP32 path: this particle's share of the reductions
   int own_ni = 0, own_nf = 0, own_cnt = 0;
@@ -1088,7 +1371,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     }
     __syncthreads();
   }
-  if (i < n) {
+  if (G > 1 || i < n) {
     const uint32_t* __restrict__ pid = buf ? p1 : p0;
     const VT vi = view[i];
     const uint32_t* __restrict__ meta = buf ? m1 : m0;
@@ -1097,19 +1380,20 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // a feature-surface particle (Sec. 3.5) takes forces from surface particles
     // only (SURF: the variant launched when the handle has any)
     const bool surf = SURF && (mi & kSurfaceBit) != 0;
-    const T hv = view_h(F, vi);
+    T hv = view_h(F, vi);
     const T qv = F.qv;
-    const T Hd = P.kappa * hv, Hd2 = Hd * Hd, invHd = T(1) / Hd;
-    const T inv_tau_v = P.inv_tau * qv;           // h in view units -> (h/tau)
-    const T qi = inv_rho_t2<D, T>(hv, inv_tau_v);  // 1/rho_t,i^2
+    T Hd = P.kappa * hv;
+    const T Hd2 = Hd * Hd, invHd = T(1) / Hd;
+    const T inv_tau_v = P.inv_tau * qv;     // h in view units -> (h/tau)
+    T qi = inv_rho_t2<D, T>(hv, inv_tau_v);  // 1/rho_t,i^2
     const T Pi = GENERAL ? pc[i] : P.P0 * qi;
     const T sP0 = sigma * P.P0;
     const T half_kappa = T(0.5) * P.kappa;
     T dsum = 0, ax = 0, ay = 0, az = 0;
     int nf = 0, ni = 0, nd = 0;
     long long sd = 0, sf = 0;
-    const uint32_t lc = lcount[i];
-    const int cnt = list_cnt(lc);
+    const uint32_t lc = lead ? lcount[i] : 0u;
+    int cnt = list_cnt(lc);
     PairRec<T>* __restrict__ pw = plist + pair_at(i, 0, cap);  // this step's force pairs, for pass B
     // FP32: the listed entries two at a time, every FP32 operation on both at
     // once, on exact differences throughout (a coarse screen first saved the
@@ -1202,7 +1486,19 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // criteria on every entry (FP64 path with current FP32 views: on those that
     // pass a screen in FP32, for_skin_list_s32)
     constexpr bool S32_OK = std::is_same<T, double>::value && !GENERAL && !DBG && !SURF;
+    // G > 1: the pairs of the group's lanes one after another, in lane order
+    auto push_all = [&](bool have, uint32_t e, bool other, T f) {
+      const unsigned m = __ballot_sync(0xffffffffu, have) & group_mask<G>();
+      if (have) {
+        store_pair(pw + 32 * __popc(m & lanes_below()), e, f);
+        ni += other;
+      }
+      pw += 32 * __popc(m);
+      nf += __popc(m);
+    };
     const T iscale = T(1) / pair_scale<D>(qi, invHd);
+    bool have = false, have_other = false;  // G > 1: what the lane's entry adds to the group's pairs
+    T have_f = 0;
     auto pair = [&](uint32_t e, const VT& vj) {
       const int j = (int)(e >> 8);
       const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
@@ -1237,14 +1533,36 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
         ax += s * dx;
         ay += s * dy;
         az += s * dz;
-        store_pair(pw, e, (qi + qj) * w * iscale);
-        pw += 32;
-        ++nf;
-        ni += other;
+        if (G == 1) {
+          store_pair(pw, e, (qi + qj) * w * iscale);
+          pw += 32;
+          ++nf;
+          ni += other;
+        } else {
+          have = true;
+          have_other = other;
+          have_f = (qi + qj) * w * iscale;
+        }
         if (DBG) sf += pid[j];
       }
     };
-    if (S32_OK && v32 && (lc & kFastBit)) {
+    if constexpr (G > 1) {
+      // lane g of the group takes entries g, g + G, ...
+      const int n_in = list_in(lc);
+      for (int k = threadIdx.x % G; __any_sync(0xffffffffu, k < cnt); k += G) {
+        have = false;
+        uint32_t e = 0;
+        if (k < cnt) {
+          e = list[list_at(i, list_row(k, n_in, cap), cap)];
+          pair(e, view[e >> 8]);
+        }
+        push_all(have, e, have_other, have_f);
+      }
+      dsum = group_sum<G>(dsum);
+      ax = group_sum<G>(ax);
+      ay = group_sum<G>(ay);
+      az = group_sum<G>(az);
+    } else if (S32_OK && v32 && (lc & kFastBit)) {
       const int4 wi = v32[i];
       const float ws = 2.0f / (float)(1 << kViewBits), wi32 = 0.5f * ws * view_w(wi), Hd32 = ws * view_w(wi);  // view units
       auto screen = [&](const int4& w) {
@@ -1259,7 +1577,42 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       for_skin_list(list, view, i, lc, cap, pair);
     }
     }
-    pcount[i] = (uint32_t)nf;
+    if constexpr (G > 1) {
+      // the 32 particles of the block to the lanes of warp 0: what follows
+      // costs a warp as much for one particle as for 32
+      __shared__ T sums[4][32];
+      __shared__ int counted[3][32];
+      ni = group_sum<G>(ni);
+      const int t = threadIdx.x / G;
+      if (threadIdx.x % G == 0) {
+        sums[0][t] = dsum;
+        sums[1][t] = ax;
+        sums[2][t] = ay;
+        sums[3][t] = az;
+        counted[0][t] = nf;
+        counted[1][t] = ni;
+        counted[2][t] = cnt;
+      }
+      __syncthreads();
+      if (threadIdx.x >= 32) return;
+      dsum = sums[0][threadIdx.x];
+      ax = sums[1][threadIdx.x];
+      ay = sums[2][threadIdx.x];
+      az = sums[3][threadIdx.x];
+      nf = counted[0][threadIdx.x];
+      ni = counted[1][threadIdx.x];
+      cnt = counted[2][threadIdx.x];
+      i = blockIdx.x * 32 + threadIdx.x;
+      lead = i < n;
+      i = min(i, n - 1);
+    }
+    // the target's lengths again (of another target where G > 1): kept over the
+    // loop they cost registers that spill
+    hv = view_h(F, view[i]);
+    Hd = P.kappa * hv;
+    qi = inv_rho_t2<D, T>(hv, P.inv_tau * qv);
+    if (G == 1) cnt = list_cnt(lcount[i]);
+    if (lead) pcount[i] = (uint32_t)nf;
     // back to physical units: rho ~ 1/H^D, a ~ (view length)^-(D+1)
     const T Hphys = Hd * qv;
     const T rho = GENERAL ? rho_out[i] : dsum * P.alpha / (D == 2 ? Hphys * Hphys : Hphys * Hphys * Hphys);
@@ -1281,29 +1634,31 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     const T rt = T(1) / dsqrt(qi);
     const T rc = Hphys;
     const T g = T(0.05) * rt * rc * an;
-    acc_out[i] = V4<T>{ax, ay, az, g};
-    if (!GENERAL && rho_out) rho_out[i] = rho;
+    if (lead) acc_out[i] = V4<T>{ax, ay, az, g};
+    if (!GENERAL && rho_out && lead) rho_out[i] = rho;
     if constexpr (std::is_same<T, float>::value) {
       own_rc = rc;
       own_an = an;
       own_rho = rho;
       own_rt = rt;
-      own_ni = ni;
-      own_nf = nf;
-      own_cnt = cnt;
+      own_ni = lead ? ni : 0;
+      own_nf = lead ? nf : 0;
+      own_cnt = lead ? cnt : 0;
     } else {
       const double e = (double)rho / (double)rt - 1.0;
-      part.min_rc_a = an > T(0) ? (double)rc / (double)an : DBL_MAX;
-      part.amin = an > T(0) ? (long long)i : -1;
-      part.max_a = (double)an;
-      part.sum_rho = (double)rho;
-      part.err_l2 = e * e;
-      part.err_max = fabs(e);
-      part.ipairs = ni;
-      part.fpairs = nf;
-      part.lentries = cnt;
+      if (lead) {
+        part.min_rc_a = an > T(0) ? (double)rc / (double)an : DBL_MAX;
+        part.amin = an > T(0) ? (long long)i : -1;
+        part.max_a = (double)an;
+        part.sum_rho = (double)rho;
+        part.err_l2 = e * e;
+        part.err_max = fabs(e);
+        part.ipairs = ni;
+        part.fpairs = nf;
+        part.lentries = cnt;
+      }
     }
-    if (!(isfinite(an) && isfinite(rho))) atomicOr(err, kErrNonfinite);
+    if (lead && !(isfinite(an) && isfinite(rho))) atomicOr(err, kErrNonfinite);
     if (DBG) {
       const uint32_t id = pid[i];
       dbg_count[2 * id] = nd;
@@ -1313,95 +1668,30 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     }
   }
   // the block's partial in warp 0 (the other warps are done), then the grid's
-  constexpr int NW = NT / 32;
+  constexpr int NW = G > 1 ? 1 : NT / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if constexpr (std::is_same<T, float>::value) {
     __shared__ WarpSums ws[NW];
-    warp_sums(i < n, i, own_rc, own_an, own_rho, own_rt, own_ni, own_nf, own_cnt, ws + warp);
-    __syncthreads();
-    if (warp != 0) return;
+    warp_sums(lead, i, own_rc, own_an, own_rho, own_rt, own_ni, own_nf, own_cnt, ws + warp);
+    if (NW > 1) {
+      __syncthreads();
+      if (warp != 0) return;
+    } else {
+      __syncwarp();
+    }
     part = lane < NW ? to_partial(ws[lane]) : no_partial();
+    if (NW > 1) part = warp_total<T>(part);
   } else {
-    __shared__ Partial sm[NW];
-    warp_merge<T>(part, 32);
-    if (lane == 0) sm[warp] = part;
-    __syncthreads();
-    if (warp != 0) return;
-    part = lane < NW ? sm[lane] : no_partial();
+    part = warp_total<T>(part);
+    if constexpr (NW > 1) {
+      __shared__ Partial sm[NW];
+      if (lane == 0) sm[warp] = part;
+      __syncthreads();
+      if (warp != 0) return;
+      part = warp_total<T>(lane < NW ? sm[lane] : no_partial());
+    }
   }
-  warp_merge<T>(part, NW);
-  if (!grid_total<T>(part, partials, ticket)) return;
-  if (lane == 0) {
-    const Partial& acc = part;
-    // Eq. time_step_size with v_n = 0 (the velocity reset of Algorithm 1): the
-    // first time step keeps only the body-force term, dt1 = min_i 0.25
-    // sqrt(r_c,i/|a_i|). With v~_i = a_i dt1/2 and nu_i = 0.1 r_c,i |v~_i|, the
-    // second time step's terms are
-    // r_c/(40|v~|) = m/(20 dt1) and 0.125 r_c^2/nu = 2.5 m/dt1, m = min r_c/|a|
-    // (all three are monotone in r_c,i/|a_i|, so their minima share the argmin).
-    constexpr bool f32 = std::is_same<T, float>::value;
-    const double m = !f32 ? acc.min_rc_a : acc.amin >= 0 ? (double)acc.rc / (double)acc.an : DBL_MAX;
-    double dt1 = 0.0, dt2 = 0.0;
-    if (m < DBL_MAX) {
-      dt1 = 0.25 * sqrt(m);
-      dt2 = fmin(dt1, fmin(m / (20.0 * dt1), 2.5 * m / dt1));
-    }
-    if (dt_fix) {  // prescribed step sizes
-      dt1 = dt_fix[0];
-      dt2 = dt_fix[1];
-    }
-    if (dt_rec) {
-      dt_rec[0] = dt1;
-      dt_rec[1] = dt2;
-    }
-    // the step-size history of a reverse-pass run: replay or record
-    const long long hk = step - cc.dt_base;
-    if (cc.dt_mode && cc.dt_hist && hk >= 0 && hk < cc.dt_len) {
-      if (cc.dt_mode == 2) {
-        dt1 = cc.dt_hist[2 * hk];
-        dt2 = cc.dt_hist[2 * hk + 1];
-      } else {
-        cc.dt_hist[2 * hk] = dt1;
-        cc.dt_hist[2 * hk + 1] = dt2;
-      }
-    }
-    scal->dt1 = dt1;
-    scal->dt2 = dt2;
-    scal->min_rc_a = m;
-    scal->argmin = acc.amin;
-    scal->max_a = acc.max_a;
-    scal->sum_rho = acc.sum_rho;
-    scal->err_l2 = acc.err_l2;
-    scal->err_max = f32 ? fmax(err_exact(acc.er, acc.et), 0.0) : acc.err_max;
-    scal->sigma = (double)sigma;
-    scal->ipairs = acc.ipairs / 2;
-    scal->fpairs = acc.fpairs / 2;
-    scal->lentries = acc.lentries;
-    scal->wall_moved = 0;
-    scal->step_of_stats = step;
-    if (advance && cc.auto_on && !cc.auto_done) {
-      // convergence of the partition (Sec. 3.3): the interface-pair count stays
-      // within auto_tol of the count that opened the run for auto_window steps;
-      // then the ramp of Eq. sph_st_sigma starts: t0 = this step, t1 = (1 + theta) t0
-      const long long ip = acc.ipairs / 2;
-      long long ref = cc.auto_ref;
-      int stable = cc.auto_stable;
-      if (ref >= 0 && fabs((double)(ip - ref)) <= cc.auto_tol * (double)ref) {
-        ++stable;
-      } else {
-        ref = ip;
-        stable = 0;
-      }
-      ctl->auto_ref = ref;
-      ctl->auto_stable = stable;
-      if (stable >= cc.auto_window) {
-        ctl->t0 = (double)step;
-        ctl->t1 = (1.0 + cc.auto_theta) * (double)step;
-        ctl->auto_done = 1;
-      }
-    }
-    if (advance) ctl->step = step + 1;
-  }
+  finish_step<T>(part, partials, ticket, ctl, scal, advance, dt_fix, dt_rec);
 }
 
 // --------------------------------------------------------------------------
@@ -1415,7 +1705,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
 // The new view goes to the other view buffer; a particle that moved half its
 // skin since the list was built raises need_rebuild.
 // --------------------------------------------------------------------------
-template <int D, class T, int NT>
+template <int D, class T, int NT, int G = 1>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP64 : SPH_PASSB_MIN_BLOCKS) * 256 / NT) k_pass_b(int n, StepCtl* __restrict__ ctl,
                                                 const typename ViewOf<T>::type* __restrict__ v0,
                                                 const typename ViewOf<T>::type* __restrict__ v1,
@@ -1432,23 +1722,24 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
                                                 const uint32_t* __restrict__ m1, int4* __restrict__ v32out,
                                                 int sv32, float c2w32) {
   using VT = typename ViewOf<T>::type;
-  __shared__ int moved_sm[8];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ int moved_sm[NT / 32];
+  // G lanes per particle, as pass A
+  static_assert(G == 1 || NT == 32 * G, "several lanes per particle: 32 particles per block");
+  const int slot = (blockIdx.x * NT + threadIdx.x) / G;
+  int i = G == 1 ? slot : min(slot, n - 1);
+  bool lead = slot < n;
   const int vp = ctl->vp, buf = ctl->buf;
   int moved = 0, far = 0;
-  if (i < n) {
+  if (G > 1 || i < n) {
     const VT* __restrict__ view = vp ? v1 : v0;
-    const VT vi = view[i];
-    const T hv = view_h(F, vi);
-    const T qi = inv_rho_t2<D, T>(hv, P.inv_tau * F.qv);
-    const V4<T> ai = acc[i];
+    V4<T> ai = acc[i];
     T bx = 0, by = 0, bz = 0;
     // this step's pairs as pass A left them: the geometry in a factor per pair,
     // so only the neighbour's acceleration is gathered and no distance, root or
     // kernel value is computed again. FP32, 8,388,608 particles in 3D: 1.40 ->
     // 0.86 ms, and pass A, which writes the factor, 1.59 -> 1.65; FP64, where the
     // FP64 pipe bounds both passes, 300,007 in 3D: 1.40 -> 0.43 ms.
-    const int cnt = (int)pcount[i];
+    const int cnt = lead ? (int)pcount[i] : 0;
     const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
     if constexpr (std::is_same<T, float>::value) {
       // two pairs per instruction; sums of (a_j - a_i), factor gi gj / (gi + gj)
@@ -1465,6 +1756,16 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       };
       constexpr int B = SPH_PASSB_BATCH;
       int k = 0;
+      if constexpr (G > 1) {
+        for (k = 2 * (threadIdx.x % G), p += 32 * k; k < cnt; k += 2 * G, p += 64 * G) {
+          const PairRec<T> r0 = load_pair(p);
+          PairRec<T> r1{r0.e, 0.0f};
+          if (k + 1 < cnt) r1 = load_pair(p + 32);
+          const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
+          two(r0, a0, r1, a1);
+        }
+        __syncwarp();
+      } else {
       PairRec<T> ahead[B];
       if (cnt >= B)
 #pragma unroll
@@ -1491,6 +1792,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
         two(r0, a0, r1, a1);
       }
+      }
       bx = -2.0f * (bx2.x + bx2.y);
       by = -2.0f * (by2.x + by2.y);
       bz = -2.0f * (bz2.x + bz2.y);
@@ -1503,6 +1805,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         bz += s * (ai.z - aj.z);
       };
       int k = 0;
+      if constexpr (G > 1) {
+        for (k = threadIdx.x % G, p += 32 * k; k < cnt; k += G, p += 32 * G) {
+          const PairRec<T> r0 = load_pair(p);
+          pair(r0, acc[r0.e >> 8]);
+        }
+        __syncwarp();
+      }
       for (; k + 2 <= cnt; k += 2, p += 64) {
         const PairRec<T> r0 = load_pair(p), r1 = load_pair(p + 32);
         const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
@@ -1514,6 +1823,29 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         pair(r0, acc[r0.e >> 8]);
       }
     }
+    if constexpr (G > 1) {  // the block's 32 particles to warp 0
+      __shared__ T sums[3][32];
+      bx = group_sum<G>(bx);
+      by = group_sum<G>(by);
+      bz = group_sum<G>(bz);
+      if (threadIdx.x % G == 0) {
+        sums[0][threadIdx.x / G] = bx;
+        sums[1][threadIdx.x / G] = by;
+        sums[2][threadIdx.x / G] = bz;
+      }
+      __syncthreads();
+      i = blockIdx.x * 32 + threadIdx.x;
+      lead = threadIdx.x < 32 && i < n;
+      i = min(i, n - 1);
+      bx = sums[0][threadIdx.x & 31];
+      by = sums[1][threadIdx.x & 31];
+      bz = sums[2][threadIdx.x & 31];
+      ai = acc[i];
+    }
+    if (G == 1 || threadIdx.x < 32) {
+    const VT vi = view[i];
+    const T hv = view_h(F, vi);
+    const T qi = inv_rho_t2<D, T>(hv, P.inv_tau * F.qv);
     // dW/dr / r = -20 alpha (1-q)^3 / H^(D+2); view lengths -> physical
     const T iq = F.inv_qv;
     const T km = T(-20) * P.alpha * (D == 2 ? iq * iq * iq * iq : iq * iq * iq * iq * iq) *
@@ -1535,8 +1867,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
     const T kv = T(0.5) * dt1 * dt1;  // a~ = kv B
     // a~ for the caller when asked (a run-time test: one compiled kernel, so
     // recording cannot change the arithmetic of the step)
-    if (visc_out) visc_out[i] = V4<T>{kv * bx, kv * by, kv * bz, T(0)};
-    if (move) {
+    if (visc_out && lead) visc_out[i] = V4<T>{kv * bx, kv * by, kv * bz, T(0)};
+    if (move && lead) {
     T d[3];
     d[0] = (T(0.5) * dt1 * ai.x + T(0.5) * dt2 * kv * bx) * dt2;
     d[1] = (T(0.5) * dt1 * ai.y + T(0.5) * dt2 * kv * by) * dt2;
@@ -1579,7 +1911,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       const T hn = h_of<D, T>(geo, xa);
       const VT vn = make_view<D>(F, X, hn);
       (vp ? w0 : w1)[i] = vn;
-      if (v32out) {  // FP64 path: its FP32 view of the next step (as k_view32 makes it)
+      if (v32out) {  // FP64 path: its FP32 view of the next step (as k_gather_view makes it)
         const long long half = 1LL << (sv32 - 1);
         v32out[i] = make_int4((int)((X.x + half) >> sv32), (int)((X.y + half) >> sv32),
                               D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_w(vn) * c2w32));
@@ -1594,6 +1926,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       (vp ? w0 : w1)[i] = vi;
     }
     }  // move
+    }
   }
   if (__syncthreads_or(far) && threadIdx.x == 0) ctl->need_rebuild = 1;
   int v = moved;
@@ -1675,41 +2008,68 @@ __global__ void __launch_bounds__(256) k_get_fields(int n, int which, const Step
 // --------------------------------------------------------------------------
 inline int grid_for(int n, int tb) { return (n + tb - 1) / tb; }
 
+// Small particle counts, where one thread per particle leaves most of the chip
+// idle and a thread's own chain of loads (FP64: of arithmetic) is the whole
+// time: several lanes share a particle. Steps of the circle (2D, FP32), 4,289 /
+// 16,001 particles: the list build's groups of 8 save 6 / 2 us; of a ball (3D),
+// 10,001 / 16,001: 8 / 6 us, pass B's groups 3 / 3 us; at 24,001 both lose.
+// (Pass A in FP32 gained nothing at any size.) FP64, the 4,096-particle square:
+// 74 us with 32-thread blocks alone, 48 with 4 lanes; 16,001: 97 and 95;
+// 32,001: 124 and 148.
+constexpr int kListLanes = 8, kListGroupMax = 20480;
+constexpr int kPassLanes = 8, kPassGroupMax = 16384;
+constexpr int kLanes64 = 4, kGroupMax64 = 8192;
+inline int fp64_lanes(const DevState& S) { return S.n <= kGroupMax64 ? kLanes64 : 1; }
+// Threads per block of the FP64 pair passes (FP32: DevState::pass_threads): one
+// warp of FP64 work keeps an SM's FP64 pipe busy, so small blocks spread the
+// particles evenly over the SMs. 200,003 particles in 2D, one step: 674 -> 561 us
+// (256 -> 64 threads), 300,007 in 3D: 2,264 -> 2,077; the 4,096-particle square,
+// 16 blocks of 256 on 152 SMs: 106 -> 74 us (32).
+inline int fp64_threads(const DevState& S) { return S.n <= (1 << 17) ? 32 : 64; }
+
 template <int D, class T>
-cudaError_t launch_rebuild(const DevState& S, const Grid<T>& G, const Frame<T>& F, const Geom<T>& g, T kappa,
-                           cudaStream_t st, const Grid<float>* G32, const Frame<float>* F32) {
+cudaError_t launch_rebuild(const DevState& S, int force, const Grid<T>& G, const Frame<T>& F, const Geom<T>& g,
+                           T kappa, cudaStream_t st, const Grid<float>* G32, const Frame<float>* F32) {
   using VT = typename ViewOf<T>::type;
   // the cheap per-particle kernels on a capped grid (an idle launch costs a
   // few us); the list build on one block per 256 targets: a grid capped at
   // 16 or 32 blocks per SM made its rebuilds of the 8M 3D workload slower
   // (cells 2.01 / 1.93 vs 1.86 ms per step), its blocks no longer finishing
   // and refilling the SMs independently
-  const int tb = 256, gb = rebuild_grid(S.n, tb, 8), gl = grid_for(S.n, tb);
+  const int tb = 256, gb = rebuild_grid(S.n, tb, 8);
   const LL4* X0 = (const LL4*)S.X[0];
   const LL4* X1 = (const LL4*)S.X[1];
-  k_rekey<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, X0, X1, F, G, g, S.key);
-#define SPH_LIST_BUILD(TT) k_list_build<D, TT><<<gl, tb, 0, st>>>
+  k_rekey<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, force, S.tickets + 1, X0, X1, F, G, g, S.key, S.cnt, S.scan_part);
   cudaError_t e = build_cells(S, st);
   if (e != cudaSuccess) return e;
-  k_make_view<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, 0, X0, X1, F, g, (VT*)S.view[0], (VT*)S.view[1],
-                                       (VT*)S.vbuild);
-  if constexpr (std::is_same<T, double>::value) {
-    // the FP64 path lists its pairs through an FP32 view (same frame origin,
-    // same cells, same list format)
-    if (!S.view32 || !F32 || !G32) return cudaErrorInvalidValue;
-    k_view32<D><<<gb, tb, 0, st>>>(S.n, S.ctl, X0, X1, *F32, (const V4<double>*)S.view[0],
-                                   (const V4<double>*)S.view[1], (int4*)S.view32);
-    SPH_LIST_BUILD(float)(S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], (const int4*)S.view32,
-                          (const int4*)S.view32, S.cstart, *F32, *G32, (float)kappa, S.cap, S.list, S.lcount,
-                          S.err);
-  } else {
-    SPH_LIST_BUILD(T)(S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], (const VT*)S.view[0], (const VT*)S.view[1],
-                      S.cstart, F, G, kappa, S.cap, S.list, S.lcount, S.err);
+  // the FP64 path lists its pairs through an FP32 view (same frame origin, same
+  // cells, same list format)
+  if (std::is_same<T, double>::value && (!S.view32 || !F32 || !G32)) return cudaErrorInvalidValue;
+  k_gather_view<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, S.tmp, S.key, S.cstart, (LL4*)S.X[0], (LL4*)S.X[1], S.meta[0],
+                                         S.meta[1], S.pid[0], S.pid[1], F, g, (VT*)S.view[0], (VT*)S.view[1],
+                                         (VT*)S.vbuild, (int4*)S.view32, F32 ? *F32 : Frame<float>{});
+  constexpr bool f64 = std::is_same<T, double>::value;
+  const Frame<float>* Fl = F32;
+  const Grid<float>* Gl = G32;
+  const int4 *w0 = (const int4*)S.view32, *w1 = w0;
+  if constexpr (!f64) {
+    Fl = &F;
+    Gl = &G;
+    w0 = (const int4*)S.view[0];
+    w1 = (const int4*)S.view[1];
+  }
+  const bool group = S.n <= kListGroupMax;
+  auto build = [&](auto* kernel, int blocks) {
+    kernel<<<blocks, tb, 0, st>>>(S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], w0, w1, S.cstart, *Fl, *Gl, (float)kappa,
+                                  S.cap, S.list, S.lcount, S.err);
+  };
+  if (group) build(k_list_build_group<D, kListLanes, f64>, grid_for(S.n * kListLanes, tb));
+  else build(k_list_build<D, f64>, grid_for(S.n, tb));
+  if constexpr (!f64) {
     if (S.stage && S.llist)
       k_stage<D><<<grid_for(S.n, kStageBlock), kStageBlock, 0, st>>>(S.n, S.ctl, S.list, S.lcount, S.cap, S.llist,
                                                                   S.scount, S.sj);
   }
-#undef SPH_LIST_BUILD
   return cudaGetLastError();
 }
 
@@ -1718,53 +2078,49 @@ cudaError_t launch_pass_a(const DevState& S, const Frame<T>& F, const Phys<T>& P
   using VT = typename ViewOf<T>::type;
   Geom<T> geo{};
   if (f.geo) geo = *(const Geom<T>*)f.geo;
-  const int tb = S.pass_threads == 128 ? 128 : 256, gb = grid_for(S.n, tb);
   T* rho = (T*)S.rho;
   T* pc = (T*)S.pc;
   // the FP64 path screens on its FP32 views when the caller passes their frame
   const bool s32 = std::is_same<T, double>::value && S.view32 && f.f32;
   const int4* v32 = s32 ? (const int4*)S.view32 : nullptr;
   const Frame<float> f32 = s32 ? *f.f32 : Frame<float>{};
-  if (f.general_eos)
-    k_density<D, T><<<grid_for(S.n, 256), 256, 0, st>>>(S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1],
-                                                        S.list, S.lcount, S.cap, F, P, rho, pc);
-#define SPH_PASS_A_NT(GEN, DBG, NT)                                                                             \
-  (f.surface ? k_pass_a<D, T, GEN, DBG, true, NT> : k_pass_a<D, T, GEN, DBG, false, NT>)<<<gb, tb, 0, st>>>(    \
-                                              S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1],           \
-                                              S.meta[0], S.meta[1], S.pid[0], S.pid[1], S.list, S.lcount, S.cap, \
-                                              F, P,                                                             \
-                                              pc, (V4<T>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err,   \
-                                              f.advance, S.dbg_count, S.dbg_sum, (PairRec<T>*)S.plist, S.pcount, f.dt_fix,     \
-                                              f.dt_rec, (const LL4*)S.X[0], (const LL4*)S.X[1], geo, S.llist,     \
-                                              S.scount, S.sj, v32, f32)
-#define SPH_PASS_A(GEN, DBG)           \
-  do {                                 \
-    if (tb == 128)                     \
-      SPH_PASS_A_NT(GEN, DBG, 128);    \
-    else                               \
-      SPH_PASS_A_NT(GEN, DBG, 256);    \
-  } while (0)
-  if constexpr (std::is_same<T, float>::value) {
-    if (staged_pass(S, f)) {
-      k_pass_a<D, float, false, false, false, kStageBlock, true>
-          <<<grid_for(S.n, kStageBlock), kStageBlock, kStageCap * sizeof(int4), st>>>(
-              S.n, S.ctl, (const int4*)S.view[0], (const int4*)S.view[1], S.meta[0], S.meta[1], S.pid[0], S.pid[1],
-              S.list, S.lcount, S.cap, F, P, pc, (V4<float>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err,
-              f.advance, S.dbg_count, S.dbg_sum, (PairRec<T>*)S.plist, S.pcount, f.dt_fix, f.dt_rec, (const LL4*)S.X[0],
-              (const LL4*)S.X[1], geo, S.llist, S.scount, S.sj, nullptr, Frame<float>{});
-      return cudaGetLastError();
-    }
-  }
-  if (f.general_eos) {
-    if (f.nbr_debug) SPH_PASS_A(true, true);
-    else SPH_PASS_A(true, false);
-  } else {
-    if (f.nbr_debug) SPH_PASS_A(false, true);
-    else SPH_PASS_A(false, false);
-  }
+  auto run = [&](auto* kernel, int threads, int lanes, size_t smem) {
+    kernel<<<grid_for(S.n * lanes, threads), threads, smem, st>>>(
+        S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], S.meta[0], S.meta[1], S.pid[0], S.pid[1], S.list,
+        S.lcount, S.cap, F, P, pc, (V4<T>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err, f.advance, S.dbg_count,
+        S.dbg_sum, (PairRec<T>*)S.plist, S.pcount, f.dt_fix, f.dt_rec, (const LL4*)S.X[0], (const LL4*)S.X[1], geo,
+        S.llist, S.scount, S.sj, v32, f32);
+    return cudaGetLastError();
+  };
+  const auto density = [&](auto* kernel, int threads) {
+    kernel<<<grid_for(S.n, threads), threads, 0, st>>>(S.n, S.ctl, (const VT*)S.view[0],
+                                                               (const VT*)S.view[1], S.list, S.lcount, S.cap, F, P,
+                                                               rho, pc);
+  };
+  // one block size and one of the compiled variants
+  auto pick = [&](auto nt) -> cudaError_t {
+    constexpr int NT = decltype(nt)::value;
+#define SPH_PASS_A(GEN, DBG) \
+  run(f.surface ? k_pass_a<D, T, GEN, DBG, true, NT> : k_pass_a<D, T, GEN, DBG, false, NT>, NT, 1, 0)
+    if (f.general_eos) return f.nbr_debug ? SPH_PASS_A(true, true) : SPH_PASS_A(true, false);
+    return f.nbr_debug ? SPH_PASS_A(false, true) : SPH_PASS_A(false, false);
 #undef SPH_PASS_A
-#undef SPH_PASS_A_NT
-  return cudaGetLastError();
+  };
+  if constexpr (std::is_same<T, float>::value) {
+    if (f.general_eos) density(k_density<D, T>, 256);
+    if (staged_pass(S, f))
+      return run(k_pass_a<D, T, false, false, false, kStageBlock, true>, kStageBlock, 1, kStageCap * sizeof(int4));
+    if (S.pass_threads == 128) return pick(std::integral_constant<int, 128>{});
+    return pick(std::integral_constant<int, 256>{});
+  } else {
+    const int nt = fp64_threads(S);
+    if (f.general_eos) density(k_density<D, T>, nt);
+    if (fp64_lanes(S) > 1 && !f.surface && !f.nbr_debug)
+      return f.general_eos ? run(k_pass_a<D, T, true, false, false, 32 * kLanes64, false, kLanes64>, 32 * kLanes64, kLanes64, 0)
+                           : run(k_pass_a<D, T, false, false, false, 32 * kLanes64, false, kLanes64>, 32 * kLanes64, kLanes64, 0);
+    if (nt == 32) return pick(std::integral_constant<int, 32>{});
+    return pick(std::integral_constant<int, 64>{});
+  }
 }
 
 template <int D>
@@ -1779,14 +2135,23 @@ template <int D, class T>
 cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P, const Geom<T>& g, PassFlags f,
                           cudaStream_t st) {
   using VT = typename ViewOf<T>::type;
-  const int tb = S.pass_threads == 128 ? 128 : 256, gb = grid_for(S.n, tb);
   unsigned long long* wm = (unsigned long long*)&S.scal->wall_moved;
-  (tb == 128 ? k_pass_b<D, T, 128> : k_pass_b<D, T, 256>)<<<gb, tb, 0, st>>>(
-      S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], (VT*)S.view[0], (VT*)S.view[1], (const VT*)S.vbuild,
-      (LL4*)S.X[0], (LL4*)S.X[1], (const PairRec<T>*)S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
-      f.record ? (V4<T>*)S.visc : nullptr, S.err, wm, f.move, S.meta[0], S.meta[1],
-      (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0, f.f32 ? f.f32->c2w : 0.0f);
-  return cudaGetLastError();
+  auto run = [&](auto* kernel, int threads, int lanes) {
+    kernel<<<grid_for(S.n * lanes, threads), threads, 0, st>>>(
+        S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], (VT*)S.view[0], (VT*)S.view[1], (const VT*)S.vbuild,
+        (LL4*)S.X[0], (LL4*)S.X[1], (const PairRec<T>*)S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
+        f.record ? (V4<T>*)S.visc : nullptr, S.err, wm, f.move, S.meta[0], S.meta[1],
+        (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0,
+        f.f32 ? f.f32->c2w : 0.0f);
+    return cudaGetLastError();
+  };
+  if constexpr (std::is_same<T, float>::value) {
+    if (S.n <= kPassGroupMax) return run(k_pass_b<D, T, 32 * kPassLanes, kPassLanes>, 32 * kPassLanes, kPassLanes);
+    return S.pass_threads == 128 ? run(k_pass_b<D, T, 128>, 128, 1) : run(k_pass_b<D, T, 256>, 256, 1);
+  } else {
+    if (fp64_lanes(S) > 1) return run(k_pass_b<D, T, 32 * kLanes64, kLanes64>, 32 * kLanes64, kLanes64);
+    return fp64_threads(S) == 32 ? run(k_pass_b<D, T, 32>, 32, 1) : run(k_pass_b<D, T, 64>, 64, 1);
+  }
 }
 
 template <int D, class T>
@@ -1817,8 +2182,9 @@ cudaError_t launch_get_fields(const DevState& S, int which, double* out, cudaStr
 }
 
 #define SPH_INSTANTIATE_STEP(D, T)                                                                             \
-  template cudaError_t launch_rebuild<D, T>(const DevState&, const Grid<T>&, const Frame<T>&, const Geom<T>&, \
-                                            T, cudaStream_t, const Grid<float>*, const Frame<float>*);        \
+  template cudaError_t launch_rebuild<D, T>(const DevState&, int, const Grid<T>&, const Frame<T>&,            \
+                                            const Geom<T>&, T, cudaStream_t, const Grid<float>*,              \
+                                            const Frame<float>*);                                             \
   template cudaError_t launch_pass_a<D, T>(const DevState&, const Frame<T>&, const Phys<T>&, PassFlags,       \
                                            cudaStream_t);                                                     \
   template cudaError_t launch_pass_b<D, T>(const DevState&, const Frame<T>&, const Phys<T>&, const Geom<T>&,  \
