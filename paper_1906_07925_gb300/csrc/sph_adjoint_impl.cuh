@@ -628,23 +628,40 @@ __global__ void __launch_bounds__(256) k_bwd_local(int n, const StepCtl* __restr
     T hbar = B.hb[i];
     T xx = 0, xy = 0, xz = 0;
     if (DENS) {
+      // W' of the pair with the support of i, and with that of j; entries outside
+      // both (a third of a list) stop at the distance, and W'/r = -20 c H^-(d+2)
+      // (1 - q)^3 needs no division by r
       const T rbi = B.rhob[i];
-      const T Hi = P.kappa * hi;
+      const T Hvi = P.kappa * hv, Hvi2 = Hvi * Hvi, iHvi = T(1) / Hvi, iHi = iHvi * F.inv_qv;
+      const T ci = rbi * P.alpha * ipow_d<D, T>(iHi), fi = T(-20) * ci * iHi * iHi;
+      T wh = 0;
       for_skin_list(list, view, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
         const int j = (int)(e >> 8);
         const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
         const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
-        const T r = dsqrt(dx * dx + dy * dy + dz * dz) * qv;
-        const KernelD<D, T> ki = wendland<D, T>(r, Hi, P.alpha);
-        hbar += rbi * ki.WH * P.kappa;
-        if (j == i || !(r > T(0))) return;
-        const T Hj = P.kappa * view_h(F, vj) * qv;
-        const KernelD<D, T> kj = wendland<D, T>(r, Hj, P.alpha);
-        const T c = (rbi * ki.Wr + B.rhob[j] * kj.Wr) / r;
-        xx += c * dx * qv;
-        xy += c * dy * qv;
-        xz += c * dz * qv;
+        const T r2 = dx * dx + dy * dy + dz * dz;
+        const T Hvj = P.kappa * view_h(F, vj);
+        const bool in_i = r2 < Hvi2, in_j = r2 < Hvj * Hvj && j != i;
+        if (!(in_i || in_j)) return;
+        const T r = r2 > T(0) ? pair_r<T>(r2) : T(0);
+        T c = 0;
+        if (in_i) {
+          const T q = r * iHvi, u = T(1) - q, u3 = u * u * u;
+          wh += u3 * (T(D) * u * (T(1) + T(4) * q) - T(20) * q * q);
+          c = fi * u3;
+        }
+        if (in_j) {
+          const T iHvj = drcp<T>(Hvj), u = T(1) - r * iHvj, iHj = iHvj * F.inv_qv;
+          c += T(-20) * P.alpha * B.rhob[j] * ipow_d<D, T>(iHj) * iHj * iHj * (u * u * u);
+        }
+        xx += c * dx;
+        xy += c * dy;
+        xz += c * dz;
       });
+      hbar -= ci * iHi * wh * P.kappa;
+      xx *= qv;
+      xy *= qv;
+      xz *= qv;
     }
     T xg[3], dc[8];
     field_adjoint<D, T>(F, geo, (buf ? X1 : X0)[i], hi, B.rtb[i], hbar, B.Tb[i], xg, dc);
@@ -684,18 +701,24 @@ __global__ void __launch_bounds__(256) k_obj(int n, const StepCtl* __restrict__ 
     const VT vi = view[i];
     const uint32_t ci = (buf ? m1 : m0)[i] & 0xFFu;
     const T qv = F.qv, hv = view_h(F, vi), hi = hv * qv;
-    const T Hi = P.kappa * hi, half_kappa = T(0.5) * P.kappa;
+    const T Hvi = P.kappa * hv, Hvi2 = Hvi * Hvi, iHvi = T(1) / Hvi, half_kappa = T(0.5) * P.kappa;
     T rho = 0, xx = 0, xy = 0, xz = 0, hbar = 0, wi = 0;
     for_skin_list(list, view, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
       const int j = (int)(e >> 8);
       const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
       const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
       const T r2 = dx * dx + dy * dy + dz * dz;
-      const T r = dsqrt(r2) * qv;
-      rho += wendland<D, T>(r, Hi, P.alpha).W;
       const T hvj = view_h(F, vj);
       const T Hv = half_kappa * (hv + hvj);
-      if (j == i || (e & 0xFFu) == ci || !(r2 < Hv * Hv)) return;
+      const bool face = r2 < Hv * Hv && j != i && (e & 0xFFu) != ci;
+      if (!(r2 < Hvi2 || face)) return;
+      const T rv = r2 > T(0) ? pair_r<T>(r2) : T(0);
+      if (r2 < Hvi2) {
+        const T q = rv * iHvi, u = T(1) - q, u2 = u * u;
+        rho += u2 * u2 * (T(1) + T(4) * q);
+      }
+      if (!face) return;
+      const T r = rv * qv;
       const KernelD<D, T> k = wendland<D, T>(r, Hv * qv, P.alpha);
       wi += T(0.5) * k.W;  // each unordered pair from both ends
       const T c = lambda * k.Wr / r;
@@ -704,6 +727,7 @@ __global__ void __launch_bounds__(256) k_obj(int n, const StepCtl* __restrict__ 
       xz += c * dz * qv;
       hbar += lambda * k.WH * half_kappa;
     });
+    rho *= P.alpha * ipow_d<D, T>(iHvi * F.inv_qv);
     const T rt = rho_t_of_h<D, T>(hi, P.inv_tau);
     const T e = rho / rt - T(1);
     v[0] = e * e;
