@@ -141,10 +141,13 @@ sph_status status_from_flags(sph_handle* h, int flags) {
 // polynomial-field workload: 20 steps in 2.77 ms against 2.82 at 0.15).
 inline double default_skin(int dim) { return dim == 3 ? 0.15 : 0.2; }
 
+// a skin or a list capacity of the caller's choosing keeps one skin for all
+inline bool adaptive_skin(const sph_handle* h) { return !(h->par.skin > 0) && h->par.list_capacity == 0; }
+
 // position frames and kernel grids (make_frames in sph_host.h)
 void setup_frames(sph_handle* h) {
   Frames fr;
-  make_frames(h->dom, h->par.kappa, h->par.skin > 0 ? h->par.skin : default_skin(h->dim), h->hg, fr);
+  make_frames(h->dom, h->par.kappa, h->par.skin > 0 ? h->par.skin : default_skin(h->dim), adaptive_skin(h), h->hg, fr);
   h->Ff = fr.f;
   h->Fd = fr.d;
   h->Gf = fr.gf;
@@ -160,7 +163,8 @@ void setup_frames(sph_handle* h) {
 // twice that and that plus ten standard deviations of a Poisson count (random
 // initial states cluster), plus 16.
 int auto_capacity(const sph_handle* h) {
-  const double skin = h->par.skin > 0 ? h->par.skin : default_skin(h->dim);
+  double skin = h->par.skin > 0 ? h->par.skin : default_skin(h->dim);
+  if (adaptive_skin(h)) skin = std::max(skin, 2.0 * kSkinMost);
   const double k1 = h->par.kappa * (1.0 + skin);
   const double L = std::min(h->lip_h, 0.5 / k1);
   const double g = k1 / (1.0 - L * k1);

@@ -83,7 +83,10 @@ struct Frame {
   T qv, inv_qv;          // physical length of one view unit (the finest cell edge c0)
   T q64t, inv_q64t;
   T lo[3];
-  T skin;                // list skin as a fraction of kappa h
+  // how far a particle may move from the list build, as a fraction of kappa h:
+  // skin_u while its speed is unknown, else its last step's move times skin_k
+  // plus skin_lo, at most skin_hi; held in 255ths of skin_hi (skin_q)
+  float skin_u, skin_k, skin_lo, skin_hi, skin_q;
 };
 
 // The view unit is the level-0 cell edge c0. FP32 view integers are 2^-24 c0;
@@ -139,7 +142,7 @@ struct StepCtl {
   long long step;
   double t0, t1, sigma0;
   int buf, vp, rebuild, need_rebuild;
-  int lmax, pad_;  // longest neighbour list of the last build
+  int lmax, dmax;  // of the last build: longest neighbour list, largest reach code (Frame::skin_q)
   long long rebuilds;
   // automatic start of the ramp (Sec. 3.3 convergence test): on, run length in
   // steps, relative tolerance, ramp fraction; state: current run, its opening

@@ -148,7 +148,7 @@ extern "C" sph_status sph_eval_forces_noalloc(const sph_domain* dom, const sph_f
     return SPH_ERR_INVALID_ARG;
   }
   Frames fr;
-  make_frames(*dom, params->kappa, 0.0, hg, fr);  // one evaluation: no skin
+  make_frames(*dom, params->kappa, 0.0, false, hg, fr);  // one evaluation: no skin
   Geom<float> geof;
   fill_geom<float>(*dom, *field, hfac, field->rho_scale, geof);
   Phys<float> Pf;

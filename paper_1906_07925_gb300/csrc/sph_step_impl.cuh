@@ -89,6 +89,14 @@ __device__ __forceinline__ double view_w(const V4<double>& v) { return v.w; }
 __device__ __forceinline__ float view_h(const Frame<float>& F, const int4& v) { return __int_as_float(v.w) * F.w2c; }
 __device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>& v) { return v.w; }
 
+// The build view of a particle (vbuild; FP64 path: view32 until pass B renews it):
+// its position, and in w its view_w rounded up to 16 bits of mantissa with its
+// reach code in the low byte. The reach, in view integers:
+__device__ __forceinline__ float build_w(int4 v) { return __int_as_float(v.w & ~0xFF); }
+__device__ __forceinline__ float build_reach(const Frame<float>& F, int4 v) {
+  return (float)(v.w & 0xFF) * (2.0f * F.skin_q) * build_w(v);
+}
+
 // The neighbour list of particle i has list_rows(cap) rows (list_at), split at
 // its build: the entries then inside their support (r < max(kappa h_i,
 // kappa h_ij)) fill rows 0, 1, ... in candidate order, the others the last row,
@@ -129,8 +137,6 @@ template <int D>
 __device__ __forceinline__ V4<double> make_view(const Frame<double>& F, const LL4& X, double h) {
   return V4<double>{(double)X.x * F.s2v, (double)X.y * F.s2v, D == 3 ? (double)X.z * F.s2v : 0.0, h * F.inv_qv};
 }
-__device__ __forceinline__ int4 with_w(int4 v, float w) { return make_int4(v.x, v.y, v.z, __float_as_int(w)); }
-__device__ __forceinline__ V4<double> with_w(V4<double> v, double w) { return V4<double>{v.x, v.y, v.z, w}; }
 
 #ifndef SPH_LIST_BATCH_X
 #define SPH_LIST_BATCH_X 2  // 4 spilled at the 48 / 64-register budgets of the passes using it
@@ -242,27 +248,25 @@ __device__ __forceinline__ int list_row(int k, int n_in, int cap) {
   return k < n_in ? k : list_rows(cap) - 1 - (k - n_in);
 }
 // pair(e, view of e) for every entry of the skin list of particle i, what is
-// left of the inside part before the outside part. A body of FP64 arithmetic
-// costs as much for one lane as for 32, so the lanes' inside entries have to
-// stay in step (quads with their remainders last: 3 % slower).
+// left of the inside part before the outside part, four entries in flight. A
+// body of FP64 arithmetic costs as much for one lane as for 32, so the lanes'
+// entries have to stay in step: no loop of its own for what is left (a lane with
+// 15 entries then met a lane with 16 in different loops), and not the quads'
+// order with their remainders last (3 % slower).
 template <class VT, class Fn>
 __device__ __forceinline__ void for_skin_list(const uint32_t* __restrict__ list, const VT* __restrict__ view, int i,
                                               uint32_t lc, int cap, Fn&& pair) {
   const int cnt = list_cnt(lc), n_in = list_in(lc);
-  int k = 0;
-  for (; k + 4 <= cnt; k += 4) {
+  for (int k = 0; k < cnt; k += 4) {
     uint32_t e[4];
     VT v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) e[q] = list[list_at(i, list_row(k + q, n_in, cap), cap)];
+    for (int q = 0; q < 4; ++q) e[q] = list[list_at(i, list_row(min(k + q, cnt - 1), n_in, cap), cap)];
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = view[e[q] >> 8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) pair(e[q], v[q]);
-  }
-  for (; k < cnt; ++k) {
-    const uint32_t e = list[list_at(i, list_row(k, n_in, cap), cap)];
-    pair(e, view[e >> 8]);
+    for (int q = 0; q < 4; ++q)
+      if (k + q < cnt) pair(e[q], v[q]);
   }
 }
 
@@ -277,28 +281,23 @@ __device__ __forceinline__ void for_skin_list_s32(const uint32_t* __restrict__ l
                                                   const VT* __restrict__ view, int i, uint32_t lc, int cap,
                                                   Screen&& screen, Fn&& pair) {
   const int cnt = list_cnt(lc), n_in = list_in(lc);
-  int k = 0;
-  for (; k + 4 <= cnt; k += 4) {
+  for (int k = 0; k < cnt; k += 4) {
     uint32_t e[4];
     int4 w[4];
     bool ok[4];
     VT v[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) e[q] = list[list_at(i, list_row(k + q, n_in, cap), cap)];
+    for (int q = 0; q < 4; ++q) e[q] = list[list_at(i, list_row(min(k + q, cnt - 1), n_in, cap), cap)];
 #pragma unroll
     for (int q = 0; q < 4; ++q) w[q] = v32[e[q] >> 8];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      ok[q] = screen(w[q]);
+      ok[q] = screen(w[q]) && k + q < cnt;
       if (ok[q]) v[q] = view[e[q] >> 8];
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (ok[q]) pair(e[q], v[q]);
-  }
-  for (; k < cnt; ++k) {
-    const uint32_t e = list[list_at(i, list_row(k, n_in, cap), cap)];
-    if (screen(v32[e >> 8])) pair(e, view[e >> 8]);
   }
 }
 
@@ -774,6 +773,7 @@ __global__ void __launch_bounds__(256) k_rekey(int n, StepCtl* ctl, int force, u
       ctl->need_rebuild = 0;
       ctl->rebuilds += 1;
       ctl->lmax = 0;
+      ctl->dmax = 0;
     }
   }
 }
@@ -781,14 +781,15 @@ __global__ void __launch_bounds__(256) k_rekey(int n, StepCtl* ctl, int force, u
 // Slot s of the scatter holds old index i; its rank among the cell's members by
 // particle id gives its destination (cells ordered by key, each cell by
 // particle id): the state is copied there, with the view of the new order, the
-// reference view of the skin test (w = half the skin), and in the FP64 path the
+// build view with the particle's reach until the next rebuild (X.w carries its
+// last move, see k_pass_b; zero: none yet), and in the FP64 path the
 // FP32 view its list build and pass A's screen read. (The list only has to hold
 // every pair the exact FP64 tests can accept before the next rebuild, and an
 // FP32 candidate test errs by ~1e-7 of the distance, far inside the list's
 // margins, while FP64 arithmetic runs at a small fraction of the FP32 rate.)
 template <int D, class T>
 __global__ void __launch_bounds__(256) k_gather_view(
-    int n, const StepCtl* __restrict__ ctl, const uint32_t* __restrict__ slots, const uint32_t* __restrict__ key,
+    int n, StepCtl* __restrict__ ctl, const uint32_t* __restrict__ slots, const uint32_t* __restrict__ key,
     const uint32_t* __restrict__ cstart, LL4* __restrict__ X0, LL4* __restrict__ X1, uint32_t* __restrict__ m0,
     uint32_t* __restrict__ m1, uint32_t* __restrict__ p0, uint32_t* __restrict__ p1, Frame<T> F, Geom<T> geo,
     typename ViewOf<T>::type* __restrict__ v0, typename ViewOf<T>::type* __restrict__ v1,
@@ -796,6 +797,7 @@ __global__ void __launch_bounds__(256) k_gather_view(
   if (!ctl->rebuild) return;
   const int nb = ctl->buf, vp = ctl->vp;  // new buffers; the old order lives in the other state buffer
   const uint32_t* __restrict__ pold = nb ? p0 : p1;
+  int most = 0;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
     const uint32_t i = slots[s];
     const uint32_t k = key[i];
@@ -812,45 +814,58 @@ __global__ void __launch_bounds__(256) k_gather_view(
     abs_pos<D, T>(F, X, x);
     const auto v = make_view<D>(F, X, h_of<D, T>(geo, x));
     (vp ? v1 : v0)[d] = v;
-    vbuild[d] = with_w(v, T(0.5) * F.skin * view_h(F, v));  // kappa folded in by the host
+    const float moved = __uint_as_float((uint32_t)X.w);
+    const float reach = moved > 0.0f ? fminf(fmaf(F.skin_k, moved, F.skin_lo), F.skin_hi) : F.skin_u;
+    const int code = min((int)ceilf(reach / F.skin_q), 255);
+    most = max(most, code);
     if constexpr (std::is_same<T, double>::value) {
       const long long half = 1LL << (F32.sv - 1);
-      v32[d] = make_int4((int)((X.x + half) >> F32.sv), (int)((X.y + half) >> F32.sv),
-                         D == 3 ? (int)((X.z + half) >> F32.sv) : 0, __float_as_int((float)view_w(v) * F32.c2w));
+      const int w = ((__float_as_int((float)view_w(v) * F32.c2w) + 0xFF) & ~0xFF) | code;
+      const int4 u = make_int4((int)((X.x + half) >> F32.sv), (int)((X.y + half) >> F32.sv),
+                               D == 3 ? (int)((X.z + half) >> F32.sv) : 0, w);
+      v32[d] = u;
+      vbuild[d] = V4<double>{v.x, v.y, v.z, (double)(build_reach(F32, u) * F32.vscale)};
+    } else {
+      vbuild[d] = make_int4(v.x, v.y, v.z, ((v.w + 0xFF) & ~0xFF) | code);
     }
   }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0) atomicMax(&ctl->dmax, most);
 }
 
 // Neighbour list of each particle: every j (itself included) with
-//   r < kappa max(h_i, h_j) (1 + 1e-5) + kappa lip_h s_max / 2 + s_max,
-// s = skin (kappa folded) of i and j: after both moved at most half their skin
-// (and h changed by at most lip_h times that), any pair inside the exact
+//   r < kappa max(h_i, h_j) (1 + 1e-5) + (d_i + d_j) (1 + kappa lip_h),
+// d the reaches of i and j: after both moved at most their reach (and h changed
+// by at most lip_h times that), any pair inside the exact
 // criteria is still listed. Candidates come from rows of cells of every level
 // that can hold such a j, in the order (level, z row, y row, x).
 // The list is built on FP32 views in both precisions. Lengths of the tests are
-// view integers; with w = kappa h / 2 (view_w) and m = max(w_i, w_j) the list
-// radius above is m times a constant and the larger of the supports kappa h_i
-// and kappa h_ij is w_i + m.
+// view integers; with w = kappa h / 2 (build_w) and m = max(w_i, w_j), 2 m is the
+// largest support of the pair and the larger of kappa h_i and kappa h_ij is w_i + m.
 struct ListTarget {
   float Rs, R2;          // search radius, view units
-  float wi, c, r2max;    // view integers
+  float wi, di, c1, c2, u2, r2max;  // view integers
   int l0, l1;            // levels that can hold a neighbour
-  __device__ __forceinline__ ListTarget(const Frame<float>& F, const Grid<float>& G, float kappa, const int4& vi) {
-    const float hv = view_h(F, vi), sk = F.skin * hv, lip = G.lip_h, cl = 1.0f + 0.5f * kappa * lip;
-    // search radius: bound h_j by Lipschitz continuity, iterate twice
+  __device__ __forceinline__ ListTarget(const Frame<float>& F, const Grid<float>& G, float kappa, int dmax,
+                                        const int4& vi) {
+    wi = build_w(vi);
+    di = build_reach(F, vi);
+    const float hv = wi * F.w2c, lip = G.lip_h, dv = di * F.vscale, dm = (float)dmax * F.skin_q * kappa;
+    // search radius: bound h_j by Lipschitz continuity and d_j by the largest
+    // reach of this build, iterate twice
     float hhi = hv;
-    Rs = kappa * hv * G.rfac + sk * cl;
+    c2 = 1.0f + kappa * lip;
+    Rs = kappa * hv * G.rfac + (dv + dm * hv) * c2;
     for (int it = 0; it < 2; ++it) {
-      hhi = hv * 1.00001f + lip * Rs;
-      const float shi = sk * hhi / hv;
-      Rs = kappa * hhi * G.rfac + shi * cl;
+      hhi = hv * 1.0001f + lip * Rs;
+      Rs = kappa * hhi * G.rfac + (dv + dm * hhi) * c2;
       Rs = fmaxf(Rs, kappa * hv * G.rfac);
     }
-    l0 = level_of_h(G, (hv * 0.99999f - lip * Rs) * F.qv);
+    l0 = level_of_h(G, (hv * 0.9999f - lip * Rs) * F.qv);
     l1 = level_of_h(G, hhi * F.qv);
     R2 = Rs * Rs;
-    wi = view_w(vi);
-    c = 2.0f * (1.00001f + F.skin / kappa * cl);  // skin: kappa folded in
+    c1 = 2.0f * 1.00001f;
+    u2 = 2.0f * F.skin_q;
     r2max = R2 / (F.vscale * F.vscale);
   }
   // a pair of candidates, without a branch: listed (acc), inside its support
@@ -866,8 +881,9 @@ struct ListTarget {
       r2 = fma2(dz, dz, r2);
     }
     // symmetric in i and j: j lists i whenever i lists j
-    const float2 m = make_float2(fmaxf(wi, view_w(a)), fmaxf(wi, view_w(b)));
-    const float2 rl = mul2(both(c), m), rl2 = mul2(rl, rl), hp = add2(both(wi), m), hp2 = mul2(hp, hp);
+    const float2 wj = make_float2(build_w(a), build_w(b)), m = make_float2(fmaxf(wi, wj.x), fmaxf(wi, wj.y));
+    const float2 dj = mul2(mul2(make_float2((float)(a.w & 0xFF), (float)(b.w & 0xFF)), both(u2)), wj);
+    const float2 rl = fma2(add2(both(di), dj), both(c2), mul2(both(c1), m)), rl2 = mul2(rl, rl), hp = add2(both(wi), m), hp2 = mul2(hp, hp);
     acc[0] = r2.x < fminf(rl2.x, r2max);
     acc[1] = r2.y < fminf(rl2.y, r2max);
     inside[0] = r2.x < hp2.x;
@@ -875,9 +891,9 @@ struct ListTarget {
   }
   // largest axis separation (view units) a listed pair can reach before the next rebuild
   template <int D>
-  __device__ __forceinline__ float reach(const Frame<float>& F, float kappa, const int4& vi, const int4& vj) const {
+  __device__ __forceinline__ float reach(const Frame<float>& F, const int4& vi, const int4& vj) const {
     const int d = max(max(abs(vi.x - vj.x), abs(vi.y - vj.y)), D == 3 ? abs(vi.z - vj.z) : 0);
-    return (float)d * F.vscale + F.skin / kappa * 2.0f * fmaxf(wi, view_w(vj)) * F.vscale;
+    return ((float)d + di + build_reach(F, vj)) * F.vscale;
   }
   // the coarse FP32 conversion is exact below 2^22 coarse integers = 2^(22 - kCoarseBits) c0
   static __device__ __forceinline__ bool fast(float reach) { return reach < 0.999f * (1 << (22 - kCoarseBits)); }
@@ -938,19 +954,18 @@ struct RowWalk {
 template <int D, bool REACH>
 __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(
     int n, StepCtl* __restrict__ ctl, const LL4* __restrict__ X0, const LL4* __restrict__ X1,
-    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1, const int4* __restrict__ v0,
-    const int4* __restrict__ v1, const uint32_t* __restrict__ cstart, Frame<float> F, Grid<float> G, float kappa, int cap,
+    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1, const int4* __restrict__ view,
+    const uint32_t* __restrict__ cstart, Frame<float> F, Grid<float> G, float kappa, int cap,
     uint32_t* __restrict__ list, uint32_t* __restrict__ lcount, int* __restrict__ err) {
   if (!ctl->rebuild) return;
   const int buf = ctl->buf;
-  const int4* __restrict__ view = ctl->vp ? v1 : v0;
   const uint32_t* __restrict__ meta = buf ? m1 : m0;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   int cnt = 0;  // accepted
   if (i < n) {
     const LL4 X = (buf ? X1 : X0)[i];
     const int4 vi = view[i];
-    const ListTarget t(F, G, kappa, vi);
+    const ListTarget t(F, G, kappa, ctl->dmax, vi);
     int n_in = 0, n_out = 0;  // written inside / outside entries
     const int rows = list_rows(cap);
     uint32_t* __restrict__ own = list + list_at(i, 0, cap);
@@ -968,7 +983,7 @@ __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(
         own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)j << 8) | (meta[j] & 0xFFu);
       }
       ++cnt;
-      if (REACH) reach = fmaxf(reach, t.reach<D>(F, kappa, vi, vj));
+      if (REACH) reach = fmaxf(reach, t.reach<D>(F, vi, vj));
     };
     for (int l = t.l0; l <= t.l1; ++l) {
       const RowWalk<D> w(F, G, X, t.Rs, l);
@@ -1006,7 +1021,7 @@ __global__ void __launch_bounds__(256) k_list_build_group(int n, StepCtl* __rest
                                                           const LL4* __restrict__ X0, const LL4* __restrict__ X1,
                                                           const uint32_t* __restrict__ m0,
                                                           const uint32_t* __restrict__ m1,
-                                                          const int4* __restrict__ v0, const int4* __restrict__ v1,
+                                                          const int4* __restrict__ view,
                                                           const uint32_t* __restrict__ cstart, Frame<float> F,
                                                           Grid<float> G32, float kappa, int cap,
                                                           uint32_t* __restrict__ list, uint32_t* __restrict__ lcount,
@@ -1019,11 +1034,10 @@ __global__ void __launch_bounds__(256) k_list_build_group(int n, StepCtl* __rest
   if (i < n) {  // whole groups
     const unsigned group = group_mask<G>(), below = group & lanes_below();
     const int buf = ctl->buf;
-    const int4* __restrict__ view = ctl->vp ? v1 : v0;
     const uint32_t* __restrict__ meta = buf ? m1 : m0;
     const LL4 X = (buf ? X1 : X0)[i];
     const int4 vi = view[i];
-    const ListTarget t(F, G32, kappa, vi);
+    const ListTarget t(F, G32, kappa, ctl->dmax, vi);
     const int rows = list_rows(cap);
     uint32_t* __restrict__ own = list + list_at(i, 0, cap);
     int n_in = 0, n_out = 0, cnt = 0;  // written inside / outside entries, accepted: uniform over the group
@@ -1041,8 +1055,8 @@ __global__ void __launch_bounds__(256) k_list_build_group(int n, StepCtl* __rest
             const int4 a = view[j], b = view[two ? j + 1 : j];
             t.test<D>(vi, a, b, acc, inside);
             acc[1] = acc[1] && two;
-            if (REACH && acc[0]) reach = fmaxf(reach, t.reach<D>(F, kappa, vi, a));
-            if (REACH && acc[1]) reach = fmaxf(reach, t.reach<D>(F, kappa, vi, b));
+            if (REACH && acc[0]) reach = fmaxf(reach, t.reach<D>(F, vi, a));
+            if (REACH && acc[1]) reach = fmaxf(reach, t.reach<D>(F, vi, b));
           }
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
@@ -1812,15 +1826,13 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         }
         __syncwarp();
       }
-      for (; k + 2 <= cnt; k += 2, p += 64) {
-        const PairRec<T> r0 = load_pair(p), r1 = load_pair(p + 32);
+      for (; k < cnt; k += 2, p += 64) {  // a zero factor where there is no second pair
+        const PairRec<T> r0 = load_pair(p);
+        PairRec<T> r1{T(0), r0.e, 0u};
+        if (k + 1 < cnt) r1 = load_pair(p + 32);
         const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
         pair(r0, a0);
-        pair(r1, a1);
-      }
-      if (k < cnt) {
-        const PairRec<T> r0 = load_pair(p);
-        pair(r0, acc[r0.e >> 8]);
+        if (k + 1 < cnt) pair(r1, a1);
       }
     }
     if constexpr (G > 1) {  // the block's 32 particles to warp 0
@@ -1906,6 +1918,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         }
         abs_pos<D, T>(F, X, xa);
       }
+      // the move in units of kappa h, for the next list's reach (never zero: that
+      // would mean none yet)
+      const float mx = (float)d[0], my = (float)d[1], mz = (float)d[2];
+      X.w = (long long)__float_as_uint(
+          fmaxf(sqrtf(mx * mx + my * my + mz * mz) / (float)(P.kappa * hv * F.qv), 1e-30f));
       Xs[i] = X;
       // smoothing length at the new position (the target field of the next step)
       const T hn = h_of<D, T>(geo, xa);
@@ -1920,7 +1937,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       const VT vb = vbuild[i];
       const T ex = vd(F, vn.x, vb.x), ey = vd(F, vn.y, vb.y);
       const T ez = D == 3 ? vd(F, vn.z, vb.z) : T(0);
-      const T lim = view_w(vb);
+      T lim;  // the reach, view units
+      if constexpr (std::is_same<T, float>::value) lim = build_reach(F, vb) * F.vscale;
+      else lim = vb.w;
       far = (ex * ex + ey * ey + ez * ez) >= lim * lim;
     } else {
       (vp ? w0 : w1)[i] = vi;
@@ -2051,16 +2070,14 @@ cudaError_t launch_rebuild(const DevState& S, int force, const Grid<T>& G, const
   constexpr bool f64 = std::is_same<T, double>::value;
   const Frame<float>* Fl = F32;
   const Grid<float>* Gl = G32;
-  const int4 *w0 = (const int4*)S.view32, *w1 = w0;
+  const int4* view = (const int4*)(f64 ? S.view32 : S.vbuild);
   if constexpr (!f64) {
     Fl = &F;
     Gl = &G;
-    w0 = (const int4*)S.view[0];
-    w1 = (const int4*)S.view[1];
   }
   const bool group = S.n <= kListGroupMax;
   auto build = [&](auto* kernel, int blocks) {
-    kernel<<<blocks, tb, 0, st>>>(S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], w0, w1, S.cstart, *Fl, *Gl, (float)kappa,
+    kernel<<<blocks, tb, 0, st>>>(S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], view, S.cstart, *Fl, *Gl, (float)kappa,
                                   S.cap, S.list, S.lcount, S.err);
   };
   if (group) build(k_list_build_group<D, kListLanes, f64>, grid_for(S.n * kListLanes, tb));
