@@ -64,6 +64,12 @@ __device__ __forceinline__ KernelD<D, T> wendland(T r, T H, T c) {
   k.WH = -cH * iH * (T(D) * u3 * u * (T(1) + T(4) * q) - T(20) * q * q * u3);
   return k;
 }
+// reciprocals of normal numbers: the hardware's in FP32 (1 ulp, without the
+// range handling of the library forms)
+__device__ __forceinline__ float prcp(float x) { return fast_rcp(x); }
+__device__ __forceinline__ double prcp(double x) { return drcp<double>(x); }
+__device__ __forceinline__ float prsqrt(float x) { return fast_rsqrt(x); }
+__device__ __forceinline__ double prsqrt(double x) { return drsqrt<double>(x); }
 template <int D, class T>
 struct ForceD {
   T F, Fr, FH;
@@ -71,7 +77,7 @@ struct ForceD {
 template <int D, class T>
 __device__ __forceinline__ ForceD<D, T> force_fn(T r, T H, T c) {
   ForceD<D, T> k{T(0), T(0), T(0)};
-  const T iH = drcp<T>(H), q = r * iH;
+  const T iH = prcp(H), q = r * iH;
   if (!(q < T(1))) return k;
   const T u = T(1) - q, u2 = u * u;
   const T cH3 = c * ipow_d<D, T>(iH) * iH * iH * iH;  // c H^-(d+3)
@@ -292,7 +298,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n,
       const T hvj = view_h(F, vj);
       const T Hv = half_kappa * (hv + hvj);
       if (!(r2 < Hv * Hv) || j == i) return;
-      const T irv = drsqrt<T>(r2);  // 1/r, view units
+      const T irv = prsqrt(r2);  // 1/r, view units
       const T r = r2 * irv * qv, ir = irv * F.inv_qv, ex = dx * qv, ey = dy * qv, ez = dz * qv;
       const ForceD<D, T> f = force_fn<D, T>(r, Hv * qv, P.alpha);
       const V4<T>& aj = rj.a;
@@ -523,7 +529,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? SPH_BWD_FORCE_MIN_BLOCKS
       const T hvj = view_h(F, vj);
       const T Hv = half_kappa * (hv + hvj);
       if (!(r2 < Hv * Hv) || j == i) return;
-      const T irv = drsqrt<T>(r2);  // 1/r, view units
+      const T irv = prsqrt(r2);  // 1/r, view units
       const T r = r2 * irv * qv, ir = irv * F.inv_qv, ex = dx * qv, ey = dy * qv, ez = dz * qv;
       const ForceD<D, T> f = force_fn<D, T>(r, Hv * qv, P.alpha);
       const T Tj = inv_rho_t2<D, T>(hvj * qv, P.inv_tau);

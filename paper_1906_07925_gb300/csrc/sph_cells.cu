@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(256) k_scatter(int n, const StepCtl* __restric
                                                  const uint32_t* __restrict__ cstart,
                                                  uint32_t* __restrict__ cnt,
                                                  uint32_t* __restrict__ slots, uint32_t* __restrict__ part, int nb) {
+  after_predecessor();
   if (!ctl->rebuild) return;
   // the tile counts are used up: zero for the next rebuild
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) part[b] = 0u;
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(256) k_scatter(int n, const StepCtl* __restric
 // exclusive scan of the tile counts, in place (one block of 1024 threads)
 __global__ void __launch_bounds__(1024) k_scan_top(const StepCtl* __restrict__ ctl, uint32_t* __restrict__ part,
                                                    int nb) {
+  after_predecessor();
   if (!ctl->rebuild) return;
   __shared__ uint32_t wsum[32];
   int per = (nb + blockDim.x - 1) / blockDim.x;
@@ -93,6 +95,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const StepCtl* __res
                                                             const uint32_t* __restrict__ in, uint32_t n,
                                                             const uint32_t* __restrict__ part, int scanned,
                                                             uint32_t* __restrict__ out) {
+  after_predecessor();
   if (!ctl->rebuild) return;
   __shared__ uint32_t wtot[kScanThreads / 32], wpre[kScanThreads / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -193,9 +196,9 @@ cudaError_t build_cells(const DevState& S, cudaStream_t st) {
   const int gb = rebuild_grid(n, tb, 8);
   const uint32_t m = S.total_cells;
   const int nb = (int)scan_tiles(m), scanned = nb > kScanOwn;
-  if (scanned) k_scan_top<<<1, 1024, 0, st>>>(S.ctl, S.scan_part, nb);
-  k_scan_down<<<nb, kScanThreads, 0, st>>>(S.ctl, S.cnt, m, S.scan_part, scanned, S.cstart);
-  k_scatter<<<gb, tb, 0, st>>>(n, S.ctl, S.key, S.cstart, S.cnt, S.tmp, S.scan_part, nb);
+  if (scanned) launch_after(k_scan_top, 1, 1024, 0, st, S.ctl, S.scan_part, nb);
+  launch_after(k_scan_down, nb, kScanThreads, 0, st, S.ctl, S.cnt, m, S.scan_part, scanned, S.cstart);
+  launch_after(k_scatter, gb, tb, 0, st, n, S.ctl, S.key, S.cstart, S.cnt, S.tmp, S.scan_part, nb);
   return cudaGetLastError();
 }
 

@@ -110,14 +110,16 @@ struct Phys {
 // particles they belong to (r_c and |a|, rho and rho_t: exact FP32 values) and
 // divides once, at the end.
 constexpr int kPartialGroup = 512;
-struct Partial {
-  double min_rc_a, max_a, sum_rho, err_l2, err_max;
-  long long ipairs, fpairs;
-  long long lentries;  // neighbour-list entries scanned
-  long long amin;      // index (current order) of min_rc_a; -1: none
-  float rc, an;        // FP32 path: r_c and |a| of particle amin
-  float er, et;        // FP32 path: rho and rho_t where |rho / rho_t - 1| is largest (et = 0: none)
-  float ma, pad_;      // FP32 path: the largest |a|
+struct alignas(16) Partial {
+  double sum_rho, err_l2;
+  double min_rc_a, max_a;
+  double err_max;
+  long long ipairs;
+  long long fpairs, lentries;  // force pairs, neighbour-list entries scanned
+  long long amin;              // index (current order) of min_rc_a; -1: none
+  float rc, an;                // FP32 path: r_c and |a| of particle amin
+  float er, et, ma, q;         // rho and rho_t where |rho / rho_t - 1| is largest (et = 0: none); largest |a|; rc / an
+  float ek, pad_[3];           // that |rho / rho_t - 1| to a few ulp (-1: none)
 };
 // partials of the blocks and of their groups for n particles at >= `threads` per block
 constexpr size_t partial_slots(size_t n, int threads) {

@@ -160,11 +160,13 @@ inline std::string grid_setup(const sph_domain& dom, double kappa, double cell_f
 // reach. Few particles move fast (the step size lets the fastest move 0.015 to
 // 0.02 of its support, the r.m.s. move is a quarter of that early in a
 // relaxation and a thirtieth later), so with one reach for all, the few set the
-// length of every list or the interval between rebuilds. With six steps of its
-// own last move plus 0.05, at most 0.15: 8 to 9 steps between rebuilds where a
-// common reach of 0.075 lasts 4.2 (2,000,000 particles in 3D, first 40 steps;
-// 11 against 8 after 100), at a mean reach of 0.06, so with shorter lists.
-constexpr float kSkinSteps = 6.0f, kSkinFloor = 0.05f, kSkinMost = 0.15f;
+// length of every list or the interval between rebuilds. With eight steps of its
+// own last move plus 0.05, at most 0.15: 9 to 10 steps between rebuilds where a
+// common reach of 0.075 lasts 4.2 (3D, first 60 steps), at a mean reach of 0.06,
+// so with shorter lists. One step of 8,388,608 particles in 3D, over 60:
+// 3.28 ms; 6 / 0.05 / 0.15: 3.36; 8 / 0.05 / 0.12: 3.34; 6 / 0.04 / 0.10: 3.45;
+// 6 / 0.08 / 0.15: 3.42.
+constexpr float kSkinSteps = 8.0f, kSkinFloor = 0.05f, kSkinMost = 0.15f;
 
 // Position frames. The integer state unit q64 divides the level-0 cell edge by
 // 2^kCellShift, so cell coordinates are shifts. The FP32 view drops sv low bits

@@ -103,6 +103,44 @@ inline int device_sms() {
   }();
   return sms;
 }
+// Launch of a rebuild kernel, which follows another of the same rebuild: it may
+// be set up while its predecessor still runs (programmatic dependent launch) and
+// waits for it on the device, by after_predecessor(), before it touches memory.
+// On most steps these kernels exit at once and are mostly launch latency, which
+// this hides (circle of 4,289 particles 36 -> 33 us per step). Not for kernels
+// with work on every step: blocks that start early crowd onto the SMs that the
+// predecessor leaves first (the reverse pass of 20,011 FP64 particles in 3D took
+// 13.6 ms so, 11.5 without).
+template <class... K, class... A>
+inline cudaError_t launch_after(void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, (K)args...);
+}
+// the successor may be set up from here on
+__device__ __forceinline__ void let_successor() {
+#if defined(__CUDA_ARCH__)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+// First statement of a kernel launched by launch_after: the predecessor is
+// complete and its writes are visible; then the successor may be set up.
+// (Waiting first keeps the chain: a kernel that exits at once has still waited.)
+__device__ __forceinline__ void after_predecessor() {
+#if defined(__CUDA_ARCH__)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
+  let_successor();
+}
+
 // Grid of a predicated list-rebuild kernel: grid-stride over n with at most
 // per_sm blocks per SM. Most steps do not rebuild, and such a kernel then
 // exits at once: with one block per 256 particles an 8M-particle grid took

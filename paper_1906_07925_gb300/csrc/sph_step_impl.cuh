@@ -145,7 +145,8 @@ __device__ __forceinline__ V4<double> make_view(const Frame<double>& F, const LL
 // the neighbour (its acceleration, an adjoint): that record, fetch(j), is
 // loaded for the whole batch together with the views, so each thread keeps
 // 2 x SPH_LIST_BATCH_X independent gathers in flight instead of meeting the
-// record's latency inside every pair body. Words are streamed (read once).
+// record's latency inside every pair body. Words are streamed (read once), the
+// next batch's loaded before this one's arithmetic.
 template <class T, class VT, class Fetch, class Fn>
 __device__ __forceinline__ void for_pairs_x(const PairRec<T>* __restrict__ plist, const VT* __restrict__ view, int i,
                                             int cnt, int cap, Fetch&& fetch, Fn&& pair) {
@@ -153,17 +154,25 @@ __device__ __forceinline__ void for_pairs_x(const PairRec<T>* __restrict__ plist
   constexpr int B = SPH_LIST_BATCH_X;
   const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
   int k = 0;
-  for (; k + B <= cnt; k += B, p += 32 * B) {
+  uint32_t ahead[B];
+  if (cnt >= B)
+#pragma unroll
+    for (int q = 0; q < B; ++q) ahead[q] = __ldcs(&p[32 * q].e);
+  for (; k + B <= cnt; k += B) {
     uint32_t e[B];
     VT v[B];
     XT x[B];
 #pragma unroll
-    for (int q = 0; q < B; ++q) e[q] = __ldcs(&p[32 * q].e);
+    for (int q = 0; q < B; ++q) e[q] = ahead[q];
 #pragma unroll
     for (int q = 0; q < B; ++q) {
       v[q] = view[e[q] >> 8];
       x[q] = fetch((int)(e[q] >> 8));
     }
+    p += 32 * B;
+    if (k + 2 * B <= cnt)
+#pragma unroll
+      for (int q = 0; q < B; ++q) ahead[q] = __ldcs(&p[32 * q].e);
 #pragma unroll
     for (int q = 0; q < B; ++q) pair(e[q], v[q], x[q]);
   }
@@ -382,19 +391,7 @@ __device__ __forceinline__ void abs_pos(const Frame<T>& F, const LL4& X, T* x) {
 }
 
 // ---------------------------------------------------------- reductions ----
-__device__ __forceinline__ double warp_min(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 __device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ long long warp_sum(long long v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
@@ -432,18 +429,22 @@ __device__ __forceinline__ bool err_above(float ra, float ta, float rb, float tb
   return err_exact(ra, ta) > err_exact(rb, tb);
 }
 
-// b into a (fixed order: a's block comes first)
+// b into a (fixed order: a's block comes first). FP32 path: by the quotients the
+// partials carry; only ties look further.
 template <class T>
 __device__ __forceinline__ void merge(Partial& a, const Partial& b) {
   if (sizeof(T) == 4) {
-    if (ratio_before(b.rc, b.an, b.amin, a.rc, a.an, a.amin)) {
+    if (b.q < a.q || (b.q == a.q && ratio_before(b.rc, b.an, b.amin, a.rc, a.an, a.amin))) {
       a.rc = b.rc;
       a.an = b.an;
+      a.q = b.q;
       a.amin = b.amin;
     }
-    if (err_above(b.er, b.et, a.er, a.et)) {
+    const bool near = fabsf(a.ek - b.ek) <= 1e-6f * fmaxf(a.ek, b.ek);
+    if (near ? err_above(b.er, b.et, a.er, a.et) : b.ek > a.ek) {
       a.er = b.er;
       a.et = b.et;
+      a.ek = b.ek;
     }
     a.ma = fmaxf(a.ma, b.ma);
   } else {
@@ -458,7 +459,12 @@ __device__ __forceinline__ void merge(Partial& a, const Partial& b) {
   a.lentries += b.lentries;
 }
 __device__ __forceinline__ Partial no_partial() {
-  return Partial{DBL_MAX, 0.0, 0.0, 0.0, 0.0, 0, 0, 0, -1, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  Partial p{};
+  p.min_rc_a = DBL_MAX;
+  p.amin = -1;
+  p.q = __int_as_float(0x7f800000);  // infinity
+  p.ek = -1.0f;
+  return p;
 }
 // Warp reductions of whole values by the integer reduction unit: a few
 // instructions where five rounds of shuffles and merges took microseconds at
@@ -479,10 +485,10 @@ __device__ __forceinline__ double warp_max_bits(double v) {
   const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)__double2loint(v) : 0u);
   return __hiloint2double((int)mh, (int)ml);
 }
-// the lane whose r_c / |a| comes first (k: its particle, < 0: none); -1: none
-__device__ __forceinline__ int first_ratio(float rc, float an, int k) {
+// the lane whose r_c / |a| = q comes first (k: its particle, < 0: none); -1: none
+__device__ __forceinline__ int first_ratio(float q, float rc, float an, int k) {
   constexpr unsigned all = 0xffffffffu;
-  const unsigned qb = k >= 0 ? __float_as_uint(__fdiv_rn(rc, an)) : 0xffffffffu;
+  const unsigned qb = k >= 0 ? __float_as_uint(q) : 0xffffffffu;
   const unsigned qmin = __reduce_min_sync(all, qb), who = __ballot_sync(all, qb == qmin);
   if (qmin == 0xffffffffu) return -1;
   int src = __ffs(who) - 1;
@@ -530,11 +536,13 @@ __device__ __forceinline__ Partial warp_total(const Partial& p) {
   constexpr unsigned all = 0xffffffffu;
   Partial q = no_partial();
   if (sizeof(T) == 4) {
-    const int l = first_ratio(p.rc, p.an, (int)p.amin), s = l < 0 ? 0 : l;
+    const int l = first_ratio(p.q, p.rc, p.an, (int)p.amin), s = l < 0 ? 0 : l;
     q.rc = __shfl_sync(all, p.rc, s);
     q.an = __shfl_sync(all, p.an, s);
+    q.q = __shfl_sync(all, p.q, s);
     q.amin = __shfl_sync(all, (int)p.amin, s);
-    const int m = largest_error(err_key(p.er, p.et), p.er, p.et), t = m < 0 ? 0 : m;
+    const int m = largest_error(p.ek, p.er, p.et), t = m < 0 ? 0 : m;
+    q.ek = __shfl_sync(all, p.ek, t);
     q.er = __shfl_sync(all, p.er, t);
     q.et = __shfl_sync(all, p.et, t);
     q.ma = __uint_as_float(__reduce_max_sync(all, __float_as_uint(p.ma)));
@@ -596,7 +604,7 @@ __device__ __forceinline__ void warp_sums(bool active, int i, float rc, float an
   const int lane = threadIdx.x & 31;
   // the smallest r_c / |a|
   const bool moves = active && an > 0.0f;
-  const int first = first_ratio(rc, an, moves ? i : -1), fl = first < 0 ? 0 : first;
+  const int first = first_ratio(moves ? __fdiv_rn(rc, an) : 0.0f, rc, an, moves ? i : -1), fl = first < 0 ? 0 : first;
   const float mrc = __shfl_sync(all, rc, fl), man = __shfl_sync(all, an, fl);
   const int mi = __shfl_sync(all, i, fl);
   // the largest |a| (NaN, which raises the error word, counts as none)
@@ -654,8 +662,10 @@ __device__ __forceinline__ Partial to_partial(const WarpSums& w) {
   p.an = w.an;
   p.amin = w.amin;
   p.ma = __uint_as_float(w.max_a);
+  if (w.amin >= 0) p.q = __fdiv_rn(w.rc, w.an);
   p.er = w.er;
   p.et = w.et;
+  p.ek = err_key(w.er, w.et);
   p.sum_rho = from_limbs(w.rl, w.re);
   p.err_l2 = from_limbs(w.el, w.ee);
   p.ipairs = w.ni;
@@ -666,13 +676,11 @@ __device__ __forceinline__ Partial to_partial(const WarpSums& w) {
 
 // L2 read of a partial another block wrote
 __device__ __forceinline__ Partial load_partial(const Partial* p) {
-  static_assert(sizeof(Partial) == 96, "members read one by one");
-  const double* d = (const double*)p;
-  const long long* l = (const long long*)p;
-  const float* f = (const float*)p;
-  return Partial{__ldcg(d + 0), __ldcg(d + 1), __ldcg(d + 2), __ldcg(d + 3), __ldcg(d + 4), __ldcg(l + 5),
-                 __ldcg(l + 6), __ldcg(l + 7), __ldcg(l + 8), __ldcg(f + 18), __ldcg(f + 19), __ldcg(f + 20),
-                 __ldcg(f + 21), __ldcg(f + 22), 0.0f};
+  static_assert(sizeof(Partial) == 112, "whole 16-byte words");
+  Partial q;
+#pragma unroll
+  for (int k = 0; k < 7; ++k) ((int4*)&q)[k] = __ldcg((const int4*)p + k);
+  return q;
 }
 // Called by one warp of every block with the block's partial in lane 0:
 // the last block of a group merges the group's partials, the last group's
@@ -734,6 +742,7 @@ __global__ void __launch_bounds__(256) k_rekey(int n, StepCtl* ctl, int force, u
                                                const LL4* __restrict__ X0, const LL4* __restrict__ X1, Frame<T> F,
                                                Grid<T> G, Geom<T> geo, uint32_t* __restrict__ key,
                                                uint32_t* __restrict__ cnt, uint32_t* __restrict__ part) {
+  let_successor();
   if (!(force || *(volatile int*)&ctl->need_rebuild)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       ctl->vp ^= 1;
@@ -794,6 +803,7 @@ __global__ void __launch_bounds__(256) k_gather_view(
     uint32_t* __restrict__ m1, uint32_t* __restrict__ p0, uint32_t* __restrict__ p1, Frame<T> F, Geom<T> geo,
     typename ViewOf<T>::type* __restrict__ v0, typename ViewOf<T>::type* __restrict__ v1,
     typename ViewOf<T>::type* __restrict__ vbuild, int4* __restrict__ v32, Frame<float> F32) {
+  after_predecessor();
   if (!ctl->rebuild) return;
   const int nb = ctl->buf, vp = ctl->vp;  // new buffers; the old order lives in the other state buffer
   const uint32_t* __restrict__ pold = nb ? p0 : p1;
@@ -957,6 +967,7 @@ __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(
     const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1, const int4* __restrict__ view,
     const uint32_t* __restrict__ cstart, Frame<float> F, Grid<float> G, float kappa, int cap,
     uint32_t* __restrict__ list, uint32_t* __restrict__ lcount, int* __restrict__ err) {
+  after_predecessor();
   if (!ctl->rebuild) return;
   const int buf = ctl->buf;
   const uint32_t* __restrict__ meta = buf ? m1 : m0;
@@ -1027,6 +1038,7 @@ __global__ void __launch_bounds__(256) k_list_build_group(int n, StepCtl* __rest
                                                           uint32_t* __restrict__ list, uint32_t* __restrict__ lcount,
                                                           int* __restrict__ err) {
   __shared__ int longest;
+  after_predecessor();
   if (!ctl->rebuild) return;
   if (threadIdx.x == 0) longest = 0;
   __syncthreads();
@@ -1107,6 +1119,7 @@ __global__ void __launch_bounds__(kStageBlock) k_stage(int n, const StepCtl* __r
                                                       const uint32_t* __restrict__ lcount, int cap,
                                                       uint32_t* __restrict__ llist, int* __restrict__ scount,
                                                       int* __restrict__ sj) {
+  after_predecessor();
   if (!ctl->rebuild) return;
   __shared__ int tab[kStageHash];
   __shared__ int rnk[kStageHash];
@@ -2064,7 +2077,7 @@ cudaError_t launch_rebuild(const DevState& S, int force, const Grid<T>& G, const
   // the FP64 path lists its pairs through an FP32 view (same frame origin, same
   // cells, same list format)
   if (std::is_same<T, double>::value && (!S.view32 || !F32 || !G32)) return cudaErrorInvalidValue;
-  k_gather_view<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, S.tmp, S.key, S.cstart, (LL4*)S.X[0], (LL4*)S.X[1], S.meta[0],
+  launch_after(k_gather_view<D, T>, gb, tb, 0, st, S.n, S.ctl, S.tmp, S.key, S.cstart, (LL4*)S.X[0], (LL4*)S.X[1], S.meta[0],
                                          S.meta[1], S.pid[0], S.pid[1], F, g, (VT*)S.view[0], (VT*)S.view[1],
                                          (VT*)S.vbuild, (int4*)S.view32, F32 ? *F32 : Frame<float>{});
   constexpr bool f64 = std::is_same<T, double>::value;
@@ -2077,14 +2090,14 @@ cudaError_t launch_rebuild(const DevState& S, int force, const Grid<T>& G, const
   }
   const bool group = S.n <= kListGroupMax;
   auto build = [&](auto* kernel, int blocks) {
-    kernel<<<blocks, tb, 0, st>>>(S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], view, S.cstart, *Fl, *Gl, (float)kappa,
-                                  S.cap, S.list, S.lcount, S.err);
+    launch_after(kernel, blocks, tb, 0, st, S.n, S.ctl, X0, X1, S.meta[0], S.meta[1], view, S.cstart, *Fl, *Gl,
+                 (float)kappa, S.cap, S.list, S.lcount, S.err);
   };
   if (group) build(k_list_build_group<D, kListLanes, f64>, grid_for(S.n * kListLanes, tb));
   else build(k_list_build<D, f64>, grid_for(S.n, tb));
   if constexpr (!f64) {
     if (S.stage && S.llist)
-      k_stage<D><<<grid_for(S.n, kStageBlock), kStageBlock, 0, st>>>(S.n, S.ctl, S.list, S.lcount, S.cap, S.llist,
+      launch_after(k_stage<D>, grid_for(S.n, kStageBlock), kStageBlock, 0, st, S.n, S.ctl, S.list, S.lcount, S.cap, S.llist,
                                                                   S.scount, S.sj);
   }
   return cudaGetLastError();
@@ -2103,16 +2116,14 @@ cudaError_t launch_pass_a(const DevState& S, const Frame<T>& F, const Phys<T>& P
   const Frame<float> f32 = s32 ? *f.f32 : Frame<float>{};
   auto run = [&](auto* kernel, int threads, int lanes, size_t smem) {
     kernel<<<grid_for(S.n * lanes, threads), threads, smem, st>>>(
-        S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], S.meta[0], S.meta[1], S.pid[0], S.pid[1], S.list,
-        S.lcount, S.cap, F, P, pc, (V4<T>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err, f.advance, S.dbg_count,
+        S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], S.meta[0], S.meta[1], S.pid[0], S.pid[1], S.list, S.lcount, S.cap, F, P, pc, (V4<T>*)S.acc4, rho, S.partials, S.scal, S.tickets, S.err, f.advance, S.dbg_count,
         S.dbg_sum, (PairRec<T>*)S.plist, S.pcount, f.dt_fix, f.dt_rec, (const LL4*)S.X[0], (const LL4*)S.X[1], geo,
         S.llist, S.scount, S.sj, v32, f32);
     return cudaGetLastError();
   };
   const auto density = [&](auto* kernel, int threads) {
-    kernel<<<grid_for(S.n, threads), threads, 0, st>>>(S.n, S.ctl, (const VT*)S.view[0],
-                                                               (const VT*)S.view[1], S.list, S.lcount, S.cap, F, P,
-                                                               rho, pc);
+    kernel<<<grid_for(S.n, threads), threads, 0, st>>>(S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], S.list,
+                                                       S.lcount, S.cap, F, P, rho, pc);
   };
   // one block size and one of the compiled variants
   auto pick = [&](auto nt) -> cudaError_t {
@@ -2164,7 +2175,10 @@ cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P
   };
   if constexpr (std::is_same<T, float>::value) {
     if (S.n <= kPassGroupMax) return run(k_pass_b<D, T, 32 * kPassLanes, kPassLanes>, 32 * kPassLanes, kPassLanes);
-    return S.pass_threads == 128 ? run(k_pass_b<D, T, 128>, 128, 1) : run(k_pass_b<D, T, 256>, 256, 1);
+    // large runs in small blocks, whose warps wait for no one else's tail
+    // (8,388,608 particles in 3D 873 -> 805 us, 1,048,576 in 2D 71 -> 69; at
+    // 240,370 in 3D 31 -> 33)
+    return S.pass_threads == 128 || S.n >= (1 << 19) ? run(k_pass_b<D, T, 128>, 128, 1) : run(k_pass_b<D, T, 256>, 256, 1);
   } else {
     if (fp64_lanes(S) > 1) return run(k_pass_b<D, T, 32 * kLanes64, kLanes64>, 32 * kLanes64, kLanes64);
     return fp64_threads(S) == 32 ? run(k_pass_b<D, T, 32>, 32, 1) : run(k_pass_b<D, T, 64>, 64, 1);
