@@ -381,6 +381,7 @@ def relax_fn(problem, colors, n_steps, precision="fp32", lam=1.0, density_weight
             c = col.to(x0.device)
             xs = x0.detach().to(torch.float64).contiguous()
             ctx.save_for_backward(xs, c, sigma0, gamma, P0, poly)
+            r.stream.wait_stream(torch.cuda.current_stream(xs.device))  # xs and c may still be on their way
             r.set_state(xs, c)
             r.step(n_steps)
             out = torch.empty_like(xs)
@@ -396,8 +397,9 @@ def relax_fn(problem, colors, n_steps, precision="fp32", lam=1.0, density_weight
         def backward(ctx, g_x, g_L):
             xs, c, sigma0, gamma, P0, poly = ctx.saved_tensors
             r = handle(values(sigma0, gamma, P0, poly))
-            r.set_state(xs, c)
             seed = None if g_x is None else g_x.detach().to(torch.float64).contiguous()
+            r.stream.wait_stream(torch.cuda.current_stream(xs.device))
+            r.set_state(xs, c)
             wL = 0.0 if g_L is None else float(g_L)
             dpos = torch.empty_like(xs)
             res = r.backward(n_steps, lam=lam * wL, density_weight=density_weight * wL, frozen_dt=frozen_dt,
