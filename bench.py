@@ -63,10 +63,9 @@ WORKLOADS = {
 # are extra traffic by design and are not counted.
 ALG_BYTES = {"cells": 54, "pass_a": 33, "pass_b": 49}
 ALG_BYTES_FP64 = {"cells": 92, "pass_a": 56, "pass_b": 83}
-# launches per step (gamma = 2): gate; rekey, count, 3 scan, scatter, gather,
-# make_view, list_build (predicated: they exit at once unless the list is
-# rebuilt); pass A; pass B; with the staged pass A one more predicated
-# rebuild kernel (the blocks' neighbour sets)
+# launches per step (gamma = 2): rekey, scan, scatter, gather, list_build (they
+# exit at once unless the list is rebuilt); pass A; pass B; with the staged pass A
+# one more predicated rebuild kernel (the blocks' neighbour sets)
 KERNELS_PER_STEP = 7
 # pair arithmetic (FP32 flop, counted from the equations as the kernels evaluate
 # them): distance of a pair 10 (differences, squared norm, root), density term 8

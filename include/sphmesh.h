@@ -107,13 +107,14 @@ typedef struct {
   int32_t kernel_id;   /* 0: Wendland C2 (the only one) */
   uint64_t seed;       /* seed of the initial sampling (Philox4x32-10) */
   double cell_factor;  /* finest cell edge / smallest support; 0 -> 1.0 */
-  int32_t block_size;  /* threads per block of the pair passes: 0 (256), 128 or 256 */
+  int32_t block_size;  /* threads per block of the FP32 pair passes: 0 (256), 128 or 256 */
   int32_t use_graph;   /* 1: sph_step replays a captured CUDA graph of one step */
   int32_t record_fields; /* 1: keep rho, a_n and a~ of the last step for sph_get_field */
   int32_t list_capacity; /* neighbour-list entries per particle; 0 -> auto */
   double skin;           /* neighbour-list skin as a fraction of the support kappa h;
-                            0 -> 0.15 in 3D, 0.2 in 2D; the list is rebuilt when a particle has moved
-                            half its skin (results do not depend on it) */
+                            the list is rebuilt when a particle has moved half its skin (results do
+                            not depend on it). 0 -> each particle's own, from its last move (0.15 in
+                            3D, 0.2 in 2D before any); a given list_capacity keeps those for all */
 } sph_params;
 
 typedef struct {

@@ -133,12 +133,9 @@ sph_status status_from_flags(sph_handle* h, int flags) {
   return SPH_OK;
 }
 
-// list skin (fraction of kappa h) when params.skin = 0: a longer list costs
-// every step, a shorter one more frequent rebuilds. 3D: on the 8M-particle
-// graded workload (20 graph-replayed steps after 5 warm-up steps) 0.15 took
-// 5.94 ms per step against 6.6 / 6.33 / 6.16 ms for 0.12 / 0.2 / 0.25 (5.93
-// vs 6.16 ms for 0.15 / 0.2 over 50 steps). 2D: 0.2 (the 262,144-particle
-// polynomial-field workload: 20 steps in 2.77 ms against 2.82 at 0.15).
+// list skin (fraction of kappa h) of the first list when params.skin = 0, before
+// any particle's speed is known (then kSkinSteps in sph_host.h): a longer list
+// costs every step, a shorter one more frequent rebuilds
 inline double default_skin(int dim) { return dim == 3 ? 0.15 : 0.2; }
 
 // a skin or a list capacity of the caller's choosing keeps one skin for all
@@ -164,7 +161,10 @@ void setup_frames(sph_handle* h) {
 // initial states cluster), plus 16.
 int auto_capacity(const sph_handle* h) {
   double skin = h->par.skin > 0 ? h->par.skin : default_skin(h->dim);
-  if (adaptive_skin(h)) skin = std::max(skin, 2.0 * kSkinMost);
+  // adaptive reach: a pair of the fastest particles is listed to 0.3, but lists
+  // are shorter on average than with one skin of 0.15, so 0.2 for the bound below
+  // (3D: 150 entries; all neighbours fast: 74 expected, 126 at six deviations)
+  if (adaptive_skin(h)) skin = std::max(skin, 0.2);
   const double k1 = h->par.kappa * (1.0 + skin);
   const double L = std::min(h->lip_h, 0.5 / k1);
   const double g = k1 / (1.0 - L * k1);
