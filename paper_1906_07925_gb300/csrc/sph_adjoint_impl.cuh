@@ -97,6 +97,10 @@ __device__ __forceinline__ float warp_sum_t(float v) {
 }
 __device__ __forceinline__ double warp_sum_t(double v) { return warp_sum(v); }
 
+// The blocks' sums are added in two levels, groups of kAdjGroup blocks and then
+// the groups, one value per warp at a time: one block adding everybody's with
+// all its warps took 800 FP64 warp instructions for the eleven values of
+// k_bwd_force, 16 cycles each.
 template <int M, class T>
 __device__ bool block_partials(T (&v)[M], double* __restrict__ part, unsigned* __restrict__ ticket, double* out) {
   __shared__ double sm[8][M];
@@ -114,36 +118,34 @@ __device__ bool block_partials(T (&v)[M], double* __restrict__ part, unsigned* _
     for (int k = 0; k < nw; ++k) s += sm[k][threadIdx.x];
     part[(size_t)blockIdx.x * kAdjPartials + threadIdx.x] = s;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  const int nb = gridDim.x, ng = (nb + kAdjGroup - 1) / kAdjGroup, g = blockIdx.x / kAdjGroup, b0 = g * kAdjGroup;
+  // true in the block that adds `n` entries from `first` last of `arrivals`
+  auto gather = [&](unsigned* t, int arrivals, int first, int n) -> bool {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      last = atomicAdd(t, 1u) == (unsigned)(arrivals - 1);
+    }
+    __syncthreads();
+    if (!last) return false;
     __threadfence();
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    for (int q = w; q < M; q += nw) {
+      double s = 0.0;
+      for (int b = lane; b < n; b += 32) s += __ldcg(part + (size_t)(first + b) * kAdjPartials + q);
+      s = warp_sum(s);
+      if (lane == 0) res[q] = s;
+    }
+    if (threadIdx.x == 0) *t = 0u;
+    __syncthreads();
+    return true;
+  };
+  if (!gather(ticket + 1 + g, min(kAdjGroup, nb - b0), b0, min(kAdjGroup, nb - b0))) return false;
+  if (ng > 1) {
+    if (threadIdx.x < M) part[(size_t)(nb + g) * kAdjPartials + threadIdx.x] = res[threadIdx.x];
+    if (!gather(ticket, ng, nb, ng)) return false;
   }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  // every thread sums a fixed stride of the block partials, then a fixed tree
-  double a[M];
-#pragma unroll
-  for (int q = 0; q < M; ++q) a[q] = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < M; ++q) a[q] += __ldcg(part + (size_t)b * kAdjPartials + q);
-#pragma unroll
-  for (int q = 0; q < M; ++q) {
-    const double x = warp_sum(a[q]);
-    if (lane == 0) sm[w][q] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x < M) {
-    double s = 0.0;
-    for (int k = 0; k < nw; ++k) s += sm[k][threadIdx.x];
-    res[threadIdx.x] = s;
-  }
-  __syncthreads();
 #pragma unroll
   for (int q = 0; q < M; ++q) out[q] = res[q];
-  if (threadIdx.x == 0) *ticket = 0u;
   return true;
 }
 
@@ -787,7 +789,9 @@ template <int D, class T>
 cudaError_t launch_bwd_step(const DevState& S, const Frame<T>& F, const Phys<T>& P, const Geom<T>& geo,
                             const AdjBufs<T>& B, int recomputed_dt, int general_eos, cudaStream_t st) {
   using VT = typename ViewOf<T>::type;
-  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 256, gb = grid_for(S.n, tb);
+  // small blocks: warps that are done wait for the block's slowest (barrier
+  // stalls were a sixth of k_bwd_visc at 256 threads)
+  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 128, gb = grid_for(S.n, tb);
   if (S.n <= 0) return cudaSuccess;
   const VT* w0 = (const VT*)S.view[0];
   const VT* w1 = (const VT*)S.view[1];
@@ -813,7 +817,9 @@ template <int D, class T>
 cudaError_t launch_objective(const DevState& S, const Frame<T>& F, const Phys<T>& P, const Geom<T>& geo,
                              const AdjBufs<T>& B, double wd, double lambda, cudaStream_t st) {
   using VT = typename ViewOf<T>::type;
-  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 256, gb = grid_for(S.n, tb);
+  // small blocks: warps that are done wait for the block's slowest (barrier
+  // stalls were a sixth of k_bwd_visc at 256 threads)
+  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 128, gb = grid_for(S.n, tb);
   if (S.n <= 0) return cudaSuccess;
   const VT* w0 = (const VT*)S.view[0];
   const VT* w1 = (const VT*)S.view[1];

@@ -505,13 +505,13 @@ sph_status ensure_adj(sph_handle* h) {
   SPH_TRY(grab(h, p, N * t1)); a.Tb = p;
   SPH_TRY(grab(h, p, N * t1)); a.rtb = p;
   SPH_TRY(grab(h, p, N * t1)); a.rhob = p;
-  SPH_TRY(grab(h, a.part, nb * kAdjPartials));
+  SPH_TRY(grab(h, a.part, (nb + nb / kAdjGroup + 2) * kAdjPartials));
   SPH_TRY(grab(h, a.acc, (size_t)kAdjSlots));
   SPH_TRY(grab(h, a.g[0], N * d));
   SPH_TRY(grab(h, a.g[1], N * d));
-  SPH_TRY(grab(h, a.ticket, 4));
+  SPH_TRY(grab(h, a.ticket, nb / kAdjGroup + 3));
   SPH_TRY(grab(h, a.col, N));
-  SPH_CUDA(h, cudaMemsetAsync(a.ticket, 0, 16, h->stream));
+  SPH_CUDA(h, cudaMemsetAsync(a.ticket, 0, sizeof(unsigned) * (nb / kAdjGroup + 3), h->stream));
   a.ready = true;
   return SPH_OK;
 }

@@ -204,6 +204,7 @@ enum AdjSlot : int {
   kAdjSlots = 16
 };
 constexpr int kAdjPartials = 12;  // doubles per block partial
+constexpr int kAdjGroup = 64;     // blocks whose partials are added together first
 
 template <class T>
 struct AdjBufs {
