@@ -112,7 +112,7 @@ typedef struct {
   int32_t record_fields; /* 1: keep rho, a_n and a~ of the last step for sph_get_field */
   int32_t list_capacity; /* neighbour-list entries per particle; 0 -> auto */
   double skin;           /* neighbour-list skin as a fraction of the support kappa h;
-                            the list is rebuilt when a particle has moved half its skin (results do
+                            the list is rebuilt when a particle has moved half of it (results do
                             not depend on it). 0 -> each particle's own, from its last move (0.15 in
                             3D, 0.2 in 2D before any); a given list_capacity keeps those for all */
 } sph_params;
@@ -487,7 +487,7 @@ void sph_destroy(sph_handle* h);
  * problem needs must fit in SPH_NOALLOC_MAX_CELLS cells (raise
  * params->cell_factor otherwise); FP32 split precision only; field->rho_scale
  * must be given (> 0). Anything beyond: SPH_ERR_INVALID_ARG, nothing launched.
- * The scratch array (about 35 MB) is held by every GPU that loads the library
+ * The scratch array (about 50 MB) is held by every GPU that loads the library
  * until the process exits. A particle with more than 95 neighbours inside its
  * support makes the call fail with SPH_ERR_CELL_OVERFLOW.
  *

@@ -100,7 +100,8 @@ __device__ __forceinline__ double warp_sum_t(double v) { return warp_sum(v); }
 // The blocks' sums are added in two levels, groups of kAdjGroup blocks and then
 // the groups, one value per warp at a time: one block adding everybody's with
 // all its warps took 800 FP64 warp instructions for the eleven values of
-// k_bwd_force, 16 cycles each.
+// k_bwd_force, 16 cycles each (262,144 particles in 2D, 1,024 blocks of 256: 20
+// reverse steps 6.27 -> 6.12 ms with 2,048 blocks of 128).
 template <int M, class T>
 __device__ bool block_partials(T (&v)[M], double* __restrict__ part, unsigned* __restrict__ ticket, double* out) {
   __shared__ double sm[8][M];

@@ -1489,7 +1489,7 @@ sph_status sph_backward(sph_handle* h, int32_t K, const sph_objective* obj, cons
 
 // ================================================================ batch ==
 // Many independent instances stepped by one CUDA graph per step. Instance k's
-// step (its 12 kernels, predicated on its own list-rebuild flag) sits on
+// step (its 7 kernels, those of a rebuild predicated on its own list-rebuild flag) sits on
 // branch b(k) of the graph; the branches fork from and join to the batch's
 // stream, so instances on different branches run concurrently and fill the
 // SMs that one small instance leaves idle. Instances are dealt to branches

@@ -139,7 +139,7 @@ struct Scalars {
 // Surface-tension schedule (Eq. sph_st_sigma), step counter and the
 // neighbour-list bookkeeping. `buf` selects the buffer holding the state in its
 // current order, `vp` the current view buffer; `need_rebuild` is raised by
-// pass B when a particle has moved half its skin since the list was built.
+// pass B when a particle has moved its reach since the list was built.
 struct StepCtl {
   long long step;
   double t0, t1, sigma0;

@@ -10,7 +10,8 @@
 //
 // Neighbour list (the neighbour search of Algorithm 1). The list of particle i holds every j
 // (itself included) that can come within kappa max(h_i, h_j) before some
-// particle has moved half its skin; it is rebuilt, on the device, only then.
+// particle has moved its reach (its share of the skin, k_gather_view); it is
+// rebuilt, on the device, only then.
 // The criterion is symmetric, so i also finds every j whose own support
 // reaches i (the reverse pass gathers over such pairs).
 // Passes A and B re-test the exact criteria of the current step for every
@@ -1729,8 +1730,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
 //   a~_i = (dt1^2 / 2) B_i,
 //   B_i  = sum_j HM(g_i, g_j) (1/rho_t,i^2 + 1/rho_t,j^2) (dW/dr / r)(a_i - a_j),
 //   v_i  = dt1 a_i / 2 + dt2 a~_i / 2,   r_i += v_i dt2.
-// The new view goes to the other view buffer; a particle that moved half its
-// skin since the list was built raises need_rebuild.
+// The new view goes to the other view buffer; a particle that moved its
+// reach since the list was built raises need_rebuild.
+// Bound by the gather of the neighbour's acceleration, one per force pair: the
+// pair's geometry factor comes from pass A's record (8,388,608 particles in 3D,
+// FP32: 1.40 -> 0.77 ms with 128-thread blocks; 300,007 in FP64: 1.40 -> 0.43).
 // --------------------------------------------------------------------------
 template <int D, class T, int NT, int G = 1>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP64 : SPH_PASSB_MIN_BLOCKS) * 256 / NT) k_pass_b(int n, StepCtl* __restrict__ ctl,
