@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(256) k_bwd_local(int n, const StepCtl* __restr
       // both (a third of a list) stop at the distance, and W'/r = -20 c H^-(d+2)
       // (1 - q)^3 needs no division by r
       const T rbi = B.rhob[i];
-      const T Hvi = P.kappa * hv, Hvi2 = Hvi * Hvi, iHvi = T(1) / Hvi, iHi = iHvi * F.inv_qv;
+      const T Hvi = P.kappa * hv, Hvi2 = Hvi * Hvi, iHvi = T(1) / Hvi, iHi = T(1) / (P.kappa * hi);
       const T ci = rbi * P.alpha * ipow_d<D, T>(iHi), fi = T(-20) * ci * iHi * iHi;
       T wh = 0;
       for_skin_list(list, view, i, lcount[i], cap, [&](uint32_t e, const VT& vj) {
@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(256) k_bwd_local(int n, const StepCtl* __restr
         const T Hvj = P.kappa * view_h(F, vj);
         const bool in_i = r2 < Hvi2, in_j = r2 < Hvj * Hvj && j != i;
         if (!(in_i || in_j)) return;
-        const T r = r2 > T(0) ? pair_r<T>(r2) : T(0);
+        const T r = dsqrt(r2);
         T c = 0;
         if (in_i) {
           const T q = r * iHvi, u = T(1) - q, u3 = u * u * u;
@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(256) k_bwd_local(int n, const StepCtl* __restr
           c = fi * u3;
         }
         if (in_j) {
-          const T iHvj = drcp<T>(Hvj), u = T(1) - r * iHvj, iHj = iHvj * F.inv_qv;
+          const T iHj = drcp<T>(Hvj * qv), u = T(1) - r * qv * iHj;
           c += T(-20) * P.alpha * B.rhob[j] * ipow_d<D, T>(iHj) * iHj * iHj * (u * u * u);
         }
         xx += c * dx;
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(256) k_obj(int n, const StepCtl* __restrict__ 
       const T Hv = half_kappa * (hv + hvj);
       const bool face = r2 < Hv * Hv && j != i && (e & 0xFFu) != ci;
       if (!(r2 < Hvi2 || face)) return;
-      const T rv = r2 > T(0) ? pair_r<T>(r2) : T(0);
+      const T rv = dsqrt(r2);
       if (r2 < Hvi2) {
         const T q = rv * iHvi, u = T(1) - q, u2 = u * u;
         rho += u2 * u2 * (T(1) + T(4) * q);
@@ -736,7 +736,9 @@ __global__ void __launch_bounds__(256) k_obj(int n, const StepCtl* __restrict__ 
       xz += c * dz * qv;
       hbar += lambda * k.WH * half_kappa;
     });
-    rho *= P.alpha * ipow_d<D, T>(iHvi * F.inv_qv);
+    // with the same h as rho_t below, and (above) the rounded root: what is off
+    // alike in every particle does not cancel in rho / rho_t - 1
+    rho *= P.alpha * ipow_d<D, T>(T(1) / (P.kappa * hi));
     const T rt = rho_t_of_h<D, T>(hi, P.inv_tau);
     const T e = rho / rt - T(1);
     v[0] = e * e;
