@@ -170,12 +170,21 @@ class Relaxation:
     def __exit__(self, *a):
         self.close()
 
+    def _after(self, *tensors):
+        """Order the handle's stream after what the caller's streams still have to
+        write to (or read of) these CUDA tensors. The library is done with them
+        when a call that takes them returns."""
+        cuda = self._torch.cuda
+        for d in {t.device for t in tensors if t is not None and t.is_cuda}:
+            self.stream.wait_stream(cuda.current_stream(d))
+
     # ------------------------------------------------------------------- API
     def set_state(self, pos, col):
         torch = self._torch
         if isinstance(pos, torch.Tensor) and pos.is_cuda:
             pos = pos.to(torch.float64).contiguous()
             col = col.to(torch.uint8).contiguous()
+            self._after(pos, col)
             self._check(self.lib.sph_set_state(self.h, pos.data_ptr(), col.data_ptr(), 1))
             return
         pos = np.ascontiguousarray(pos, dtype=np.float64)
@@ -212,6 +221,7 @@ class Relaxation:
     def positions(self, out=None):
         """(n, dim) float64 in particle-id order: numpy, or into a CUDA tensor `out`."""
         if out is not None:
+            self._after(out)
             self._check(self.lib.sph_get_positions(self.h, out.data_ptr(), 1))
             return out
         x = np.empty((self.n, self.dim), np.float64)
@@ -239,6 +249,7 @@ class Relaxation:
             if dt_dev is None or dt_dev.shape[0] != max(int(n_steps), 0) or dt_dev.device != out.device:
                 dt_dev = torch.zeros((max(int(n_steps), 0), 2), dtype=torch.float64, device=out.device)
                 self._dt_dev = dt_dev
+            self._after(out, seed, dt, dt_dev)
             self._check(self.lib.sph_backward(self.h, int(n_steps), C.byref(obj),
                                               None if seed is None else seed.data_ptr(),
                                               None if dt is None else dt.data_ptr(),
@@ -381,7 +392,6 @@ def relax_fn(problem, colors, n_steps, precision="fp32", lam=1.0, density_weight
             c = col.to(x0.device)
             xs = x0.detach().to(torch.float64).contiguous()
             ctx.save_for_backward(xs, c, sigma0, gamma, P0, poly)
-            r.stream.wait_stream(torch.cuda.current_stream(xs.device))  # xs and c may still be on their way
             r.set_state(xs, c)
             r.step(n_steps)
             out = torch.empty_like(xs)
@@ -398,7 +408,6 @@ def relax_fn(problem, colors, n_steps, precision="fp32", lam=1.0, density_weight
             xs, c, sigma0, gamma, P0, poly = ctx.saved_tensors
             r = handle(values(sigma0, gamma, P0, poly))
             seed = None if g_x is None else g_x.detach().to(torch.float64).contiguous()
-            r.stream.wait_stream(torch.cuda.current_stream(xs.device))
             r.set_state(xs, c)
             wL = 0.0 if g_L is None else float(g_L)
             dpos = torch.empty_like(xs)
