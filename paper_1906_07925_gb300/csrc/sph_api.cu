@@ -128,7 +128,7 @@ sph_status status_from_flags(sph_handle* h, int flags) {
   if (flags & kErrNonfinite) return fail(h, SPH_ERR_NONFINITE, "non-finite density, force or position");
   if (flags & kErrOutOfDomain) return fail(h, SPH_ERR_OUT_OF_DOMAIN, "a particle was outside the box");
   if (flags & kErrListOverflow)
-    return fail(h, SPH_ERR_CELL_OVERFLOW, "a neighbour list exceeded its capacity (raise params.list_capacity)");
+    return fail(h, SPH_ERR_CELL_OVERFLOW, "a neighbour list exceeded its capacity, at the common reach too (raise params.list_capacity)");
   if (flags & kErrTimeout) return fail(h, SPH_ERR_TIMEOUT, "a bounded device loop gave up");
   return SPH_OK;
 }
@@ -158,13 +158,13 @@ void setup_frames(sph_handle* h) {
 // L the field's Lipschitz bound of h), and inside that ball the number density
 // (tau/h)^d is at most (tau/h_i)^d / (1 - L g)^d. The capacity is the larger of
 // twice that and that plus ten standard deviations of a Poisson count (random
-// initial states cluster), plus 16.
+// initial states cluster), plus 16. That is for one skin: with the particles' own
+// reach a pair of fast ones is listed further out (0.3), so there is less room
+// over the mean (3D, no grading: 152 entries for 51 at the skin of 0.15, for 74
+// where all are fast); a list that does not fit is cut to the common reach
+// (k_list_build).
 int auto_capacity(const sph_handle* h) {
-  double skin = h->par.skin > 0 ? h->par.skin : default_skin(h->dim);
-  // adaptive reach: a pair of the fastest particles is listed to 0.3, but lists
-  // are shorter on average than with one skin of 0.15, so 0.2 for the bound below
-  // (3D: 150 entries; all neighbours fast: 74 expected, 126 at six deviations)
-  if (adaptive_skin(h)) skin = std::max(skin, 0.2);
+  const double skin = h->par.skin > 0 ? h->par.skin : default_skin(h->dim);
   const double k1 = h->par.kappa * (1.0 + skin);
   const double L = std::min(h->lip_h, 0.5 / k1);
   const double g = k1 / (1.0 - L * k1);
@@ -336,6 +336,7 @@ sph_status write_ctl_all(sph_handle* h) {
   c.vp = 0;
   c.rebuild = 0;
   c.need_rebuild = 1;
+  c.reach_cap = 255;
   c.rebuilds = 0;
   c.auto_on = h->auto_window > 0;
   c.auto_window = h->auto_window;

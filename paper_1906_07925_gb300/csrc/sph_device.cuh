@@ -87,6 +87,7 @@ struct Frame {
   // skin_u while its speed is unknown, else its last step's move times skin_k
   // plus skin_lo, at most skin_hi; held in 255ths of skin_hi (skin_q)
   float skin_u, skin_k, skin_lo, skin_hi, skin_q;
+  int code_u;            // skin_u in units of skin_q, rounded down: the common reach
 };
 
 // The view unit is the level-0 cell edge c0. FP32 view integers are 2^-24 c0;
@@ -145,6 +146,8 @@ struct StepCtl {
   double t0, t1, sigma0;
   int buf, vp, rebuild, need_rebuild;
   int lmax, dmax;  // of the last build: longest neighbour list, largest reach code (Frame::skin_q)
+  int reach_cap, pad_;  // no particle may move further than this code (255, or the common
+                        // reach: some list of the last build did not fit at the particles' own)
   long long rebuilds;
   // automatic start of the ramp (Sec. 3.3 convergence test): on, run length in
   // steps, relative tolerance, ramp fraction; state: current run, its opening

@@ -204,6 +204,7 @@ inline void make_frames(const sph_domain& dom, double kappa, double skin, bool a
     F.skin_lo = adaptive ? kSkinFloor : F.skin_u;
     F.skin_hi = adaptive ? std::max(kSkinMost, F.skin_u) : F.skin_u;
     F.skin_q = std::max(F.skin_hi, 1e-6f) / 255.0f;
+    F.code_u = std::max((int)std::floor(F.skin_u / F.skin_q - 0.5f), 0);
   };
   fill(out.f);
   fill(out.d);

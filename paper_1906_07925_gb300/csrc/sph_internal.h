@@ -21,7 +21,7 @@ struct DevState {
   uint32_t* meta[2] = {nullptr, nullptr};  // colour
   uint32_t* pid[2] = {nullptr, nullptr};   // particle id
   void* view[2] = {nullptr, nullptr};    // int4 (FP32) or double4 (FP64)
-  void* vbuild = nullptr;                // view at the list build, w = half skin
+  void* vbuild = nullptr;                // view at the list build with the particle's reach (FP32: build_reach, FP64: coded_reach)
   void* view32 = nullptr;                // FP64 path: FP32 view (list build; pass A's screen)
   uint32_t* key = nullptr;               // cell key (old order, rebuild only)
   uint32_t* tmp = nullptr;               // scatter slots

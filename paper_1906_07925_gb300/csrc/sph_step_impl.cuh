@@ -94,8 +94,17 @@ __device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>&
 // its position, and in w its view_w rounded up to 16 bits of mantissa with its
 // reach code in the low byte. The reach, in view integers:
 __device__ __forceinline__ float build_w(int4 v) { return __int_as_float(v.w & ~0xFF); }
-__device__ __forceinline__ float build_reach(const Frame<float>& F, int4 v) {
-  return (float)(v.w & 0xFF) * (2.0f * F.skin_q) * build_w(v);
+__device__ __forceinline__ float build_reach(const Frame<float>& F, int4 v, int most = 255) {
+  return (float)min(v.w & 0xFF, most) * (2.0f * F.skin_q) * build_w(v);
+}
+// FP64 path: pass B reads the reach itself (view units) with its code in the low
+// byte, where a float's mantissa leaves zeros
+__device__ __forceinline__ double with_code(float reach, int code) {
+  return __longlong_as_double(__double_as_longlong((double)reach) | code);
+}
+__device__ __forceinline__ double coded_reach(double w, int most) {
+  const int code = (int)(__double_as_longlong(w) & 0xFF);
+  return code > most ? w * (double)((float)most / (float)code) : w;
 }
 
 // The neighbour list of particle i has list_rows(cap) rows (list_at), split at
@@ -784,6 +793,7 @@ __global__ void __launch_bounds__(256) k_rekey(int n, StepCtl* ctl, int force, u
       ctl->rebuilds += 1;
       ctl->lmax = 0;
       ctl->dmax = 0;
+      ctl->reach_cap = 255;
     }
   }
 }
@@ -808,6 +818,7 @@ __global__ void __launch_bounds__(256) k_gather_view(
   if (!ctl->rebuild) return;
   const int nb = ctl->buf, vp = ctl->vp;  // new buffers; the old order lives in the other state buffer
   const uint32_t* __restrict__ pold = nb ? p0 : p1;
+  const int first = min((int)ceilf(F.skin_u / F.skin_q), 255);  // while the speed is unknown
   int most = 0;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
     const uint32_t i = slots[s];
@@ -826,8 +837,8 @@ __global__ void __launch_bounds__(256) k_gather_view(
     const auto v = make_view<D>(F, X, h_of<D, T>(geo, x));
     (vp ? v1 : v0)[d] = v;
     const float moved = __uint_as_float((uint32_t)X.w);
-    const float reach = moved > 0.0f ? fminf(fmaf(F.skin_k, moved, F.skin_lo), F.skin_hi) : F.skin_u;
-    const int code = min((int)ceilf(reach / F.skin_q), 255);
+    const float reach = fminf(fmaf(F.skin_k, moved, F.skin_lo), F.skin_hi);
+    const int code = moved > 0.0f && F.skin_k > 0.0f ? min((int)ceilf(reach / F.skin_q), 255) : first;
     most = max(most, code);
     if constexpr (std::is_same<T, double>::value) {
       const long long half = 1LL << (F32.sv - 1);
@@ -835,7 +846,7 @@ __global__ void __launch_bounds__(256) k_gather_view(
       const int4 u = make_int4((int)((X.x + half) >> F32.sv), (int)((X.y + half) >> F32.sv),
                                D == 3 ? (int)((X.z + half) >> F32.sv) : 0, w);
       v32[d] = u;
-      vbuild[d] = V4<double>{v.x, v.y, v.z, (double)(build_reach(F32, u) * F32.vscale)};
+      vbuild[d] = V4<double>{v.x, v.y, v.z, with_code(build_reach(F32, u) * F32.vscale, code)};
     } else {
       vbuild[d] = make_int4(v.x, v.y, v.z, ((v.w + 0xFF) & ~0xFF) | code);
     }
@@ -850,17 +861,27 @@ __global__ void __launch_bounds__(256) k_gather_view(
 // by at most lip_h times that), any pair inside the exact
 // criteria is still listed. Candidates come from rows of cells of every level
 // that can hold such a j, in the order (level, z row, y row, x).
+// CUT: a list that does not fit at these reaches is made again with d_i and d_j at
+// most the common reach (Frame::code_u) and the change of h bounded by the longer
+// of the two moves, max(d_i, d_j) kappa lip_h: no longer than a list with one skin
+// of twice the common reach. From then to the next rebuild no particle may move
+// further than that (ctl->reach_cap), which is less than what the other lists
+// allow for, so all of them hold every pair.
 // The list is built on FP32 views in both precisions. Lengths of the tests are
 // view integers; with w = kappa h / 2 (build_w) and m = max(w_i, w_j), 2 m is the
 // largest support of the pair and the larger of kappa h_i and kappa h_ij is w_i + m.
+template <bool CUT>
 struct ListTarget {
   float Rs, R2;          // search radius, view units
   float wi, di, c1, c2, u2, r2max;  // view integers
   int l0, l1;            // levels that can hold a neighbour
+  int most;              // CUT: the largest code
   __device__ __forceinline__ ListTarget(const Frame<float>& F, const Grid<float>& G, float kappa, int dmax,
                                         const int4& vi) {
+    most = F.code_u;
+    if (CUT) dmax = min(dmax, most);
     wi = build_w(vi);
-    di = build_reach(F, vi);
+    di = build_reach(F, vi, CUT ? most : 255);
     const float hv = wi * F.w2c, lip = G.lip_h, dv = di * F.vscale, dm = (float)dmax * F.skin_q * kappa;
     // search radius: bound h_j by Lipschitz continuity and d_j by the largest
     // reach of this build, iterate twice
@@ -878,6 +899,10 @@ struct ListTarget {
     c1 = 2.0f * 1.00001f;
     u2 = 2.0f * F.skin_q;
     r2max = R2 / (F.vscale * F.vscale);
+    if (CUT) c2 = kappa * lip;
+  }
+  __device__ __forceinline__ float code(const int4& v) const {
+    return (float)(CUT ? min(v.w & 0xFF, most) : v.w & 0xFF);
   }
   // a pair of candidates, without a branch: listed (acc), inside its support
   // now (density or force: the front of the list)
@@ -893,8 +918,11 @@ struct ListTarget {
     }
     // symmetric in i and j: j lists i whenever i lists j
     const float2 wj = make_float2(build_w(a), build_w(b)), m = make_float2(fmaxf(wi, wj.x), fmaxf(wi, wj.y));
-    const float2 dj = mul2(mul2(make_float2((float)(a.w & 0xFF), (float)(b.w & 0xFF)), both(u2)), wj);
-    const float2 rl = fma2(add2(both(di), dj), both(c2), mul2(both(c1), m)), rl2 = mul2(rl, rl), hp = add2(both(wi), m), hp2 = mul2(hp, hp);
+    const float2 dj = mul2(mul2(make_float2(code(a), code(b)), both(u2)), wj), d = add2(both(di), dj);
+    float2 rl = mul2(both(c1), m);
+    if (CUT) rl = add2(fma2(make_float2(fmaxf(di, dj.x), fmaxf(di, dj.y)), both(c2), rl), d);
+    else rl = fma2(d, both(c2), rl);
+    const float2 rl2 = mul2(rl, rl), hp = add2(both(wi), m), hp2 = mul2(hp, hp);
     acc[0] = r2.x < fminf(rl2.x, r2max);
     acc[1] = r2.y < fminf(rl2.y, r2max);
     inside[0] = r2.x < hp2.x;
@@ -960,144 +988,195 @@ struct RowWalk {
   }
 };
 
-// One thread per particle. REACH: certify the coarse FP32 test (kFastBit, read
-// by the FP64 path).
+// What a walk over the candidates found: entries accepted (cnt), written inside
+// and outside, the largest axis separation (REACH).
+struct ListCount {
+  int cnt, n_in, n_out;
+  float reach;
+};
+// One thread's list. REACH: certify the coarse FP32 test (kFastBit, read by the
+// FP64 path).
+template <int D, bool REACH, bool CUT>
+__device__ __forceinline__ ListCount walk_list(const Frame<float>& F, const Grid<float>& G, float kappa, int dmax,
+                                               const LL4& X, const int4& vi, const int4* __restrict__ view,
+                                               const uint32_t* __restrict__ meta,
+                                               const uint32_t* __restrict__ cstart, int cap,
+                                               uint32_t* __restrict__ own) {
+  const ListTarget<CUT> t(F, G, kappa, dmax, vi);
+  const int rows = list_rows(cap);
+  ListCount c{0, 0, 0, 0.0f};
+  // only the list store is conditional: most candidates fail, and a branch
+  // over the tests ran for a few lanes of the warp in nearly every iteration.
+  // Bound by issue slots (lanes of a warp have different rows and row lengths:
+  // 11 of 32 active); two candidates per instruction, with the lengths of the
+  // tests relative to w, take 31 % off a rebuild (8,388,608 particles in 3D:
+  // 1.48 -> 1.03 ms per step at a rebuild every four steps).
+  auto take = [&](int j, const int4& vj, bool acc, bool inside) {
+    if (!acc) return;
+    if (c.cnt < cap) {
+      const int row = inside ? c.n_in++ : rows - 1 - c.n_out++;
+      own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)j << 8) | (meta[j] & 0xFFu);
+    }
+    ++c.cnt;
+    if (REACH) c.reach = fmaxf(c.reach, t.template reach<D>(F, vi, vj));
+  };
+  for (int l = t.l0; l <= t.l1; ++l) {
+    const RowWalk<D> w(F, G, X, t.Rs, l);
+    for (int dz = w.zlo; dz <= w.zhi; ++dz) {
+      for (int dy = w.ylo; dy <= w.yhi; ++dy) {
+        int j, je;
+        if (!w.row(cstart, dz, dy, t.R2, j, je)) continue;
+        // candidates in ascending order, two at a time (an odd last one twice)
+        for (; j < je; j += 2) {
+          const bool two = j + 1 < je;
+          const int4 a = view[j], b = view[two ? j + 1 : j];
+          bool acc[2], inside[2];
+          t.template test<D>(vi, a, b, acc, inside);
+          take(j, a, acc[0], inside[0]);
+          take(j + 1, b, acc[1] && two, inside[1]);
+        }
+      }
+    }
+  }
+  return c;
+}
+// The same list made by a group of G lanes: lane g walks candidate rows g,
+// g + G, ... and the group's lanes test one candidate each at a time; accepted
+// ones take their places in lane order. cnt, n_in, n_out: uniform over the group.
+template <int D, int G, bool REACH, bool CUT>
+__device__ __forceinline__ ListCount walk_list_group(const Frame<float>& F, const Grid<float>& G32, float kappa,
+                                                     int dmax, const LL4& X, const int4& vi,
+                                                     const int4* __restrict__ view,
+                                                     const uint32_t* __restrict__ meta,
+                                                     const uint32_t* __restrict__ cstart, int cap,
+                                                     uint32_t* __restrict__ own) {
+  const unsigned group = group_mask<G>(), below = group & lanes_below();
+  const ListTarget<CUT> t(F, G32, kappa, dmax, vi);
+  const int rows = list_rows(cap);
+  ListCount c{0, 0, 0, 0.0f};
+  for (int l = t.l0; l <= t.l1; ++l) {
+    const RowWalk<D> w(F, G32, X, t.Rs, l);
+    const int ny = w.yhi - w.ylo + 1, nr = ny * (w.zhi - w.zlo + 1);
+    for (int r = threadIdx.x % G; __any_sync(group, r < nr); r += G) {
+      int j = 0, je = 0;
+      if (r < nr) w.row(cstart, w.zlo + r / ny, w.ylo + r % ny, t.R2, j, je);
+      for (; __any_sync(group, j < je); j += 2) {
+        bool acc[2] = {false, false}, inside[2] = {false, false};
+        if (j < je) {
+          const bool two = j + 1 < je;
+          const int4 a = view[j], b = view[two ? j + 1 : j];
+          t.template test<D>(vi, a, b, acc, inside);
+          acc[1] = acc[1] && two;
+          if (REACH && acc[0]) c.reach = fmaxf(c.reach, t.template reach<D>(F, vi, a));
+          if (REACH && acc[1]) c.reach = fmaxf(c.reach, t.template reach<D>(F, vi, b));
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          unsigned all = __ballot_sync(group, acc[q]), in = __ballot_sync(group, acc[q] && inside[q]);
+          c.cnt += __popc(all);
+          if (c.cnt > cap) {  // a full list keeps the first of them
+            for (int room = cap - c.n_in - c.n_out; __popc(all) > room;) all &= ~(1u << (31 - __clz(all)));
+            in &= all;
+          }
+          if (all >> (threadIdx.x & 31) & 1u) {
+            const int row = inside[q] ? c.n_in + __popc(in & below) : rows - 1 - (c.n_out + __popc(all & ~in & below));
+            own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)(j + q) << 8) | (meta[j + q] & 0xFFu);
+          }
+          c.n_in += __popc(in);
+          c.n_out += __popc(all & ~in);
+        }
+      }
+    }
+  }
+  for (int o = 1; o < G; o <<= 1) c.reach = fmaxf(c.reach, __shfl_xor_sync(group, c.reach, o));
+  return c;
+}
+__device__ __forceinline__ uint32_t list_counts(const ListCount& c, bool reach) {
+  return (uint32_t)c.n_in | ((uint32_t)c.n_out << kOutShift) |
+         (reach && ListTarget<false>::fast(c.reach) ? kFastBit : 0u);
+}
+// A list that did not fit, again at the common reach (G: lanes that make it). A
+// function of its own, called last and with nothing but the kernel's parameters:
+// it hardly ever runs, and neither its registers nor its arguments take any from
+// the walk.
+template <int D, int G, bool REACH>
+__device__ __noinline__ void cut_list(StepCtl* ctl, const LL4* X0, const LL4* X1, const uint32_t* m0,
+                                      const uint32_t* m1, const int4* view, const uint32_t* cstart,
+                                      const Frame<float>& F, const Grid<float>& Gr, float kappa, int cap,
+                                      uint32_t* list, uint32_t* lcount, int* err) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G, buf = ctl->buf;
+  const uint32_t* meta = buf ? m1 : m0;
+  const LL4 X = (buf ? X1 : X0)[i];
+  uint32_t* own = list + list_at(i, 0, cap);
+  ListCount c;
+  if constexpr (G == 1) c = walk_list<D, REACH, true>(F, Gr, kappa, ctl->dmax, X, view[i], view, meta, cstart, cap, own);
+  else c = walk_list_group<D, G, REACH, true>(F, Gr, kappa, ctl->dmax, X, view[i], view, meta, cstart, cap, own);
+  if (threadIdx.x % G != 0) return;
+  lcount[i] = list_counts(c, REACH);
+  atomicMin(&ctl->reach_cap, F.code_u);
+  atomicMax(&ctl->lmax, c.cnt);
+  if (c.cnt > cap) atomicOr(err, kErrListOverflow);
+}
+
+// One thread per particle.
 template <int D, bool REACH>
 __global__ void __launch_bounds__(256, SPH_LIST_MIN_BLOCKS) k_list_build(
     int n, StepCtl* __restrict__ ctl, const LL4* __restrict__ X0, const LL4* __restrict__ X1,
     const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1, const int4* __restrict__ view,
-    const uint32_t* __restrict__ cstart, Frame<float> F, Grid<float> G, float kappa, int cap,
-    uint32_t* __restrict__ list, uint32_t* __restrict__ lcount, int* __restrict__ err) {
+    const uint32_t* __restrict__ cstart, const __grid_constant__ Frame<float> F,
+    const __grid_constant__ Grid<float> G, float kappa, int cap, uint32_t* __restrict__ list,
+    uint32_t* __restrict__ lcount, int* __restrict__ err) {
   after_predecessor();
   if (!ctl->rebuild) return;
   const int buf = ctl->buf;
   const uint32_t* __restrict__ meta = buf ? m1 : m0;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int cnt = 0;  // accepted
+  int cnt = 0;
   if (i < n) {
     const LL4 X = (buf ? X1 : X0)[i];
-    const int4 vi = view[i];
-    const ListTarget t(F, G, kappa, ctl->dmax, vi);
-    int n_in = 0, n_out = 0;  // written inside / outside entries
-    const int rows = list_rows(cap);
-    uint32_t* __restrict__ own = list + list_at(i, 0, cap);
-    float reach = 0.0f;
-    // only the list store is conditional: most candidates fail, and a branch
-    // over the tests ran for a few lanes of the warp in nearly every iteration.
-    // Bound by issue slots (lanes of a warp have different rows and row lengths:
-    // 11 of 32 active); two candidates per instruction, with the lengths of the
-    // tests relative to w, take 31 % off a rebuild (8,388,608 particles in 3D:
-    // 1.48 -> 1.03 ms per step at a rebuild every four steps).
-    auto take = [&](int j, const int4& vj, bool acc, bool inside) {
-      if (!acc) return;
-      if (cnt < cap) {
-        const int row = inside ? n_in++ : rows - 1 - n_out++;
-        own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)j << 8) | (meta[j] & 0xFFu);
-      }
-      ++cnt;
-      if (REACH) reach = fmaxf(reach, t.reach<D>(F, vi, vj));
-    };
-    for (int l = t.l0; l <= t.l1; ++l) {
-      const RowWalk<D> w(F, G, X, t.Rs, l);
-      for (int dz = w.zlo; dz <= w.zhi; ++dz) {
-        for (int dy = w.ylo; dy <= w.yhi; ++dy) {
-          int j, je;
-          if (!w.row(cstart, dz, dy, t.R2, j, je)) continue;
-          // candidates in ascending order, two at a time (an odd last one twice)
-          for (; j < je; j += 2) {
-            const bool two = j + 1 < je;
-            const int4 a = view[j], b = view[two ? j + 1 : j];
-            bool acc[2], inside[2];
-            t.test<D>(vi, a, b, acc, inside);
-            take(j, a, acc[0], inside[0]);
-            take(j + 1, b, acc[1] && two, inside[1]);
-          }
-        }
-      }
-    }
-    lcount[i] = (uint32_t)n_in | ((uint32_t)n_out << kOutShift) | (REACH && ListTarget::fast(reach) ? kFastBit : 0u);
-    if (cnt > cap) atomicOr(err, kErrListOverflow);
+    const ListCount c = walk_list<D, REACH, false>(F, G, kappa, ctl->dmax, X, view[i], view, meta, cstart, cap,
+                                                   list + list_at(i, 0, cap));
+    lcount[i] = list_counts(c, REACH);
+    cnt = c.cnt;
   }
   // longest list of this build (one atomic per warp; every lane gets here)
-  const int wmax = __reduce_max_sync(0xffffffffu, cnt);
+  const int wmax = __reduce_max_sync(0xffffffffu, cnt <= cap ? cnt : 0);
   if ((threadIdx.x & 31) == 0 && wmax > 0) atomicMax(&ctl->lmax, wmax);
+  if (cnt > cap) cut_list<D, 1, REACH>(ctl, X0, X1, m0, m1, view, cstart, F, G, kappa, cap, list, lcount, err);
 }
 
-// The same lists with G lanes per particle: lane g walks candidate rows g,
-// g + G, ... and the group's lanes test one candidate each at a time; accepted
-// ones take their places in lane order. For particle counts that leave most of
-// the chip idle with one thread per particle, where one thread's chain of row
-// look-ups and candidate loads is the whole time (launch_rebuild).
+// G lanes per particle: for particle counts that leave most of the chip idle with
+// one thread per particle, where one thread's chain of row look-ups and candidate
+// loads is the whole time (launch_rebuild).
 template <int D, int G, bool REACH>
-__global__ void __launch_bounds__(256) k_list_build_group(int n, StepCtl* __restrict__ ctl,
-                                                          const LL4* __restrict__ X0, const LL4* __restrict__ X1,
-                                                          const uint32_t* __restrict__ m0,
-                                                          const uint32_t* __restrict__ m1,
-                                                          const int4* __restrict__ view,
-                                                          const uint32_t* __restrict__ cstart, Frame<float> F,
-                                                          Grid<float> G32, float kappa, int cap,
-                                                          uint32_t* __restrict__ list, uint32_t* __restrict__ lcount,
-                                                          int* __restrict__ err) {
+__global__ void __launch_bounds__(256) k_list_build_group(
+    int n, StepCtl* __restrict__ ctl, const LL4* __restrict__ X0, const LL4* __restrict__ X1,
+    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1, const int4* __restrict__ view,
+    const uint32_t* __restrict__ cstart, const __grid_constant__ Frame<float> F,
+    const __grid_constant__ Grid<float> G32, float kappa, int cap, uint32_t* __restrict__ list,
+    uint32_t* __restrict__ lcount, int* __restrict__ err) {
   __shared__ int longest;
   after_predecessor();
   if (!ctl->rebuild) return;
   if (threadIdx.x == 0) longest = 0;
   __syncthreads();
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G, g = threadIdx.x % G;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+  int cnt = 0;
   if (i < n) {  // whole groups
-    const unsigned group = group_mask<G>(), below = group & lanes_below();
     const int buf = ctl->buf;
     const uint32_t* __restrict__ meta = buf ? m1 : m0;
     const LL4 X = (buf ? X1 : X0)[i];
-    const int4 vi = view[i];
-    const ListTarget t(F, G32, kappa, ctl->dmax, vi);
-    const int rows = list_rows(cap);
-    uint32_t* __restrict__ own = list + list_at(i, 0, cap);
-    int n_in = 0, n_out = 0, cnt = 0;  // written inside / outside entries, accepted: uniform over the group
-    float reach = 0.0f;
-    for (int l = t.l0; l <= t.l1; ++l) {
-      const RowWalk<D> w(F, G32, X, t.Rs, l);
-      const int ny = w.yhi - w.ylo + 1, nr = ny * (w.zhi - w.zlo + 1);
-      for (int r = g; __any_sync(group, r < nr); r += G) {
-        int j = 0, je = 0;
-        if (r < nr) w.row(cstart, w.zlo + r / ny, w.ylo + r % ny, t.R2, j, je);
-        for (; __any_sync(group, j < je); j += 2) {
-          bool acc[2] = {false, false}, inside[2] = {false, false};
-          if (j < je) {
-            const bool two = j + 1 < je;
-            const int4 a = view[j], b = view[two ? j + 1 : j];
-            t.test<D>(vi, a, b, acc, inside);
-            acc[1] = acc[1] && two;
-            if (REACH && acc[0]) reach = fmaxf(reach, t.reach<D>(F, vi, a));
-            if (REACH && acc[1]) reach = fmaxf(reach, t.reach<D>(F, vi, b));
-          }
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            unsigned all = __ballot_sync(group, acc[q]), in = __ballot_sync(group, acc[q] && inside[q]);
-            cnt += __popc(all);
-            if (cnt > cap) {  // a full list keeps the first of them
-              for (int room = cap - n_in - n_out; __popc(all) > room;) all &= ~(1u << (31 - __clz(all)));
-              in &= all;
-            }
-            if (all >> (threadIdx.x & 31) & 1u) {
-              const int row = inside[q] ? n_in + __popc(in & below) : rows - 1 - (n_out + __popc(all & ~in & below));
-              own[(size_t)(row >> 2) * 128 + (row & 3)] = ((uint32_t)(j + q) << 8) | (meta[j + q] & 0xFFu);
-            }
-            n_in += __popc(in);
-            n_out += __popc(all & ~in);
-          }
-        }
-      }
-    }
-    for (int o = 1; o < G; o <<= 1) reach = fmaxf(reach, __shfl_xor_sync(group, reach, o));
-    if (g == 0) {
-      lcount[i] = (uint32_t)n_in | ((uint32_t)n_out << kOutShift) | (REACH && ListTarget::fast(reach) ? kFastBit : 0u);
-      if (cnt > cap) atomicOr(err, kErrListOverflow);
-      atomicMax(&longest, cnt);
+    const ListCount c = walk_list_group<D, G, REACH, false>(F, G32, kappa, ctl->dmax, X, view[i], view, meta, cstart,
+                                                            cap, list + list_at(i, 0, cap));
+    cnt = c.cnt;
+    if (threadIdx.x % G == 0) {
+      lcount[i] = list_counts(c, REACH);
+      if (cnt <= cap) atomicMax(&longest, cnt);
     }
   }
   __syncthreads();
   if (threadIdx.x == 0 && longest > 0) atomicMax(&ctl->lmax, longest);
+  if (cnt > cap) cut_list<D, G, REACH>(ctl, X0, X1, m0, m1, view, cstart, F, G32, kappa, cap, list, lcount, err);
 }
 
 // Staged pass A, set up at a list rebuild: one block per kStageBlock targets
@@ -1955,8 +2034,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       const T ex = vd(F, vn.x, vb.x), ey = vd(F, vn.y, vb.y);
       const T ez = D == 3 ? vd(F, vn.z, vb.z) : T(0);
       T lim;  // the reach, view units
-      if constexpr (std::is_same<T, float>::value) lim = build_reach(F, vb) * F.vscale;
-      else lim = vb.w;
+      const int most = ctl->reach_cap;
+      if constexpr (std::is_same<T, float>::value) lim = build_reach(F, vb, most) * F.vscale;
+      else lim = coded_reach(vb.w, most);
       far = (ex * ex + ey * ey + ez * ez) >= lim * lim;
     } else {
       (vp ? w0 : w1)[i] = vi;
