@@ -353,8 +353,10 @@ sph_status sph_load(sph_handle* h, const void* buf, size_t nbytes);
  *
  * Memory: the run keeps the positions (FP64, by particle id) at the start of
  * every segment of ckpt_every steps and re-runs each segment from there into a
- * tape of ckpt_every steps (each step's state, a, a~, rho and force pairs:
- * roughly 100 + 4 * list_capacity bytes per particle) just before reversing it.
+ * tape of ckpt_every steps (each step's state, a, a~, rho and the list words of
+ * its force pairs: 100 (FP32) or 156 (FP64) + 4 * list_capacity bytes per
+ * particle, with gamma != 2 another 4 + 4 * list_capacity for the neighbour list)
+ * just before reversing it.
  * Checkpoints, tape and five n-sized reverse-pass arrays are allocated once
  * through the handle's allocator (grown when K or ckpt_every grows) and kept
  * until sph_destroy.

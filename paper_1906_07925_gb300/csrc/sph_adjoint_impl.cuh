@@ -267,7 +267,7 @@ template <int D, class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n, const StepCtl* __restrict__ ctl,
                                                   const typename ViewOf<T>::type* __restrict__ v0,
                                                   const typename ViewOf<T>::type* __restrict__ v1,
-                                                  const PairRec<T>* __restrict__ plist,
+                                                  const uint32_t* __restrict__ words,
                                                   const uint32_t* __restrict__ pcount, int cap,
                                                   const V4<T>* __restrict__ acc, const Scalars* __restrict__ scal,
                                                   Frame<T> F, Phys<T> P, int recomputed_dt, AdjBufs<T> B) {
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_bwd_visc(int n,
     struct Rec {
       V4<T> a, atb;
     };
-    for_pairs_x(plist, view, i, cnt, cap, [&](int j) { return Rec{acc[j], B.atb[j]}; },
+    for_pairs_x(words, view, i, cnt, cap, [&](int j) { return Rec{acc[j], B.atb[j]}; },
                [&](uint32_t e, const VT& vj, const Rec& rj) {
       const int j = (int)(e >> 8);
       const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? SPH_BWD_FORCE_MIN_BLOCKS
                                                    const typename ViewOf<T>::type* __restrict__ v0,
                                                    const typename ViewOf<T>::type* __restrict__ v1,
                                                    const uint32_t* __restrict__ m0, const uint32_t* __restrict__ m1,
-                                                   const PairRec<T>* __restrict__ plist,
+                                                   const uint32_t* __restrict__ words,
                                                    const uint32_t* __restrict__ pcount, int cap,
                                                    const T* __restrict__ rho, const T* __restrict__ pc,
                                                    const Scalars* __restrict__ scal, Frame<T> F, Phys<T> P,
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? SPH_BWD_FORCE_MIN_BLOCKS
     T xx = 0, xy = 0, xz = 0, hbar = 0, Tbar = 0, Qbar = 0;
     T sb = 0, pb = 0;
     const int cnt = (int)pcount[i];
-    for_pairs_x(plist, view, i, cnt, cap, [&](int j) { return B.ab[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& abj) {
+    for_pairs_x(words, view, i, cnt, cap, [&](int j) { return B.ab[j]; }, [&](uint32_t e, const VT& vj, const V4<T>& abj) {
       const int j = (int)(e >> 8);
       const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
       const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
@@ -801,13 +801,13 @@ cudaError_t launch_bwd_step(const DevState& S, const Frame<T>& F, const Phys<T>&
   const V4<T>* acc = (const V4<T>*)S.acc4;
   k_bwd_out<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, (const LL4*)S.X[0], (const LL4*)S.X[1], S.pid[0], S.pid[1], acc,
                                      (const V4<T>*)S.visc, S.scal, F, geo, B);
-  k_bwd_visc<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, (const PairRec<T>*)S.plist, S.pcount, S.cap, acc, S.scal, F, P, recomputed_dt, B);
+  k_bwd_visc<D, T><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.words, S.pcount, S.cap, acc, S.scal, F, P, recomputed_dt, B);
   if (general_eos)
-    k_bwd_force<D, T, true><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], (const PairRec<T>*)S.plist, S.pcount, S.cap,
+    k_bwd_force<D, T, true><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], S.words, S.pcount, S.cap,
                                                (const T*)S.rho, (const T*)S.pc, S.scal, F, P, (const LL4*)S.X[0],
                                                (const LL4*)S.X[1], S.pid[0], S.pid[1], geo, B);
   else  // the gamma = 2 form has no density adjoint: the target-field step is fused in
-    k_bwd_force<D, T, false><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], (const PairRec<T>*)S.plist, S.pcount, S.cap,
+    k_bwd_force<D, T, false><<<gb, tb, 0, st>>>(S.n, S.ctl, w0, w1, S.meta[0], S.meta[1], S.words, S.pcount, S.cap,
                                                 (const T*)S.rho, (const T*)S.pc, S.scal, F, P, (const LL4*)S.X[0],
                                                 (const LL4*)S.X[1], S.pid[0], S.pid[1], geo, B);
   if (general_eos)

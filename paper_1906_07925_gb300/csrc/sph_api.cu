@@ -207,6 +207,7 @@ sph_status launch_step(sph_handle* h, int record, int force_rebuild = 0, cudaEve
   f.record = record;
   f.dt_fix = dt_fix;
   f.dt_rec = dt_rec;
+  f.words = tape ? tape->words : nullptr;
   const bool f64 = h->prec == SPH_PREC_FP64;
   f.geo = f64 ? (const void*)&h->geod : (const void*)&h->geof;
   f.surface = h->has_surface ? 1 : 0;
@@ -572,7 +573,9 @@ sph_status run_bwd_step(sph_handle* h, const DevState& S, const double* gin, dou
 }
 
 // Per-step record of a taped step: the state pass A used (current order), the
-// step's forward results (a, g, a~, rho, p/rho^2, this step's force pairs),
+// step's forward results (a, g, a~, rho, p/rho^2, the list words of its force
+// pairs: what pass A leaves to pass B beside them, 8 or 16 bytes a pair, the
+// reverse pass does not read),
 // its control block and scalars, and with a general EOS its neighbour list.
 // Slots are allocated once (through the handle's allocator) and reused.
 sph_status ensure_tape(sph_handle* h, int slots) {
@@ -587,7 +590,7 @@ sph_status ensure_tape(sph_handle* h, int slots) {
     SPH_TRY(grab(h, T.meta[0], N)); T.meta[1] = T.meta[0];
     SPH_TRY(grab(h, T.pid[0], N)); T.pid[1] = T.pid[0];
     SPH_TRY(grab(h, p, N * v4)); T.view[0] = T.view[1] = p;
-    SPH_TRY(grab(h, p, pair_bytes(N, h->S.cap, h->S.fp64))); T.plist = p;
+    SPH_TRY(grab(h, T.words, (N + 31) / 32 * 32 * (size_t)h->S.cap));
     SPH_TRY(grab(h, T.pcount, N));
     SPH_TRY(grab(h, p, N * v4)); T.acc4 = p;
     SPH_TRY(grab(h, p, N * v4)); T.visc = p;
@@ -628,7 +631,6 @@ sph_status capture(sph_handle* h, cudaGraphExec_t* out, Body&& body) {
 // one step writing its forward results into tape slot T (and the state into it)
 sph_status taped_step(sph_handle* h, const DevState& T, const double* dt_fix, double* dt_rec) {
   DevState S2 = h->S;
-  S2.plist = T.plist;
   S2.pcount = T.pcount;
   S2.acc4 = T.acc4;
   S2.visc = T.visc;

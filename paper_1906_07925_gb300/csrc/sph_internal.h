@@ -32,6 +32,7 @@ struct DevState {
   uint32_t* list = nullptr;              // skin lists, entries (j << 8 | colour_j), see list_at
   uint32_t* lcount = nullptr;            // entries per particle; bit 31: FP32 coarse test exact
   void* plist = nullptr;                 // the force pairs of the current step (PairRec, pass A -> B), see pair_at
+  uint32_t* words = nullptr;             // tape slot: the list words of its step's force pairs, see pair_at
   // staged pass A (FP32, 256-thread pair passes): per 256-target block its
   // distinct neighbours sj (kStageCap per block), their count scount (-1: not
   // staged) and the list again with ranks in that set (llist, as list)
@@ -156,6 +157,7 @@ struct PassFlags {
   int nbr_debug = 0;    // write neighbour-set sizes and id sums by particle id
   int advance = 1;      // count this pass as a step (sigma schedule, counter)
   int move = 1;         // pass B: integrate (0: only a~, for the reverse pass)
+  uint32_t* words = nullptr;  // pass B: a taped step's list words of the force pairs (DevState::words)
   const double* dt_fix = nullptr;  // pass A: prescribed {dt1, dt2} (device)
   double* dt_rec = nullptr;        // pass A: record {dt1, dt2} (device)
   const void* geo = nullptr;       // pass A: the Geom<T> of the handle (feature-surface normals)

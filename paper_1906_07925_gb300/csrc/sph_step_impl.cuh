@@ -157,17 +157,17 @@ __device__ __forceinline__ V4<double> make_view(const Frame<double>& F, const LL
 // 2 x SPH_LIST_BATCH_X independent gathers in flight instead of meeting the
 // record's latency inside every pair body. Words are streamed (read once), the
 // next batch's loaded before this one's arithmetic.
-template <class T, class VT, class Fetch, class Fn>
-__device__ __forceinline__ void for_pairs_x(const PairRec<T>* __restrict__ plist, const VT* __restrict__ view, int i,
+template <class VT, class Fetch, class Fn>
+__device__ __forceinline__ void for_pairs_x(const uint32_t* __restrict__ words, const VT* __restrict__ view, int i,
                                             int cnt, int cap, Fetch&& fetch, Fn&& pair) {
   using XT = decltype(fetch(0));
   constexpr int B = SPH_LIST_BATCH_X;
-  const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
+  const uint32_t* __restrict__ p = words + pair_at(i, 0, cap);
   int k = 0;
   uint32_t ahead[B];
   if (cnt >= B)
 #pragma unroll
-    for (int q = 0; q < B; ++q) ahead[q] = __ldcs(&p[32 * q].e);
+    for (int q = 0; q < B; ++q) ahead[q] = __ldcs(p + 32 * q);
   for (; k + B <= cnt; k += B) {
     uint32_t e[B];
     VT v[B];
@@ -182,12 +182,12 @@ __device__ __forceinline__ void for_pairs_x(const PairRec<T>* __restrict__ plist
     p += 32 * B;
     if (k + 2 * B <= cnt)
 #pragma unroll
-      for (int q = 0; q < B; ++q) ahead[q] = __ldcs(&p[32 * q].e);
+      for (int q = 0; q < B; ++q) ahead[q] = __ldcs(p + 32 * q);
 #pragma unroll
     for (int q = 0; q < B; ++q) pair(e[q], v[q], x[q]);
   }
   for (; k < cnt; ++k, p += 32) {
-    const uint32_t e = __ldcs(&p->e);
+    const uint32_t e = __ldcs(p);
     pair(e, view[e >> 8], fetch((int)(e >> 8)));
   }
 }
@@ -1814,8 +1814,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
 // Bound by the gather of the neighbour's acceleration, one per force pair: the
 // pair's geometry factor comes from pass A's record (8,388,608 particles in 3D,
 // FP32: 1.40 -> 0.77 ms with 128-thread blocks; 300,007 in FP64: 1.40 -> 0.43).
+// TAPE: a step of the reverse pass's tape also keeps the pairs' list words (a
+// kernel of its own that took them out of the records added 13 us to a step of
+// 262,144 particles in 2D).
 // --------------------------------------------------------------------------
-template <int D, class T, int NT, int G = 1>
+template <int D, class T, int NT, int G = 1, bool TAPE = false>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP64 : SPH_PASSB_MIN_BLOCKS) * 256 / NT) k_pass_b(int n, StepCtl* __restrict__ ctl,
                                                 const typename ViewOf<T>::type* __restrict__ v0,
                                                 const typename ViewOf<T>::type* __restrict__ v1,
@@ -1830,7 +1833,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
                                                 int* __restrict__ err, unsigned long long* __restrict__ wall_moved,
                                                 int move, const uint32_t* __restrict__ m0,
                                                 const uint32_t* __restrict__ m1, int4* __restrict__ v32out,
-                                                int sv32, float c2w32) {
+                                                int sv32, float c2w32, uint32_t* __restrict__ words) {
   using VT = typename ViewOf<T>::type;
   __shared__ int moved_sm[NT / 32];
   // G lanes per particle, as pass A
@@ -1851,6 +1854,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
     // FP64 pipe bounds both passes, 300,007 in 3D: 1.40 -> 0.43 ms.
     const int cnt = lead ? (int)pcount[i] : 0;
     const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
+    // TAPE: after the gathers of the same pairs are on their way, so that it waits
+    // for nothing of its own
+    const auto keep = [&](const PairRec<T>* q, const PairRec<T>& r) {
+      if (TAPE) __stcs(words + (q - plist), r.e);
+    };
     if constexpr (std::is_same<T, float>::value) {
       // two pairs per instruction; sums of (a_j - a_i), factor gi gj / (gi + gj)
       const float2 g2 = both(ai.w), nx2 = both(-ai.x), ny2 = both(-ai.y), nz2 = both(-ai.z);
@@ -1872,6 +1880,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
           PairRec<T> r1{r0.e, 0.0f};
           if (k + 1 < cnt) r1 = load_pair(p + 32);
           const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
+          keep(p, r0);
+          if (k + 1 < cnt) keep(p + 32, r1);
           two(r0, a0, r1, a1);
         }
         __syncwarp();
@@ -1891,6 +1901,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         if (k + 2 * B <= cnt)
 #pragma unroll
           for (int q = 0; q < B; ++q) ahead[q] = load_pair(p + 32 * q);
+        if (TAPE)
+#pragma unroll
+          for (int q = 0; q < B; ++q) keep(p + 32 * q - 32 * B, r[q]);
 #pragma unroll
         for (int q = 0; q < B; q += 2) two(r[q], a[q], r[q + 1], a[q + 1]);
       }
@@ -1900,6 +1913,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         PairRec<T> r1{r0.e, 0.0f};  // no second pair: a zero factor
         if (k + 1 < cnt) r1 = load_pair(p + 32);
         const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
+        keep(p, r0);
+        if (k + 1 < cnt) keep(p + 32, r1);
         two(r0, a0, r1, a1);
       }
       }
@@ -1918,7 +1933,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       if constexpr (G > 1) {
         for (k = threadIdx.x % G, p += 32 * k; k < cnt; k += G, p += 32 * G) {
           const PairRec<T> r0 = load_pair(p);
-          pair(r0, acc[r0.e >> 8]);
+          const V4<T> a0 = acc[r0.e >> 8];
+          keep(p, r0);
+          pair(r0, a0);
         }
         __syncwarp();
       }
@@ -1927,6 +1944,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
         PairRec<T> r1{T(0), r0.e, 0u};
         if (k + 1 < cnt) r1 = load_pair(p + 32);
         const V4<T> a0 = acc[r0.e >> 8], a1 = acc[r1.e >> 8];
+        keep(p, r0);
+        if (k + 1 < cnt) keep(p + 32, r1);
         pair(r0, a0);
         if (k + 1 < cnt) pair(r1, a1);
       }
@@ -2254,18 +2273,27 @@ cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P
         (LL4*)S.X[0], (LL4*)S.X[1], (const PairRec<T>*)S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
         f.record ? (V4<T>*)S.visc : nullptr, S.err, wm, f.move, S.meta[0], S.meta[1],
         (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0,
-        f.f32 ? f.f32->c2w : 0.0f);
+        f.f32 ? f.f32->c2w : 0.0f, f.words);
     return cudaGetLastError();
   };
+  // threads per block and lanes per particle, taped or not
+  auto pick = [&](auto nt, auto lanes) {
+    constexpr int NT = decltype(nt)::value, G = decltype(lanes)::value;
+    return f.words ? run(k_pass_b<D, T, NT, G, true>, NT, G) : run(k_pass_b<D, T, NT, G>, NT, G);
+  };
+  using one = std::integral_constant<int, 1>;
   if constexpr (std::is_same<T, float>::value) {
-    if (S.n <= kPassGroupMax) return run(k_pass_b<D, T, 32 * kPassLanes, kPassLanes>, 32 * kPassLanes, kPassLanes);
+    if (S.n <= kPassGroupMax)
+      return pick(std::integral_constant<int, 32 * kPassLanes>{}, std::integral_constant<int, kPassLanes>{});
     // large runs in small blocks, whose warps wait for no one else's tail
     // (8,388,608 particles in 3D 873 -> 805 us, 1,048,576 in 2D 71 -> 69; at
     // 240,370 in 3D 31 -> 33)
-    return S.pass_threads == 128 || S.n >= (1 << 19) ? run(k_pass_b<D, T, 128>, 128, 1) : run(k_pass_b<D, T, 256>, 256, 1);
+    if (S.pass_threads == 128 || S.n >= (1 << 19)) return pick(std::integral_constant<int, 128>{}, one{});
+    return pick(std::integral_constant<int, 256>{}, one{});
   } else {
-    if (fp64_lanes(S) > 1) return run(k_pass_b<D, T, 32 * kLanes64, kLanes64>, 32 * kLanes64, kLanes64);
-    return fp64_threads(S) == 32 ? run(k_pass_b<D, T, 32>, 32, 1) : run(k_pass_b<D, T, 64>, 64, 1);
+    if (fp64_lanes(S) > 1) return pick(std::integral_constant<int, 32 * kLanes64>{}, std::integral_constant<int, kLanes64>{});
+    if (fp64_threads(S) == 32) return pick(std::integral_constant<int, 32>{}, one{});
+    return pick(std::integral_constant<int, 64>{}, one{});
   }
 }
 
