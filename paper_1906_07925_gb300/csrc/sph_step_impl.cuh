@@ -1495,7 +1495,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     T qi = inv_rho_t2<D, T>(hv, inv_tau_v);  // 1/rho_t,i^2
     const T Pi = GENERAL ? pc[i] : P.P0 * qi;
     const T sP0 = sigma * P.P0;
-    const T half_kappa = T(0.5) * P.kappa;
+    [[maybe_unused]] const T half_kappa = T(0.5) * P.kappa;
     T dsum = 0, ax = 0, ay = 0, az = 0;
     int nf = 0, ni = 0, nd = 0;
     long long sd = 0, sf = 0;
@@ -1610,11 +1610,26 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       const int j = (int)(e >> 8);
       const T dx = vd(F, vi.x, vj.x), dy = vd(F, vi.y, vj.y);
       const T dz = D == 3 ? vd(F, vi.z, vj.z) : T(0);
-      const T r2 = dx * dx + dy * dy + dz * dz;
       const T hj = view_h(F, vj);
-      const T Hf = half_kappa * (hv + hj);
-      const bool inD = !GENERAL && r2 < Hd2;
-      const bool inF = r2 < Hf * Hf && j != i && (!surf || (meta[j] & kSurfaceBit));
+      T r2, Hf;
+      bool inD, inF;
+      if constexpr (std::is_same<T, float>::value) {
+        // the tests of the packed path, rounding for rounding (there in view
+        // integers: a power of two apart), so that diagnostics name its pairs
+        const float H = (view_w(vi) + view_w(vj)) * F.vscale, w = view_w(vi) * F.vscale;
+        r2 = fmaf(dy, dy, __fmul_rn(dx, dx));
+        if (D == 3) r2 = fmaf(dz, dz, r2);
+        Hf = H;
+        inD = r2 < __fmul_rn(4.0f * w, w);
+        inF = r2 < __fmul_rn(H, H);
+      } else {
+        r2 = dx * dx + dy * dy + dz * dz;
+        Hf = half_kappa * (hv + hj);
+        inD = r2 < Hd2;
+        inF = r2 < Hf * Hf;
+      }
+      inD = inD && !GENERAL;
+      inF = inF && j != i && (!surf || (meta[j] & kSurfaceBit));
       if (!(inD || inF)) return;
       const T r = r2 > T(0) ? pair_r<T>(r2) : T(0);
       if (inD) {
