@@ -419,7 +419,8 @@ __device__ __forceinline__ void argmin_merge(double& v, long long& k, double ov,
 // that pipe was active 58 % of a 2D pass A and 39 % of a 3D one. So the
 // reductions compare FP32 values, turn to FP64 only when those tie, and add in
 // fixed point. 10 steps of 1,048,576 particles in 2D: 3.14 -> 2.29 ms; 5 steps
-// of 8,388,608 in 3D: 25.2 -> 23.8 ms; results unchanged bit for bit.
+// of 8,388,608 in 3D: 25.2 -> 23.8 ms; positions and step sizes unchanged bit for
+// bit, the sums of the statistics nearer to their exact values.
 // r_c / |a| (FP32, correctly rounded: monotone in the exact quotient); is a
 // before b, ties by the exact quotient (products of two floats are exact in
 // FP64), then by index
@@ -597,13 +598,18 @@ struct WarpSums {
   int ni, nf, cnt;
 };
 
-// rho/rho_t - 1 = q1 + q2 by a two-float quotient (about 46 bits of the result)
-__device__ __forceinline__ void density_error(float rho, float rt, float& q1, float& q2) {
+// rho/rho_t - 1 = q1 + q2 + q3, a quotient by long division in three floats (each
+// remainder exact or carried with its rounding error): about 2^-68 of itself, so
+// that its square keeps more than an FP64 division would give
+__device__ __forceinline__ void density_error(float rho, float rt, float& q1, float& q2, float& q3) {
   const float dh = rho - rt, bb = dh - rho;
-  const float dl = (rho - (dh - bb)) - (rt + bb);
+  const float dl = (rho - (dh - bb)) - (rt + bb);  // rho - rt = dh + dl
   const float ri = __frcp_rn(rt);
   q1 = dh * ri;
-  q2 = (fmaf(-q1, rt, dh) + dl) * ri;
+  q1 = fmaf(fmaf(-q1, rt, dh), ri, q1);  // to the nearest, so that the next remainder is exact
+  const float r = fmaf(-q1, rt, dh), s = r + dl, sb = s - r, sl = (r - (s - sb)) + (dl - sb);
+  q2 = s * ri;
+  q3 = (fmaf(-q2, rt, s) + sl) * ri;
 }
 
 // every lane of the warp calls; active: this lane holds a particle. Lane 0
@@ -620,8 +626,8 @@ __device__ __forceinline__ void warp_sums(bool active, int i, float rc, float an
   // the largest |a| (NaN, which raises the error word, counts as none)
   const unsigned amax = __reduce_max_sync(all, moves ? __float_as_uint(an) : 0u);
   // the largest |rho / rho_t - 1|
-  float q1 = 0.0f, q2 = 0.0f;
-  if (active) density_error(rho, rt, q1, q2);
+  float q1 = 0.0f, q2 = 0.0f, q3 = 0.0f;
+  if (active) density_error(rho, rt, q1, q2, q3);
   const int worst = largest_error(active ? fabsf(q1) : -1.0f, rho, rt), wl = worst < 0 ? 0 : worst;
   const float er = __shfl_sync(all, rho, wl), et = __shfl_sync(all, rt, wl);
   const float emax = fabsf(__shfl_sync(all, q1, wl));
@@ -631,14 +637,15 @@ __device__ __forceinline__ void warp_sums(bool active, int i, float rc, float an
   float v = rv * exponent_scale(re);
   int rl[3], el[3];
   for (int k = 0; k < 3; ++k) rl[k] = __reduce_add_sync(all, take_limb(v));
-  // sum (rho/rho_t - 1)^2 = p + pl
-  const float p = q1 * q1, pl = fmaf(q1, q1, -p) + 2.0f * q1 * q2;
+  // sum (rho/rho_t - 1)^2: q1^2 = p + pl and 2 q1 q2 = c + cl exactly, and the rest
+  const float p = q1 * q1, pl = fmaf(q1, q1, -p), d1 = 2.0f * q1, c = d1 * q2;
+  const float cl = fmaf(q2, q2, fmaf(d1, q3, fmaf(d1, q2, -c)));
   const int ee = fixed_exponent(emax * emax * 1.00001f);  // the largest to rounding
-  const float es = exponent_scale(ee);
-  float a = p * es, b = pl * es * 4194304.0f;
+  const float es = exponent_scale(ee), limb = 4194304.0f;
+  float a = p * es, b = pl * es * limb, bc = c * es * limb, br = cl * es * limb * limb;
   el[0] = take_limb(a);
-  el[1] = take_limb(a) + take_limb(b);
-  el[2] = take_limb(a) + take_limb(b);
+  el[1] = take_limb(a) + take_limb(b) + take_limb(bc);
+  el[2] = take_limb(a) + take_limb(b) + take_limb(bc) + take_limb(br);
   for (int k = 0; k < 3; ++k) el[k] = __reduce_add_sync(all, el[k]);
   ni = __reduce_add_sync(all, ni);
   nf = __reduce_add_sync(all, nf);
