@@ -221,10 +221,8 @@ inline void make_frames(const sph_domain& dom, double kappa, double skin, bool a
   out.f.mbits = bits;
   out.f.mbias = bias;
   out.f.vscale = (float)std::ldexp(1.0, -kViewBits);
-  const double c2w = 0.5 * kappa * std::ldexp(1.0, kViewBits);
-  out.f.c2w = (float)c2w;
-  out.f.h2w = (float)(c2w / c0);
-  out.f.w2c = (float)(1.0 / c2w);
+  out.f.h2w = std::ldexp((float)(1.0 / c0), kViewBits);
+  out.f.half_kappa = out.d.half_kappa = 0.5f * (float)kappa;
   convert_grid<float>(hg, c0, out.gf);
   convert_grid<double>(hg, c0, out.gd);
 }

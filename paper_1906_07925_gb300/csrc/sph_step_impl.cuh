@@ -83,11 +83,11 @@ template <class T>
 __device__ __forceinline__ T screen_radius(T H) {
   return H * T(1.0 + 1.0 / (1 << 20)) + T(1.0 / (1 << (kCoarseBits - 2)));
 }
-// w of a view: FP32 kappa h / 2 in view integers (the support of a pair is the
-// sum of the two w), FP64 h in view units; view_h: h in view units
+// w of a view: FP32 h in view integers, FP64 h in view units; view_h: h in view
+// units (FP32: the view's own rounding and a power of two, no rounding more)
 __device__ __forceinline__ float view_w(const int4& v) { return __int_as_float(v.w); }
 __device__ __forceinline__ double view_w(const V4<double>& v) { return v.w; }
-__device__ __forceinline__ float view_h(const Frame<float>& F, const int4& v) { return __int_as_float(v.w) * F.w2c; }
+__device__ __forceinline__ float view_h(const Frame<float>& F, const int4& v) { return __int_as_float(v.w) * F.vscale; }
 __device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>& v) { return v.w; }
 
 // The build view of a particle (vbuild; FP64 path: view32 until pass B renews it):
@@ -95,7 +95,7 @@ __device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>&
 // reach code in the low byte. The reach, in view integers:
 __device__ __forceinline__ float build_w(int4 v) { return __int_as_float(v.w & ~0xFF); }
 __device__ __forceinline__ float build_reach(const Frame<float>& F, int4 v, int most = 255) {
-  return (float)min(v.w & 0xFF, most) * (2.0f * F.skin_q) * build_w(v);
+  return (float)min(v.w & 0xFF, most) * (2.0f * F.skin_q * F.half_kappa) * build_w(v);
 }
 // FP64 path: pass B reads the reach itself (view units) with its code in the low
 // byte, where a float's mantissa leaves zeros
@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(256) k_gather_view(
     most = max(most, code);
     if constexpr (std::is_same<T, double>::value) {
       const long long half = 1LL << (F32.sv - 1);
-      const int w = ((__float_as_int((float)view_w(v) * F32.c2w) + 0xFF) & ~0xFF) | code;
+      const int w = ((__float_as_int((float)view_w(v) * (float)(1 << kViewBits)) + 0xFF) & ~0xFF) | code;
       const int4 u = make_int4((int)((X.x + half) >> F32.sv), (int)((X.y + half) >> F32.sv),
                                D == 3 ? (int)((X.z + half) >> F32.sv) : 0, w);
       v32[d] = u;
@@ -875,12 +875,12 @@ __global__ void __launch_bounds__(256) k_gather_view(
 // further than that (ctl->reach_cap), which is less than what the other lists
 // allow for, so all of them hold every pair.
 // The list is built on FP32 views in both precisions. Lengths of the tests are
-// view integers; with w = kappa h / 2 (build_w) and m = max(w_i, w_j), 2 m is the
-// largest support of the pair and the larger of kappa h_i and kappa h_ij is w_i + m.
+// view integers; with w = h (build_w) and m = max(w_i, w_j), kappa m is the largest
+// support of the pair and the larger of kappa h_i and kappa h_ij is kappa (w_i + m) / 2.
 template <bool CUT>
 struct ListTarget {
   float Rs, R2;          // search radius, view units
-  float wi, di, c1, c2, u2, r2max;  // view integers
+  float wi, di, c1, c2, u2, hk, hi, r2max;  // view integers
   int l0, l1;            // levels that can hold a neighbour
   int most;              // CUT: the largest code
   __device__ __forceinline__ ListTarget(const Frame<float>& F, const Grid<float>& G, float kappa, int dmax,
@@ -889,7 +889,9 @@ struct ListTarget {
     if (CUT) dmax = min(dmax, most);
     wi = build_w(vi);
     di = build_reach(F, vi, CUT ? most : 255);
-    const float hv = wi * F.w2c, lip = G.lip_h, dv = di * F.vscale, dm = (float)dmax * F.skin_q * kappa;
+    hk = F.half_kappa;
+    hi = hk * wi;
+    const float hv = wi * F.vscale, lip = G.lip_h, dv = di * F.vscale, dm = (float)dmax * F.skin_q * kappa;
     // search radius: bound h_j by Lipschitz continuity and d_j by the largest
     // reach of this build, iterate twice
     float hhi = hv;
@@ -903,8 +905,8 @@ struct ListTarget {
     l0 = level_of_h(G, (hv * 0.9999f - lip * Rs) * F.qv);
     l1 = level_of_h(G, hhi * F.qv);
     R2 = Rs * Rs;
-    c1 = 2.0f * 1.00001f;
-    u2 = 2.0f * F.skin_q;
+    c1 = 2.0f * hk * 1.00001f;
+    u2 = 2.0f * F.skin_q * hk;
     r2max = R2 / (F.vscale * F.vscale);
     if (CUT) c2 = kappa * lip;
   }
@@ -929,7 +931,7 @@ struct ListTarget {
     float2 rl = mul2(both(c1), m);
     if (CUT) rl = add2(fma2(make_float2(fmaxf(di, dj.x), fmaxf(di, dj.y)), both(c2), rl), d);
     else rl = fma2(d, both(c2), rl);
-    const float2 rl2 = mul2(rl, rl), hp = add2(both(wi), m), hp2 = mul2(hp, hp);
+    const float2 rl2 = mul2(rl, rl), hp = fma2(m, both(hk), both(hi)), hp2 = mul2(hp, hp);
     acc[0] = r2.x < fminf(rl2.x, r2max);
     acc[1] = r2.y < fminf(rl2.y, r2max);
     inside[0] = r2.x < hp2.x;
@@ -1295,7 +1297,7 @@ __global__ void __launch_bounds__(256) k_density(int n, const StepCtl* __restric
   const uint32_t lc = lcount[i];
   T acc = 0;
   if constexpr (std::is_same<T, float>::value) {  // two entries at a time, as pass A
-    const float2 id2 = both(-0.5f / view_w(vi)), one2 = both(1.0f);
+    const float2 id2 = both(-0.5f / (F.half_kappa * view_w(vi))), one2 = both(1.0f);
     float2 ds2 = both(0.0f), dq2 = both(0.0f);
     auto two = [&](uint32_t, const VT& a, uint32_t, const VT& b, auto on0, auto on1) {
       const float2 dx = make_float2((float)(vi.x - a.x), (float)(vi.x - b.x));
@@ -1521,10 +1523,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // per SM): at 48 it spills (8,388,608 in 3D: 2.30 ms against 1.59), at 80
     // too few warps hide the gathers (1.84 ms).
     if constexpr (PACKED) {
-      // lengths in view integers, the pair's support H = w_i + w_j; powers of h_j
-      // and H relative to w_i, whose own powers come in once, after the sum
-      const float wi = view_w(vi);
-      const float2 w2 = both(wi), id2 = both(-0.5f / wi), iw2 = both(1.0f / wi), one2 = both(1.0f);
+      // lengths in view integers, the pair's support H = kappa (h_i + h_j) / 2 (the
+      // same rounding for j's pair with i), w_i = kappa h_i / 2; powers of h_j
+      // relative to h_i and of H to w_i, whose own powers come in once, after the sum
+      const float wi = F.half_kappa * view_w(vi);
+      const float2 h2 = both(view_w(vi)), w2 = both(wi), id2 = both(-0.5f / wi), ih2 = both(1.0f / view_w(vi)), one2 = both(1.0f);
       const float hd2 = 4.0f * wi * wi;  // (kappa h_i)^2
       const float sq = GENERAL ? sP0 * qi : 1.0f + sigma;
       const uint32_t own = ((uint32_t)i << 8) | ci;
@@ -1546,7 +1549,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
           if (!on0) r2.x = 1e30f;
           if (!on1) r2.y = 1e30f;
           const float2 wj = make_float2(view_w(v0), view_w(v1));
-          const float2 H = add2(w2, wj), H2 = mul2(H, H);
+          const float2 S = add2(h2, wj), H = make_float2(F.half_kappa * S.x, F.half_kappa * S.y), H2 = mul2(H, H);
           const bool f0 = r2.x < H2.x, f1 = r2.y < H2.y;
           if (!(f0 || f1 || (!GENERAL && (r2.x < hd2 || r2.y < hd2)))) return;
           const float2 r = mul2(r2, rsqrt2(r2));
@@ -1559,7 +1562,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
           const float2 nH = rcp2(make_float2(-H.x, -H.y));
           const float2 u = max2(fma2(r, nH, one2), 0.0f), g = mul2(nH, w2), g2 = mul2(g, g), g4 = mul2(g2, g2);
           const float2 w = mul2(mul2(mul2(u, u), u), D == 2 ? g4 : mul2(g4, g));  // 3D: negative (g < 0)
-          const float2 t = mul2(wj, iw2), t2 = mul2(t, t);
+          const float2 t = mul2(wj, ih2), t2 = mul2(t, t);
           const float2 ts = D == 2 ? fma2(t2, t2, one2) : fma2(mul2(t2, t2), t2, one2);  // 1 + rho_t,i^2 / rho_t,j^2
           const bool o0 = ((e0 ^ own) & 0xFFu) != 0, o1 = ((e1 ^ own) & 0xFFu) != 0;
           const float2 tw = mul2(ts, w);
@@ -1623,7 +1626,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       if constexpr (std::is_same<T, float>::value) {
         // the tests of the packed path, rounding for rounding (there in view
         // integers: a power of two apart), so that diagnostics name its pairs
-        const float H = (view_w(vi) + view_w(vj)) * F.vscale, w = view_w(vi) * F.vscale;
+        const float w = F.half_kappa * hv, H = F.half_kappa * (hv + hj);
         r2 = fmaf(dy, dy, __fmul_rn(dx, dx));
         if (D == 3) r2 = fmaf(dz, dz, r2);
         Hf = H;
@@ -1693,11 +1696,11 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       az = group_sum<G>(az);
     } else if (S32_OK && v32 && (lc & kFastBit)) {
       const int4 wi = v32[i];
-      const float ws = 2.0f / (float)(1 << kViewBits), wi32 = 0.5f * ws * view_w(wi), Hd32 = ws * view_w(wi);  // view units
+      const float ws = F32.half_kappa * F32.vscale, wi32 = ws * view_w(wi), Hd32 = 2.0f * wi32;  // view units
       auto screen = [&](const int4& w) {
         const float cx = vd_coarse(F32, wi.x, w.x), cy = vd_coarse(F32, wi.y, w.y);
         const float cz = D == 3 ? vd_coarse(F32, wi.z, w.z) : 0.0f;
-        const float Hf32 = wi32 + 0.5f * ws * view_w(w);
+        const float Hf32 = fmaf(ws, view_w(w), wi32);
         const float Hm = screen_radius<float>(Hf32 > Hd32 ? Hf32 : Hd32);
         return cx * cx + cy * cy + cz * cz < Hm * Hm;
       };
@@ -1855,7 +1858,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
                                                 int* __restrict__ err, unsigned long long* __restrict__ wall_moved,
                                                 int move, const uint32_t* __restrict__ m0,
                                                 const uint32_t* __restrict__ m1, int4* __restrict__ v32out,
-                                                int sv32, float c2w32, uint32_t* __restrict__ words) {
+                                                int sv32, uint32_t* __restrict__ words) {
   using VT = typename ViewOf<T>::type;
   __shared__ int moved_sm[NT / 32];
   // G lanes per particle, as pass A
@@ -2068,7 +2071,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       if (v32out) {  // FP64 path: its FP32 view of the next step (as k_gather_view makes it)
         const long long half = 1LL << (sv32 - 1);
         v32out[i] = make_int4((int)((X.x + half) >> sv32), (int)((X.y + half) >> sv32),
-                              D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_w(vn) * c2w32));
+                              D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_w(vn) * (float)(1 << kViewBits)));
       }
       // skin test against the view at list build
       const VT vb = vbuild[i];
@@ -2295,7 +2298,7 @@ cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P
         (LL4*)S.X[0], (LL4*)S.X[1], (const PairRec<T>*)S.plist, S.pcount, S.cap, (const V4<T>*)S.acc4, F, P, g, S.scal,
         f.record ? (V4<T>*)S.visc : nullptr, S.err, wm, f.move, S.meta[0], S.meta[1],
         (std::is_same<T, double>::value && S.view32 && f.f32) ? (int4*)S.view32 : nullptr, f.f32 ? f.f32->sv : 0,
-        f.f32 ? f.f32->c2w : 0.0f, f.words);
+        f.words);
     return cudaGetLastError();
   };
   // threads per block and lanes per particle, taped or not
