@@ -107,7 +107,8 @@ typedef struct {
   int32_t kernel_id;   /* 0: Wendland C2 (the only one) */
   uint64_t seed;       /* seed of the initial sampling (Philox4x32-10) */
   double cell_factor;  /* finest cell edge / smallest support; 0 -> 1.0 */
-  int32_t block_size;  /* threads per block of the FP32 pair passes: 0 (256), 128 or 256 */
+  int32_t block_size;  /* threads per block of the pair passes: 128, 256 or 0 (the library's choice), see
+                          sph_set_tuning */
   int32_t use_graph;   /* 1: sph_step replays a captured CUDA graph of one step */
   int32_t record_fields; /* 1: keep rho, a_n and a~ of the last step for sph_get_field */
   int32_t list_capacity; /* neighbour-list entries per particle; 0 -> auto */
@@ -221,8 +222,11 @@ sph_status sph_set_state(sph_handle* h, const double* xyz, const uint8_t* col, i
 
 /* Launch configuration (no counterpart in the paper: it changes how the work
  * is spread over the GPU, not what is computed). pass_threads: threads per
- * block of the two pair passes, 128 or 256 (0: keep; 256 at creation unless
- * params.block_size says 128); cell_factor: finest cell edge over the
+ * block of the two pair passes, 128 or 256 (0: keep; params.block_size at
+ * creation, and without either the library's choice by precision and particle
+ * count). Small counts take several lanes per particle in blocks of 32
+ * particles whatever is asked for: FP64 up to 8,192 particles, the FP32 viscous
+ * pass up to 16,384. cell_factor: finest cell edge over the
  * smallest support, > 0 (0: keep), which rebuilds the multi-resolution grid;
  * stage_views: 1 runs the density/force pass (Algorithm 1's neighbour loop,
  * Sec. 3.3) staged, 0 unstaged, -1 keeps the setting. Staged, each list
@@ -231,7 +235,7 @@ sph_status sph_set_state(sph_handle* h, const double* xyz, const uint8_t* col, i
  * unstaged) and numbers every list entry by its rank in that set; every step
  * the pass copies the block's neighbour views into shared memory once and
  * reads them there instead of gathering each pair's view from global memory.
- * It applies to FP32 handles with gamma = 2, 256 threads per block and no
+ * It applies to FP32 handles with gamma = 2, not set to 128 threads, and no
  * feature-surface particles (other configurations run unstaged) and costs a
  * second list array (4 bytes x list capacity per particle) plus 40 bytes per
  * particle of neighbour sets. The block size and staging leave every result
@@ -239,7 +243,8 @@ sph_status sph_set_state(sph_handle* h, const double* xyz, const uint8_t* col, i
  * order of each particle's sums (rounding only). The next step rebuilds the
  * neighbour list; captured graphs are re-captured. Synchronises. Errors:
  * INVALID_ARG (stage_views = 1 on an FP64 handle), OOM, CELL_OVERFLOW.
- * sph_get_tuning reads the configuration in use (any pointer may be NULL). */
+ * sph_get_tuning reads the configuration asked for, a block size of 256 where
+ * none was (any pointer may be NULL). */
 sph_status sph_set_tuning(sph_handle* h, int32_t pass_threads, double cell_factor, int32_t stage_views);
 sph_status sph_get_tuning(const sph_handle* h, int32_t* pass_threads, double* cell_factor, int32_t* stage_views);
 

@@ -794,7 +794,7 @@ cudaError_t launch_bwd_step(const DevState& S, const Frame<T>& F, const Phys<T>&
   using VT = typename ViewOf<T>::type;
   // small blocks: warps that are done wait for the block's slowest (barrier
   // stalls were a sixth of k_bwd_visc at 256 threads)
-  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 128, gb = grid_for(S.n, tb);
+  const int tb = sizeof(T) == 8 ? fp64_threads(S.n) : 128, gb = grid_for(S.n, tb);
   if (S.n <= 0) return cudaSuccess;
   const VT* w0 = (const VT*)S.view[0];
   const VT* w1 = (const VT*)S.view[1];
@@ -822,7 +822,7 @@ cudaError_t launch_objective(const DevState& S, const Frame<T>& F, const Phys<T>
   using VT = typename ViewOf<T>::type;
   // small blocks: warps that are done wait for the block's slowest (barrier
   // stalls were a sixth of k_bwd_visc at 256 threads)
-  const int tb = sizeof(T) == 8 ? fp64_threads(S) : 128, gb = grid_for(S.n, tb);
+  const int tb = sizeof(T) == 8 ? fp64_threads(S.n) : 128, gb = grid_for(S.n, tb);
   if (S.n <= 0) return cudaSuccess;
   const VT* w0 = (const VT*)S.view[0];
   const VT* w1 = (const VT*)S.view[1];

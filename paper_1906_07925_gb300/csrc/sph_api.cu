@@ -788,7 +788,7 @@ static sph_status create_impl(sph_handle* h, const sph_domain* dom, const sph_fi
   S.dim = d;
   S.fp64 = h->prec == SPH_PREC_FP64;
   S.cap = h->par.list_capacity > 0 ? h->par.list_capacity : std::min(auto_capacity(h), kMaxListCapacity);
-  S.pass_threads = h->par.block_size == 128 ? 128 : 256;
+  S.pass_threads = h->par.block_size;
   const size_t v4 = S.fp64 ? 32 : 16, t1 = S.fp64 ? 8 : 4;
   const size_t N = (size_t)std::max<int64_t>(n_particles, 1);
   uint8_t* tmpb;
@@ -990,7 +990,7 @@ sph_status sph_set_tuning(sph_handle* h, int32_t pass_threads, double cell_facto
 
 sph_status sph_get_tuning(const sph_handle* h, int32_t* pass_threads, double* cell_factor, int32_t* stage_views) {
   if (!h) return SPH_ERR_INVALID_ARG;
-  if (pass_threads) *pass_threads = h->S.pass_threads;
+  if (pass_threads) *pass_threads = h->S.pass_threads ? h->S.pass_threads : 256;
   if (cell_factor) *cell_factor = h->par.cell_factor > 0 ? h->par.cell_factor : 1.0;
   if (stage_views) *stage_views = h->S.stage;
   return SPH_OK;
@@ -1663,10 +1663,14 @@ sph_status sph_batch_tune(sph_batch* b, const int32_t* candidates, int32_t n_can
     }
     return SPH_OK;
   };
-  // the same launch configuration on every instance
+  // the same launch configuration on every instance; the block size it had, if
+  // none was ever chosen (the library's own rules, reported as 256)
+  sph_handle* h0 = b->inst[0];
+  const int threads0 = h0->S.pass_threads;
   auto configure = [&](const sph_batch_trial& c) -> sph_status {
     for (sph_handle* h : b->inst) {
-      sph_status s = sph_set_tuning(h, c.pass_threads, c.cell_factor, h->S.fp64 ? -1 : c.stage_views);
+      h->S.pass_threads = !threads0 && c.pass_threads == 256 ? 0 : c.pass_threads;
+      sph_status s = sph_set_tuning(h, 0, c.cell_factor, h->S.fp64 ? -1 : c.stage_views);
       if (s != SPH_OK) return s;
     }
     return SPH_OK;
@@ -1699,10 +1703,9 @@ sph_status sph_batch_tune(sph_batch* b, const int32_t* candidates, int32_t n_can
     *ms_out = ms;
     return SPH_OK;
   };
-  sph_handle* h0 = b->inst[0];
   sph_batch_trial best{};
   best.branches = 0;
-  best.pass_threads = h0->S.pass_threads;
+  best.pass_threads = threads0 ? threads0 : 256;
   best.cell_factor = h0->par.cell_factor > 0 ? h0->par.cell_factor : 1.0;
   best.stage_views = h0->S.stage;
   float best_ms = 0.0f;
@@ -1722,10 +1725,10 @@ sph_status sph_batch_tune(sph_batch* b, const int32_t* candidates, int32_t n_can
   // the pair passes, cell factor
   const int threads_alt[] = {128, 256};
   const double cf_alt[] = {0.75, 1.0, 1.5};
-  const int threads0 = best.pass_threads;
+  const int threads1 = best.pass_threads;
   const double cf0 = best.cell_factor;
   for (int v : threads_alt) {
-    if (st != SPH_OK || v == threads0) continue;
+    if (st != SPH_OK || v == threads1) continue;
     sph_batch_trial t = best;
     t.pass_threads = v;
     float ms = 0.0f;

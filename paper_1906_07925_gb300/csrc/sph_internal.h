@@ -16,7 +16,7 @@ namespace sph {
 // ctl->vp (pass B writes the next step's views while pass A/B read the current).
 struct DevState {
   int n = 0, dim = 2, fp64 = 0, cap = 0;
-  int pass_threads = 256;  // threads per block of the pair passes (128 or 256)
+  int pass_threads = 0;  // threads per block of the pair passes (128 or 256; 0: the rules of pass_a_shape, pass_b_shape)
   void* X[2] = {nullptr, nullptr};       // int64 x, y, z (+ pad) per particle
   uint32_t* meta[2] = {nullptr, nullptr};  // colour
   uint32_t* pid[2] = {nullptr, nullptr};   // particle id
@@ -151,6 +151,43 @@ inline int rebuild_grid(int n, int tb, int per_sm) {
   return g < 1 ? 1 : (g < cap ? g : cap);
 }
 
+// Small particle counts, where one thread per particle leaves most of the chip
+// idle and a thread's own chain of loads (FP64: of arithmetic) is the whole
+// time: several lanes share a particle. Steps of the circle (2D, FP32), 4,289 /
+// 16,001 particles: the list build's groups of 8 save 6 / 2 us; of a ball (3D),
+// 10,001 / 16,001: 8 / 6 us, pass B's groups 3 / 3 us; at 24,001 both lose.
+// (Pass A in FP32 gained nothing at any size.) FP64, the 4,096-particle square:
+// 74 us with 32-thread blocks alone, 48 with 4 lanes; 16,001: 97 and 95;
+// 32,001: 124 and 148.
+constexpr int kListLanes = 8, kListGroupMax = 20480;
+constexpr int kPassLanes = 8, kPassGroupMax = 16384;
+constexpr int kLanes64 = 4, kGroupMax64 = 8192;
+// Threads per block of the FP64 pair passes where the caller has not chosen: one
+// warp of FP64 work keeps an SM's FP64 pipe busy, so small blocks spread the
+// particles evenly over the SMs. 200,003 particles in 2D, one step: 674 -> 561 us
+// (256 -> 64 threads), 300,007 in 3D: 2,264 -> 2,077; the 4,096-particle square,
+// 16 blocks of 256 on 152 SMs: 106 -> 74 us (32).
+inline int fp64_threads(int n) { return n <= (1 << 17) ? 32 : 64; }
+// Launch of a pair pass: threads per block and lanes per particle. The rules
+// choose where the caller has not (DevState::pass_threads); groups of lanes make
+// blocks of 32 particles whatever the caller chose.
+struct PassShape {
+  int threads, lanes;
+};
+inline PassShape pass_a_shape(const DevState& S, bool groups) {
+  if (!S.fp64) return {S.pass_threads == 128 ? 128 : 256, 1};
+  if (groups && S.n <= kGroupMax64) return {32 * kLanes64, kLanes64};
+  return {S.pass_threads ? S.pass_threads : fp64_threads(S.n), 1};
+}
+inline PassShape pass_b_shape(const DevState& S) {
+  if (S.fp64) return pass_a_shape(S, true);
+  if (S.n <= kPassGroupMax) return {32 * kPassLanes, kPassLanes};
+  // large runs in small blocks, whose warps wait for no one else's tail
+  // (8,388,608 particles in 3D 873 -> 805 us, 1,048,576 in 2D 71 -> 69; at
+  // 240,370 in 3D 31 -> 33)
+  return {S.pass_threads ? S.pass_threads : S.n >= (1 << 19) ? 128 : 256, 1};
+}
+
 struct PassFlags {
   int general_eos = 0;  // gamma != 2: density pass first, pressure p/rho^2
   int record = 0;       // keep rho and a~ for output
@@ -180,7 +217,7 @@ cudaError_t prepare_staged_pass();
 // whether pass A runs staged for these flags (the variant exists for FP32,
 // gamma = 2, no feature-surface particles, no neighbour diagnostics, 256 threads)
 inline bool staged_pass(const DevState& S, const PassFlags& f) {
-  return S.stage && !S.fp64 && S.pass_threads == 256 && !f.general_eos && !f.nbr_debug && !f.surface;
+  return S.stage && !S.fp64 && S.pass_threads != 128 && !f.general_eos && !f.nbr_debug && !f.surface;
 }
 template <int D, class T>
 cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P, const Geom<T>& g, PassFlags f,

@@ -1461,7 +1461,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
   static_assert(G == 1 || (sizeof(T) == 8 && !DBG && !SURF && NT == 32 * G),
                 "several lanes per particle: FP64, 32 particles per block");
   extern __shared__ __align__(16) unsigned char stage_smem[];
-  // G lanes per particle (fp64_lanes): all of a warp's lanes stay together in
+  // G lanes per particle (pass_a_shape): all of a warp's lanes stay together in
   // the loop, those past the end with an empty list; warp 0 holds the block's 32
   // particles afterwards
   const int slot = (blockIdx.x * NT + threadIdx.x) / G;
@@ -2168,25 +2168,6 @@ __global__ void __launch_bounds__(256) k_get_fields(int n, int which, const Step
 // --------------------------------------------------------------------------
 inline int grid_for(int n, int tb) { return (n + tb - 1) / tb; }
 
-// Small particle counts, where one thread per particle leaves most of the chip
-// idle and a thread's own chain of loads (FP64: of arithmetic) is the whole
-// time: several lanes share a particle. Steps of the circle (2D, FP32), 4,289 /
-// 16,001 particles: the list build's groups of 8 save 6 / 2 us; of a ball (3D),
-// 10,001 / 16,001: 8 / 6 us, pass B's groups 3 / 3 us; at 24,001 both lose.
-// (Pass A in FP32 gained nothing at any size.) FP64, the 4,096-particle square:
-// 74 us with 32-thread blocks alone, 48 with 4 lanes; 16,001: 97 and 95;
-// 32,001: 124 and 148.
-constexpr int kListLanes = 8, kListGroupMax = 20480;
-constexpr int kPassLanes = 8, kPassGroupMax = 16384;
-constexpr int kLanes64 = 4, kGroupMax64 = 8192;
-inline int fp64_lanes(const DevState& S) { return S.n <= kGroupMax64 ? kLanes64 : 1; }
-// Threads per block of the FP64 pair passes (FP32: DevState::pass_threads): one
-// warp of FP64 work keeps an SM's FP64 pipe busy, so small blocks spread the
-// particles evenly over the SMs. 200,003 particles in 2D, one step: 674 -> 561 us
-// (256 -> 64 threads), 300,007 in 3D: 2,264 -> 2,077; the 4,096-particle square,
-// 16 blocks of 256 on 152 SMs: 106 -> 74 us (32).
-inline int fp64_threads(const DevState& S) { return S.n <= (1 << 17) ? 32 : 64; }
-
 template <int D, class T>
 cudaError_t launch_rebuild(const DevState& S, int force, const Grid<T>& G, const Frame<T>& F, const Geom<T>& g,
                            T kappa, cudaStream_t st, const Grid<float>* G32, const Frame<float>* F32) {
@@ -2253,30 +2234,34 @@ cudaError_t launch_pass_a(const DevState& S, const Frame<T>& F, const Phys<T>& P
     kernel<<<grid_for(S.n, threads), threads, 0, st>>>(S.n, S.ctl, (const VT*)S.view[0], (const VT*)S.view[1], S.list,
                                                        S.lcount, S.cap, F, P, rho, pc);
   };
-  // one block size and one of the compiled variants
+  // one of the compiled variants at one block size (the diagnostics at one only)
   auto pick = [&](auto nt) -> cudaError_t {
     constexpr int NT = decltype(nt)::value;
-#define SPH_PASS_A(GEN, DBG) \
-  run(f.surface ? k_pass_a<D, T, GEN, DBG, true, NT> : k_pass_a<D, T, GEN, DBG, false, NT>, NT, 1, 0)
-    if (f.general_eos) return f.nbr_debug ? SPH_PASS_A(true, true) : SPH_PASS_A(true, false);
-    return f.nbr_debug ? SPH_PASS_A(false, true) : SPH_PASS_A(false, false);
-#undef SPH_PASS_A
+    if (f.general_eos)
+      return run(f.surface ? k_pass_a<D, T, true, false, true, NT> : k_pass_a<D, T, true, false, false, NT>, NT, 1, 0);
+    return run(f.surface ? k_pass_a<D, T, false, false, true, NT> : k_pass_a<D, T, false, false, false, NT>, NT, 1, 0);
   };
-  if constexpr (std::is_same<T, float>::value) {
-    if (f.general_eos) density(k_density<D, T>, 256);
-    if (staged_pass(S, f))
-      return run(k_pass_a<D, T, false, false, false, kStageBlock, true>, kStageBlock, 1, kStageCap * sizeof(int4));
-    if (S.pass_threads == 128) return pick(std::integral_constant<int, 128>{});
-    return pick(std::integral_constant<int, 256>{});
-  } else {
-    const int nt = fp64_threads(S);
-    if (f.general_eos) density(k_density<D, T>, nt);
-    if (fp64_lanes(S) > 1 && !f.surface && !f.nbr_debug)
-      return f.general_eos ? run(k_pass_a<D, T, true, false, false, 32 * kLanes64, false, kLanes64>, 32 * kLanes64, kLanes64, 0)
-                           : run(k_pass_a<D, T, false, false, false, 32 * kLanes64, false, kLanes64>, 32 * kLanes64, kLanes64, 0);
-    if (nt == 32) return pick(std::integral_constant<int, 32>{});
-    return pick(std::integral_constant<int, 64>{});
+  auto diagnose = [&](auto nt) -> cudaError_t {
+    constexpr int NT = decltype(nt)::value;
+    if (f.general_eos)
+      return run(f.surface ? k_pass_a<D, T, true, true, true, NT> : k_pass_a<D, T, true, true, false, NT>, NT, 1, 0);
+    return run(f.surface ? k_pass_a<D, T, false, true, true, NT> : k_pass_a<D, T, false, true, false, NT>, NT, 1, 0);
+  };
+  constexpr bool f64 = std::is_same<T, double>::value;
+  if (f.general_eos) density(k_density<D, T>, f64 ? fp64_threads(S.n) : 256);
+  if (f.nbr_debug) return diagnose(std::integral_constant<int, f64 ? 64 : 256>{});
+  const PassShape shape = pass_a_shape(S, !f.surface);
+  if constexpr (f64) {
+    if (shape.lanes > 1)
+      return f.general_eos ? run(k_pass_a<D, T, true, false, false, 32 * kLanes64, false, kLanes64>, shape.threads, kLanes64, 0)
+                           : run(k_pass_a<D, T, false, false, false, 32 * kLanes64, false, kLanes64>, shape.threads, kLanes64, 0);
+    if (shape.threads == 32) return pick(std::integral_constant<int, 32>{});
+    if (shape.threads == 64) return pick(std::integral_constant<int, 64>{});
+  } else if (staged_pass(S, f)) {
+    return run(k_pass_a<D, T, false, false, false, kStageBlock, true>, kStageBlock, 1, kStageCap * sizeof(int4));
   }
+  if (shape.threads == 128) return pick(std::integral_constant<int, 128>{});
+  return pick(std::integral_constant<int, 256>{});
 }
 
 template <int D>
@@ -2307,19 +2292,17 @@ cudaError_t launch_pass_b(const DevState& S, const Frame<T>& F, const Phys<T>& P
     return f.words ? run(k_pass_b<D, T, NT, G, true>, NT, G) : run(k_pass_b<D, T, NT, G>, NT, G);
   };
   using one = std::integral_constant<int, 1>;
+  const PassShape shape = pass_b_shape(S);
   if constexpr (std::is_same<T, float>::value) {
-    if (S.n <= kPassGroupMax)
+    if (shape.lanes > 1)
       return pick(std::integral_constant<int, 32 * kPassLanes>{}, std::integral_constant<int, kPassLanes>{});
-    // large runs in small blocks, whose warps wait for no one else's tail
-    // (8,388,608 particles in 3D 873 -> 805 us, 1,048,576 in 2D 71 -> 69; at
-    // 240,370 in 3D 31 -> 33)
-    if (S.pass_threads == 128 || S.n >= (1 << 19)) return pick(std::integral_constant<int, 128>{}, one{});
-    return pick(std::integral_constant<int, 256>{}, one{});
   } else {
-    if (fp64_lanes(S) > 1) return pick(std::integral_constant<int, 32 * kLanes64>{}, std::integral_constant<int, kLanes64>{});
-    if (fp64_threads(S) == 32) return pick(std::integral_constant<int, 32>{}, one{});
-    return pick(std::integral_constant<int, 64>{}, one{});
+    if (shape.lanes > 1) return pick(std::integral_constant<int, 32 * kLanes64>{}, std::integral_constant<int, kLanes64>{});
+    if (shape.threads == 32) return pick(std::integral_constant<int, 32>{}, one{});
+    if (shape.threads == 64) return pick(std::integral_constant<int, 64>{}, one{});
   }
+  if (shape.threads == 128) return pick(std::integral_constant<int, 128>{}, one{});
+  return pick(std::integral_constant<int, 256>{}, one{});
 }
 
 template <int D, class T>
