@@ -79,8 +79,8 @@ struct Frame {
   int mbits;             // FP32: bits of 1.5 * 2^(23 - kCoarseBits); adding d encodes d 2^-kCoarseBits
   float mbias;           // FP32: 1.5 * 2^(23 - kCoarseBits)
   float vscale;          // FP32: 2^-kViewBits, one view integer in view units
-  float h2w;             // FP32: h -> view integers, the same rounding as inv_qv a power of two away
   float half_kappa;      // kappa / 2: the support of a pair is half_kappa (h_i + h_j)
+  float hk_int;          // FP32: the same from h in view units to a support in view integers
   T qv, inv_qv;          // physical length of one view unit (the finest cell edge c0)
   T q64t, inv_q64t;
   T lo[3];

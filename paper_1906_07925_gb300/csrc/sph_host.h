@@ -221,8 +221,8 @@ inline void make_frames(const sph_domain& dom, double kappa, double skin, bool a
   out.f.mbits = bits;
   out.f.mbias = bias;
   out.f.vscale = (float)std::ldexp(1.0, -kViewBits);
-  out.f.h2w = std::ldexp((float)(1.0 / c0), kViewBits);
   out.f.half_kappa = out.d.half_kappa = 0.5f * (float)kappa;
+  out.f.hk_int = out.d.hk_int = std::ldexp(out.f.half_kappa, kViewBits);
   convert_grid<float>(hg, c0, out.gf);
   convert_grid<double>(hg, c0, out.gd);
 }

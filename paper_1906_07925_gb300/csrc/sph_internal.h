@@ -72,7 +72,7 @@ __host__ __device__ inline size_t pair_at(int i, int k, int cap) {
 }
 // A force pair as pass A leaves it to pass B: the list word and what the viscous
 // force needs of the pair's geometry, f = (1/rho_t,i^2 + 1/rho_t,j^2) (1 - q)^3
-// / H^(D+2) (FP32: over a factor of the target alone, pair_scale).
+// / H^(D+2) (FP32: over a factor common to all pairs, pair_scale).
 template <class T> struct PairRec;
 template <> struct alignas(8) PairRec<float> { uint32_t e; float f; };
 template <> struct alignas(16) PairRec<double> { double f; uint32_t e, pad; };
@@ -153,12 +153,16 @@ inline int rebuild_grid(int n, int tb, int per_sm) {
 
 // Small particle counts, where one thread per particle leaves most of the chip
 // idle and a thread's own chain of loads (FP64: of arithmetic) is the whole
-// time: several lanes share a particle. Steps of the circle (2D, FP32), 4,289 /
-// 16,001 particles: the list build's groups of 8 save 6 / 2 us; of a ball (3D),
-// 10,001 / 16,001: 8 / 6 us, pass B's groups 3 / 3 us; at 24,001 both lose.
-// (Pass A in FP32 gained nothing at any size.) FP64, the 4,096-particle square:
-// 74 us with 32-thread blocks alone, 48 with 4 lanes; 16,001: 97 and 95;
-// 32,001: 124 and 148.
+// time: several lanes share a particle. One step, us, without and with groups:
+//   list build (8 lanes): 6 / 2 less for the circle (2D, FP32) of 4,289 / 16,001
+//     particles, 8 / 6 for a ball (3D) of 10,001 / 16,001; at 24,001 both lose
+//   FP32 pass B (8 lanes), graded hole (2D) and inclusion (3D): 4,096 29.2 / 27.2
+//     and 92.3 / 90.1, 16,384 29.4 / 29.3 and 77.8 / 76.4, 20,480 31.2 / 30.6 and
+//     71.8 / 73.6, 24,576 31.3 / 33.3 and 76.1 / 78.2
+//   FP64 passes (4 lanes), the same: 4,096 72 / 46 and 206 / 129, 8,192 72 / 54 and
+//     202 / 148, 12,288 74 / 67 and 195 / 166, 16,384 80 / 83 and 195 / 191, 24,576
+//     93 / 113 and 229 / 272: the gain ends past 12,288, the line is well inside it
+// (Pass A in FP32 gained nothing at any size.)
 constexpr int kListLanes = 8, kListGroupMax = 20480;
 constexpr int kPassLanes = 8, kPassGroupMax = 16384;
 constexpr int kLanes64 = 4, kGroupMax64 = 8192;
@@ -166,7 +170,10 @@ constexpr int kLanes64 = 4, kGroupMax64 = 8192;
 // warp of FP64 work keeps an SM's FP64 pipe busy, so small blocks spread the
 // particles evenly over the SMs. 200,003 particles in 2D, one step: 674 -> 561 us
 // (256 -> 64 threads), 300,007 in 3D: 2,264 -> 2,077; the 4,096-particle square,
-// 16 blocks of 256 on 152 SMs: 106 -> 74 us (32).
+// 16 blocks of 256 on 152 SMs: 106 -> 74 us (32). Between 32 and 64 it matters
+// little: 32,768 in 2D / 3D 107 / 246 against 115 / 267 us, 131,072 325 / 792
+// against 329 / 795, 200,000 483 / 1,166 against 487 / 1,169; past the line 64
+// halves the partials that the end of pass A merges.
 inline int fp64_threads(int n) { return n <= (1 << 17) ? 32 : 64; }
 // Launch of a pair pass: threads per block and lanes per particle. The rules
 // choose where the caller has not (DevState::pass_threads); groups of lanes make
@@ -182,9 +189,10 @@ inline PassShape pass_a_shape(const DevState& S, bool groups) {
 inline PassShape pass_b_shape(const DevState& S) {
   if (S.fp64) return pass_a_shape(S, true);
   if (S.n <= kPassGroupMax) return {32 * kPassLanes, kPassLanes};
-  // large runs in small blocks, whose warps wait for no one else's tail
-  // (8,388,608 particles in 3D 873 -> 805 us, 1,048,576 in 2D 71 -> 69; at
-  // 240,370 in 3D 31 -> 33)
+  // large runs in small blocks, whose warps wait for no one else's tail: with 128
+  // threads for 256, 8,388,608 particles in 3D 873 -> 805 us, 1,048,576 in 3D 112 ->
+  // 105 and in 2D 66 -> 64, 524,288 62 -> 54 and 32 -> 31; 393,216 and 262,144 the
+  // same to the event clock's 2 us, 240,370 in 3D 31 -> 33
   return {S.pass_threads ? S.pass_threads : S.n >= (1 << 19) ? 128 : 256, 1};
 }
 

@@ -83,11 +83,10 @@ template <class T>
 __device__ __forceinline__ T screen_radius(T H) {
   return H * T(1.0 + 1.0 / (1 << 20)) + T(1.0 / (1 << (kCoarseBits - 2)));
 }
-// w of a view: FP32 h in view integers, FP64 h in view units; view_h: h in view
-// units (FP32: the view's own rounding and a power of two, no rounding more)
+// w of a view, h in view units
 __device__ __forceinline__ float view_w(const int4& v) { return __int_as_float(v.w); }
 __device__ __forceinline__ double view_w(const V4<double>& v) { return v.w; }
-__device__ __forceinline__ float view_h(const Frame<float>& F, const int4& v) { return __int_as_float(v.w) * F.vscale; }
+__device__ __forceinline__ float view_h(const Frame<float>&, const int4& v) { return __int_as_float(v.w); }
 __device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>& v) { return v.w; }
 
 // The build view of a particle (vbuild; FP64 path: view32 until pass B renews it):
@@ -95,7 +94,7 @@ __device__ __forceinline__ double view_h(const Frame<double>&, const V4<double>&
 // reach code in the low byte. The reach, in view integers:
 __device__ __forceinline__ float build_w(int4 v) { return __int_as_float(v.w & ~0xFF); }
 __device__ __forceinline__ float build_reach(const Frame<float>& F, int4 v, int most = 255) {
-  return (float)min(v.w & 0xFF, most) * (2.0f * F.skin_q * F.half_kappa) * build_w(v);
+  return (float)min(v.w & 0xFF, most) * (2.0f * F.skin_q * F.hk_int) * build_w(v);
 }
 // FP64 path: pass B reads the reach itself (view units) with its code in the low
 // byte, where a float's mantissa leaves zeros
@@ -141,7 +140,7 @@ template <int D>
 __device__ __forceinline__ int4 make_view(const Frame<float>& F, const LL4& X, float h) {
   const long long half = 1LL << (F.sv - 1);
   return make_int4((int)((X.x + half) >> F.sv), (int)((X.y + half) >> F.sv), D == 3 ? (int)((X.z + half) >> F.sv) : 0,
-                   __float_as_int(h * F.h2w));
+                   __float_as_int(h * F.inv_qv));
 }
 template <int D>
 __device__ __forceinline__ V4<double> make_view(const Frame<double>& F, const LL4& X, double h) {
@@ -207,15 +206,12 @@ __device__ __forceinline__ PairRec<double> load_pair(const PairRec<double>* p) {
   const uint4 v = __ldcs((const uint4*)p);
   return PairRec<double>{__longlong_as_double((long long)v.x | (long long)v.y << 32), v.z, 0u};
 }
-// the target's factor of its pair records: FP32 records hold powers of h_j and
-// of the support relative to w_i = kappa h_i / 2, and 1 + rho_t,i^2/rho_t,j^2
+// the factor that all FP32 pair records leave out: (h / tau)^(2 D) of one view unit
+// (common), and the sign of their odd power of -1/H in 3D
 template <int D>
-__device__ __forceinline__ float pair_scale(float qi, float invHd) {
-  const float iw = 2.0f * invHd, iw4 = iw * iw * iw * iw;
-  return qi * (D == 2 ? iw4 : -iw4 * iw);
-}
+__device__ __forceinline__ float pair_scale(float common) { return D == 2 ? common : -common; }
 template <int D>
-__device__ __forceinline__ double pair_scale(double, double) { return 1.0; }
+__device__ __forceinline__ double pair_scale(double) { return 1.0; }
 
 // The skin list of particle i as quads of entries (split at its build, see
 // kFastBit), in the order: full quads of the inside part, full quads of the
@@ -358,6 +354,14 @@ __device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a product and a sum that stay two roundings (packed ones were fused to one fma,
+// also where both name their rounding; the scalar forms are not)
+__device__ __forceinline__ float2 mul2_apart(float2 a, float2 b) {
+  return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 add2_apart(float2 a, float2 b) {
+  return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
 __device__ __forceinline__ float2 max2(float2 a, float b) { return make_float2(fmaxf(a.x, b), fmaxf(a.y, b)); }
 // hardware reciprocal (1 ulp) and reciprocal square root of normal numbers
 __device__ __forceinline__ float fast_rcp(float x) {
@@ -849,7 +853,7 @@ __global__ void __launch_bounds__(256) k_gather_view(
     most = max(most, code);
     if constexpr (std::is_same<T, double>::value) {
       const long long half = 1LL << (F32.sv - 1);
-      const int w = ((__float_as_int((float)view_w(v) * (float)(1 << kViewBits)) + 0xFF) & ~0xFF) | code;
+      const int w = ((__float_as_int((float)view_w(v)) + 0xFF) & ~0xFF) | code;
       const int4 u = make_int4((int)((X.x + half) >> F32.sv), (int)((X.y + half) >> F32.sv),
                                D == 3 ? (int)((X.z + half) >> F32.sv) : 0, w);
       v32[d] = u;
@@ -875,12 +879,12 @@ __global__ void __launch_bounds__(256) k_gather_view(
 // further than that (ctl->reach_cap), which is less than what the other lists
 // allow for, so all of them hold every pair.
 // The list is built on FP32 views in both precisions. Lengths of the tests are
-// view integers; with w = h (build_w) and m = max(w_i, w_j), kappa m is the largest
+// view integers; with w = h (build_w, view units) and m = max(w_i, w_j), kappa m is the largest
 // support of the pair and the larger of kappa h_i and kappa h_ij is kappa (w_i + m) / 2.
 template <bool CUT>
 struct ListTarget {
   float Rs, R2;          // search radius, view units
-  float wi, di, c1, c2, u2, hk, hi, r2max;  // view integers
+  float wi, di, c1, c2, u2, hk, hi, r2max;  // view integers (wi: view units)
   int l0, l1;            // levels that can hold a neighbour
   int most;              // CUT: the largest code
   __device__ __forceinline__ ListTarget(const Frame<float>& F, const Grid<float>& G, float kappa, int dmax,
@@ -889,9 +893,9 @@ struct ListTarget {
     if (CUT) dmax = min(dmax, most);
     wi = build_w(vi);
     di = build_reach(F, vi, CUT ? most : 255);
-    hk = F.half_kappa;
+    hk = F.hk_int;
     hi = hk * wi;
-    const float hv = wi * F.vscale, lip = G.lip_h, dv = di * F.vscale, dm = (float)dmax * F.skin_q * kappa;
+    const float hv = wi, lip = G.lip_h, dv = di * F.vscale, dm = (float)dmax * F.skin_q * kappa;
     // search radius: bound h_j by Lipschitz continuity and d_j by the largest
     // reach of this build, iterate twice
     float hhi = hv;
@@ -1297,7 +1301,7 @@ __global__ void __launch_bounds__(256) k_density(int n, const StepCtl* __restric
   const uint32_t lc = lcount[i];
   T acc = 0;
   if constexpr (std::is_same<T, float>::value) {  // two entries at a time, as pass A
-    const float2 id2 = both(-0.5f / (F.half_kappa * view_w(vi))), one2 = both(1.0f);
+    const float2 id2 = both(-0.5f / (F.hk_int * view_w(vi))), one2 = both(1.0f);
     float2 ds2 = both(0.0f), dq2 = both(0.0f);
     auto two = [&](uint32_t, const VT& a, uint32_t, const VT& b, auto on0, auto on1) {
       const float2 dx = make_float2((float)(vi.x - a.x), (float)(vi.x - b.x));
@@ -1523,13 +1527,23 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // per SM): at 48 it spills (8,388,608 in 3D: 2.30 ms against 1.59), at 80
     // too few warps hide the gathers (1.84 ms).
     if constexpr (PACKED) {
-      // lengths in view integers, the pair's support H = kappa (h_i + h_j) / 2 (the
-      // same rounding for j's pair with i), w_i = kappa h_i / 2; powers of h_j
-      // relative to h_i and of H to w_i, whose own powers come in once, after the sum
-      const float wi = F.half_kappa * view_w(vi);
-      const float2 h2 = both(view_w(vi)), w2 = both(wi), id2 = both(-0.5f / wi), ih2 = both(1.0f / view_w(vi)), one2 = both(1.0f);
+      // distances and supports H = kappa (h_i + h_j) / 2 in view integers, powers of
+      // h and of H in view units; what all pairs have in common (pair_scale, P0)
+      // comes in once, after the sum. A pair's terms round alike for both its ends,
+      // so that the forces of a pair cancel exactly: with powers relative to the
+      // target's h they did not, and after 8 steps of 20,011 particles in 2D the
+      // gradients by positions were off by 6.3e-7 instead of 5.7e-7, that by sigma0 by
+      // 2.7e-7 instead of 1.7e-7 (means over 80 starts; in 3D 5.3e-7 and 2.3e-7).
+      const float wi = F.hk_int * view_w(vi);  // kappa h_i / 2
+      const float2 h2 = both(view_w(vi)), id2 = both(-0.5f / wi), one2 = both(1.0f), unit2 = both((float)(1 << kViewBits));
+      const auto power = [](float2 h) {  // h^(2 D), rounded before it enters a sum
+        const float2 t2 = mul2(h, h), t4 = mul2_apart(t2, t2);
+        return D == 2 ? t4 : mul2_apart(t4, t2);
+      };
+      const float2 qi2 = power(h2);
       const float hd2 = 4.0f * wi * wi;  // (kappa h_i)^2
-      const float sq = GENERAL ? sP0 * qi : 1.0f + sigma;
+      const float common = inv_rho_t2<D, float>(1.0f, inv_tau_v);  // (h / tau)^(2 D) from h in view units
+      const float sq = GENERAL ? sP0 * common : 1.0f + sigma;
       const uint32_t own = ((uint32_t)i << 8) | ci;
       uint32_t counts = 0;  // force pairs, of them other colours << 16
       float dq = 0.0f;
@@ -1548,8 +1562,8 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
           r2 = make_float2(fmaxf(r2.x, 1.0f), fmaxf(r2.y, 1.0f));  // 1 for the particle itself: r = 2^-24 c0, dx = 0
           if (!on0) r2.x = 1e30f;
           if (!on1) r2.y = 1e30f;
-          const float2 wj = make_float2(view_w(v0), view_w(v1));
-          const float2 S = add2(h2, wj), H = make_float2(F.half_kappa * S.x, F.half_kappa * S.y), H2 = mul2(H, H);
+          const float2 hj = make_float2(view_w(v0), view_w(v1));
+          const float2 S = add2(h2, hj), H = make_float2(F.hk_int * S.x, F.hk_int * S.y), H2 = mul2(H, H);
           const bool f0 = r2.x < H2.x, f1 = r2.y < H2.y;
           if (!(f0 || f1 || (!GENERAL && (r2.x < hd2 || r2.y < hd2)))) return;
           const float2 r = mul2(r2, rsqrt2(r2));
@@ -1560,10 +1574,9 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
             dq += m.x + m.y;
           }
           const float2 nH = rcp2(make_float2(-H.x, -H.y));
-          const float2 u = max2(fma2(r, nH, one2), 0.0f), g = mul2(nH, w2), g2 = mul2(g, g), g4 = mul2(g2, g2);
+          const float2 u = max2(fma2(r, nH, one2), 0.0f), g = mul2(nH, unit2), g2 = mul2(g, g), g4 = mul2(g2, g2);
           const float2 w = mul2(mul2(mul2(u, u), u), D == 2 ? g4 : mul2(g4, g));  // 3D: negative (g < 0)
-          const float2 t = mul2(wj, ih2), t2 = mul2(t, t);
-          const float2 ts = D == 2 ? fma2(t2, t2, one2) : fma2(mul2(t2, t2), t2, one2);  // 1 + rho_t,i^2 / rho_t,j^2
+          const float2 ts = add2_apart(qi2, power(hj));  // 1 / rho_t,i^2 + 1 / rho_t,j^2 over `common`
           const bool o0 = ((e0 ^ own) & 0xFFu) != 0, o1 = ((e1 ^ own) & 0xFFu) != 0;
           const float2 tw = mul2(ts, w);
           float2 s;
@@ -1593,8 +1606,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       dsum -= 4.0f * dq;  // dq holds the terms in -q
       nf = counts & 0xFFFFu;
       ni = counts >> 16;
-      // back to view units: w_i^-(D+2), and P0/rho_t,i^2 (or the pressures themselves)
-      const float back = F.vscale * pair_scale<D>(GENERAL ? 1.0f : P.P0 * qi, invHd);
+      const float back = F.vscale * pair_scale<D>(GENERAL ? 1.0f : P.P0 * common);
       ax = (ax2.x + ax2.y) * back;
       ay = (ay2.x + ay2.y) * back;
       az = (az2.x + az2.y) * back;
@@ -1613,7 +1625,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       pw += 32 * __popc(m);
       nf += __popc(m);
     };
-    const T iscale = T(1) / pair_scale<D>(qi, invHd);
+    const T iscale = T(1) / pair_scale<D>(inv_rho_t2<D, T>(T(1), inv_tau_v));
     bool have = false, have_other = false;  // G > 1: what the lane's entry adds to the group's pairs
     T have_f = 0;
     auto pair = [&](uint32_t e, const VT& vj) {
@@ -1696,7 +1708,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
       az = group_sum<G>(az);
     } else if (S32_OK && v32 && (lc & kFastBit)) {
       const int4 wi = v32[i];
-      const float ws = F32.half_kappa * F32.vscale, wi32 = ws * view_w(wi), Hd32 = 2.0f * wi32;  // view units
+      const float ws = F32.half_kappa, wi32 = ws * view_w(wi), Hd32 = 2.0f * wi32;  // view units
       auto screen = [&](const int4& w) {
         const float cx = vd_coarse(F32, wi.x, w.x), cy = vd_coarse(F32, wi.y, w.y);
         const float cz = D == 3 ? vd_coarse(F32, wi.z, w.z) : 0.0f;
@@ -1838,7 +1850,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
 // reach since the list was built raises need_rebuild.
 // Bound by the gather of the neighbour's acceleration, one per force pair: the
 // pair's geometry factor comes from pass A's record (8,388,608 particles in 3D,
-// FP32: 1.40 -> 0.77 ms with 128-thread blocks; 300,007 in FP64: 1.40 -> 0.43).
+// FP32: 1.40 -> 0.74 ms with 128-thread blocks; 300,007 in FP64: 1.40 -> 0.43).
 // TAPE: a step of the reverse pass's tape also keeps the pairs' list words (a
 // kernel of its own that took them out of the records added 13 us to a step of
 // 262,144 particles in 2D).
@@ -1997,11 +2009,10 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
     if (G == 1 || threadIdx.x < 32) {
     const VT vi = view[i];
     const T hv = view_h(F, vi);
-    const T qi = inv_rho_t2<D, T>(hv, P.inv_tau * F.qv);
     // dW/dr / r = -20 alpha (1-q)^3 / H^(D+2); view lengths -> physical
     const T iq = F.inv_qv;
     const T km = T(-20) * P.alpha * (D == 2 ? iq * iq * iq * iq : iq * iq * iq * iq * iq) *
-                 pair_scale<D>(qi, T(1) / (P.kappa * hv));
+                 pair_scale<D>(inv_rho_t2<D, T>(T(1), P.inv_tau * F.qv));
     bx *= km;
     by *= km;
     bz *= km;
@@ -2071,7 +2082,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
       if (v32out) {  // FP64 path: its FP32 view of the next step (as k_gather_view makes it)
         const long long half = 1LL << (sv32 - 1);
         v32out[i] = make_int4((int)((X.x + half) >> sv32), (int)((X.y + half) >> sv32),
-                              D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_w(vn) * (float)(1 << kViewBits)));
+                              D == 3 ? (int)((X.z + half) >> sv32) : 0, __float_as_int((float)view_w(vn)));
       }
       // skin test against the view at list build
       const VT vb = vbuild[i];
