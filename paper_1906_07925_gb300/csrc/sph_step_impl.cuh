@@ -1434,10 +1434,11 @@ __device__ __noinline__ void finish_step(Partial part, Partial* partials, unsign
 // e_ij = (r_i - r_j)/r_ij, h_ij = (h_i + h_j)/2, and for the Wendland C2 kernel
 // of support H: dW/dr e_ij = -20 alpha (1 - q)^3 (r_i - r_j) / H^(D+2).
 // Writes a_i and g_i = 0.05 rho_t,i r_c,i |a_i| (eta_i = dt1 g_i, Eq.
-// viscosity_coefficient with v~ = a dt1 / 2); FP64 block partials of
-// min r_c/|a|, max |a|, sum rho, sum (rho/rho_t - 1)^2, max |rho/rho_t - 1|,
-// pair counts; the last block reduces them in fixed order and sets dt1, dt2
-// (Eq. time_step_size, see below).
+// viscosity_coefficient with v~ = a dt1 / 2), the force pairs for pass B, and
+// block partials (FP32: fixed-point sums and the particles of the extrema,
+// WarpSums; FP64: values) of min r_c/|a|, max |a|, sum rho, sum (rho/rho_t - 1)^2,
+// max |rho/rho_t - 1|, pair counts; the last block reduces them in fixed order and
+// sets dt1, dt2 (Eq. time_step_size, see finish_step).
 // --------------------------------------------------------------------------
 template <int D, class T, bool GENERAL, bool DBG, bool SURF, int NT, bool STG = false, int G = 1>
 __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64 : SPH_PASS_MIN_BLOCKS) * 256 / NT) k_pass_a(int n, StepCtl* ctl,
@@ -1522,10 +1523,10 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASS_MIN_BLOCKS_FP64
     // nothing and needs no test; only an iteration in which neither entry is
     // inside is skipped. What bounds it: the latency of the view gathers (issue
     // slots 51 % busy, L1 data pipe 56 %). With the reductions above, at
-    // 1,048,576 particles: 304 -> 227 us in 3D (249 -> 144 million warp
-    // instructions), 216 -> 126 us in 2D. 64 registers (four 256-thread blocks
-    // per SM): at 48 it spills (8,388,608 in 3D: 2.30 ms against 1.59), at 80
-    // too few warps hide the gathers (1.84 ms).
+    // 1,048,576 particles: 304 -> 231 us in 3D (249 -> 144 million warp
+    // instructions), 216 -> 114 us in 2D; 8,388,608 in 3D 1.50 ms. 64 registers
+    // (four 256-thread blocks per SM): an earlier form at 48 spilled (2.30 ms
+    // against 1.59), at 80 too few warps hid the gathers (1.84 ms).
     if constexpr (PACKED) {
       // distances and supports H = kappa (h_i + h_j) / 2 in view integers, powers of
       // h and of H in view units; what all pairs have in common (pair_scale, P0)
@@ -1887,7 +1888,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 8 ? SPH_PASSB_MIN_BLOCKS_FP6
     // this step's pairs as pass A left them: the geometry in a factor per pair,
     // so only the neighbour's acceleration is gathered and no distance, root or
     // kernel value is computed again. FP32, 8,388,608 particles in 3D: 1.40 ->
-    // 0.86 ms, and pass A, which writes the factor, 1.59 -> 1.65; FP64, where the
+    // 0.74 ms, and pass A, which writes the factor, 0.06 ms longer; FP64, where the
     // FP64 pipe bounds both passes, 300,007 in 3D: 1.40 -> 0.43 ms.
     const int cnt = lead ? (int)pcount[i] : 0;
     const PairRec<T>* __restrict__ p = plist + pair_at(i, 0, cap);
