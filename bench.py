@@ -65,8 +65,10 @@ ALG_BYTES = {"cells": 54, "pass_a": 33, "pass_b": 49}
 ALG_BYTES_FP64 = {"cells": 92, "pass_a": 56, "pass_b": 83}
 # launches per step (gamma = 2): rekey, scan, scatter, gather, list_build (they
 # exit at once unless the list is rebuilt); pass A; pass B; with the staged pass A
-# one more predicated rebuild kernel (the blocks' neighbour sets)
+# one more predicated rebuild kernel (the blocks' neighbour sets), with more cells
+# than the scan takes in one level (csrc/sph_cells.cu) another
 KERNELS_PER_STEP = 7
+SCAN_ONE_LEVEL = 2048 * 4096
 # pair arithmetic (FP32 flop, counted from the equations as the kernels evaluate
 # them): distance of a pair 10 (differences, squared norm, root), density term 8
 # (Eq. density_sum), pressure + surface-tension term 30 (Eqs.
@@ -313,7 +315,7 @@ def run_gpu(args, wl, rank, world):
     e2e = {"value": job_rate(n, world, args.steps, e2e_s), "unit": METRIC,
            "h2d_bytes_per_step": (n * d * 8 + n) / args.steps, "d2h_bytes_per_step": (n * d * 8 + 128) / args.steps}
     info = dict(grid=r.grid(), stats=st, stats_e2e=st2, stage=dict(r.stage_info(), enabled=staged),
-                kernels_per_step=KERNELS_PER_STEP + (1 if staged else 0))
+                kernels_per_step=KERNELS_PER_STEP + (1 if staged else 0) + (1 if r.grid()["base"][-1] > SCAN_ONE_LEVEL else 0))
     r.close()
     out = dict(ms=ms, ms_step=ms_step, value=value, clocks=ck, phase_ms=phase_ms, e2e=e2e, info=info)
     if not args.no_extras and wl["precision"] == "fp32":

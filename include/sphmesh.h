@@ -115,7 +115,8 @@ typedef struct {
   double skin;           /* neighbour-list skin as a fraction of the support kappa h;
                             the list is rebuilt when a particle has moved half of it (results do
                             not depend on it). 0 -> each particle's own, from its last move (0.15 in
-                            3D, 0.2 in 2D before any); a given list_capacity keeps those for all */
+                            3D, 0.2 in 2D before any, and wherever a list does not fit otherwise); a
+                            given list_capacity keeps those for all */
 } sph_params;
 
 typedef struct {
